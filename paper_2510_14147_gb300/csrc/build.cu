@@ -1,15 +1,12 @@
 // build.cu -- cover-tree construction on the GPU (Algorithm 1 SplitVertex and
 // Algorithm 2 BuildLevel of the paper, Sec. IV-A).
 //
-// All hubs created in one round are split together.  One split iteration is
-// two launches over every hub of the round:
-//   k_hub_step      -- per hub: take the farthest point found by the previous
-//                      pass (largest D, lowest position on ties, as the strict
-//                      comparison of Algorithm 1 in scan order); stop the hub
-//                      once it lies within 2^(l-1), else make it the next centre;
-//   k_dist_update   -- per point of an active hub: d = d(p, newest centre);
-//                      if d < D[p] then D[p] = d, L[p] = new label (strict <);
-//                      then the hub's argmax of D by a packed 64-bit atomicMax.
+// All hubs created in one round are split together, in passes over every hub
+// of the round that each take a batch of centres (see k_net_update_l2):
+// farthest-first among the farthest points that the blocks of the pass report,
+// while they lie beyond 2^(l-1); every point keeps the distance D and the
+// label L of its nearest centre so far (strict <).  Small hubs (L2) are split
+// whole in one CTA each.
 // When every hub has stopped, the round's points are partitioned by
 // (hub, label) with a stable radix sort; each child's centre is moved to the
 // front of its range, its radius is the max of D over its range, and a child
@@ -24,6 +21,7 @@
 #include <cstdio>
 #include <memory>
 #include <mutex>
+#include <type_traits>
 #include <vector>
 #include <algorithm>
 
@@ -55,69 +53,55 @@ __device__ __forceinline__ float round_radius_up(float r, int metric) {
     return __fadd_ru(t, 0x1p-64f);
 }
 
-// ---- L2 distance of a point row to a centre row held in shared memory.
-// TPD threads cooperate on one distance; lane j reads float4s j, j+TPD, ...
-// The shuffles name only the TPD lanes of the caller's group, so groups of
-// one warp may take different branches around the call.
-template <int TPD>
-__device__ __forceinline__ float group_sqdist(const float4 *__restrict__ row, const float4 *cen,
-                                              int nq, int j) {
-    float acc = 0.f;
-#pragma unroll 4
-    for (int k = j; k < nq; k += TPD) {
-        float4 a = __ldg(row + k);
-        float4 b = cen[k];
-        float dx = a.x - b.x, dy = a.y - b.y, dz = a.z - b.z, dw = a.w - b.w;
-        acc = fmaf(dx, dx, acc);
-        acc = fmaf(dy, dy, acc);
-        acc = fmaf(dz, dz, acc);
-        acc = fmaf(dw, dw, acc);
-    }
-    const unsigned mask = TPD == 32 ? 0xffffffffu : (((1u << TPD) - 1u) << ((threadIdx.x & 31) & ~(TPD - 1)));
+// ---- L2 distances of a row held in registers.  TPD lanes share one row:
+// lane j holds its float4s j, j + TPD, ... (NV of them; NV = 0: rows too long
+// for registers, read again for every distance).  The other row comes from
+// shared or global memory.  Callers run whole warps converged.
+template <int TPD, int NV>
+struct RowRegs {
+    float4 v[NV ? NV : 1];
+    const float4 *row;
+    __device__ __forceinline__ void load(const float4 *r, int nq, int j) {
+        row = r;
 #pragma unroll
-    for (int o = TPD / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(mask, acc, o, TPD);
-    return acc;
-}
-
-constexpr int UPD_PASSES = 8;  // passes of a block over its chunk in k_dist_update_l2
-
-// The same distance with the row staged in shared memory by the calling lane
-// (lane j copied float4s j, j + TPD, ... and reads only those): the same
-// operations in the same order, so the same value.
-template <int TPD>
-__device__ __forceinline__ float group_sqdist_staged(const float4 *row, const float4 *cen, int nq, int j) {
-    float acc = 0.f;
-#pragma unroll 4
-    for (int k = j; k < nq; k += TPD) {
-        float4 a = row[k];
-        float4 b = cen[k];
-        float dx = a.x - b.x, dy = a.y - b.y, dz = a.z - b.z, dw = a.w - b.w;
-        acc = fmaf(dx, dx, acc);
-        acc = fmaf(dy, dy, acc);
-        acc = fmaf(dz, dz, acc);
-        acc = fmaf(dw, dw, acc);
+        for (int u = 0; u < NV; ++u) {
+            const int k = j + u * TPD;
+            v[u] = k < nq ? __ldg(r + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
     }
-    const unsigned mask = TPD == 32 ? 0xffffffffu : (((1u << TPD) - 1u) << ((threadIdx.x & 31) & ~(TPD - 1)));
+    __device__ __forceinline__ void zero() {
+        row = nullptr;
 #pragma unroll
-    for (int o = TPD / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(mask, acc, o, TPD);
-    return acc;
-}
-__device__ __forceinline__ void stage_copy16(void *smem, const void *gmem) {
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem));
-}
-__device__ __forceinline__ void stage_commit() { asm volatile("cp.async.commit_group;\n" ::); }
-template <int N>
-__device__ __forceinline__ void stage_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N)); }
-// Staged passes keep UPD_STAGES buffers of G rows in shared memory: the rows
-// of passes p + 1 and p + 2 are in flight while pass p is computed.
-constexpr int UPD_STAGES = 3;
-constexpr int UPD_STAGE_F4 = 1024;  // float4s of one buffer (G rows of nq float4s) that allow staging
+        for (int u = 0; u < NV; ++u) v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    // squared distance to `other`, the same in all TPD lanes
+    __device__ __forceinline__ float sqdist(const float4 *other, int nq, int j) const {
+        float acc = 0.f;
+        auto add = [&](const float4 a, const float4 b) {
+            const float dx = a.x - b.x, dy = a.y - b.y, dz = a.z - b.z, dw = a.w - b.w;
+            acc = fmaf(dx, dx, acc);
+            acc = fmaf(dy, dy, acc);
+            acc = fmaf(dz, dz, acc);
+            acc = fmaf(dw, dw, acc);
+        };
+        if (NV) {
+#pragma unroll
+            for (int u = 0; u < NV; ++u) {
+                const int k = j + u * TPD;
+                if (k < nq) add(v[u], other[k]);
+            }
+        } else if (row) {
+            for (int k = j; k < nq; k += TPD) add(__ldg(row + k), other[k]);
+        }
+#pragma unroll
+        for (int o = TPD / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o, TPD);
+        return acc;
+    }
+};
 
 struct Hubs {
-    int32_t *begin, *count, *node, *nc, *cur, *done, *level;
-    int32_t *flat;     // 1: the split stopped early and every child is a leaf block
-    int32_t *covered;  // points within the split threshold after the last pass (L2)
+    int32_t *begin, *count, *node, *nc, *m, *done, *level;
+    int32_t *flat;  // 1: the split stopped early and every child is a leaf block
     float *thr;
     unsigned long long *key;
 };
@@ -135,285 +119,588 @@ __device__ __forceinline__ bool flat_split(int nc, int covered) {
     return nc >= FLAT_MIN_CENTRES && covered <= nc + (nc >> 3);
 }
 
-// The next split step of a hub, taken inside the update pass by the hub's
-// last block to finish (its arrival completes the hub's count in `arrive`;
-// every other block of the hub has written its distances and its key by
-// then): k_hub_step for that hub, then k_centre_dists for its new centre.
-// One launch per split iteration instead of three; nothing waits -- the
-// blocks only count their arrivals.
-struct Step {
-    int32_t *arrive;      // per hub: blocks of the pass that have finished (reset by the last)
-    int32_t *active_out;  // hubs that took a new centre
-    int32_t *cpos;        // centre positions per hub label
-    float *dcc;           // distances of the new centre to the hub's centres (read by the pass, then rewritten)
+// ---- Splitting in batches of centres.
+//
+// A hub's split takes centres until every point lies within the threshold
+// 2^(l-1) of one.  Taken one at a time, the farthest point first, that is a
+// chain of as many dependent passes as the hub has children (1250 launches
+// for 121k uniform points in 16-D, 480 for 50k DNA strings, 700 a level for a
+// million 256-bit codes), each as long as a launch and a round trip to memory
+// (about 15 us) whatever its work.  Here a pass takes up to NET_M centres:
+//   update -- every point of the hub against the batch (its row is read
+//             once); each warp then reports its farthest point;
+//   select -- one CTA per hub reduces the reports to NET_C candidates and
+//             takes the next batch from them farthest-first: the first is the
+//             hub's farthest point, each next one the candidate farthest from
+//             every centre including those just taken, while above the
+//             threshold;
+//   dists  -- distances of the batch to the hub's centres, for the triangle-
+//             inequality test of the next update.
+// The centres are a net as before (pairwise farther apart than the threshold,
+// every point within it); only their order among near-equals differs.
+// Measured (build stage, before -> after): see k_net_update_l2.
+constexpr int NET_M = 32;    // centres of a batch
+constexpr int NET_C = 128;   // candidates of a selection
+constexpr int NET_KEYS = 8;  // farthest-point reports of a chunk
+
+// A chunk of a hub's points: {hub, first position, index of its reports}.
+struct Chunks {
+    const int4 *list;
+    int len;                     // points per chunk
+    unsigned long long *keys;    // NET_KEYS per chunk: (distance, position) of a part's farthest point
+    int32_t *cov;                // NET_KEYS per chunk: points of the part within the threshold
+};
+// The hub's batch: positions of its centres; their labels are nc - m ...
+struct Batch {
+    int32_t *pos;     // NET_M per listed hub
+    int32_t *cpos;    // centre positions by hub label (begin + label)
+    float *dcc;       // (begin + label) x NET_M: distance of the label's centre to the batch's centres
 };
 
 template <int TPD>
-__device__ __noinline__ void step_tail(const float *__restrict__ X, int dp, const int32_t *__restrict__ ids,
-                                       Hubs hb, int h, float4 *cen, Step st) {
-    __shared__ int s_act, s_nc, s_cur;
-    if (threadIdx.x == 0) {
-        const unsigned long long k = atomicAdd(&hb.key[h], 0ull);  // every block's maximum has landed
-        const float v = key_value(k);
-        const int covered = atomicExch(&hb.covered[h], 0);           // every block's count has landed
-        s_act = 0;
-        if (k == 0ull || !(v > hb.thr[h])) {
-            hb.done[h] = 1;
-        } else if (flat_split(hb.nc[h], covered)) {
-            hb.done[h] = 1;
-            hb.flat[h] = 1;
-        } else {
-            const int b = hb.begin[h], nc = hb.nc[h];
-            const int cur = (int32_t)key_pos(k);
-            hb.cur[h] = cur;
-            st.cpos[b] = b;  // label 0: the hub's own centre
-            st.cpos[b + nc] = cur;
-            hb.nc[h] = nc + 1;
-            hb.key[h] = 0ull;
-            atomicAdd(st.active_out, 1);
-            s_act = 1;
-            s_nc = nc + 1;
-            s_cur = cur;
-        }
-        st.arrive[h] = 0;
+constexpr int net_passes() { return TPD == 1 ? 1 : TPD == 2 ? 2 : 4; }
+
+// The farthest point and the number of covered points of a warp's points.
+__device__ __forceinline__ void net_report(unsigned long long best, int cov, const Chunks &ch, int slot) {
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long v = __shfl_xor_sync(0xffffffffu, best, o);
+        best = v > best ? v : best;
+        cov += __shfl_xor_sync(0xffffffffu, cov, o);
     }
-    __syncthreads();
-    if (!s_act) return;
-    const int b = hb.begin[h], nc = s_nc, nq = dp >> 2;
-    const float4 *crow = reinterpret_cast<const float4 *>(X + (size_t)ids[s_cur] * dp);
-    for (int i = threadIdx.x; i < nq; i += blockDim.x) cen[i] = crow[i];
-    __syncthreads();
-    constexpr int G = BT / TPD;
-    const int g = threadIdx.x / TPD, j = threadIdx.x % TPD;
-    // the row of label L (its centre's point id), the next step's loaded
-    // while this step's distance is computed
-    auto row_of = [&](int L) { return ids[st.cpos[b + (L < nc ? L : 0)]]; };
-    int rid = row_of(g);
-    for (int L0 = 0; L0 < nc; L0 += G) {  // every group runs the same number of steps
-        const int L = L0 + g;
-        const int nrid = L0 + G < nc ? row_of(L + G) : 0;
-        const float dd = sqrtf(group_sqdist<TPD>(reinterpret_cast<const float4 *>(X + (size_t)rid * dp), cen, nq, j));
-        if (L < nc && j == 0) st.dcc[b + L] = dd;
-        rid = nrid;
+    if ((threadIdx.x & 31) == 0) {
+        ch.keys[slot] = best;
+        ch.cov[slot] = cov;
     }
 }
 
-// Pruning (L2): a point labelled L cannot come closer to the new centre c
-// than D when d(c, centre L) >= 2 D (triangle inequality); such points keep D
-// and L without reading their row.  dcc[begin + L] = d(c, centre L) of the
-// hub (nullptr: no pruning).  STAGE: the rows of the chunk's passes are
-// copied into shared memory two passes ahead (cp.async), so that a group's
-// eight passes do not wait on memory one after another; otherwise each pass
-// reads its rows from global memory.
-template <int TPD, bool STAGE>
-__global__ void __launch_bounds__(BT, 4) k_dist_update_l2(
-    const float *__restrict__ X, int dp, const int32_t *__restrict__ ids, float *__restrict__ D,
-    int32_t *__restrict__ lab, const int32_t *__restrict__ chunk_hub,
-    const int32_t *__restrict__ chunk_start, int chunk_len, Hubs hb, const float *dcc, Step st) {
-    extern __shared__ float4 cen[];
-    int c = blockIdx.x;
-    int h = chunk_hub[c];
+// L2 update pass: TPD lanes per point, its row in registers, the batch's
+// centres in shared memory.  PRUNE: a point labelled L cannot come closer to
+// centre c than its distance D when d(c, centre L) >= 2 D (triangle
+// inequality, with a margin for the fp32 errors); each point computes only
+// the distances its mask leaves, and the row is not read when none is left.
+// The test costs one 128-byte read per point, so it pays for rows longer than
+// that (dp > 16); shorter rows compute every distance.  root: the first pass
+// (D infinite) also reduces the farthest point of all into *root.
+// Bound by the centres' shared-memory reads and the FP32 pipe where little is
+// pruned, by the latency of one chunk where the hub is small.
+// Build stage of 1M x 128 (mixture), 121k x 16 (uniform), 174k x 64 (mixture):
+// 18.6 / 22.7 / 9.6 ms with one centre per pass -> 10.6 / 3.5 / 4.0 ms.
+template <int TPD, int NV, bool PRUNE>
+__global__ void __launch_bounds__(BT) k_net_update_l2(const float *__restrict__ X, int dp,
+                                                      const int32_t *__restrict__ ids, float *__restrict__ D,
+                                                      int32_t *__restrict__ lab, Chunks ch, Hubs hb, Batch bt,
+                                                      const int32_t *__restrict__ hslot,
+                                                      unsigned long long *__restrict__ root) {
+    extern __shared__ float4 cen[];  // m x nq
+    constexpr int P = net_passes<TPD>(), G = BT / TPD;
+    const int4 ck = ch.list[blockIdx.x];
+    const int h = ck.x, start = ck.y;
     if (hb.done[h]) return;
-    int start = chunk_start[c];
-    const int hbeg = hb.begin[h];
-    int end = min(start + chunk_len, hbeg + hb.count[h]);
-    int cpos = hb.cur[h];
-    int lbl = hb.nc[h] - 1;
-    int nq = dp >> 2;
-    const float4 *crow = reinterpret_cast<const float4 *>(X + (size_t)ids[cpos] * dp);
-    for (int i = threadIdx.x; i < nq; i += blockDim.x) cen[i] = crow[i];
-    constexpr int G = BT / TPD;
-    int g = threadIdx.x / TPD, j = threadIdx.x % TPD;
-    // the chunk's passes (chunk_len = UPD_PASSES * G): distances, labels and
-    // ids of every pass first, then the pruning test, then the distances --
-    // three round trips to memory per chunk instead of three per pass
-    float cur[UPD_PASSES];
-    int lb[UPD_PASSES], pid[UPD_PASSES];
-    bool far[UPD_PASSES];
+    const int hbeg = hb.begin[h], m = hb.m[h], lbl0 = hb.nc[h] - m, nq = dp >> 2;
+    const int end = min(start + ch.len, hbeg + hb.count[h]);
+    const float thr = hb.thr[h];
+    const int32_t *bpos = bt.pos + (size_t)hslot[h] * NET_M;
+    for (int i = threadIdx.x; i < m * nq; i += BT) {
+        const int c = i / nq, k = i - c * nq;
+        cen[i] = __ldg(reinterpret_cast<const float4 *>(X + (size_t)ids[bpos[c]] * dp) + k);
+    }
+    const int g = threadIdx.x / TPD, j = threadIdx.x % TPD, lane = threadIdx.x & 31;
+    float cur[P];
+    int lb[P], pid[P];
+    unsigned mask[P];
 #pragma unroll
-    for (int p = 0; p < UPD_PASSES; ++p) {
+    for (int p = 0; p < P; ++p) {
         const int pos = start + p * G + g;
         const bool valid = pos < end;
         cur[p] = valid ? D[pos] : 0.f;
-        lb[p] = valid ? lab[pos] : 0;
+        lb[p] = valid && PRUNE ? lab[pos] : 0;
         pid[p] = valid ? ids[pos] : 0;
-        far[p] = !valid;
+        mask[p] = valid && m ? 0xffffffffu >> (32 - m) : 0u;
     }
-    if (dcc) {
+    if (PRUNE && m && !root) {
 #pragma unroll
-        for (int p = 0; p < UPD_PASSES; ++p)
-            if (!far[p]) far[p] = dcc[hbeg + lb[p]] >= 2.0f * cur[p] * (1.0f + 0x1p-12f) + 0x1p-60f;
-    }
-    // STAGE: buffer b holds G rows of nq float4s after the centre row; a lane
-    // copies (and later reads) only its own float4s of its group's row
-    float4 *stage = cen + nq;
-    auto issue = [&](int p) {
-        if (p < UPD_PASSES && !far[p]) {
-            const float4 *row = reinterpret_cast<const float4 *>(X + (size_t)pid[p] * dp);
-            float4 *dst = stage + ((size_t)(p % UPD_STAGES) * G + g) * nq;
-            for (int k = j; k < nq; k += TPD) stage_copy16(dst + k, row + k);
-        }
-        stage_commit();
-    };
-    if (STAGE) {
-        issue(0);
-        issue(1);
-    }
-    __syncthreads();  // the centre row
-    unsigned long long best = 0ull;
-#pragma unroll
-    for (int p = 0; p < UPD_PASSES; ++p) {
-        const int pos = start + p * G + g;
-        if (STAGE) issue(p + 2);
-        if (!far[p]) {  // the same for the group's TPD lanes
-            float s;
-            if (STAGE) {
-                stage_wait<UPD_STAGES - 1>();  // this lane's copies of pass p have landed
-                s = group_sqdist_staged<TPD>(stage + ((size_t)(p % UPD_STAGES) * G + g) * nq, cen, nq, j);
-            } else {
-                s = group_sqdist<TPD>(reinterpret_cast<const float4 *>(X + (size_t)pid[p] * dp), cen, nq, j);
+        for (int p = 0; p < P; ++p) {
+            if (!mask[p]) continue;
+            const float lim = 2.0f * cur[p] * (1.0f + 0x1p-12f) + 0x1p-60f;
+            const float4 *row = reinterpret_cast<const float4 *>(bt.dcc + (size_t)(hbeg + lb[p]) * NET_M);
+            unsigned near = 0u;
+            for (int q = j; 4 * q < m; q += TPD) {  // entries at and past m are masked out
+                const float4 d = row[q];
+                near |= ((d.x < lim ? 1u : 0u) | (d.y < lim ? 2u : 0u) | (d.z < lim ? 4u : 0u) |
+                         (d.w < lim ? 8u : 0u)) << (4 * q);
             }
-            if (j == 0) {
-                float d = sqrtf(s);
-                if (d < cur[p]) {
+            mask[p] &= near;  // this lane's part; the group's parts are combined below
+        }
+#pragma unroll
+        for (int p = 0; p < P; ++p)
+#pragma unroll
+            for (int o = TPD / 2; o > 0; o >>= 1) mask[p] |= __shfl_xor_sync(0xffffffffu, mask[p], o, TPD);
+    }
+    __syncthreads();  // the centres
+    unsigned long long best = 0ull;
+    int cov = 0;
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+        const int pos = start + p * G + g;
+        unsigned mk = mask[p];
+        if (__any_sync(0xffffffffu, mk != 0u)) {
+            RowRegs<TPD, NV> r;
+            if (mk) r.load(reinterpret_cast<const float4 *>(X + (size_t)pid[p] * dp), nq, j);
+            else r.zero();
+            float sb = INFINITY;
+            int ib = 0;
+            if (PRUNE) {
+                do {  // each group its next centre
+                    const int i = mk ? __ffs(mk) - 1 : 0;
+                    const float s = r.sqdist(cen + i * nq, nq, j);
+                    if (mk && s < sb) {
+                        sb = s;
+                        ib = i;
+                    }
+                    mk &= mk - 1u;
+                } while (__any_sync(0xffffffffu, mk != 0u));
+            } else {
+                for (int i = 0; i < m; ++i) {
+                    const float s = r.sqdist(cen + i * nq, nq, j);
+                    if (s < sb) {
+                        sb = s;
+                        ib = i;
+                    }
+                }
+                if (!mk) sb = INFINITY;
+            }
+            const float d = sqrtf(sb);
+            if (d < cur[p]) {
+                cur[p] = d;
+                if (j == 0) {
                     D[pos] = d;
-                    lab[pos] = lbl;
-                    cur[p] = d;
+                    lab[pos] = lbl0 + ib;
                 }
             }
         }
         if (pos < end && j == 0) {
-            unsigned long long k = pack_max_key(cur[p], (uint32_t)pos);
+            const unsigned long long k = pack_max_key(cur[p], (uint32_t)pos);
             best = k > best ? k : best;
+            cov += cur[p] <= thr;
         }
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        unsigned long long v = __shfl_xor_sync(0xffffffffu, best, o);
-        best = v > best ? v : best;
+    net_report(best, cov, ch, ck.z * NET_KEYS + (threadIdx.x >> 5));
+    if (root) {
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long v = __shfl_xor_sync(0xffffffffu, best, o);
+            best = v > best ? v : best;
+        }
+        if (lane == 0) atomicMax(root, best);
     }
-    // points now within the split threshold (the flat-split test)
-    const float thr = hb.thr[h];
+}
+
+// Reduces the reports of a hub's chunks to at most C candidates above the
+// threshold (slot s: the farthest of the reports s, s + C, ...), in cd / cp
+// (distance, position); returns their number, and the hub's covered points in
+// *covered.  Called by a whole block of at least C threads; ends with a barrier.
+template <int C>
+__device__ __forceinline__ int net_candidates(const Chunks &ch, int64_t first, int n_rep, float thr, float *cd,
+                                              int32_t *cp, int *covered) {
+    __shared__ unsigned long long slot[C];
+    __shared__ int s_n[C / 32], s_cov[32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    for (int i = threadIdx.x; i < C; i += blockDim.x) slot[i] = 0ull;
+    __syncthreads();
     int cov = 0;
-#pragma unroll
-    for (int p = 0; p < UPD_PASSES; ++p) cov += (j == 0 && start + p * G + g < end && cur[p] <= thr) ? 1 : 0;
+    unsigned long long best = 0ull;  // blockDim.x is a multiple of C: a thread's reports share a slot
+    for (int i = threadIdx.x; i < n_rep; i += blockDim.x) {
+        const unsigned long long k = ch.keys[first + i];
+        best = k > best ? k : best;
+        cov += ch.cov[first + i];
+    }
+    if (best && key_value(best) > thr) atomicMax(&slot[threadIdx.x % C], best);
     for (int o = 16; o > 0; o >>= 1) cov += __shfl_xor_sync(0xffffffffu, cov, o);
-    // the block's maximum key and count go to the hub in one atomic each (a
-    // block's chunk lies in one hub); then, with pruning, the block arrives
-    // and the hub's last block takes its next step
-    __shared__ unsigned long long s_best[BT / 32];
-    __shared__ int s_cov[BT / 32];
-    __shared__ int s_last;
-    if ((threadIdx.x & 31) == 0) {
-        s_best[threadIdx.x >> 5] = best;
-        s_cov[threadIdx.x >> 5] = cov;
-    }
-    if (st.arrive) __threadfence();  // this thread's D and lab writes, before the block's arrival
+    if (lane == 0) s_cov[w] = cov;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long bk = 0ull;
-        int bc = 0;
+    unsigned long long k = 0ull;
+    unsigned bal = 0u;
+    if (threadIdx.x < C) {
+        k = slot[threadIdx.x];
+        bal = __ballot_sync(0xffffffffu, k != 0ull);
+        if (lane == 0) s_n[w] = __popc(bal);
+    }
+    __syncthreads();
+    int total = 0, base = 0;
 #pragma unroll
-        for (int w = 0; w < BT / 32; ++w) {
-            bk = s_best[w] > bk ? s_best[w] : bk;
-            bc += s_cov[w];
-        }
-        if (bk) atomicMax(&hb.key[h], bk);
-        if (bc) atomicAdd(&hb.covered[h], bc);
-        if (st.arrive) {
-            __threadfence();  // the key and the count, before the arrival
-            const int blocks = (hb.count[h] + chunk_len - 1) / chunk_len;  // all of the hub's chunks run
-            s_last = atomicAdd(&st.arrive[h], 1) == blocks - 1;
-        }
+    for (int i = 0; i < C / 32; ++i) {
+        if (i < w) base += s_n[i];
+        total += s_n[i];
     }
-    if (st.arrive) {
-        __syncthreads();
-        if (s_last) {
-            __threadfence();
-            step_tail<TPD>(X, dp, ids, hb, h, cen, st);
-        }
+    if (k) {
+        const int at = base + __popc(bal & lanemask_lt());
+        cd[at] = key_value(k);
+        cp[at] = (int32_t)key_pos(k);
     }
+    int c = 0;
+    for (int i = 0; i < nw; ++i) c += s_cov[i];
+    *covered = c;
+    __syncthreads();
+    return total;
 }
 
-// The hub step's decision in the hub's last block (thread 0; every block's
-// key and count have landed): the next centre from the hub's largest key, or
-// the hub is done (nothing above the split threshold, or a flat split where
-// `flat_check`).  The same decision as k_hub_step.
-__device__ __forceinline__ void step_decide(Hubs hb, int h, Step st, bool flat_check) {
-    const unsigned long long k = atomicAdd(&hb.key[h], 0ull);
-    const float v = key_value(k);
-    const int covered = atomicExch(&hb.covered[h], 0);
-    if (k == 0ull || !(v > hb.thr[h])) {
-        hb.done[h] = 1;
-    } else if (flat_check && flat_split(hb.nc[h], covered)) {
-        hb.done[h] = 1;
-        hb.flat[h] = 1;
-    } else {
-        hb.cur[h] = (int32_t)key_pos(k);
-        hb.nc[h] += 1;
-        hb.key[h] = 0ull;
-        atomicAdd(st.active_out, 1);
-    }
-    st.arrive[h] = 0;
-}
-
-// A block's arrival at the end of an update pass (its writes and atomics
-// fenced first): true in every thread of the hub's last block to arrive.
-__device__ __forceinline__ bool last_to_arrive(Step st, int h, int blocks) {
-    __shared__ int s_last;
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) s_last = atomicAdd(&st.arrive[h], 1) == blocks - 1;
-    __syncthreads();
-    if (s_last) __threadfence();
-    return s_last;
-}
-
-// Edit distance: one thread per point; the newest centre is the pattern of
-// the bit-parallel recurrence, its match masks in shared memory.
-template <int W>
-__global__ void __launch_bounds__(BT) k_dist_update_lev(
-    const uint8_t *__restrict__ S, const int64_t *__restrict__ off, const int32_t *__restrict__ ids,
-    float *__restrict__ D, int32_t *__restrict__ lab, const int32_t *__restrict__ chunk_hub,
-    const int32_t *__restrict__ chunk_start, int chunk_len, Hubs hb, Step st) {
-    __shared__ uint64_t peq[256 * W];
-    int c = blockIdx.x;
-    int h = chunk_hub[c];
-    if (hb.done[h]) return;
-    int start = chunk_start[c];
-    int end = min(start + chunk_len, hb.begin[h] + hb.count[h]);
-    int cid = ids[hb.cur[h]];
-    int lbl = hb.nc[h] - 1;
-    const uint8_t *pat = S + off[cid];
-    int m = (int)(off[cid + 1] - off[cid]);
-    lev_build_peq<W>(peq, pat, m);
-    __syncthreads();
+// The farthest of n candidates (lowest index among equals) as (distance bits,
+// ~index); every warp computes it for itself.
+__device__ __forceinline__ unsigned long long net_farthest(const float *cd, int n) {
     unsigned long long best = 0ull;
-    for (int base = start; base < end; base += blockDim.x) {
-        int pos = base + threadIdx.x;
-        if (pos < end) {
-            int id = ids[pos];
-            const uint8_t *txt = S + off[id];
-            int n = (int)(off[id + 1] - off[id]);
-            float cur = D[pos];
-            int cutoff = isinf(cur) ? INT_MAX / 2 : (int)cur - 1;
-            int d = lev_myers<W>(peq, m, txt, n, cutoff);
-            if (d <= cutoff && (float)d < cur) {
-                D[pos] = (float)d;
-                lab[pos] = lbl;
-                cur = (float)d;
-            }
-            unsigned long long k = pack_max_key(cur, (uint32_t)pos);
-            best = k > best ? k : best;
-        }
+    for (int i = threadIdx.x & 31; i < n; i += 32) {
+        const unsigned long long k = pack_max_key(cd[i], (uint32_t)i);
+        best = k > best ? k : best;
     }
+#pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-        unsigned long long v = __shfl_xor_sync(0xffffffffu, best, o);
+        const unsigned long long v = __shfl_xor_sync(0xffffffffu, best, o);
         best = v > best ? v : best;
     }
-    if ((threadIdx.x & 31) == 0 && best) atomicMax(&hb.key[h], best);
-    if (st.arrive) {  // the hub's last block takes its next step (no flat-split test: no counts here)
-        const int blocks = (hb.count[h] + chunk_len - 1) / chunk_len;  // all of the hub's chunks run
-        if (last_to_arrive(st, h, blocks) && threadIdx.x == 0) step_decide(hb, h, st, false);
+    return best;
+}
+
+// A hub's batch taken (thread 0): m centres after the nc it had, or done.
+__device__ __forceinline__ void net_take(Hubs hb, int h, int m, bool flat, int32_t *active) {
+    hb.m[h] = m;
+    hb.nc[h] += m;
+    if (m == 0) hb.done[h] = 1;
+    if (flat) hb.flat[h] = 1;
+    if (m) atomicAdd(active, 1);
+}
+
+// The next batch of a hub (one CTA per listed hub {hub, slot}).  The
+// candidates' rows are staged in shared memory where they fit.
+template <int TPD>
+__global__ void __launch_bounds__(BT) k_net_select_l2(const float *__restrict__ X, int dp,
+                                                      const int32_t *__restrict__ ids, const int2 *__restrict__ hlist,
+                                                      Hubs hb, const int64_t *__restrict__ coff, Chunks ch, Batch bt,
+                                                      int mcap, int staged, int32_t *__restrict__ active) {
+    extern __shared__ float4 rows[];  // NET_C x nq if staged
+    __shared__ float cd[NET_C];
+    __shared__ int32_t cp[NET_C];
+    const int2 hs = hlist[blockIdx.x];
+    const int h = hs.x;
+    if (hb.done[h]) return;
+    const int b = hb.begin[h], nc = hb.nc[h], nq = dp >> 2;
+    const float thr = hb.thr[h];
+    const int n_rep = (hb.count[h] + ch.len - 1) / ch.len * NET_KEYS;
+    int covered;
+    const int n = net_candidates<NET_C>(ch, coff[hs.y] * NET_KEYS, n_rep, thr, cd, cp, &covered);
+    const bool flat = n > 0 && flat_split(nc, covered);
+    if (n == 0 || flat) {
+        if (threadIdx.x == 0) net_take(hb, h, 0, flat, active);
+        return;
+    }
+    if (staged) {
+        for (int i = threadIdx.x; i < n * nq; i += BT) {
+            const int c = i / nq, k = i - c * nq;
+            rows[i] = __ldg(reinterpret_cast<const float4 *>(X + (size_t)ids[cp[c]] * dp) + k);
+        }
+        __syncthreads();
+    }
+    auto row_of = [&](int c) -> const float4 * {
+        return staged ? rows + c * nq : reinterpret_cast<const float4 *>(X + (size_t)ids[cp[c]] * dp);
+    };
+    constexpr int G = BT / TPD;
+    const int g = threadIdx.x / TPD, j = threadIdx.x % TPD;
+    int m = 0;
+    while (m < mcap) {
+        const unsigned long long f = net_farthest(cd, n);
+        if (!(key_value(f) > thr)) break;
+        const int pick = (int)key_pos(f);
+        if (threadIdx.x == 0) {
+            bt.pos[(size_t)hs.y * NET_M + m] = cp[pick];
+            bt.cpos[b + nc + m] = cp[pick];
+        }
+        ++m;
+        __syncthreads();  // every warp has read cd
+        const float4 *pr = row_of(pick);
+        for (int c0 = 0; c0 < n; c0 += G) {
+            const int c = c0 + g;
+            float acc = 0.f;
+            if (c < n) {
+                const float4 *cr = row_of(c);
+#pragma unroll 4
+                for (int k = j; k < nq; k += TPD) {
+                    const float4 x = pr[k], y = cr[k];
+                    const float dx = x.x - y.x, dy = x.y - y.y, dz = x.z - y.z, dw = x.w - y.w;
+                    acc = fmaf(dx, dx, acc);
+                    acc = fmaf(dy, dy, acc);
+                    acc = fmaf(dz, dz, acc);
+                    acc = fmaf(dw, dw, acc);
+                }
+            }
+#pragma unroll
+            for (int o = TPD / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o, TPD);
+            if (c < n && j == 0) cd[c] = fminf(cd[c], sqrtf(acc));
+        }
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        if (nc == 1) bt.cpos[b] = b;  // label 0: the hub's own centre
+        net_take(hb, h, m, false, active);
+    }
+}
+
+// Distances of a hub's centres (labels below nc) to its new batch: blocks
+// (hub, y) over the labels, TPD lanes per label.
+template <int TPD, int NV>
+__global__ void __launch_bounds__(BT) k_net_dists_l2(const float *__restrict__ X, int dp,
+                                                     const int32_t *__restrict__ ids, const int2 *__restrict__ hlist,
+                                                     Hubs hb, Batch bt) {
+    extern __shared__ float4 cen[];  // m x nq
+    const int2 hs = hlist[blockIdx.x];
+    const int h = hs.x;
+    if (hb.done[h]) return;
+    const int b = hb.begin[h], nc = hb.nc[h], m = hb.m[h], nq = dp >> 2;
+    constexpr int G = BT / TPD;
+    if ((int)blockIdx.y * G >= nc) return;
+    const int32_t *bpos = bt.pos + (size_t)hs.y * NET_M;
+    for (int i = threadIdx.x; i < m * nq; i += BT) {
+        const int c = i / nq, k = i - c * nq;
+        cen[i] = __ldg(reinterpret_cast<const float4 *>(X + (size_t)ids[bpos[c]] * dp) + k);
+    }
+    __syncthreads();
+    const int g = threadIdx.x / TPD, j = threadIdx.x % TPD;
+    for (int L0 = blockIdx.y * G; L0 < nc; L0 += gridDim.y * G) {  // the same number of steps in every group
+        const int L = L0 + g;
+        RowRegs<TPD, NV> r;
+        r.load(reinterpret_cast<const float4 *>(X + (size_t)ids[bt.cpos[b + min(L, nc - 1)]] * dp), nq, j);
+        float *out = bt.dcc + (size_t)(b + L) * NET_M;
+        for (int i = 0; i < m; ++i) {
+            const float s = r.sqdist(cen + i * nq, nq, j);
+            if (L < nc && j == 0) out[i] = sqrtf(s);
+        }
+    }
+}
+
+// ---- Edit distance: the same passes.  Strings are re-coded to the A bytes
+// that occur (match masks of A entries), and each update block compacts the
+// (point, centre) pairs that the triangle inequality leaves, so that its
+// threads run the recurrence on full warps.
+constexpr int LEV_P = 64;     // points per chunk
+constexpr int LEV_C = 64;     // candidates of a selection
+
+__global__ void k_present(const uint8_t *__restrict__ s, int64_t nbytes, int32_t *__restrict__ present) {
+    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < nbytes) present[s[i]] = 1;
+}
+// code[byte] = its rank among the bytes that occur; *A = their number.
+__global__ void k_codes(const int32_t *__restrict__ present, uint8_t *__restrict__ code, int32_t *__restrict__ A) {
+    __shared__ int s_w[8];
+    const int t = threadIdx.x, lane = t & 31;
+    const bool p = present[t] != 0;
+    const unsigned bal = __ballot_sync(0xffffffffu, p);
+    if (lane == 0) s_w[t >> 5] = __popc(bal);
+    __syncthreads();
+    int base = 0, total = 0;
+    for (int w = 0; w < 8; ++w) {
+        if (w < (t >> 5)) base += s_w[w];
+        total += s_w[w];
+    }
+    code[t] = (uint8_t)(p ? base + __popc(bal & lanemask_lt()) : 0);
+    if (t == 0) *A = total;
+}
+__global__ void k_recode(const uint8_t *__restrict__ s, int64_t nbytes, const uint8_t *__restrict__ code,
+                         uint8_t *__restrict__ out) {
+    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < nbytes) out[i] = code[s[i]];
+}
+
+struct Strings {
+    const uint8_t *s;    // codes below A
+    const int64_t *off;
+    int A;
+};
+
+// Match masks of one string over A codes, by the whole block (barriers inside).
+template <int W>
+__device__ __forceinline__ void lev_masks(uint64_t *peq, const uint8_t *pat, int m, int A) {
+    for (int i = threadIdx.x; i < A * W; i += blockDim.x) peq[i] = 0ull;
+    __syncthreads();
+    for (int i = threadIdx.x; i < m; i += blockDim.x)
+        atomicOr((unsigned long long *)&peq[pat[i] * W + (i >> 6)], 1ull << (i & 63));
+    __syncthreads();
+}
+
+template <int W>
+__global__ void __launch_bounds__(BT) k_net_update_lev(Strings S, const int32_t *__restrict__ ids,
+                                                       float *__restrict__ D, int32_t *__restrict__ lab, Chunks ch,
+                                                       Hubs hb, Batch bt, const int32_t *__restrict__ hslot, int prune,
+                                                       unsigned long long *__restrict__ root) {
+    extern __shared__ uint64_t speq[];  // m x A x W
+    __shared__ int sd[LEV_P], sid[LEV_P], clen[NET_M];
+    __shared__ unsigned skey[LEV_P];    // (distance << 8) | centre of the point's best so far
+    __shared__ uint16_t pairs[LEV_P * NET_M];
+    __shared__ int s_n;
+    const int4 ck = ch.list[blockIdx.x];
+    const int h = ck.x, start = ck.y;
+    if (hb.done[h]) return;
+    const int hbeg = hb.begin[h], m = hb.m[h], lbl0 = hb.nc[h] - m;
+    const int np = min(ch.len, hbeg + hb.count[h] - start);
+    const int32_t *bpos = bt.pos + (size_t)hslot[h] * NET_M;
+    const int t = threadIdx.x;
+    for (int i = t; i < m * S.A * W; i += BT) speq[i] = 0ull;
+    float cur = 0.f;
+    if (t < LEV_P) {
+        if (t < np) {
+            cur = D[start + t];
+            sid[t] = ids[start + t];
+        }
+        sd[t] = isinf(cur) ? INT_MAX / 4 : (int)cur;
+        skey[t] = 0xffffffffu;
+    }
+    if (t < m) {
+        const int c = ids[bpos[t]];
+        clen[t] = (int)(S.off[c + 1] - S.off[c]);
+    }
+    if (t == 0) s_n = 0;
+    __syncthreads();
+    for (int c = 0; c < m; ++c) {
+        const uint8_t *pat = S.s + S.off[ids[bpos[c]]];
+        for (int i = t; i < clen[c]; i += BT)
+            atomicOr((unsigned long long *)&speq[((size_t)c * S.A + pat[i]) * W + (i >> 6)], 1ull << (i & 63));
+    }
+    // the pairs left by the triangle inequality: d(c, p) >= d(c, centre of p) - D(p)
+    for (int i0 = 0; i0 < m * LEV_P; i0 += BT) {
+        const int i = i0 + t, c = i / LEV_P, p = i % LEV_P;
+        bool keep = c < m && p < np;
+        if (keep && prune)
+            keep = bt.dcc[(size_t)(hbeg + lab[start + p]) * NET_M + c] < 2.0f * (float)sd[p];
+        const unsigned bal = __ballot_sync(0xffffffffu, keep);
+        int base = 0;
+        if ((t & 31) == 0 && bal) base = atomicAdd(&s_n, __popc(bal));
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (keep) pairs[base + __popc(bal & lanemask_lt())] = (uint16_t)(c * LEV_P + p);
+    }
+    __syncthreads();
+    const int n = s_n;
+    for (int i = t; i < n; i += BT) {
+        const int c = pairs[i] / LEV_P, p = pairs[i] % LEV_P;
+        const int id = sid[p];
+        // a distance above the best so far cannot win; an equal one wins by its lower centre
+        const unsigned seen = *(volatile unsigned *)&skey[p];
+        const int k = min(sd[p] - 1, (int)(seen >> 8));
+        const int d = lev_myers<W>(speq + (size_t)c * S.A * W, clen[c], S.s + S.off[id],
+                                   (int)(S.off[id + 1] - S.off[id]), k);
+        if (d <= k) atomicMin(&skey[p], ((unsigned)d << 8) | (unsigned)c);
+    }
+    __syncthreads();
+    if (t < LEV_P) {  // two warps: reports of eight points each
+        unsigned long long best = 0ull;
+        if (t < np) {
+            const unsigned k = skey[t];
+            if (k != 0xffffffffu) {
+                cur = (float)(k >> 8);
+                D[start + t] = cur;
+                lab[start + t] = lbl0 + (int)(k & 255u);
+            }
+            best = pack_max_key(cur, (uint32_t)(start + t));
+        }
+#pragma unroll
+        for (int o = LEV_P / NET_KEYS / 2; o > 0; o >>= 1) {
+            const unsigned long long v = __shfl_xor_sync(0xffffffffu, best, o);
+            best = v > best ? v : best;
+        }
+        if (t % (LEV_P / NET_KEYS) == 0) {
+            ch.keys[ck.z * NET_KEYS + t / (LEV_P / NET_KEYS)] = best;
+            ch.cov[ck.z * NET_KEYS + t / (LEV_P / NET_KEYS)] = 0;  // no flat-split test for edit distance
+            if (root) atomicMax(root, best);
+        }
+    }
+}
+
+// Selection in three launches: the candidates, all their mutual distances
+// (one block per candidate: a distance takes tens of microseconds, so they
+// are not left to the picks' chain), and the picks.
+struct LevCands {
+    int32_t *n;          // per listed hub
+    float *d;            // LEV_C per listed hub
+    int32_t *pos;
+    uint16_t *pair;      // LEV_C x LEV_C per listed hub
+};
+__global__ void __launch_bounds__(BT) k_net_cands_lev(const int2 *__restrict__ hlist, Hubs hb,
+                                                      const int64_t *__restrict__ coff, Chunks ch, LevCands lc) {
+    __shared__ float cd[LEV_C];
+    __shared__ int32_t cp[LEV_C];
+    const int2 hs = hlist[blockIdx.x];
+    if (hb.done[hs.x]) return;
+    const int n_rep = (hb.count[hs.x] + ch.len - 1) / ch.len * NET_KEYS;
+    int covered;
+    const int n = net_candidates<LEV_C>(ch, coff[hs.y] * NET_KEYS, n_rep, hb.thr[hs.x], cd, cp, &covered);
+    if (threadIdx.x < n) {
+        lc.d[(size_t)blockIdx.x * LEV_C + threadIdx.x] = cd[threadIdx.x];
+        lc.pos[(size_t)blockIdx.x * LEV_C + threadIdx.x] = cp[threadIdx.x];
+    }
+    if (threadIdx.x == 0) lc.n[blockIdx.x] = n;
+}
+template <int W>
+__global__ void __launch_bounds__(LEV_C) k_net_pairs_lev(Strings S, const int32_t *__restrict__ ids,
+                                                         const int2 *__restrict__ hlist, Hubs hb, LevCands lc) {
+    extern __shared__ uint64_t speq[];  // A x W
+    const int i = blockIdx.x, a = blockIdx.y, t = threadIdx.x;
+    if (hb.done[hlist[i].x]) return;
+    const int n = lc.n[i];
+    if (a >= n) return;
+    const int32_t *pos = lc.pos + (size_t)i * LEV_C;
+    const int ia = ids[pos[a]];
+    const int la = (int)(S.off[ia + 1] - S.off[ia]);
+    lev_masks<W>(speq, S.s + S.off[ia], la, S.A);
+    if (t < n && t >= a) {
+        const int ib = ids[pos[t]];
+        const int d = t == a ? 0 : lev_myers<W>(speq, la, S.s + S.off[ib], (int)(S.off[ib + 1] - S.off[ib]), INT_MAX / 2);
+        uint16_t *pr = lc.pair + (size_t)i * LEV_C * LEV_C;
+        pr[a * LEV_C + t] = (uint16_t)d;
+        pr[t * LEV_C + a] = (uint16_t)d;
+    }
+}
+__global__ void __launch_bounds__(32) k_net_pick_lev(const int2 *__restrict__ hlist, Hubs hb, Batch bt, LevCands lc,
+                                                     int mcap, int32_t *__restrict__ active) {
+    __shared__ float cd[LEV_C];
+    const int2 hs = hlist[blockIdx.x];
+    const int h = hs.x, lane = threadIdx.x;
+    if (hb.done[h]) return;
+    const int n = lc.n[blockIdx.x], b = hb.begin[h], nc = hb.nc[h];
+    const float thr = hb.thr[h];
+    const size_t o = (size_t)blockIdx.x * LEV_C;
+    for (int i = lane; i < n; i += 32) cd[i] = lc.d[o + i];
+    __syncwarp();
+    int m = 0;
+    while (m < mcap && n) {
+        const unsigned long long f = net_farthest(cd, n);
+        if (!(key_value(f) > thr)) break;
+        const int pick = (int)key_pos(f);
+        if (lane == 0) {
+            bt.pos[(size_t)hs.y * NET_M + m] = lc.pos[o + pick];
+            bt.cpos[b + nc + m] = lc.pos[o + pick];
+        }
+        ++m;
+        __syncwarp();
+        const uint16_t *pr = lc.pair + (o + pick) * LEV_C;
+        for (int i = lane; i < n; i += 32) cd[i] = fminf(cd[i], (float)pr[i]);
+        __syncwarp();
+    }
+    if (lane == 0) {
+        if (nc == 1) bt.cpos[b] = b;  // label 0: the hub's own centre
+        net_take(hb, h, m, false, active);
+    }
+}
+// Distances of a hub's centres to its new batch: block (hub, batch centre).
+template <int W>
+__global__ void __launch_bounds__(128) k_net_dists_lev(Strings S, const int32_t *__restrict__ ids,
+                                                       const int2 *__restrict__ hlist, Hubs hb, Batch bt) {
+    extern __shared__ uint64_t speq[];  // A x W
+    const int2 hs = hlist[blockIdx.x];
+    const int h = hs.x, c = blockIdx.y;
+    if (hb.done[h] || c >= hb.m[h]) return;
+    const int b = hb.begin[h], nc = hb.nc[h];
+    const int id = ids[bt.pos[(size_t)hs.y * NET_M + c]];
+    const int m = (int)(S.off[id + 1] - S.off[id]);
+    lev_masks<W>(speq, S.s + S.off[id], m, S.A);
+    for (int L = threadIdx.x; L < nc; L += blockDim.x) {
+        const int il = ids[bt.cpos[b + L]];
+        bt.dcc[(size_t)(b + L) * NET_M + c] =
+            (float)lev_myers<W>(speq, m, S.s + S.off[il], (int)(S.off[il + 1] - S.off[il]), INT_MAX / 2);
     }
 }
 
@@ -447,54 +734,111 @@ __global__ void k_pack_bits(const uint8_t *__restrict__ src, int64_t n, int dim,
     dst[i] = v;
 }
 
-// Hamming: one thread per point against the newest centre (its row in shared
-// memory); also counts the hub's points within the split threshold.
-__global__ void __launch_bounds__(BT) k_dist_update_ham(
-    const uint32_t *__restrict__ X, int wp, const int32_t *__restrict__ ids, float *__restrict__ D,
-    int32_t *__restrict__ lab, const int32_t *__restrict__ chunk_hub, const int32_t *__restrict__ chunk_start,
-    int chunk_len, Hubs hb, Step st) {
-    extern __shared__ uint4 hcen[];
-    const int c = blockIdx.x;
-    const int h = chunk_hub[c];
+// Hamming update pass: one thread per point, its row in registers (NQ 16-byte
+// pieces; 0: longer rows, read again for every centre), the batch's centres in
+// shared memory.  A distance is a few population counts, so nothing is pruned.
+template <int NQ>
+__global__ void __launch_bounds__(BT) k_net_update_ham(const uint32_t *__restrict__ X, int wp,
+                                                       const int32_t *__restrict__ ids, float *__restrict__ D,
+                                                       int32_t *__restrict__ lab, Chunks ch, Hubs hb, Batch bt,
+                                                       const int32_t *__restrict__ hslot,
+                                                       unsigned long long *__restrict__ root) {
+    extern __shared__ uint4 hcen[];  // m x nq
+    const int4 ck = ch.list[blockIdx.x];
+    const int h = ck.x, start = ck.y;
     if (hb.done[h]) return;
-    const int start = chunk_start[c];
-    const int end = min(start + chunk_len, hb.begin[h] + hb.count[h]);
-    const int nq = wp >> 2;
-    const uint4 *crow = reinterpret_cast<const uint4 *>(X + (size_t)ids[hb.cur[h]] * wp);
-    for (int i = threadIdx.x; i < nq; i += blockDim.x) hcen[i] = crow[i];
+    const int hbeg = hb.begin[h], m = hb.m[h], lbl0 = hb.nc[h] - m, nq = NQ ? NQ : wp >> 2;
+    const int end = min(start + ch.len, hbeg + hb.count[h]);
+    const int32_t *bpos = bt.pos + (size_t)hslot[h] * NET_M;
+    for (int i = threadIdx.x; i < m * nq; i += BT) {
+        const int c = i / nq, k = i - c * nq;
+        hcen[i] = reinterpret_cast<const uint4 *>(X + (size_t)ids[bpos[c]] * wp)[k];
+    }
+    const int pos = start + threadIdx.x;  // ch.len = BT
+    const bool valid = pos < end;
+    float cur = valid ? D[pos] : 0.f;
+    const uint4 *row = reinterpret_cast<const uint4 *>(X + (size_t)(valid ? ids[pos] : 0) * wp);
+    uint4 v[NQ ? NQ : 1];
+#pragma unroll
+    for (int k = 0; k < NQ; ++k) v[k] = m ? __ldg(row + k) : make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
-    const int lbl = hb.nc[h] - 1;
-    const float thr = hb.thr[h];
-    unsigned long long best = 0ull;
-    int cov = 0;
-    for (int base = start; base < end; base += blockDim.x) {
-        const int pos = base + threadIdx.x;
-        if (pos < end) {
-            float cur = D[pos];
-            const int d = ham_dist4(reinterpret_cast<const uint4 *>(X + (size_t)ids[pos] * wp), hcen, nq);
-            if ((float)d < cur) {
-                D[pos] = (float)d;
-                lab[pos] = lbl;
-                cur = (float)d;
+    int db = INT_MAX, ib = 0;
+    for (int c = 0; c < m; ++c) {
+        int d = 0;
+        if (NQ) {
+#pragma unroll
+            for (int k = 0; k < NQ; ++k) {
+                const uint4 y = hcen[c * nq + k];
+                d += __popc(v[k].x ^ y.x) + __popc(v[k].y ^ y.y) + __popc(v[k].z ^ y.z) + __popc(v[k].w ^ y.w);
             }
-            cov += cur <= thr;
-            const unsigned long long k = pack_max_key(cur, (uint32_t)pos);
-            best = k > best ? k : best;
+        } else {
+            d = ham_dist4(row, hcen + c * nq, nq);
+        }
+        if (d < db) {
+            db = d;
+            ib = c;
         }
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long v = __shfl_xor_sync(0xffffffffu, best, o);
-        best = v > best ? v : best;
-        cov += __shfl_xor_sync(0xffffffffu, cov, o);
+    unsigned long long best = 0ull;
+    int cov = 0;
+    if (valid) {
+        if (m && (float)db < cur) {
+            cur = (float)db;
+            D[pos] = cur;
+            lab[pos] = lbl0 + ib;
+        }
+        best = pack_max_key(cur, (uint32_t)pos);
+        cov = cur <= hb.thr[h];
     }
-    if ((threadIdx.x & 31) == 0) {
-        if (best) atomicMax(&hb.key[h], best);
-        if (cov) atomicAdd(&hb.covered[h], cov);
+    net_report(best, cov, ch, ck.z * NET_KEYS + (threadIdx.x >> 5));
+    if (root) {
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long k = __shfl_xor_sync(0xffffffffu, best, o);
+            best = k > best ? k : best;
+        }
+        if ((threadIdx.x & 31) == 0) atomicMax(root, best);
     }
-    if (st.arrive) {  // the hub's last block takes its next step
-        const int blocks = (hb.count[h] + chunk_len - 1) / chunk_len;  // all of the hub's chunks run
-        if (last_to_arrive(st, h, blocks) && threadIdx.x == 0) step_decide(hb, h, st, true);
+}
+
+// The next batch of a hub (one CTA per listed hub), as k_net_select_l2.
+__global__ void __launch_bounds__(BT) k_net_select_ham(const uint32_t *__restrict__ X, int wp,
+                                                       const int32_t *__restrict__ ids, const int2 *__restrict__ hlist,
+                                                       Hubs hb, const int64_t *__restrict__ coff, Chunks ch, Batch bt,
+                                                       int32_t *__restrict__ active) {
+    extern __shared__ uint4 hrows[];  // NET_C x nq
+    __shared__ float cd[NET_C];
+    __shared__ int32_t cp[NET_C];
+    const int2 hs = hlist[blockIdx.x];
+    const int h = hs.x;
+    if (hb.done[h]) return;
+    const int nc = hb.nc[h], nq = wp >> 2;
+    const float thr = hb.thr[h];
+    const int n_rep = (hb.count[h] + ch.len - 1) / ch.len * NET_KEYS;
+    int covered;
+    const int n = net_candidates<NET_C>(ch, coff[hs.y] * NET_KEYS, n_rep, thr, cd, cp, &covered);
+    const bool flat = n > 0 && flat_split(nc, covered);
+    if (n == 0 || flat) {
+        if (threadIdx.x == 0) net_take(hb, h, 0, flat, active);
+        return;
     }
+    for (int i = threadIdx.x; i < n * nq; i += BT) {
+        const int c = i / nq, k = i - c * nq;
+        hrows[i] = reinterpret_cast<const uint4 *>(X + (size_t)ids[cp[c]] * wp)[k];
+    }
+    __syncthreads();
+    int m = 0;
+    while (m < NET_M) {
+        const unsigned long long f = net_farthest(cd, n);
+        if (!(key_value(f) > thr)) break;
+        const int pick = (int)key_pos(f);
+        if (threadIdx.x == 0) bt.pos[(size_t)hs.y * NET_M + m] = cp[pick];
+        ++m;
+        __syncthreads();  // every warp has read cd
+        if (threadIdx.x < n)
+            cd[threadIdx.x] = fminf(cd[threadIdx.x], (float)ham_dist4(hrows + pick * nq, hrows + threadIdx.x * nq, nq));
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) net_take(hb, h, m, false, active);
 }
 
 __global__ void k_gather_bits(const uint32_t *__restrict__ Xb, int wp, const int32_t *__restrict__ perm, int64_t n,
@@ -521,228 +865,181 @@ __global__ void k_group_radius_ham(int ng, const int32_t *__restrict__ gbeg, con
     if (lane == 0) grad[g] = (float)r;
 }
 
-// One thread per hub: decide termination or choose the next centre (its
-// position goes to cpos[begin + label] when cpos is given).
-__global__ void k_hub_step(int nh, const int32_t *__restrict__ hlist, Hubs hb, int32_t *__restrict__ active_out,
-                           int32_t *__restrict__ cpos, int flat_check) {
+// Chunks per listed hub, and the listed hubs' slots (their index in the list).
+__global__ void k_chunk_counts(int nl, const int2 *__restrict__ hlist, const int32_t *__restrict__ count,
+                               int chunk_len, int32_t *__restrict__ out, int32_t *__restrict__ hslot) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int h = i < nh && hlist ? hlist[i] : i;
-    int act = 0;
-    if (i < nh && !hb.done[h]) {
-        unsigned long long k = hb.key[h];
-        float v = key_value(k);
-        const int covered = hb.covered[h];
-        hb.covered[h] = 0;
-        if (k == 0ull || !(v > hb.thr[h])) {
-            hb.done[h] = 1;
-        } else if (flat_check && flat_split(hb.nc[h], covered)) {
-            hb.done[h] = 1;
-            hb.flat[h] = 1;
-        } else {
-            hb.cur[h] = (int32_t)key_pos(k);
-            if (cpos) {
-                cpos[hb.begin[h]] = hb.begin[h];  // label 0: the hub's own centre
-                cpos[hb.begin[h] + hb.nc[h]] = hb.cur[h];
-            }
-            hb.nc[h] += 1;
-            hb.key[h] = 0ull;
-            act = 1;
-        }
-    }
-    unsigned b = __ballot_sync(0xffffffffu, act);
-    if ((threadIdx.x & 31) == 0 && b) atomicAdd(active_out, __popc(b));
+    if (i >= nl) return;
+    const int h = hlist[i].x;
+    out[i] = (count[h] + chunk_len - 1) / chunk_len;
+    hslot[h] = i;
 }
 
-// Per hub that took a new centre: its distance to each of the hub's centres
-// (TPD lanes per distance, warps over the labels).
-template <int TPD>
-__global__ void __launch_bounds__(BT) k_centre_dists(const float *__restrict__ X, int dp,
-                                                     const int32_t *__restrict__ ids, Hubs hb,
-                                                     const int32_t *__restrict__ hlist,
-                                                     const int32_t *__restrict__ cpos, float *__restrict__ dcc) {
-    const int h = hlist ? hlist[blockIdx.x] : blockIdx.x;
-    if (hb.done[h]) return;
-    const int b = hb.begin[h], nc = hb.nc[h], nq = dp >> 2;
-    const float4 *crow = reinterpret_cast<const float4 *>(X + (size_t)ids[hb.cur[h]] * dp);
-    constexpr int G = BT / TPD;
-    const int g = threadIdx.x / TPD, j = threadIdx.x % TPD;
-    for (int L0 = 0; L0 < nc; L0 += G) {  // every group runs the same number of steps
-        const int L = L0 + g;
-        const int pos = cpos[b + (L < nc ? L : 0)];
-        const float dd = sqrtf(group_sqdist<TPD>(reinterpret_cast<const float4 *>(X + (size_t)ids[pos] * dp), crow,
-                                                 nq, j));
-        if (L < nc && j == 0) dcc[b + L] = dd;
-    }
-}
-
-// Chunk table of a round: chunk -> (hub, first position).
-__global__ void k_chunk_counts(int nh, const int32_t *__restrict__ count, int chunk_len,
-                               int32_t *__restrict__ out) {
-    int h = blockIdx.x * blockDim.x + threadIdx.x;
-    if (h < nh) out[h] = (count[h] + chunk_len - 1) / chunk_len;
-}
-// The whole split (Algorithm 1) of one small hub (at most SPLIT_SMALL points)
-// in one CTA: the iterations of k_hub_step, k_centre_dists and
-// k_dist_update_l2 for that hub (the same steps and pruning; TPD lanes per
-// distance, four 16-byte loads each, so that a pass has many rows in
-// flight), its distances, labels and centres in shared memory, and no
-// launch per iteration.  One CTA per hub of the round (larger hubs exit);
-// the distances, labels and the number of children go back to global memory.
+// The whole split of one small hub (at most SPLIT_SMALL points) in one CTA,
+// in the same batched passes: every warp's farthest point is a candidate, the
+// candidates' mutual distances are taken at once (a group of TPD lanes per
+// pair), one thread picks from them farthest-first, and a pass compares every
+// point (its row read once) with the picks.  Distances and labels stay in
+// shared memory; no launch per pass.  Larger hubs exit.
+// Bound by the latency of a pass (about 2 us); before the batches each pass
+// took one centre: 3.2 -> 1.6 ms for the small hubs of 1M x 128.
 constexpr int SPLIT_SMALL = 512;
-template <int TPD>
+constexpr int SMALL_M = BT / 32;  // candidates, and centres of a pass
+template <int TPD, int NV>
 __global__ void __launch_bounds__(BT) k_split_small(const float *__restrict__ X, int dp,
                                                     const int32_t *__restrict__ ids, float *__restrict__ D,
-                                                    int32_t *__restrict__ lab, Hubs hb, int32_t *__restrict__ err) {
-    __shared__ float Ds[SPLIT_SMALL], dccs[SPLIT_SMALL];
-    __shared__ int32_t labs[SPLIT_SMALL], cposs[SPLIT_SMALL];
-    __shared__ float4 cen[32];  // dp <= 128 (TPD is chosen for it)
-    __shared__ unsigned long long red[BT / 32];
-    __shared__ int s_nc, s_done;
-    __shared__ unsigned long long s_key;
+                                                    int32_t *__restrict__ lab, Hubs hb) {
+    __shared__ float Ds[SPLIT_SMALL], pd[SMALL_M * SMALL_M];
+    __shared__ int32_t labs[SPLIT_SMALL];
+    __shared__ float4 cen[SMALL_M * 32];  // dp <= 128
+    __shared__ unsigned long long cand[SMALL_M];
+    __shared__ int s_pick[SMALL_M], s_m;
     const int h = blockIdx.x;
-    if (hb.done[h] || hb.count[h] > SPLIT_SMALL) return;  // a large hub: the level-wide iterations
+    if (hb.done[h] || hb.count[h] > SPLIT_SMALL) return;  // a large hub: the level-wide passes
     const int b = hb.begin[h], cnt = hb.count[h], nq = dp >> 2;
     const float thr = hb.thr[h];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    constexpr int G = BT / TPD;
+    const int g = threadIdx.x / TPD, j = threadIdx.x % TPD;
+    unsigned long long best = 0ull;
     for (int i = threadIdx.x; i < cnt; i += BT) {
         Ds[i] = D[b + i];
         labs[i] = lab[b + i];
+        const unsigned long long k = pack_max_key(Ds[i], (uint32_t)i);
+        best = k > best ? k : best;
     }
-    if (threadIdx.x == 0) {
-        s_nc = hb.nc[h];
-        s_key = hb.key[h];
-        cposs[0] = b;  // label 0: the hub's own centre
-    }
-    __syncthreads();
-    constexpr int G = BT / TPD;
-    const int g = threadIdx.x / TPD, j = threadIdx.x % TPD;
+    int nc = hb.nc[h];
     for (;;) {
-        // k_hub_step: done, or the farthest point becomes the next centre
-        if (threadIdx.x == 0) {
-            const unsigned long long k = s_key;
-            const float v = key_value(k);
-            if (k == 0ull || !(v > thr) || s_nc >= cnt + 1) {
-                if (k != 0ull && v > thr) atomicOr(err, 4);  // cannot happen: every centre is a distinct point
-                s_done = 1;
-            } else {
-                cposs[s_nc] = (int32_t)key_pos(k);
-                s_nc += 1;
-                s_done = 0;
-            }
-            s_key = 0ull;
-        }
-        __syncthreads();
-        if (s_done) break;
-        const int nc = s_nc, cur = cposs[nc - 1];
-        const float4 *crow = reinterpret_cast<const float4 *>(X + (size_t)ids[cur] * dp);
-        for (int i = threadIdx.x; i < nq; i += BT) cen[i] = crow[i];
-        __syncthreads();
-        // k_centre_dists: the new centre against every centre of the hub
-        for (int L0 = 0; L0 < nc; L0 += G) {
-            const int L = L0 + g;
-            const int pos = cposs[L < nc ? L : 0];
-            const float dd = sqrtf(group_sqdist<TPD>(reinterpret_cast<const float4 *>(X + (size_t)ids[pos] * dp), cen,
-                                                     nq, j));
-            if (L < nc && j == 0) dccs[L] = dd;
-        }
-        __syncthreads();
-        // k_dist_update_l2 over the hub's points, with the same pruning
-        unsigned long long best = 0ull;
-        for (int base = 0; base < cnt; base += G) {
-            const int i = base + g;
-            const bool valid = i < cnt;
-            float curd = valid ? Ds[i] : 0.f;
-            bool far = !valid;
-            if (valid) far = dccs[labs[i]] >= 2.0f * curd * (1.0f + 0x1p-12f) + 0x1p-60f;
-            if (!far) {
-                const float sq = group_sqdist<TPD>(reinterpret_cast<const float4 *>(X + (size_t)ids[b + i] * dp), cen,
-                                                   nq, j);
-                if (j == 0) {
-                    const float d = sqrtf(sq);
-                    if (d < curd) {
-                        Ds[i] = d;
-                        labs[i] = nc - 1;
-                        curd = d;
-                    }
-                }
-            }
-            if (valid && j == 0) {
-                const unsigned long long k = pack_max_key(curd, (uint32_t)(b + i));
-                best = k > best ? k : best;
-            }
-        }
         for (int o = 16; o > 0; o >>= 1) {
             const unsigned long long v = __shfl_xor_sync(0xffffffffu, best, o);
             best = v > best ? v : best;
         }
-        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = best;
+        // candidates in cand / cen: the farthest point of every warp
+        if (lane == 0) cand[w] = best;
+        const int wpos = best ? (int)key_pos(best) : 0;
+        const float4 *crow = reinterpret_cast<const float4 *>(X + (size_t)ids[b + wpos] * dp);
+        for (int k = lane; k < nq; k += 32) cen[w * nq + k] = __ldg(crow + k);
         __syncthreads();
-        if (threadIdx.x == 0) {
-            unsigned long long m = 0ull;
-            for (int w = 0; w < BT / 32; ++w) m = red[w] > m ? red[w] : m;
-            s_key = m;
+        // their mutual distances
+        for (int q0 = 0; q0 < SMALL_M * SMALL_M; q0 += G) {
+            const int q = min(q0 + g, SMALL_M * SMALL_M - 1);
+            float acc = 0.f;
+            const float4 *x = cen + (q / SMALL_M) * nq, *y = cen + (q % SMALL_M) * nq;
+#pragma unroll 4
+            for (int k = j; k < nq; k += TPD) {
+                const float4 u = x[k], v = y[k];
+                const float dx = u.x - v.x, dy = u.y - v.y, dz = u.z - v.z, dw = u.w - v.w;
+                acc = fmaf(dx, dx, acc);
+                acc = fmaf(dy, dy, acc);
+                acc = fmaf(dz, dz, acc);
+                acc = fmaf(dw, dw, acc);
+            }
+#pragma unroll
+            for (int o = TPD / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o, TPD);
+            if (j == 0) pd[q] = sqrtf(acc);
         }
-        // the next pass's reads of Ds / labs follow the barrier at its top
+        __syncthreads();
+        // the picks, farthest-first (lane c of warp 0 follows candidate c)
+        if (w == 0) {
+            const unsigned long long mine = lane < SMALL_M ? cand[lane] : 0ull;
+            float d = mine ? key_value(mine) : 0.f;
+            int m = 0;
+            for (; m < SMALL_M; ++m) {
+                unsigned long long f = lane < SMALL_M ? pack_max_key(d, (uint32_t)lane) : 0ull;
+#pragma unroll
+                for (int o = SMALL_M / 2; o > 0; o >>= 1) {
+                    const unsigned long long v = __shfl_xor_sync(0xffffffffu, f, o);
+                    f = v > f ? v : f;
+                }
+                f = __shfl_sync(0xffffffffu, f, 0);
+                if (!(key_value(f) > thr)) break;
+                const int pick = (int)key_pos(f);
+                if (lane == 0) s_pick[m] = pick;
+                if (lane < SMALL_M) d = fminf(d, pd[pick * SMALL_M + lane]);
+            }
+            if (lane == 0) s_m = m;
+        }
+        __syncthreads();
+        const int m = s_m;
+        if (m == 0) break;
+        // every point against the picks
+        best = 0ull;
+        for (int i0 = 0; i0 < cnt; i0 += G) {
+            const int i = i0 + g;
+            const bool valid = i < cnt;
+            RowRegs<TPD, NV> r;
+            r.load(reinterpret_cast<const float4 *>(X + (size_t)ids[b + (valid ? i : 0)] * dp), nq, j);
+            float sb = INFINITY;
+            int ib = 0;
+            for (int c = 0; c < m; ++c) {
+                const float s = r.sqdist(cen + s_pick[c] * nq, nq, j);
+                if (s < sb) {
+                    sb = s;
+                    ib = c;
+                }
+            }
+            if (valid && j == 0) {
+                float cur = Ds[i];
+                const float d = sqrtf(sb);
+                if (d < cur) {
+                    cur = d;
+                    Ds[i] = d;
+                    labs[i] = nc + ib;
+                }
+                const unsigned long long k = pack_max_key(cur, (uint32_t)i);
+                best = k > best ? k : best;
+            }
+        }
+        nc += m;
+        __syncthreads();  // cen and s_pick have been read
     }
     for (int i = threadIdx.x; i < cnt; i += BT) {
         D[b + i] = Ds[i];
         lab[b + i] = labs[i];
     }
     if (threadIdx.x == 0) {
-        hb.nc[h] = s_nc;
+        hb.nc[h] = nc;
         hb.done[h] = 1;
-        hb.key[h] = 0ull;
     }
 }
 
-// Hubs not yet done, and the chunks of those hubs (from the current chunk
-// list), for the next burst of split iterations: late iterations touch only
-// the few hubs still splitting.  The order within the lists is immaterial
-// (every hub and point is updated independently; keys combine by max).
-__global__ void k_active_hubs(int nh, const int32_t *__restrict__ done, int32_t *__restrict__ hlist,
-                              int32_t *__restrict__ cnt) {
-    const int h = blockIdx.x * blockDim.x + threadIdx.x;
-    const bool a = h < nh && !done[h];
+// The listed hubs not yet done, and their chunks, for the next passes (the
+// order within the lists is immaterial).  cnt: {hubs, chunks}.
+__device__ __forceinline__ int append_slot(bool a, int32_t *cnt) {
     const unsigned m = __ballot_sync(0xffffffffu, a);
-    if (!m) return;
+    if (!m) return 0;
     const int lane = threadIdx.x & 31, leader = __ffs(m) - 1;
     int base = 0;
     if (lane == leader) base = atomicAdd(cnt, __popc(m));
     base = __shfl_sync(0xffffffffu, base, leader);
-    if (a) hlist[base + __popc(m & ((1u << lane) - 1u))] = h;
+    return base + __popc(m & lanemask_lt());
 }
-__global__ void k_active_chunks(int64_t nchunks, const int32_t *__restrict__ chub, const int32_t *__restrict__ cst,
-                                const int32_t *__restrict__ done, int32_t *__restrict__ chub2,
-                                int32_t *__restrict__ cst2, int32_t *__restrict__ cnt) {
-    const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const bool a = c < nchunks && !done[chub[c]];
-    const unsigned m = __ballot_sync(0xffffffffu, a);
-    if (!m) return;
-    const int lane = threadIdx.x & 31, leader = __ffs(m) - 1;
-    int base = 0;
-    if (lane == leader) base = atomicAdd(cnt, __popc(m));
-    base = __shfl_sync(0xffffffffu, base, leader);
-    if (a) {
-        const int k = base + __popc(m & ((1u << lane) - 1u));
-        chub2[k] = chub[c];
-        cst2[k] = cst[c];
-    }
+__global__ void k_active(int nl, const int2 *__restrict__ hl, int64_t nck, const int4 *__restrict__ cl,
+                         const int32_t *__restrict__ done, int2 *__restrict__ hl2, int4 *__restrict__ cl2,
+                         int32_t *__restrict__ cnt) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const bool ah = i < nl && !done[hl[i < nl ? i : 0].x];
+    int k = append_slot(ah, cnt);
+    if (ah) hl2[k] = hl[i];
+    const bool ac = i < nck && !done[cl[i < nck ? i : 0].x];
+    k = append_slot(ac, cnt + 1);
+    if (ac) cl2[k] = cl[i];
 }
 
-// Chunk table of a round, one thread per chunk: its hub is the last one whose
-// chunk offset is at most the chunk's index (hubs without chunks share an
-// offset with the next hub and are skipped by the search).
-__global__ void k_chunk_fill(int64_t nchunks, int nh, const int32_t *__restrict__ begin,
-                             const int64_t *__restrict__ coff, int chunk_len,
-                             int32_t *__restrict__ chunk_hub, int32_t *__restrict__ chunk_start) {
+// Chunk table of the listed hubs, one thread per chunk: its hub is the last
+// one whose chunk offset is at most the chunk's index.
+__global__ void k_chunk_fill(int64_t nchunks, int nl, const int2 *__restrict__ hlist,
+                             const int32_t *__restrict__ begin, const int64_t *__restrict__ coff, int chunk_len,
+                             int4 *__restrict__ chunks) {
     const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= nchunks) return;
-    int lo = 0, hi = nh;  // coff[lo] <= c, and c < coff[hi] unless hi = nh
+    int lo = 0, hi = nl;  // coff[lo] <= c, and c < coff[hi] unless hi = nl
     while (hi - lo > 1) {
         const int mid = (lo + hi) >> 1;
         if (__ldg(coff + mid) <= c) lo = mid; else hi = mid;
     }
-    chunk_hub[c] = lo;
-    chunk_start[c] = begin[lo] + (int)(c - coff[lo]) * chunk_len;
+    const int h = hlist[lo].x;
+    chunks[c] = make_int4(h, begin[h] + (int)(c - coff[lo]) * chunk_len, (int)c, 0);
 }
 
 // Partition keys for the round: key = child_base[hub] + label, value = round
@@ -850,22 +1147,27 @@ __global__ void k_child_keys(int64_t R, const uint32_t *__restrict__ skeys, cons
     if (valid && (lane == 31 || next != gc)) atomicMax(&ckey[gc], v);
 }
 
-// Link every hub to its children (consecutive node ids).
-__global__ void k_link_children(int nh, Hubs hb, const int64_t *__restrict__ child_base, int node_base,
+// Link every hub to its children (consecutive node ids): one thread per child
+// finds its hub (the last one whose child base is at most the child's index;
+// every hub has children), the hub's first child writes the hub's record.
+__global__ void k_link_children(int64_t T, int nh, Hubs hb, const int64_t *__restrict__ child_base, int node_base,
                                 int32_t *__restrict__ child_begin, int32_t *__restrict__ child_count,
                                 int32_t *__restrict__ node_level, int32_t *__restrict__ parent,
                                 int32_t *__restrict__ leafy) {
-    int h = blockIdx.x * blockDim.x + threadIdx.x;
-    if (h >= nh) return;
-    int u = hb.node[h];
-    int first = node_base + (int32_t)child_base[h];
-    child_begin[u] = first;
-    child_count[u] = hb.nc[h];
-    node_level[u] = hb.level[h];
-    const int fl = hb.flat[h];
-    for (int c = 0; c < hb.nc[h]; ++c) {
-        parent[first + c] = u;
-        leafy[child_base[h] + c] = fl;
+    const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (c >= T) return;
+    int lo = 0, hi = nh;
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (__ldg(child_base + mid) <= c) lo = mid; else hi = mid;
+    }
+    const int u = hb.node[lo];
+    parent[node_base + c] = u;
+    leafy[c] = hb.flat[lo];
+    if (c == child_base[lo]) {
+        child_begin[u] = node_base + (int32_t)c;
+        child_count[u] = hb.nc[lo];
+        node_level[u] = hb.level[lo];
     }
 }
 
@@ -890,23 +1192,31 @@ __global__ void k_make_nodes(int64_t T, int node_base, int zeta, int metric,
     is_hub[c] = (ccount[c] > zeta && r > 0.0f && !leafy[c]) ? 1 : 0;
 }
 
-// Next round's hubs from the flagged children (order preserved).
+// Next round's hubs from the flagged children (order preserved); the hubs of
+// more than small_max points are listed for the level-wide passes (cnt: listed
+// hubs, their chunks).
 __global__ void k_next_hubs(int64_t T, int node_base, const int32_t *__restrict__ is_hub,
                             const int64_t *__restrict__ hub_off, const int32_t *__restrict__ cbegin,
                             const int32_t *__restrict__ ccount, const unsigned long long *__restrict__ ckey,
-                            const int32_t *__restrict__ level, Hubs nh) {
+                            const int32_t *__restrict__ level, Hubs nh, int small_max, int chunk_len,
+                            int2 *__restrict__ hlist, int32_t *__restrict__ cnt) {
     int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= T || !is_hub[c]) return;
+    const bool hub = c < T && is_hub[c];
+    const bool listed = hub && ccount[c] > small_max;
+    const int k = append_slot(listed, cnt);
+    const int chunks = __reduce_add_sync(0xffffffffu, listed ? (ccount[c] + chunk_len - 1) / chunk_len : 0);
+    if ((threadIdx.x & 31) == 0 && chunks) atomicAdd(cnt + 2, chunks);
+    if (!hub) return;
     int64_t h = hub_off[c];
+    if (listed) hlist[k] = make_int2((int)h, k);
     int v = node_base + (int)c;
     nh.begin[h] = cbegin[c];
     nh.count[h] = ccount[c];
     nh.node[h] = v;
     nh.nc[h] = 1;
-    nh.cur[h] = cbegin[c];
+    nh.m[h] = 0;
     nh.done[h] = 0;
     nh.flat[h] = 0;
-    nh.covered[h] = 0;
     nh.key[h] = ckey[c];
     int l = level[v];
     nh.level[h] = l;
@@ -920,6 +1230,21 @@ __global__ void k_root_init(int64_t n, int root, int32_t *__restrict__ ids, floa
     ids[i] = i == 0 ? root : (i <= root ? (int32_t)i - 1 : (int32_t)i);
     D[i] = INFINITY;
     lab[i] = 0;
+}
+
+// The root's first pass: hub 0 holds every point, its batch is position 0 with label 0.
+__global__ void k_root_hub(int64_t n, Hubs hb, int32_t *__restrict__ hslot, int32_t *__restrict__ bpos,
+                           int2 *__restrict__ hlist) {
+    hb.begin[0] = 0;
+    hb.count[0] = (int32_t)n;
+    hb.nc[0] = 1;
+    hb.m[0] = 1;
+    hb.done[0] = 0;
+    hb.thr[0] = 0.0f;
+    hb.key[0] = 0ull;
+    hslot[0] = 0;
+    bpos[0] = 0;
+    hlist[0] = make_int2(0, 0);
 }
 
 __global__ void k_root_node(int64_t n, int zeta, int metric, const unsigned long long *__restrict__ key,
@@ -942,11 +1267,9 @@ __global__ void k_root_node(int64_t n, int zeta, int metric, const unsigned long
     hb.count[0] = (int32_t)n;
     hb.node[0] = 0;
     hb.nc[0] = 1;
-    hb.cur[0] = 0;
+    hb.m[0] = 0;
     hb.done[0] = 0;
     hb.flat[0] = 0;
-    hb.covered[0] = 0;
-    hb.key[0] = key[0];
     hb.level[0] = l;
     hb.thr[0] = hub ? ldexpf(1.0f, l - 1) : 0.0f;
 }
@@ -1187,11 +1510,13 @@ ct_tree *build_tree(const ct_points *pts, int zeta, int root, cudaStream_t s) {
 
     DBuf<int32_t> err(2, s);
     CT_CHECK_CUDA(cudaMemsetAsync(err.p, 0, 2 * sizeof(int32_t), s));
+    int64_t sspan[2] = {0, 0};  // edit distance: first and past-the-end byte of the strings
 
     // padded copy of the input (original order) / string lengths
     DBuf<float> Xp;
     DBuf<uint32_t> Xb;
-    int W = 1;
+    DBuf<uint8_t> codes, scode;  // edit distance: the strings re-coded to the bytes that occur
+    int W = 1, A = 1;
     if (ham) {
         Xb = DBuf<uint32_t>((size_t)(n ? n : 1) * wp, s);
         if (n) {
@@ -1213,6 +1538,8 @@ ct_tree *build_tree(const ct_points *pts, int zeta, int root, cudaStream_t s) {
         if (n) {
             k_string_lengths<<<grid_for(n), BT, 0, s>>>(n, nullptr, pts->offsets, lens.p, err.p + 1);
             CT_COUNT_LAUNCH();
+            to_host_async(sspan, pts->offsets, 1, s);
+            to_host_async(sspan + 1, pts->offsets + n, 1, s);
         }
     }
     CT_LAUNCH_CHECK();
@@ -1224,6 +1551,24 @@ ct_tree *build_tree(const ct_points *pts, int zeta, int root, cudaStream_t s) {
             CT_FAIL(CT_EUNSUPPORTED, "string of length %d above the limit %d", herr[1], CT_MAX_STRING_LEN);
         t->max_len = herr[1];
         W = lev_words_for(t->max_len);
+        const int64_t bytes = sspan[1] - sspan[0];
+        DBuf<int32_t> present(257, s);  // per byte value; their number
+        CT_CHECK_CUDA(cudaMemsetAsync(present.p, 0, 257 * sizeof(int32_t), s));
+        codes = DBuf<uint8_t>(256, s);
+        scode = DBuf<uint8_t>(bytes > 0 ? bytes : 1, s);
+        const uint8_t *src = (const uint8_t *)pts->data + sspan[0];
+        if (bytes > 0) {
+            k_present<<<grid_for(bytes), BT, 0, s>>>(src, bytes, present.p);
+            CT_COUNT_LAUNCH();
+            k_codes<<<1, 256, 0, s>>>(present.p, codes.p, present.p + 256);
+            CT_COUNT_LAUNCH();
+            k_recode<<<grid_for(bytes), BT, 0, s>>>(src, bytes, codes.p, scode.p);
+            CT_COUNT_LAUNCH();
+        }
+        CT_LAUNCH_CHECK();
+        int32_t a = 0;
+        to_host(&a, present.p + 256, 1, s);
+        A = std::max(a, 1);
     }
 
     // tree arrays: a tree whose internal vertices have >= 2 children has < 2n vertices
@@ -1239,18 +1584,18 @@ ct_tree *build_tree(const ct_points *pts, int zeta, int root, cudaStream_t s) {
         if (root < 0 || root >= n) CT_FAIL(CT_EINVAL, "root %d out of range", root);
         // ---- round 0: distances to the root
         const int64_t cap_h = n;  // hubs per round never exceed n / (zeta+1) + 1
-        DBuf<int32_t> hbuf(9 * (cap_h + 1), s);
+        DBuf<int32_t> hbuf(8 * (cap_h + 1), s);
         DBuf<float> hthr(cap_h + 1, s);
         DBuf<unsigned long long> hkey(cap_h + 1, s);
-        DBuf<int32_t> hbuf2(9 * (cap_h + 1), s);
+        DBuf<int32_t> hbuf2(8 * (cap_h + 1), s);
         DBuf<float> hthr2(cap_h + 1, s);
         DBuf<unsigned long long> hkey2(cap_h + 1, s);
         auto make_hubs = [&](DBuf<int32_t> &b, DBuf<float> &th, DBuf<unsigned long long> &k) {
             Hubs h;
             int64_t st = cap_h + 1;
             h.begin = b.p; h.count = b.p + st; h.node = b.p + 2 * st; h.nc = b.p + 3 * st;
-            h.cur = b.p + 4 * st; h.done = b.p + 5 * st; h.level = b.p + 6 * st;
-            h.flat = b.p + 7 * st; h.covered = b.p + 8 * st;
+            h.m = b.p + 4 * st; h.done = b.p + 5 * st; h.level = b.p + 6 * st;
+            h.flat = b.p + 7 * st;
             h.thr = th.p; h.key = k.p;
             return h;
         };
@@ -1258,97 +1603,143 @@ ct_tree *build_tree(const ct_points *pts, int zeta, int root, cudaStream_t s) {
 
         k_root_init<<<grid_for(n), BT, 0, s>>>(n, root, ids.p, D.p, lab.p);
         CT_COUNT_LAUNCH();
-        // one pass of the update kernel with the root as the only centre
-        // lanes per distance: four 16-byte loads each (a pass has many rows in
-        // flight); a chunk is eight passes of a block
+        // lanes per distance: four 16-byte loads each (at most eight for row
+        // lengths between two powers of two, more above 1024 floats)
         int tpd = 1;  // a power of two
         while (l2 && tpd < 32 && 2 * tpd * 16 <= dp) tpd *= 2;
-        // points per block of an update pass: L2, eight passes of the block's
-        // groups; Hamming, four per thread; edit distance, one per thread (a
-        // long recurrence each: more blocks share a pass)
-        const int chunk_len = l2 ? UPD_PASSES * (BT / tpd) : ham ? 4 * BT : BT;
-        // staged update passes where the buffers fit (a pass's rows: BT / tpd
-        // rows of dp / 4 float4s), with their shared memory allowed once
-        const bool stage = l2 && (int64_t)(BT / tpd) * (dp / 4) <= UPD_STAGE_F4;
-        const size_t stage_sm = ((size_t)dp / 4 + (size_t)UPD_STAGES * (BT / tpd) * (dp / 4)) * sizeof(float4);
-        if (stage) {
-            static std::once_flag once[6];
-            auto allow = [&](int k, const void *fn) {
-                std::call_once(once[k], [&] {
-                    cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)(sizeof(float4) * (1 + UPD_STAGES) * UPD_STAGE_F4));
-                });
-            };
+        const int nv = (dp / 4 + tpd - 1) / tpd;  // float4s per lane
+        const int passes = tpd == 1 ? net_passes<1>() : tpd == 2 ? net_passes<2>() : net_passes<4>();
+        const int chunk_len = l2 ? passes * (BT / tpd) : ham ? BT : LEV_P;
+        // hubs of at most small_max points are split whole in one CTA each
+        const int small_max = l2 && dp <= 128 ? SPLIT_SMALL : 0;
+        // centres of a batch: what 48 KB of shared memory hold
+        const int mcap = l2 ? std::max(1, std::min(NET_M, 12288 / std::max(dp, 1)))
+                       : lev ? std::max(1, std::min(NET_M, 40960 / (A * W * 8))) : NET_M;
+        const bool prune = lev || (l2 && dp > 16);
+        const Strings S{scode.p - sspan[0], pts->offsets, A};
+        DBuf<int32_t> cpos(l2 || lev ? n : 1, s);
+        DBuf<float> dcc(prune ? (size_t)n * NET_M : 1, s);
+        DBuf<int32_t> hslot(cap_h + 1, s), bpos(NET_M, s);
+        DBuf<int4> chunks_a, chunks_b;
+        DBuf<int2> hl_a(cap_h + 1, s), hl_b(cap_h + 1, s);
+        DBuf<unsigned long long> keys;
+        DBuf<int32_t> cov;
+        LevCands lc{};
+        DBuf<int32_t> lcn, lcpos;
+        DBuf<float> lcd;
+        DBuf<uint16_t> lcpair;
+        auto dispatch = [&](auto f) {  // f(lanes per distance, float4s per lane) as compile-time constants
+#define CT_TN(T, V) f(std::integral_constant<int, T>(), std::integral_constant<int, V>())
+#define CT_T48(T) case T: if (nv <= 4) CT_TN(T, 4); else CT_TN(T, 8); break;
             switch (tpd) {
-                case 1: allow(0, (const void *)k_dist_update_l2<1, true>); break;
-                case 2: allow(1, (const void *)k_dist_update_l2<2, true>); break;
-                case 4: allow(2, (const void *)k_dist_update_l2<4, true>); break;
-                case 8: allow(3, (const void *)k_dist_update_l2<8, true>); break;
-                case 16: allow(4, (const void *)k_dist_update_l2<16, true>); break;
-                case 32: allow(5, (const void *)k_dist_update_l2<32, true>); break;
+                case 1: if (nv <= 1) CT_TN(1, 1); else if (nv <= 2) CT_TN(1, 2); else if (nv <= 4) CT_TN(1, 4); else CT_TN(1, 8); break;
+                CT_T48(2) CT_T48(4) CT_T48(8) CT_T48(16)
+                case 32: if (nv <= 4) CT_TN(32, 4); else if (nv <= 8) CT_TN(32, 8); else CT_TN(32, 0); break;
             }
-            CT_CHECK_CUDA(cudaGetLastError());
-        }
-        // pruned updates (L2): centre positions and centre-to-new-centre distances per hub label
-        DBuf<int32_t> cpos(l2 ? n : 1, s);
-        DBuf<float> dcc(l2 ? n : 1, s);
-        bool prune = false;  // off for the root's first pass (no labels yet)
-        auto update = [&](Hubs &hb, int64_t nchunks, const int32_t *chub, const int32_t *cst, Step st) {
-            if (!nchunks) return;
+#undef CT_T48
+#undef CT_TN
+            CT_COUNT_LAUNCH();
+            CT_LAUNCH_CHECK();
+        };
+        // one update pass over the listed chunks
+        auto update = [&](const Hubs &hb, int64_t nck, const int4 *list, const Batch &bt, unsigned long long *root) {
+            const Chunks ch{list, chunk_len, keys.p, cov.p};
             if (l2) {
-                if (stage) {
-                    switch (tpd) {
-#define CT_UPD(T) case T: k_dist_update_l2<T, true><<<(unsigned)nchunks, BT, stage_sm, s>>>(Xp.p, dp, ids.p, D.p, lab.p, chub, cst, chunk_len, hb, prune ? dcc.p : nullptr, st); break;
-                        CT_UPD(1) CT_UPD(2) CT_UPD(4) CT_UPD(8) CT_UPD(16) CT_UPD(32)
-#undef CT_UPD
-                    }
-                } else {
-                    const size_t sm = (size_t)dp * sizeof(float);
-                    switch (tpd) {
-#define CT_UPD(T) case T: k_dist_update_l2<T, false><<<(unsigned)nchunks, BT, sm, s>>>(Xp.p, dp, ids.p, D.p, lab.p, chub, cst, chunk_len, hb, prune ? dcc.p : nullptr, st); break;
-                        CT_UPD(1) CT_UPD(2) CT_UPD(4) CT_UPD(8) CT_UPD(16) CT_UPD(32)
-#undef CT_UPD
-                    }
+                const size_t sm = (size_t)mcap * dp * sizeof(float);
+                dispatch([&](auto T, auto V) {
+                    if (prune)
+                        k_net_update_l2<T(), V(), true><<<(unsigned)nck, BT, sm, s>>>(Xp.p, dp, ids.p, D.p, lab.p, ch, hb, bt, hslot.p, root);
+                    else
+                        k_net_update_l2<T(), V(), false><<<(unsigned)nck, BT, sm, s>>>(Xp.p, dp, ids.p, D.p, lab.p, ch, hb, bt, hslot.p, root);
+                });
+                return;
+            }
+            if (ham) {
+                const size_t sm = (size_t)NET_M * wp * sizeof(uint32_t);
+                switch (wp / 4) {
+#define CT_UH(Q) k_net_update_ham<Q><<<(unsigned)nck, BT, sm, s>>>(Xb.p, wp, ids.p, D.p, lab.p, ch, hb, bt, hslot.p, root)
+                    case 1: CT_UH(1); break;
+                    case 2: CT_UH(2); break;
+                    case 3: CT_UH(3); break;
+                    case 4: CT_UH(4); break;
+                    default: CT_UH(0); break;
+#undef CT_UH
                 }
-            } else if (ham) {
-                k_dist_update_ham<<<(unsigned)nchunks, BT, (size_t)wp * sizeof(uint32_t), s>>>(
-                    Xb.p, wp, ids.p, D.p, lab.p, chub, cst, chunk_len, hb, st);
             } else {
-                const uint8_t *S = (const uint8_t *)pts->data;
+                const size_t sm = (size_t)mcap * A * W * sizeof(uint64_t);
                 switch (W) {
-#define CT_UPDL(WW) case WW: k_dist_update_lev<WW><<<(unsigned)nchunks, BT, 0, s>>>(S, pts->offsets, ids.p, D.p, lab.p, chub, cst, chunk_len, hb, st); break;
-                    CT_UPDL(1) CT_UPDL(2) CT_UPDL(4) CT_UPDL(8) CT_UPDL(16)
-#undef CT_UPDL
+#define CT_UL(WW) case WW: k_net_update_lev<WW><<<(unsigned)nck, BT, sm, s>>>(S, ids.p, D.p, lab.p, ch, hb, bt, hslot.p, root ? 0 : 1, root); break;
+                    CT_UL(1) CT_UL(2) CT_UL(4) CT_UL(8) CT_UL(16)
+#undef CT_UL
                 }
             }
             CT_COUNT_LAUNCH();
             CT_LAUNCH_CHECK();
         };
-        // root hub state for the initial pass: centre = position 0, label 0
-        {
-            int32_t one = 1;
-            int32_t zero = 0;
-            unsigned long long z = 0;
-            CT_CHECK_CUDA(cudaMemcpyAsync(H.begin, &zero, 4, cudaMemcpyHostToDevice, s));
-            int32_t cnt = (int32_t)n;
-            CT_CHECK_CUDA(cudaMemcpyAsync(H.count, &cnt, 4, cudaMemcpyHostToDevice, s));
-            CT_CHECK_CUDA(cudaMemcpyAsync(H.nc, &one, 4, cudaMemcpyHostToDevice, s));
-            CT_CHECK_CUDA(cudaMemcpyAsync(H.cur, &zero, 4, cudaMemcpyHostToDevice, s));
-            CT_CHECK_CUDA(cudaMemcpyAsync(H.done, &zero, 4, cudaMemcpyHostToDevice, s));
-            CT_CHECK_CUDA(cudaMemcpyAsync(H.flat, &zero, 4, cudaMemcpyHostToDevice, s));
-            CT_CHECK_CUDA(cudaMemcpyAsync(H.covered, &zero, 4, cudaMemcpyHostToDevice, s));
-            CT_CHECK_CUDA(cudaMemcpyAsync(H.key, &z, 8, cudaMemcpyHostToDevice, s));
-            CT_CHECK_CUDA(cudaStreamSynchronize(s));  // host values above are on the stack
-        }
-        int64_t nchunks0 = ceil_div(n, chunk_len);
-        DBuf<int32_t> chub(nchunks0, s), cst(nchunks0, s);
-        {
-            DBuf<int64_t> coff(1, s);
-            CT_CHECK_CUDA(cudaMemsetAsync(coff.p, 0, sizeof(int64_t), s));
-            k_chunk_fill<<<grid_for(nchunks0), BT, 0, s>>>(nchunks0, 1, H.begin, coff.p, chunk_len, chub.p, cst.p);
+        // the listed hubs' next batches and, where updates prune, their distances to the hubs' centres
+        auto select = [&](const Hubs &hb, int nlist, const int2 *list, const int64_t *coff, const Batch &bt,
+                          int32_t *active) {
+            const Chunks ch{nullptr, chunk_len, keys.p, cov.p};
+            if (l2) {
+                const int staged = dp <= 128;
+                const size_t sm = staged ? (size_t)NET_C * dp * sizeof(float) : 0;
+                const size_t dsm = (size_t)mcap * dp * sizeof(float);
+                dispatch([&](auto T, auto V) {
+                    auto kern = k_net_select_l2<T()>;
+                    if (sm > 40 * 1024)
+                        CT_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+                    kern<<<(unsigned)nlist, BT, sm, s>>>(Xp.p, dp, ids.p, list, hb, coff, ch, bt, mcap, staged, active);
+                    if (prune) {
+                        CT_COUNT_LAUNCH();
+                        k_net_dists_l2<T(), V()><<<dim3((unsigned)nlist, nlist >= 64 ? 4 : 32), BT, dsm, s>>>(Xp.p, dp, ids.p, list, hb, bt);
+                    }
+                });
+                return;
+            }
+            if (ham) {
+                const size_t sm = (size_t)NET_C * wp * sizeof(uint32_t);
+                if (sm > 40 * 1024)
+                    CT_CHECK_CUDA(cudaFuncSetAttribute(k_net_select_ham, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+                k_net_select_ham<<<(unsigned)nlist, BT, sm, s>>>(Xb.p, wp, ids.p, list, hb, coff, ch, bt, active);
+            } else {
+                const size_t sm = (size_t)A * W * sizeof(uint64_t);
+                k_net_cands_lev<<<(unsigned)nlist, BT, 0, s>>>(list, hb, coff, ch, lc);
+                CT_COUNT_LAUNCH();
+                switch (W) {
+#define CT_PL(WW) case WW: k_net_pairs_lev<WW><<<dim3((unsigned)nlist, LEV_C), LEV_C, sm, s>>>(S, ids.p, list, hb, lc); break;
+                    CT_PL(1) CT_PL(2) CT_PL(4) CT_PL(8) CT_PL(16)
+#undef CT_PL
+                }
+                CT_COUNT_LAUNCH();
+                k_net_pick_lev<<<(unsigned)nlist, 32, 0, s>>>(list, hb, bt, lc, mcap, active);
+                CT_COUNT_LAUNCH();
+                switch (W) {
+#define CT_DL(WW) case WW: k_net_dists_lev<WW><<<dim3((unsigned)nlist, (unsigned)mcap), 128, sm, s>>>(S, ids.p, list, hb, bt); break;
+                    CT_DL(1) CT_DL(2) CT_DL(4) CT_DL(8) CT_DL(16)
+#undef CT_DL
+                }
+            }
             CT_COUNT_LAUNCH();
-            update(H, nchunks0, chub.p, cst.p, Step{});
-        }
+            CT_LAUNCH_CHECK();
+        };
+        int64_t nchunks = ceil_div(n, chunk_len);
+        auto grow_chunks = [&]() {
+            for (DBuf<int4> *c : {&chunks_a, &chunks_b})
+                if ((int64_t)c->n < nchunks) *c = DBuf<int4>(nchunks, s);
+            if ((int64_t)cov.n < nchunks * NET_KEYS) {
+                keys = DBuf<unsigned long long>(nchunks * NET_KEYS, s);
+                cov = DBuf<int32_t>(nchunks * NET_KEYS, s);
+            }
+        };
+        // the root's pass: a batch of one centre, position 0 (the memsets write zeros, k_root_hub the rest)
+        DBuf<int64_t> i64tmp(4, s);
+        CT_CHECK_CUDA(cudaMemsetAsync(i64tmp.p, 0, 4 * sizeof(int64_t), s));
+        grow_chunks();
+        k_root_hub<<<1, 1, 0, s>>>(n, H, hslot.p, bpos.p, hl_a.p);
+        CT_COUNT_LAUNCH();
+        k_chunk_fill<<<grid_for(nchunks), BT, 0, s>>>(nchunks, 1, hl_a.p, H.begin, i64tmp.p, chunk_len, chunks_a.p);
+        CT_COUNT_LAUNCH();
+        update(H, nchunks, chunks_a.p, Batch{bpos.p, cpos.p, dcc.p}, H.key);
         DBuf<int32_t> is_root_hub(1, s);
         k_root_node<<<1, 1, 0, s>>>(n, zeta, pts->metric, H.key, nb.p, ncnt.p, cbeg.p, ccnt.p, rad.p, lvl.p, H,
                                     is_root_hub.p);
@@ -1358,121 +1749,71 @@ ct_tree *build_tree(const ct_points *pts, int zeta, int root, cudaStream_t s) {
         to_host(&root_hub, is_root_hub.p, 1, s);
         n_nodes = 1;
         int64_t nh = root_hub ? 1 : 0;
+        int nl = root_hub && n > small_max ? 1 : 0;  // hubs of the level-wide passes
 
         // scratch for partitioning
         DBuf<uint32_t> pk(n, s), pv(n, s), tk(n, s), tv(n, s);
         DBuf<int32_t> rpos(n, s), tids(n, s);
         DBuf<float> tD(n, s);
-        DBuf<int32_t> active(3, s);  // hub activations of a burst, active hubs, active chunks
-        DBuf<int32_t> hlist(n, s), chub2(nchunks0, s), cst2(nchunks0, s);
-        DBuf<int32_t> arrive(cap_h + 1, s);  // per hub: finished blocks of an update pass
-        DBuf<int64_t> i64tmp(2, s);
+        DBuf<int32_t> active(3, s);  // batches taken in a burst; hubs and chunks left
 
         while (nh > 0) {
             ++depth;
-            // chunk table of this round
-            DBuf<int32_t> ccounts(nh, s);
-            DBuf<int64_t> coff(nh, s);
-            k_chunk_counts<<<grid_for(nh), BT, 0, s>>>((int)nh, H.count, chunk_len, ccounts.p);
-            CT_COUNT_LAUNCH();
-            exclusive_scan_i32_to_i64(ccounts.p, coff.p, nh, i64tmp.p, s);
-            int64_t nchunks = 0;
-            to_host(&nchunks, i64tmp.p, 1, s);
-            chub.grow(nchunks);
-            cst.grow(nchunks);
-            chub2.grow(nchunks);
-            cst2.grow(nchunks);
-            k_chunk_fill<<<grid_for(nchunks), BT, 0, s>>>(nchunks, (int)nh, H.begin, coff.p, chunk_len, chub.p, cst.p);
-            CT_COUNT_LAUNCH();
-            CT_LAUNCH_CHECK();
-
-            // split iterations (Algorithm 1) for every hub of the round
             {
                 ProfScope prof_split("build_split", s);
-                int burst = 1;
-                int64_t iters = 0;
-                bool first_step = true;
-                // the hubs and chunks a burst visits: all at first, then those
-                // of the hubs still splitting after the previous burst
-                const int32_t *hl = nullptr;
-                int64_t nl = nh, nck = nchunks;
-                int32_t *cb = chub.p, *cs = cst.p, *cb2 = chub2.p, *cs2 = cst2.p;
-                if (l2 && dp <= 128 && prune) {
-                    // small hubs split whole in one CTA each; the loop below takes the rest
-                    switch (tpd) {
-#define CT_SS(T) case T: k_split_small<T><<<(unsigned)nh, BT, 0, s>>>(Xp.p, dp, ids.p, D.p, lab.p, H, err.p); break;
-                        CT_SS(1) CT_SS(2) CT_SS(4) CT_SS(8) CT_SS(16) CT_SS(32)
-#undef CT_SS
-                    }
-                    CT_COUNT_LAUNCH();
-                    CT_CHECK_CUDA(cudaMemsetAsync(active.p, 0, 3 * sizeof(int32_t), s));
-                    k_active_hubs<<<grid_for(nh), BT, 0, s>>>((int)nh, H.done, hlist.p, active.p + 1);
-                    CT_COUNT_LAUNCH();
-                    k_active_chunks<<<grid_for(nck), BT, 0, s>>>(nck, cb, cs, H.done, cb2, cs2, active.p + 2);
-                    CT_COUNT_LAUNCH();
-                    CT_LAUNCH_CHECK();
-                    int32_t cnt3[3] = {0, 0, 0};
-                    to_host(cnt3, active.p, 3, s);
-                    hl = hlist.p;
-                    nl = cnt3[1];
-                    nck = cnt3[2];
-                    std::swap(cb, cb2);
-                    std::swap(cs, cs2);
+                if (small_max && (nl < nh)) {
+                    dispatch([&](auto T, auto V) {
+                        if constexpr (T() <= 8)
+                            k_split_small<T(), V()><<<(unsigned)nh, BT, 0, s>>>(Xp.p, dp, ids.p, D.p, lab.p, H);
+                    });
                 }
-                for (; nl > 0;) {
-                    // every iteration adds a distinct centre to some hub, so
-                    // no hub is active after n + 1 of them; a burst of up to
-                    // 16 may run past the last useful iteration
-                    if (iters > n + 2 + 16) CT_FAIL(CT_ECUDA, "split loop did not terminate");
-                    iters += burst;
-                    CT_CHECK_CUDA(cudaMemsetAsync(active.p, 0, 3 * sizeof(int32_t), s));
-                    if (l2) {
-                        // the level's first step by its own kernels; every later
-                        // step is taken inside the update pass by each hub's last block
-                        if (first_step) {
-                            CT_CHECK_CUDA(cudaMemsetAsync(arrive.p, 0, nh * sizeof(int32_t), s));
-                            k_hub_step<<<grid_for(nl), BT, 0, s>>>((int)nl, hl, H, active.p, cpos.p, 1);
-                            CT_COUNT_LAUNCH();
-                            switch (tpd) {
-#define CT_CD(T) case T: k_centre_dists<T><<<(unsigned)nl, BT, 0, s>>>(Xp.p, dp, ids.p, H, hl, cpos.p, dcc.p); break;
-                                CT_CD(1) CT_CD(2) CT_CD(4) CT_CD(8) CT_CD(16) CT_CD(32)
-#undef CT_CD
-                            }
-                            CT_COUNT_LAUNCH();
-                            prune = true;
-                            first_step = false;
-                        }
-                        const Step st{arrive.p, active.p, cpos.p, dcc.p};
-                        for (int it = 0; it < burst; ++it) update(H, nck, cb, cs, st);
-                    } else {
-                        // the level's first step by k_hub_step; every later step
-                        // is taken inside the update pass by each hub's last block
-                        if (first_step) {
-                            CT_CHECK_CUDA(cudaMemsetAsync(arrive.p, 0, nh * sizeof(int32_t), s));
-                            k_hub_step<<<grid_for(nl), BT, 0, s>>>((int)nl, hl, H, active.p, nullptr, ham ? 1 : 0);
-                            CT_COUNT_LAUNCH();
-                            first_step = false;
-                        }
-                        const Step st{arrive.p, active.p, nullptr, nullptr};
-                        for (int it = 0; it < burst; ++it) update(H, nck, cb, cs, st);
+                if (nl) {
+                    // the listed hubs' chunk table
+                    DBuf<int32_t> ccounts(nl, s);
+                    DBuf<int64_t> coff(nl, s);
+                    grow_chunks();
+                    if ((int64_t)bpos.n < (int64_t)nl * NET_M) bpos = DBuf<int32_t>((size_t)nl * NET_M, s);
+                    if (lev && (int64_t)lcn.n < nl) {
+                        lcn = DBuf<int32_t>(nl, s);
+                        lcpos = DBuf<int32_t>((size_t)nl * LEV_C, s);
+                        lcd = DBuf<float>((size_t)nl * LEV_C, s);
+                        lcpair = DBuf<uint16_t>((size_t)nl * LEV_C * LEV_C, s);
+                        lc = LevCands{lcn.p, lcd.p, lcpos.p, lcpair.p};
                     }
-                    k_active_hubs<<<grid_for(nh), BT, 0, s>>>((int)nh, H.done, hlist.p, active.p + 1);
+                    k_chunk_counts<<<grid_for(nl), BT, 0, s>>>(nl, hl_a.p, H.count, chunk_len, ccounts.p, hslot.p);
                     CT_COUNT_LAUNCH();
-                    if (nck) {
-                        k_active_chunks<<<grid_for(nck), BT, 0, s>>>(nck, cb, cs, H.done, cb2, cs2, active.p + 2);
-                        CT_COUNT_LAUNCH();
-                    }
+                    exclusive_scan_i32_to_i64(ccounts.p, coff.p, nl, nullptr, s);
+                    k_chunk_fill<<<grid_for(nchunks), BT, 0, s>>>(nchunks, nl, hl_a.p, H.begin, coff.p, chunk_len,
+                                                                  chunks_a.p);
+                    CT_COUNT_LAUNCH();
                     CT_LAUNCH_CHECK();
-                    int32_t act[3] = {0, 0, 0};
-                    to_host(act, active.p, 3, s);
-                    if (act[0] == 0) break;
-                    hl = hlist.p;
-                    nl = act[1];
-                    nck = act[2];
-                    std::swap(cb, cb2);
-                    std::swap(cs, cs2);
-                    if (nl == 0) break;
-                    burst = burst < 16 ? burst * 2 : 16;
+                    const Batch bt{bpos.p, cpos.p, dcc.p};
+                    int2 *hl = hl_a.p, *hl2 = hl_b.p;
+                    int4 *cl = chunks_a.p, *cl2 = chunks_b.p;
+                    int64_t nck = nchunks;
+                    // bursts of passes (the first compares nothing: it reports the farthest points), then the
+                    // hubs and chunks still splitting
+                    int64_t done_passes = 0;
+                    for (int burst = 2; nl > 0; burst = std::min(2 * burst, 8)) {
+                        // every pass gives each hub left a new centre: none is left after n + 1 passes
+                        if (done_passes > n + 2) CT_FAIL(CT_ECUDA, "split loop did not terminate");
+                        done_passes += burst;
+                        CT_CHECK_CUDA(cudaMemsetAsync(active.p, 0, 3 * sizeof(int32_t), s));
+                        for (int it = 0; it < burst; ++it) {
+                            update(H, nck, cl, bt, nullptr);
+                            select(H, nl, hl, coff.p, bt, active.p);
+                        }
+                        k_active<<<grid_for(std::max<int64_t>(nl, nck)), BT, 0, s>>>(nl, hl, nck, cl, H.done, hl2, cl2,
+                                                                                    active.p + 1);
+                        CT_COUNT_LAUNCH();
+                        CT_LAUNCH_CHECK();
+                        int32_t act[3] = {0, 0, 0};
+                        to_host(act, active.p, 3, s);
+                        nl = act[1];
+                        nck = act[2];
+                        std::swap(hl, hl2);
+                        std::swap(cl, cl2);
+                    }
                 }
             }
 
@@ -1505,24 +1846,28 @@ ct_tree *build_tree(const ct_points *pts, int zeta, int root, cudaStream_t s) {
             CT_COUNT_LAUNCH();
             k_child_keys<<<grid_for(R), BT, 0, s>>>(R, pk.p, rpos.p, D.p, ckey.p);
             CT_COUNT_LAUNCH();
-            k_link_children<<<grid_for(nh), BT, 0, s>>>((int)nh, H, child_base.p, n_nodes, cbeg.p, ccnt.p, lvl.p, par.p,
-                                                         leafy.p);
+            k_link_children<<<grid_for(T), BT, 0, s>>>(T, (int)nh, H, child_base.p, n_nodes, cbeg.p, ccnt.p, lvl.p,
+                                                       par.p, leafy.p);
             CT_COUNT_LAUNCH();
             k_make_nodes<<<grid_for(T), BT, 0, s>>>(T, n_nodes, zeta, pts->metric, cbegin.p, ccount.p, ckey.p,
                                                     nb.p, ncnt.p, cbeg.p, ccnt.p, rad.p, lvl.p, leafy.p, is_hub.p);
             CT_COUNT_LAUNCH();
             DBuf<int64_t> hub_off(T, s);
+            CT_CHECK_CUDA(cudaMemsetAsync(i64tmp.p + 1, 0, 2 * sizeof(int64_t), s));
             exclusive_scan_i32_to_i64(is_hub.p, hub_off.p, T, i64tmp.p, s);
-            int64_t nh2 = 0;
-            to_host(&nh2, i64tmp.p, 1, s);
-            if (nh2 > cap_h) CT_FAIL(CT_ECUDA, "hub capacity exceeded");
+            // a hub has more than zeta points: at most n / (zeta + 1) of them, within cap_h
             k_next_hubs<<<grid_for(T), BT, 0, s>>>(T, n_nodes, is_hub.p, hub_off.p, cbegin.p, ccount.p, ckey.p, lvl.p,
-                                                   H2);
+                                                   H2, small_max, chunk_len, hl_a.p,
+                                                   reinterpret_cast<int32_t *>(i64tmp.p + 1));
             CT_COUNT_LAUNCH();
             CT_LAUNCH_CHECK();
+            int64_t next[3] = {0, 0, 0};  // hubs; listed hubs (int32); their chunks (int32)
+            to_host(next, i64tmp.p, 3, s);
             n_nodes += (int)T;
             std::swap(H, H2);
-            nh = nh2;
+            nh = next[0];
+            nl = (int32_t)next[1];
+            nchunks = (int32_t)next[2];
         }
         int32_t e2 = 0;
         to_host(&e2, err.p, 1, s);
