@@ -23,6 +23,7 @@
 #include <cstring>
 #include <cuda.h>
 #include <mutex>
+#include <type_traits>
 
 #include "lev.cuh"
 #include "profile.cuh"
@@ -119,8 +120,12 @@ __device__ __forceinline__ int cloud_of_group(const Views &V, int gg) {
 //
 // One pass: every warp appends the candidate leaf blocks of its groups to
 // private chunks of a shared pool; a group's candidates form one or more
-// segments (group, pool offset, count).  If the pool runs out, the host reruns
-// the pass with the exact size.
+// segments (group, pool offset, count).  If the pool runs out, the walks stop
+// where they are: a warp that finds no chunk for its next step stores the
+// ranges on its stack, and the work it takes after that, in the resume list;
+// the host grows the pool and walks the list on.  (The pass used to be rerun
+// from the start: 19.5 of 63 ms on 121k x 16 uniform points and 23 of 60 ms
+// on a million codes went into two full passes.)
 
 constexpr int POOL_CHUNK = 2048;
 
@@ -133,8 +138,15 @@ struct Pool {
     int32_t *nseg;
     int64_t seg_cap;
     unsigned long long *total;  // candidates of all groups
-    int32_t *overflow;
+    int32_t *overflow;          // 1: out of chunks; 2: out of segments or of the resume list
+    // work left when the pool ran out, as items (group, first vertex, count or
+    // -1: the whole group); null: walks go on, counting without writing
+    int4 *resume = nullptr;
+    int32_t *n_resume = nullptr;
+    int32_t *n_whole = nullptr;  // whole groups among them
+    int resume_cap = 0;
 };
+constexpr int POOL_STOPPED = 1;
 
 // Walks stopped at a step limit leave their stack's ranges here, as items
 // (global group, first vertex, count, -) that the next round walks.
@@ -167,10 +179,44 @@ __device__ __forceinline__ void pool_close(const Pool &P, int g, PoolCursor &pc)
             P.seg_begin[idx] = pc.seg_begin;
             P.seg_count[idx] = pc.seg_count;
         } else {
-            atomicOr(P.overflow, 1);
+            atomicOr(P.overflow, 2);
         }
     }
     pc.seg_count = 0;
+}
+
+// A new chunk for the next step's 32 vertices; false when the pool is out.
+__device__ __forceinline__ bool pool_more(const Pool &P, int g, PoolCursor &pc) {
+    pool_close(P, g, pc);
+    unsigned long long c = 0ull;
+    if ((threadIdx.x & 31) == 0) {
+        c = atomicAdd(P.next, (unsigned long long)POOL_CHUNK);
+        if ((int64_t)c + POOL_CHUNK > P.cap) {
+            atomicOr(P.overflow, 1);
+            c = ~0ull;
+        }
+    }
+    c = __shfl_sync(0xffffffffu, c, 0);
+    if (c == ~0ull) {
+        pc.cur = -1;
+        pc.fill = POOL_CHUNK;
+        return false;
+    }
+    pc.cur = (int64_t)c;
+    pc.fill = 0;
+    pc.seg_begin = pc.cur;
+    return true;
+}
+__device__ __forceinline__ void resume_put(const Pool &P, int at, int4 item) {
+    if (at < P.resume_cap) P.resume[at] = item;
+    else atomicOr(P.overflow, 2);
+}
+// Leaves one work item (group, range; count 0: the whole group) for the next pass.
+__device__ __forceinline__ void resume_item(const Pool &P, int g, int2 start) {
+    if ((threadIdx.x & 31) == 0) {
+        if (start.y == 0) atomicAdd(P.n_whole, 1);
+        resume_put(P, atomicAdd(P.n_resume, 1), make_int4(g, start.x, start.y ? start.y : -1, 0));
+    }
 }
 
 // Appends the values of the lanes with `flag` set, in lane order.
@@ -223,9 +269,13 @@ __device__ __forceinline__ int walk_group(const TreeView &tv, int2 *__restrict__
                                           const Pool &P, PoolCursor &pc, unsigned long long &evals,
                                           int32_t *__restrict__ err, const Spill *sp, Tester tester) {
     const int lane = threadIdx.x & 31;
-    int n_cand = 0;
+    int n_cand = 0, status = 0;
     pc.seg_begin = pc.cur + pc.fill;
     pc.seg_count = 0;
+    if (P.resume && pc.fill > POOL_CHUNK - 32 && !pool_more(P, g, pc)) {
+        resume_item(P, g, start);
+        return POOL_STOPPED;
+    }
     if (start.y == 0 && tv.child_count[0] == 0) {  // the root is a leaf block: it is the only candidate
         pool_append(P, g, pc, lane == 0, 0u);
         n_cand = 1;
@@ -251,6 +301,18 @@ __device__ __forceinline__ int walk_group(const TreeView &tv, int2 *__restrict__
                 // (count 0, skipped), and the walk is finished here
                 for (int i = base + lane; i < sp->cap; i += 32) sp->items[i] = make_int4(g, 0, 0, 0);
                 limit = INT_MAX;
+            }
+            // resumable walks have room for every vertex of a step before it begins
+            if (P.resume && pc.fill > POOL_CHUNK - 32 && !pool_more(P, g, pc)) {
+                int base = 0;
+                if (lane == 0) base = atomicAdd(P.n_resume, top);
+                base = __shfl_sync(0xffffffffu, base, 0);
+                for (int i = lane; i < top; i += 32) {
+                    const int2 r = stack[i];
+                    resume_put(P, base + i, make_int4(g, r.x, r.y, 0));
+                }
+                status = POOL_STOPPED;
+                break;
             }
             // the step's vertices: the top ranges of the stack, newest first,
             // until the 32 lanes are filled (lane i reads the i-th range from
@@ -309,7 +371,7 @@ __device__ __forceinline__ int walk_group(const TreeView &tv, int2 *__restrict__
     }
     pool_close(P, g, pc);
     if (lane == 0) atomicAdd(P.total, (unsigned long long)n_cand);
-    return 0;
+    return status;
 }
 
 // Vertices the warp tested for group g (for fitting the predictor; the rounds
@@ -393,6 +455,7 @@ __global__ void __launch_bounds__(TRAV_WARPS * 32, 8) k_traverse_l2(
     }
     const int n_work = in_items ? min(*in_count, in_cap) : n_order;
     const Spill *sp = out.items ? &out : nullptr;
+    bool full = false;  // the pool had no chunk for this warp
     for (;;) {
         // work is taken dynamically: walks differ widely in length
         int gi = 0;
@@ -403,11 +466,15 @@ __global__ void __launch_bounds__(TRAV_WARPS * 32, 8) k_traverse_l2(
         int2 start = make_int2(0, 0);
         if (in_items) {
             const int4 w = in_items[gi];
-            if (w.z <= 0) continue;  // an empty range (a stop that did not fit)
+            if (w.z == 0) continue;  // an empty range (a stop that did not fit)
             gg = w.x;
-            start = make_int2(w.y, w.z);
+            if (w.z > 0) start = make_int2(w.y, w.z);
         } else {
             gg = order[gi];
+        }
+        if (full) {
+            resume_item(P, gg, start);
+            continue;
         }
         const int c = cloud_of_group(V, gg);
         const TreeView &tv = V.tv[c];
@@ -427,7 +494,9 @@ __global__ void __launch_bounds__(TRAV_WARPS * 32, 8) k_traverse_l2(
             }
         };
         const unsigned long long e0 = evals;
-        if (walk_group(tv, stack, cap, gg, start, P, pc, evals, err, sp, tester) < 0) return;
+        const int ws = walk_group(tv, stack, cap, gg, start, P, pc, evals, err, sp, tester);
+        if (ws < 0) return;
+        full = ws == POOL_STOPPED;
         if (gvisit) group_visits(gvisit, gg, evals - e0);
         __syncwarp();
     }
@@ -458,6 +527,7 @@ __global__ void __launch_bounds__(32) k_traverse_lev(
     }
     const int n_work = in_items ? min(*in_count, in_cap) : tv.n_groups;
     const Spill *sp = out.items ? &out : nullptr;
+    bool full = false;  // the pool had no chunk for this warp
     for (;;) {
         int gi = 0;
         if (lane == 0) gi = atomicAdd(next_group, 1);
@@ -467,11 +537,15 @@ __global__ void __launch_bounds__(32) k_traverse_lev(
         int2 start = make_int2(0, 0);
         if (in_items) {
             const int4 w = in_items[gi];
-            if (w.z <= 0) continue;  // an empty range (a stop that did not fit)
+            if (w.z == 0) continue;  // an empty range (a stop that did not fit)
             g = w.x;
-            start = make_int2(w.y, w.z);
+            if (w.z > 0) start = make_int2(w.y, w.z);
         } else {
             g = tv.group_order[gi];
+        }
+        if (full) {
+            resume_item(P, g, start);
+            continue;
         }
         int cpos = tv.group_begin[g];
         const uint8_t *pat = tv.sdata + tv.soff[cpos];
@@ -489,7 +563,9 @@ __global__ void __launch_bounds__(32) k_traverse_lev(
             return lev_myers<W>(peq, m, txt, n, k) <= k;
         };
         const unsigned long long e0 = evals;
-        if (walk_group(tv, stack, cap, g, start, P, pc, evals, err, sp, tester) < 0) return;
+        const int ws = walk_group(tv, stack, cap, g, start, P, pc, evals, err, sp, tester);
+        if (ws < 0) return;
+        full = ws == POOL_STOPPED;
         if (gvisit) group_visits(gvisit, g, evals - e0);
         __syncwarp();
     }
@@ -540,6 +616,7 @@ __global__ void __launch_bounds__(32) k_traverse_ham(
     }
     const int n_work = in_items ? min(*in_count, in_cap) : tv.n_groups;
     const Spill *sp = out.items ? &out : nullptr;
+    bool full = false;  // the pool had no chunk for this warp
     for (;;) {
         int gi = 0;
         if (lane == 0) gi = atomicAdd(next_group, 1);
@@ -549,11 +626,15 @@ __global__ void __launch_bounds__(32) k_traverse_ham(
         int2 start = make_int2(0, 0);
         if (in_items) {
             const int4 w = in_items[gi];
-            if (w.z <= 0) continue;  // an empty range (a stop that did not fit)
+            if (w.z == 0) continue;  // an empty range (a stop that did not fit)
             g = w.x;
-            start = make_int2(w.y, w.z);
+            if (w.z > 0) start = make_int2(w.y, w.z);
         } else {
             g = tv.group_order[gi];
+        }
+        if (full) {
+            resume_item(P, g, start);
+            continue;
         }
         const uint4 *crow = reinterpret_cast<const uint4 *>(tv.bits + (size_t)tv.group_begin[g] * tv.wp);
         __syncwarp();
@@ -567,7 +648,9 @@ __global__ void __launch_bounds__(32) k_traverse_ham(
             return ham_rows(cen, row, nq) <= k;
         };
         const unsigned long long e0 = evals;
-        if (walk_group(tv, stack, cap, g, start, P, pc, evals, err, sp, tester) < 0) return;
+        const int ws = walk_group(tv, stack, cap, g, start, P, pc, evals, err, sp, tester);
+        if (ws < 0) return;
+        full = ws == POOL_STOPPED;
         if (gvisit) group_visits(gvisit, g, evals - e0);
         __syncwarp();
     }
@@ -3273,11 +3356,15 @@ int64_t pool_capacity_guess(int64_t n, int64_t G, const TravLaunch &tl) {
 void launch_traversal(const Views &V, int64_t G, int max_dp, int max_len, bool l2, const int32_t *order,
                       const Pool &P, int2 *stacks, int cap, const TravLaunch &tl, unsigned long long *st,
                       int32_t *err, int32_t *next_group, int4 *const spill[2], int32_t *spill_cnt, int spill_cap,
-                      longlong2 *cursors, cudaStream_t s, int32_t *gvisit = nullptr) {
+                      longlong2 *cursors, cudaStream_t s, int32_t *gvisit = nullptr, const int4 *resumed = nullptr,
+                      const int32_t *n_resumed = nullptr, int resumed_cap = 0) {
     // P.next .. P.overflow are the four 64-bit words of one counter block
+    // (kept when a resume list is walked on, as are gvisit and the cursors)
     CT_CHECK_CUDA(cudaMemsetAsync(next_group, 0, sizeof(int32_t), s));
-    CT_CHECK_CUDA(cudaMemsetAsync(P.next, 0, 4 * sizeof(unsigned long long), s));
-    if (gvisit && G > 0) CT_CHECK_CUDA(cudaMemsetAsync(gvisit, 0, (size_t)G * sizeof(int32_t), s));
+    if (!resumed) {
+        CT_CHECK_CUDA(cudaMemsetAsync(P.next, 0, 4 * sizeof(unsigned long long), s));
+        if (gvisit && G > 0) CT_CHECK_CUDA(cudaMemsetAsync(gvisit, 0, (size_t)G * sizeof(int32_t), s));
+    }
     if (G == 0) return;
     if (l2) {
         const size_t tsm = (size_t)TRAV_WARPS * max_dp * sizeof(float);
@@ -3285,8 +3372,9 @@ void launch_traversal(const Views &V, int64_t G, int max_dp, int max_len, bool l
             CT_CHECK_CUDA(cudaFuncSetAttribute(k_traverse_l2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tsm));
         CT_CHECK_CUDA(cudaMemsetAsync(spill_cnt, 0, 2 * sizeof(int32_t), s));
         for (int r = 0; r <= TRAV_ROUNDS; ++r) {
-            const int4 *in = r ? spill[(r - 1) & 1] : nullptr;
-            const int32_t *in_cnt = r ? spill_cnt + ((r - 1) & 1) : nullptr;
+            const int4 *in = r ? spill[(r - 1) & 1] : resumed;
+            const int32_t *in_cnt = r ? spill_cnt + ((r - 1) & 1) : n_resumed;
+            const int in_cap = r ? spill_cap : resumed_cap;
             Spill out{nullptr, spill_cnt + (r & 1), spill_cap, INT_MAX};
             if (r < TRAV_ROUNDS) {
                 out.items = spill[r & 1];
@@ -3296,7 +3384,7 @@ void launch_traversal(const Views &V, int64_t G, int max_dp, int max_len, bool l
                 CT_CHECK_CUDA(cudaMemsetAsync(next_group, 0, sizeof(int32_t), s));
                 CT_CHECK_CUDA(cudaMemsetAsync(spill_cnt + (r & 1), 0, sizeof(int32_t), s));
             }
-            k_traverse_l2<<<tl.blocks, TRAV_WARPS * 32, tsm, s>>>(V, order, (int)G, in, in_cnt, spill_cap, out, P,
+            k_traverse_l2<<<tl.blocks, TRAV_WARPS * 32, tsm, s>>>(V, order, (int)G, in, in_cnt, in_cap, out, P,
                                                                    cursors, stacks, cap, st, err, next_group,
                                                                    gvisit, max_dp >> 2);
             CT_COUNT_LAUNCH();
@@ -3308,8 +3396,9 @@ void launch_traversal(const Views &V, int64_t G, int max_dp, int max_len, bool l
         const bool ham = tv.wp != 0;
         CT_CHECK_CUDA(cudaMemsetAsync(spill_cnt, 0, 2 * sizeof(int32_t), s));
         for (int r = 0; r <= TRAV_ROUNDS; ++r) {
-            const int4 *in = r ? spill[(r - 1) & 1] : nullptr;
-            const int32_t *in_cnt = r ? spill_cnt + ((r - 1) & 1) : nullptr;
+            const int4 *in = r ? spill[(r - 1) & 1] : resumed;
+            const int32_t *in_cnt = r ? spill_cnt + ((r - 1) & 1) : n_resumed;
+            const int in_cap = r ? spill_cap : resumed_cap;
             Spill out{nullptr, spill_cnt + (r & 1), spill_cap, INT_MAX};
             if (r < TRAV_ROUNDS) {
                 out.items = spill[r & 1];
@@ -3320,12 +3409,12 @@ void launch_traversal(const Views &V, int64_t G, int max_dp, int max_len, bool l
                 CT_CHECK_CUDA(cudaMemsetAsync(spill_cnt + (r & 1), 0, sizeof(int32_t), s));
             }
             if (ham) {
-                k_traverse_ham<<<tl.blocks, 32, 0, s>>>(tv, V.qp[0], in, in_cnt, spill_cap, out, P, cursors, stacks,
+                k_traverse_ham<<<tl.blocks, 32, 0, s>>>(tv, V.qp[0], in, in_cnt, in_cap, out, P, cursors, stacks,
                                                         cap, st, err, next_group, gvisit);
             } else {
                 switch (lev_words_for(max_len)) {
 #define CT_TL(WW) \
-    case WW: k_traverse_lev<WW><<<tl.blocks, 32, 0, s>>>(tv, V.qp[0], in, in_cnt, spill_cap, out, P, cursors, stacks, cap, st, err, next_group, gvisit); break;
+    case WW: k_traverse_lev<WW><<<tl.blocks, 32, 0, s>>>(tv, V.qp[0], in, in_cnt, in_cap, out, P, cursors, stacks, cap, st, err, next_group, gvisit); break;
                     CT_TL(1) CT_TL(2) CT_TL(4) CT_TL(8) CT_TL(16)
 #undef CT_TL
                 }
@@ -3526,33 +3615,81 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
     DBuf<int32_t> spill_cnt(2, s);
     int4 *const spills[2] = {spill_a.p, spill_b.p};
     DBuf<longlong2> cursors(tl.warps, s);
-    int64_t pool_cap = pool_capacity_guess(n, G, tl);
+    // a pool of whole chunks; work left when it runs out goes to a resume list
+    // (at most every group, a full spill buffer a round and the stacks of the
+    // warps; a list that is too short restarts the pass with a larger pool)
+    int64_t pool_cap = ceil_div(pool_capacity_guess(n, G, tl), POOL_CHUNK) * POOL_CHUNK;
+    const int resume_cap = (int)std::min<int64_t>(G + 2LL * spill_cap + 65536, 1 << 26);
     DBuf<uint32_t> pool;
+    DBuf<int4> resume[2];
+    DBuf<int32_t> rctr(3, s);  // entries of the two lists, whole groups
     DBuf<int32_t> seg_group, seg_count;
     DBuf<int64_t> seg_begin;
     unsigned long long hc[4] = {0, 0, 0, 0};
+    int64_t seg_cap = 0;
     Pool P{};
-    for (int attempt = 0;; ++attempt) {
+    for (int pass = 0;; ++pass) {
         // a segment per walk (groups, stored ranges) and per chunk a walk crosses
-        const int64_t seg_cap = G + (int64_t)TRAV_ROUNDS * spill_cap + pool_cap / POOL_CHUNK + tl.warps + 16;
-        pool = DBuf<uint32_t>(pool_cap, s);
-        seg_group = DBuf<int32_t>(seg_cap, s);
-        seg_count = DBuf<int32_t>(seg_cap, s);
-        seg_begin = DBuf<int64_t>(seg_cap, s);
+        const int64_t old_seg = seg_cap, nseg0 = pass ? (int64_t)(uint32_t)hc[1] : 0;
+        seg_cap = old_seg + G + (int64_t)TRAV_ROUNDS * spill_cap + pool_cap / POOL_CHUNK + tl.warps + 16 +
+                  (pass ? resume_cap : 0);
+        auto grown = [&](auto &buf, int64_t cap_new, int64_t used) {  // a larger copy
+            std::decay_t<decltype(buf)> b((size_t)cap_new, s);
+            if (used) CT_CHECK_CUDA(cudaMemcpyAsync(b.p, buf.p, (size_t)used * sizeof(*b.p), cudaMemcpyDeviceToDevice, s));
+            buf = std::move(b);
+        };
+        grown(pool, pool_cap, pass ? P.cap : 0);
+        grown(seg_group, seg_cap, nseg0);
+        grown(seg_count, seg_cap, nseg0);
+        grown(seg_begin, seg_cap, nseg0);
+        const int cur = pass & 1;  // this pass writes list cur and reads the other
+        if (!resume[cur].p) resume[cur] = DBuf<int4>(resume_cap, s);
+        CT_CHECK_CUDA(cudaMemsetAsync(rctr.p + cur, 0, sizeof(int32_t), s));
+        CT_CHECK_CUDA(cudaMemsetAsync(rctr.p + 2, 0, sizeof(int32_t), s));
         P = Pool{pool.p, pool_cap, ctr.p, seg_group.p, seg_count.p, seg_begin.p,
-                 reinterpret_cast<int32_t *>(ctr.p + 1), seg_cap, ctr.p + 2, reinterpret_cast<int32_t *>(ctr.p + 3)};
+                 reinterpret_cast<int32_t *>(ctr.p + 1), seg_cap, ctr.p + 2, reinterpret_cast<int32_t *>(ctr.p + 3),
+                 resume[cur].p, rctr.p + cur, rctr.p + 2, resume_cap};
         {
             ProfScope ps("traverse", s);
             launch_traversal(V, G, max_dp, max_len, l2, order, P, stacks.p, cap, tl, st.p, err, next_group.p, spills,
-                             spill_cnt.p, spill_cap, cursors.p, s, gvisit);
+                             spill_cnt.p, spill_cap, cursors.p, s, gvisit, pass ? resume[cur ^ 1].p : nullptr,
+                             rctr.p + (cur ^ 1), resume_cap);
         }
         to_host(hc, ctr.p, 4, s);
-        if (!(uint32_t)hc[3]) break;
-        if (attempt >= 1) CT_FAIL(CT_ECUDA, "candidate pool overflowed twice");
-        pool_cap = (int64_t)hc[2] + 2LL * tl.warps * POOL_CHUNK + POOL_CHUNK;
-        CT_CHECK_CUDA(cudaMemsetAsync(st.p, 0, ST_N * sizeof(unsigned long long), s));
+        const uint32_t full = (uint32_t)hc[3];
+        if (!full) break;
+        if (pass >= 16) CT_FAIL(CT_ECUDA, "the candidate pool overflowed %d times", pass);
+        // the size the walked groups ask for (the longest walks come first), at
+        // least double, within half of the free memory if that is still larger
+        int32_t whole = 0;
+        to_host(&whole, rctr.p + 2, 1, s);
+        const double walked = std::max(1.0, (double)(G - whole));
+        double want = std::max(2.0 * (double)pool_cap,
+                               1.1 * (double)hc[2] * (double)G / walked + 2.0 * (double)tl.warps * POOL_CHUNK);
+        size_t fr = 0, tot = 0;
+        if (cudaMemGetInfo(&fr, &tot) == cudaSuccess) {
+            const double lim = std::max(1.125 * (double)pool_cap, (double)fr / 2 / sizeof(uint32_t));
+            want = std::min(want, lim);
+        } else {
+            cudaGetLastError();
+        }
+        const unsigned long long used = (unsigned long long)pool_cap;
+        pool_cap = ceil_div((int64_t)want, POOL_CHUNK) * POOL_CHUNK;
+        if (full & 2u) {  // work was lost: from the start
+            pass = -1;
+            pool.reset();
+            seg_cap = 0;
+            CT_CHECK_CUDA(cudaMemsetAsync(st.p, 0, ST_N * sizeof(unsigned long long), s));
+            continue;
+        }
+        // every chunk below the old capacity is taken; the counters of the walked part stay
+        CT_CHECK_CUDA(cudaMemcpyAsync(ctr.p, &used, sizeof(used), cudaMemcpyHostToDevice, s));
+        CT_CHECK_CUDA(cudaMemsetAsync(ctr.p + 3, 0, sizeof(unsigned long long), s));
+        CT_CHECK_CUDA(cudaStreamSynchronize(s));  // `used` is on the stack
     }
     stacks.reset();
+    resume[0].reset();
+    resume[1].reset();
     const int64_t n_cand = (int64_t)hc[2];
     int nseg = (int)(uint32_t)hc[1];
     // each group's candidates in one range (segments become one per group)
