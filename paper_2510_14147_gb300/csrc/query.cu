@@ -1721,62 +1721,118 @@ constexpr int TC_KL = 1024;             // kept pairs rechecked per round
 // which keeps every edge with a 4x margin on the fp32 terms.  The slack
 // relative to eps grows with |x - m| / eps (about 2^-10 of it); rows are
 // copied into the MMA's layout unchanged, so the count pass converts nothing.
-constexpr int H16_MB = 1024;  // blocks of the column-mean partial sums
+//
+// Any m keeps the bound; the column means only keep |x - m| small, so they are
+// taken from a strided sample of at most H16_SAMPLE points.  The three
+// launches serve every cloud of a batch (a serial sum of 1024 partials per
+// cloud used to take 83 us each: 1.9 ms for 20 clouds, 5.0 ms for 60, now
+// 0.1 and 0.2; 1M x 128: 0.36 -> 0.17 ms, bound by its 0.77 GB of traffic).
+constexpr int H16_MB = 64;        // blocks of a cloud's column sums
+constexpr int H16_SAMPLE = 16384; // points of a cloud's column sums
+constexpr int H16_T = 256;
 constexpr float H16_REL = 0x1.01p-11f, H16_ABS = 0x1p-20f, H16_ABS2 = 0x1p-14f;
 constexpr float H16_NORM_UP = 1.0f + 0x1p-16f;
 
-// Partial column sums: block b adds points b, b + H16_MB, ...; thread k is
-// coordinate k (dp <= 128).
-__global__ void k_col_partial(const float *__restrict__ pts, int64_t n, int dp, float *__restrict__ partial) {
-    const int k = threadIdx.x;
-    if (k >= dp) return;
-    float acc = 0.f;
-    for (int64_t i = blockIdx.x; i < n; i += gridDim.x) acc += __ldg(pts + i * dp + k);
-    partial[(size_t)blockIdx.x * dp + k] = acc;
+// Per cloud: its fp16 rows, norms, means and {s, s eps_up} (null: FP32 tiles).
+struct H16Out {
+    uint4 *h16[kMaxClouds];
+    float *n16[kMaxClouds], *mean[kMaxClouds], *scal[kMaxClouds];
+};
+
+// Partial column sums of a cloud's sample: block (b, cloud) adds the sampled
+// points b R, b R + 1, ... (R rows of dp / 4 threads at a time; dp <= 128).
+__global__ void __launch_bounds__(H16_T) k_h16_sums(const __grid_constant__ Views V, float *__restrict__ partial) {
+    const int c = blockIdx.y;
+    if (!V.h16[c]) return;
+    const int64_t n = V.rbase[c + 1] - V.rbase[c];
+    const int64_t ns = n < H16_SAMPLE ? n : H16_SAMPLE, step = n / ns;
+    const int nq = V.tv[c].dp >> 2, R = H16_T / nq, r = threadIdx.x / nq, q = threadIdx.x % nq;
+    __shared__ float4 sh[H16_T];
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (r < R) {
+        for (int64_t i = (int64_t)blockIdx.x * R + r; i < ns; i += (int64_t)gridDim.x * R) {
+            const float4 x = __ldg(reinterpret_cast<const float4 *>(V.tv[c].pts) + i * step * nq + q);
+            acc.x += x.x;
+            acc.y += x.y;
+            acc.z += x.z;
+            acc.w += x.w;
+        }
+    }
+    sh[threadIdx.x] = acc;
+    __syncthreads();
+    if (r == 0) {
+        for (int k = 1; k < R; ++k) {
+            const float4 x = sh[k * nq + q];
+            acc.x += x.x;
+            acc.y += x.y;
+            acc.z += x.z;
+            acc.w += x.w;
+        }
+        reinterpret_cast<float4 *>(partial)[((size_t)c * H16_MB + blockIdx.x) * 32 + q] = acc;
+    }
 }
 
-// Column means (partials added in block order) and the scale: every point is
-// within r_root of the root centre, so |x_k - m_k| <= |x - m| <= 2 r_root;
-// s = 2^(14 - e) with max(2 r_root, eps) < 2^e.  scal = {s, s eps_up}.
-__global__ void k_col_final(const float *__restrict__ partial, int dp, int64_t n, const float *__restrict__ radius,
-                            float eps_up, float *__restrict__ mean, float *__restrict__ scal) {
-    const int k = threadIdx.x;
-    if (k < dp) {
+// Column means and the scale of each cloud: every point is within r_root of
+// the root centre, and so is the sample's mean, so |x_k - m_k| <= |x - m| <=
+// 2 r_root; s = 2^(14 - e) with max(2 r_root, eps) < 2^e.  scal = {s, s eps_up}.
+__global__ void __launch_bounds__(128) k_h16_means(const __grid_constant__ Views V,
+                                                   const __grid_constant__ H16Out out,
+                                                   const float *__restrict__ partial) {
+    const int c = blockIdx.x, k = threadIdx.x;
+    if (!V.h16[c]) return;
+    const int64_t n = V.rbase[c + 1] - V.rbase[c];
+    const int64_t ns = n < H16_SAMPLE ? n : H16_SAMPLE;
+    if (k < V.tv[c].dp) {
         double acc = 0.0;
-        for (int b = 0; b < H16_MB; ++b) acc += (double)partial[(size_t)b * dp + k];
-        mean[k] = n ? (float)(acc / (double)n) : 0.f;
+#pragma unroll 16
+        for (int b = 0; b < H16_MB; ++b) acc += (double)partial[((size_t)c * H16_MB + b) * 128 + k];
+        out.mean[c][k] = (float)(acc / (double)ns);
     }
     if (k == 0) {
-        const float M = fmaxf(2.0f * radius[0] * (1.0f + 0x1p-10f), eps_up);
+        const float eps_up = V.qp[c].eps_up;
+        const float M = fmaxf(2.0f * V.tv[c].radius[0] * (1.0f + 0x1p-10f), eps_up);
         float s = 0x1p-100f;
         if (M <= 0x1p100f) {
             int e;
             frexpf(fmaxf(M, 0x1p-100f), &e);  // M < 2^e
             s = ldexpf(1.0f, 14 - e);
         }
-        scal[0] = s;
-        scal[1] = s * eps_up;
+        out.scal[c][0] = s;
+        out.scal[c][1] = s * eps_up;
     }
 }
 
 // Rows in tree order -> fp16 rows and their squared norms; sixteen lanes per
-// row, lane j converts halves 8j .. 8j + 7 (one 16-byte chunk).
-__global__ void k_to_h16(const float *__restrict__ pts, int64_t n, int dp, int kp, const float *__restrict__ mean,
-                         const float *__restrict__ scal, uint4 *__restrict__ h16, float *__restrict__ n16) {
+// row (of all clouds, concatenated), lane j converts halves 8j .. 8j + 7 (one
+// 16-byte chunk).
+__global__ void __launch_bounds__(H16_T) k_to_h16(const __grid_constant__ Views V,
+                                                  const __grid_constant__ H16Out out) {
     const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t row = gid >> 4;
-    const int j = (int)(gid & 15), kc = kp >> 3;
-    const float s = scal[0];
+    const int64_t grow = gid >> 4;
+    const int j = (int)(gid & 15);
+    int c = 0;
+    if (V.nc > 1) {
+        int lo = 0, hi = V.nc;
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (V.rbase[mid] <= grow) lo = mid; else hi = mid;
+        }
+        c = lo;
+    }
+    const bool on = grow < V.rbase[V.nc] && V.h16[c];
+    const int64_t row = grow - V.rbase[c];
+    const int dp = V.tv[c].dp, kc = 8 * ((dp + 63) >> 6);
     float sq = 0.f;
-    if (row < n && j < kc) {
+    if (on && j < kc) {
+        const float s = out.scal[c][0];
         float v[8];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int k = 8 * j + 4 * h;
             float4 x = make_float4(0.f, 0.f, 0.f, 0.f), m = x;
             if (k < dp) {  // dp is a multiple of 4
-                x = __ldg(reinterpret_cast<const float4 *>(pts + row * dp + k));
-                m = __ldg(reinterpret_cast<const float4 *>(mean + k));
+                x = __ldg(reinterpret_cast<const float4 *>(V.tv[c].pts + row * dp + k));
+                m = __ldg(reinterpret_cast<const float4 *>(out.mean[c] + k));
             }
             v[4 * h + 0] = (x.x - m.x) * s;
             v[4 * h + 1] = (x.y - m.y) * s;
@@ -1792,11 +1848,11 @@ __global__ void k_to_h16(const float *__restrict__ pts, int64_t n, int dp, int k
             sq = fmaf(f.x, f.x, sq);
             sq = fmaf(f.y, f.y, sq);
         }
-        h16[row * kc + j] = make_uint4(w[0], w[1], w[2], w[3]);
+        out.h16[c][row * kc + j] = make_uint4(w[0], w[1], w[2], w[3]);
     }
 #pragma unroll
     for (int o = 8; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o, 16);
-    if (j == 0 && row < n) n16[row] = sq;
+    if (on && j == 0) out.n16[c][row] = sq;
 }
 
 constexpr int TC_T = 256;   // threads per CTA (two CTAs per SM)
@@ -3526,34 +3582,50 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
     }
     if (V.rbase[C] >= 0x7fffffffLL) CT_FAIL(CT_EOVERFLOW, "a batch above 2^31 points");
     // fp16 rows of the clouds that take the tensor-core filter
-    std::vector<DBuf<uint4>> h16s;
-    std::vector<DBuf<float>> f16s;
+    DBuf<uint4> h16s;
+    DBuf<float> f16s;  // per cloud: means (dp), {s, s eps_up, -, -}, norms (n, rounded up to 4)
     if (any_tc) {
         ProfScope ps("rows_f16", s);
-        DBuf<float> partial;
+        int64_t rows = 0, floats = 0;
+        for (int c = 0; c < C; ++c) {
+            if (!V.use_tc[c]) continue;
+            const int dp = trees[c]->dp;
+            rows += trees[c]->n * (8 * ((dp + 63) / 64));  // rows of 64-half K blocks
+            floats += dp + 4 + ceil_div(trees[c]->n, 4) * 4;
+        }
+        h16s = DBuf<uint4>((size_t)(rows ? rows : 1), s);
+        f16s = DBuf<float>((size_t)(floats ? floats : 1), s);
+        DBuf<float> partial((size_t)C * H16_MB * 128, s);
+        H16Out ho{};
+        rows = floats = 0;
+        bool any = false;
         for (int c = 0; c < C; ++c) {
             if (!V.use_tc[c]) continue;
             const ct_tree *tc = trees[c];
-            const int64_t nc = tc->n;
-            if (nc == 0) continue;  // no work items
-            const int dp = tc->dp, kp = 64 * ((dp + 63) / 64);  // rows of 64-half K blocks
-            h16s.emplace_back((size_t)nc * (kp / 8), s);
-            f16s.emplace_back((size_t)dp + 4 + nc, s);  // means (dp: a multiple of 4), {s, s eps_up}, norms
-            float *mean = f16s.back().p, *scal = mean + dp, *nrm = scal + 4;
-            partial.grow((size_t)H16_MB * dp);
-            k_col_partial<<<H16_MB, 128, 0, s>>>(tc->pts, nc, dp, partial.p);
+            if (tc->n == 0) continue;  // no work items
+            any = true;
+            const int dp = tc->dp, kp = 64 * ((dp + 63) / 64);
+            ho.h16[c] = h16s.p + rows;
+            ho.mean[c] = f16s.p + floats;
+            ho.scal[c] = ho.mean[c] + dp;
+            ho.n16[c] = ho.scal[c] + 4;
+            rows += tc->n * (kp / 8);
+            floats += dp + 4 + ceil_div(tc->n, 4) * 4;
+            encode_rows_f16(&V.tmap[c], ho.h16[c], tc->n, kp);
+            V.h16[c] = ho.h16[c];
+            V.n16[c] = ho.n16[c];
+            V.s16[c] = ho.scal[c];
+        }
+        if (any) {
+            k_h16_sums<<<dim3(H16_MB, (unsigned)C), H16_T, 0, s>>>(V, partial.p);
             CT_COUNT_LAUNCH();
             CT_LAUNCH_CHECK();
-            k_col_final<<<1, 128, 0, s>>>(partial.p, dp, nc, tc->radius, V.qp[c].eps_up, mean, scal);
+            k_h16_means<<<(unsigned)C, 128, 0, s>>>(V, ho, partial.p);
             CT_COUNT_LAUNCH();
             CT_LAUNCH_CHECK();
-            k_to_h16<<<grid_for(nc * 16, 256), 256, 0, s>>>(tc->pts, nc, dp, kp, mean, scal, h16s.back().p, nrm);
+            k_to_h16<<<grid_for(V.rbase[C] * 16, H16_T), H16_T, 0, s>>>(V, ho);
             CT_COUNT_LAUNCH();
             CT_LAUNCH_CHECK();
-            encode_rows_f16(&V.tmap[c], h16s.back().p, nc, kp);
-            V.h16[c] = h16s.back().p;
-            V.n16[c] = nrm;
-            V.s16[c] = scal;
         }
     }
     const int64_t n = V.rbase[C];
