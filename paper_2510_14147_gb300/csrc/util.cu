@@ -131,8 +131,10 @@ __device__ __forceinline__ int64_t block_exclusive_scan(int64_t v, int64_t *sh, 
     return warp_prefix + x - v;
 }
 
-// Single-block exclusive scan over `n` int64 (n up to any size, looped).
-__global__ void k_scan_single(int64_t *__restrict__ a, int64_t n, int64_t *__restrict__ total_dev) {
+// Single-block exclusive scan over `n` values (n up to any size, looped); out
+// may alias in.
+template <class T>
+__global__ void k_scan_single(const T *in, int64_t *out, int64_t n, int64_t *__restrict__ total_dev) {
     __shared__ int64_t sh[32];
     int64_t carry = 0;
     for (int64_t base = 0; base < n; base += (int64_t)blockDim.x * SCAN_ITEMS) {
@@ -140,14 +142,14 @@ __global__ void k_scan_single(int64_t *__restrict__ a, int64_t n, int64_t *__res
         int64_t loc = 0;
         int64_t idx0 = base + (int64_t)threadIdx.x * SCAN_ITEMS;
         for (int i = 0; i < SCAN_ITEMS; ++i) {
-            v[i] = idx0 + i < n ? a[idx0 + i] : 0;
+            v[i] = idx0 + i < n ? (int64_t)in[idx0 + i] : 0;
             loc += v[i];
         }
         int64_t tot;
         int64_t pre = block_exclusive_scan(loc, sh, tot);
         int64_t run = carry + pre;
         for (int i = 0; i < SCAN_ITEMS; ++i) {
-            if (idx0 + i < n) a[idx0 + i] = run;
+            if (idx0 + i < n) out[idx0 + i] = run;
             run += v[i];
         }
         carry += tot;
@@ -175,6 +177,19 @@ __global__ void k_tile_scan(const T *__restrict__ in, int64_t *__restrict__ out,
     }
 }
 
+// Up to SCAN_SMALL values one block scans them in one launch of about 4 us per
+// 8192 (the three launches take 9 us whatever the size; the lines cross at
+// about 20000).
+constexpr int64_t SCAN_SMALL = 16384;
+template <class T>
+static bool scan_small(const T *in, int64_t *out, int64_t n, int64_t *total_dev, cudaStream_t s) {
+    if (n > SCAN_SMALL) return false;
+    k_scan_single<T><<<1, 1024, 0, s>>>(in, out, n, total_dev);
+    CT_COUNT_LAUNCH();
+    CT_LAUNCH_CHECK();
+    return true;
+}
+
 template <class T>
 static void exclusive_scan_impl(const T *in, int64_t *out, int64_t n, int64_t *total_dev,
                                 cudaStream_t s) {
@@ -182,11 +197,12 @@ static void exclusive_scan_impl(const T *in, int64_t *out, int64_t n, int64_t *t
         if (total_dev) CT_CHECK_CUDA(cudaMemsetAsync(total_dev, 0, sizeof(int64_t), s));
         return;
     }
+    if (scan_small(in, out, n, total_dev, s)) return;
     int64_t tiles = ceil_div(n, SCAN_TILE);
     DBuf<int64_t> sums(tiles, s);
     k_tile_sums<T><<<(unsigned)tiles, SCAN_THREADS, 0, s>>>(in, n, sums.p);
     CT_COUNT_LAUNCH();
-    k_scan_single<<<1, 1024, 0, s>>>(sums.p, tiles, total_dev);
+    k_scan_single<int64_t><<<1, 1024, 0, s>>>(sums.p, sums.p, tiles, total_dev);
     CT_COUNT_LAUNCH();
     k_tile_scan<T><<<(unsigned)tiles, SCAN_THREADS, 0, s>>>(in, out, n, sums.p);
     CT_COUNT_LAUNCH();
@@ -206,10 +222,11 @@ void exclusive_scan_i32_to_i64_into(const int32_t *in, int64_t *out, int64_t n, 
         if (total_dev) CT_CHECK_CUDA(cudaMemsetAsync(total_dev, 0, sizeof(int64_t), s));
         return;
     }
+    if (scan_small(in, out, n, total_dev, s)) return;
     int64_t tiles = ceil_div(n, SCAN_TILE);
     k_tile_sums<int32_t><<<(unsigned)tiles, SCAN_THREADS, 0, s>>>(in, n, tile_sums);
     CT_COUNT_LAUNCH();
-    k_scan_single<<<1, 1024, 0, s>>>(tile_sums, tiles, total_dev);
+    k_scan_single<int64_t><<<1, 1024, 0, s>>>(tile_sums, tile_sums, tiles, total_dev);
     CT_COUNT_LAUNCH();
     k_tile_scan<int32_t><<<(unsigned)tiles, SCAN_THREADS, 0, s>>>(in, out, n, tile_sums);
     CT_COUNT_LAUNCH();
@@ -297,10 +314,95 @@ __global__ void k_rs_scatter(const K *__restrict__ keys, const uint32_t *__restr
     }
 }
 
+// The whole sort of a small array in one block and one launch (a multi-block
+// pass is five launches of 3 to 12 us each whatever the size).  Each warp owns
+// a contiguous part, so that counting its digits and ranking them in order
+// keeps the sort stable; the passes go back and forth between the two buffers
+// in global memory, read through L2 by the block that wrote them.
+// 4 to 10 us per pass up to RS_SMALL keys.
+constexpr int RSS_THREADS = 1024, RSS_WARPS = RSS_THREADS / 32;
+constexpr int64_t RS_SMALL = 32768;
+template <class K>
+__global__ void __launch_bounds__(RSS_THREADS) k_rs_small(K *k0, uint32_t *v0, K *k1, uint32_t *v1, int n,
+                                                          int passes) {
+    __shared__ uint32_t cnt[RSS_WARPS][256];
+    __shared__ uint32_t wsum[8];
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+    const int per = ((n + RSS_THREADS - 1) / RSS_THREADS) * 32;  // keys of a warp
+    const int beg = min(n, w * per), end = min(n, beg + per);
+    for (int p = 0; p < passes; ++p) {
+        const K *sk = p & 1 ? k1 : k0;
+        const uint32_t *sv = p & 1 ? v1 : v0;
+        K *dk = p & 1 ? k0 : k1;
+        uint32_t *dv = p & 1 ? v0 : v1;
+        const int shift = 8 * p;
+        for (int i = l; i < 256; i += 32) cnt[w][i] = 0u;
+        __syncwarp();
+        for (int i = beg + l; i < end; i += 32) atomicAdd(&cnt[w][(uint32_t)(__ldcg(sk + i) >> shift) & 255u], 1u);
+        __syncthreads();
+        // exclusive prefix over (digit, warp): digit d by thread d
+        uint32_t tot = 0, x = 0;
+        if (threadIdx.x < 256) {
+            for (int q = 0; q < RSS_WARPS; ++q) {
+                const uint32_t c = cnt[q][threadIdx.x];
+                cnt[q][threadIdx.x] = tot;
+                tot += c;
+            }
+            x = tot;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+                if (l >= o) x += y;
+            }
+            if (l == 31) wsum[w] = x;
+        }
+        __syncthreads();
+        if (threadIdx.x < 256) {
+            uint32_t base = x - tot;
+            for (int q = 0; q < w; ++q) base += wsum[q];
+            for (int q = 0; q < RSS_WARPS; ++q) cnt[q][threadIdx.x] += base;
+        }
+        __syncthreads();
+        for (int i0 = beg; i0 < end; i0 += 32) {
+            const int i = i0 + l;
+            const bool valid = i < end;
+            const K key = valid ? __ldcg(sk + i) : (K)0;
+            const uint32_t val = valid ? __ldcg(sv + i) : 0u;
+            const uint32_t d = valid ? (uint32_t)(key >> shift) & 255u : 256u + l;
+            const unsigned peers = __match_any_sync(0xffffffffu, d);
+            const int leader = __ffs(peers) - 1;
+            uint32_t at = 0;
+            if (valid && l == leader) {
+                at = cnt[w][d];
+                cnt[w][d] = at + __popc(peers);
+            }
+            at = __shfl_sync(0xffffffffu, at, leader) + __popc(peers & lanemask_lt());
+            if (valid) {
+                __stcg(dk + at, key);
+                __stcg(dv + at, val);
+            }
+            __syncwarp();
+        }
+        __threadfence();
+        __syncthreads();
+    }
+}
+
 template <class K>
 static void radix_sort_impl(K *keys, uint32_t *vals, K *tk, uint32_t *tv, int64_t n, int key_bits,
                             cudaStream_t s) {
     if (n <= 1 || key_bits <= 0) return;
+    if (n <= RS_SMALL) {
+        const int passes = (key_bits + 7) / 8;
+        k_rs_small<K><<<1, RSS_THREADS, 0, s>>>(keys, vals, tk, tv, (int)n, passes);
+        CT_COUNT_LAUNCH();
+        CT_LAUNCH_CHECK();
+        if (passes & 1) {
+            CT_CHECK_CUDA(cudaMemcpyAsync(keys, tk, n * sizeof(K), cudaMemcpyDeviceToDevice, s));
+            CT_CHECK_CUDA(cudaMemcpyAsync(vals, tv, n * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s));
+        }
+        return;
+    }
     int64_t tiles = ceil_div(n, RS_TILE);
     DBuf<int32_t> hist(256 * tiles, s);
     DBuf<int64_t> offs(256 * tiles, s);
