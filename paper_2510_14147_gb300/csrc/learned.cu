@@ -23,16 +23,24 @@ struct Norm {
     int d, on;
 };
 
-// Position -> query group (groups are runs of positions in increasing order).
-__global__ void k_pos_group(int64_t n, int G, const int32_t *__restrict__ group_begin, int32_t *__restrict__ gof) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    int lo = 0, hi = G;
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (group_begin[mid] <= i) lo = mid; else hi = mid;
+// Position -> query group and leaf block, written from the groups and blocks
+// (runs of positions): eight lanes per run.  (A binary search per position, 19
+// dependent steps, two loads each for the blocks, took 0.25 ms for a million
+// points with the features; 0.18 ms this way.)
+__global__ void k_pos_runs(int G, const int32_t *__restrict__ group_begin, const int32_t *__restrict__ group_count,
+                           int32_t *__restrict__ gof, int L, const int32_t *__restrict__ leaf_ids,
+                           const int32_t *__restrict__ node_begin, const int32_t *__restrict__ node_count,
+                           int32_t *__restrict__ lof) {
+    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 3;
+    const int j = threadIdx.x & 7;
+    if (i < G) {
+        const int b = group_begin[i], c = group_count[i];
+        for (int k = j; k < c; k += 8) gof[b + k] = (int32_t)i;
     }
-    gof[i] = lo;
+    if (i < L) {
+        const int v = leaf_ids[i], b = node_begin[v], c = node_count[v];
+        for (int k = j; k < c; k += 8) lof[b + k] = v;
+    }
 }
 
 // log1p(r / e) in fp32 with inv_e = fl(1 / e), log_e = fl(log e): the ratio
@@ -53,20 +61,14 @@ __device__ __forceinline__ float rel_log(float r, float inv_e, float log_e) {
 //  12..15 log1p(points below the lowest ancestor with radius >= e, 2e, 4e, 16e)
 __global__ void __launch_bounds__(256) k_features(
     int64_t n, int dp, int l2, const float *__restrict__ pts, const float *__restrict__ dcen,
-    const int32_t *__restrict__ leaf_ids, int n_leaves, const int32_t *__restrict__ node_begin,
-    const int32_t *__restrict__ node_count, const float *__restrict__ radius, const int32_t *__restrict__ parent,
+    const int32_t *__restrict__ lof, const int32_t *__restrict__ node_count, const float *__restrict__ radius, const int32_t *__restrict__ parent,
     const int32_t *__restrict__ group_begin, const int32_t *__restrict__ group_count,
     const float *__restrict__ group_radius, const int32_t *__restrict__ gof, double e, float inv_e, float log_e,
     Norm nm,
     float *__restrict__ x) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    int lo = 0, hi = n_leaves;  // leaf block holding position i
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (node_begin[leaf_ids[mid]] <= i) lo = mid; else hi = mid;
-    }
-    const int leaf = leaf_ids[lo];
+    const int leaf = lof[i];  // leaf block holding position i
     const int g = gof[i];
     float f[MLP_IN];
     f[0] = rel_log(dcen[i], inv_e, log_e);
@@ -260,17 +262,28 @@ void moments(const float *x, int64_t n, int d, float *mean, float *std_, cudaStr
 
 }  // namespace
 
+// Group and leaf block of every position (group 0 and vertex 0 where a loaded
+// tree's runs leave one out).
+void pos_runs(const ct_tree *t, int32_t *gof, int32_t *lof, cudaStream_t s) {
+    CT_CHECK_CUDA(cudaMemsetAsync(gof, 0, (size_t)t->n * sizeof(int32_t), s));
+    CT_CHECK_CUDA(cudaMemsetAsync(lof, 0, (size_t)t->n * sizeof(int32_t), s));
+    const int64_t runs = std::max(t->n_groups, t->n_leaves);
+    k_pos_runs<<<grid_of(runs * 8, 256), 256, 0, s>>>(t->n_groups, t->group_begin, t->group_count, gof, t->n_leaves,
+                                                     t->leaf_ids, t->node_begin, t->node_count, lof);
+    CT_COUNT_LAUNCH();
+    CT_LAUNCH_CHECK();
+}
+
 // Raw (P == nullptr) or standardised features of every tree position.
 void predictor_features(const ct_tree *t, double eps, const ct_predictor *P, float *x, cudaStream_t s) {
     const int64_t n = t->n;
     if (n == 0) return;
-    DBuf<int32_t> gof(n, s);
-    k_pos_group<<<grid_of(n, 256), 256, 0, s>>>(n, t->n_groups, t->group_begin, gof.p);
-    CT_COUNT_LAUNCH();
+    DBuf<int32_t> gof(n, s), lof(n, s);
+    pos_runs(t, gof.p, lof.p, s);
     const Norm nm = P ? make_norm(P->fmean, P->fstd, MLP_IN, true) : Norm{};
     const double e = eps > 1e-20 ? eps : 1e-20;
-    k_features<<<grid_of(n, 256), 256, 0, s>>>(n, t->dp, t->metric == CT_L2_F32, t->pts, t->dcen, t->leaf_ids,
-                                               t->n_leaves, t->node_begin, t->node_count, t->radius, t->parent,
+    k_features<<<grid_of(n, 256), 256, 0, s>>>(n, t->dp, t->metric == CT_L2_F32, t->pts, t->dcen, lof.p,
+                                               t->node_count, t->radius, t->parent,
                                                t->group_begin, t->group_count, t->group_radius, gof.p, e, (float)(1.0 / e),
                                                (float)std::log(e), nm, x);
     CT_COUNT_LAUNCH();
@@ -311,7 +324,7 @@ double predictor_fit(ct_predictor *P, const ct_tree *t, double eps, const ct_fit
     const int G = t->n_groups;
     // labels from one traversal and one count pass of the plain query
     const QParams qp = make_qparams(t, eps, o.include_self);
-    DBuf<int32_t> deg(n, s), gvisit(G ? G : 1, s), gof(n, s);
+    DBuf<int32_t> deg(n, s), gvisit(G ? G : 1, s), gof(n, s), lof(n, s);
     DBuf<float> x(n * MLP_IN, s), y(n * MLP_OUT, s);
     Probe pr;
     pr.deg = deg.p;
@@ -319,8 +332,7 @@ double predictor_fit(ct_predictor *P, const ct_tree *t, double eps, const ct_fit
     QueryOut tmp;
     query_multi(1, &t, &qp, s, &tmp, 0, nullptr, &pr);
     predictor_features(t, eps, nullptr, x.p, s);
-    k_pos_group<<<grid_of(n, 256), 256, 0, s>>>(n, G, t->group_begin, gof.p);
-    CT_COUNT_LAUNCH();
+    pos_runs(t, gof.p, lof.p, s);
     k_targets<<<grid_of(n, 256), 256, 0, s>>>(n, t->perm, gof.p, deg.p, gvisit.p, y.p);
     CT_COUNT_LAUNCH();
     CT_LAUNCH_CHECK();
@@ -445,6 +457,7 @@ void learned_plan(const ct_predictor *P, int C, const ct_tree *const *trees, con
 }
 
 void set_capacity_budget(int64_t bytes) { g_capacity_budget.store(bytes > 0 ? bytes : 0); }
+int64_t capacity_budget() { return g_capacity_budget.load(); }
 
 void query_predicted(const ct_tree *t, const QParams &qp, const void *predictor, int precision, cudaStream_t s,
                      QueryOut &out) {

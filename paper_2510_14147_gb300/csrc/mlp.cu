@@ -125,36 +125,86 @@ __global__ void k_to_half(const float *__restrict__ w, __half *__restrict__ wh) 
     if (e < MLP_NPARAMS) wh[e] = __float2half_rn(w[e]);
 }
 
-// Inference: thread per sample, fp16 weights in shared memory, fp32 sums.
-__global__ void __launch_bounds__(128) k_mlp_predict(const __half *__restrict__ wh, const float *__restrict__ x,
-                                                     int64_t n, float *__restrict__ y) {
-    __shared__ __half sw[MLP_NPARAMS];
-    for (int e = threadIdx.x; e < MLP_NPARAMS; e += blockDim.x) sw[e] = wh[e];
+// Packed fp32 pairs: two independent IEEE round-to-nearest operations.
+__device__ __forceinline__ unsigned long long pack2(float lo, float hi) {
+    unsigned long long d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+    return d;
+}
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ float lo2(unsigned long long v) { return __uint_as_float((uint32_t)v); }
+__device__ __forceinline__ float hi2(unsigned long long v) { return __uint_as_float((uint32_t)(v >> 32)); }
+__device__ __forceinline__ unsigned long long relu2(unsigned long long v) {
+    return pack2(fmaxf(lo2(v), 0.f), fmaxf(hi2(v), 0.f));
+}
+
+// Inference with fp16-rounded weights and fp32 sums: two samples per thread
+// in packed fp32, each weight widened once per block and kept twice in shared
+// memory, so that one 16-byte read feeds two packed FMAs.  (One sample per
+// thread, converting each weight at each use, was bound by issue: 0.56 ms for
+// a million samples, 0.32 ms now; the FMAs alone take 0.14 ms.)
+constexpr int PT = 128;
+__global__ void __launch_bounds__(PT) k_mlp_predict(const __half *__restrict__ wh, const float *__restrict__ x,
+                                                    int64_t n, float *__restrict__ y) {
+    __shared__ __align__(16) unsigned long long sw[MLP_NPARAMS];
+    for (int e = threadIdx.x; e < MLP_NPARAMS; e += PT) {
+        const float w = __half2float(wh[e]);
+        sw[e] = pack2(w, w);
+    }
     __syncthreads();
-    const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= n) return;
-    float xi[MLP_IN], h1[MLP_HID];
+    const int64_t s0 = (int64_t)blockIdx.x * 2 * PT + threadIdx.x, s1 = s0 + PT;
+    if (s0 >= n) return;
+    const float *xa = x + s0 * MLP_IN, *xb = x + (s1 < n ? s1 : s0) * MLP_IN;
+    unsigned long long xi[MLP_IN], h1[MLP_HID];
+    if ((reinterpret_cast<uintptr_t>(x) & 15) == 0) {
 #pragma unroll
-    for (int k = 0; k < MLP_IN; ++k) xi[k] = x[s * MLP_IN + k];
+        for (int k = 0; k < MLP_IN; k += 4) {
+            const float4 a = *reinterpret_cast<const float4 *>(xa + k), b = *reinterpret_cast<const float4 *>(xb + k);
+            xi[k] = pack2(a.x, b.x);
+            xi[k + 1] = pack2(a.y, b.y);
+            xi[k + 2] = pack2(a.z, b.z);
+            xi[k + 3] = pack2(a.w, b.w);
+        }
+    } else {  // a caller's rows at any float
+#pragma unroll
+        for (int k = 0; k < MLP_IN; ++k) xi[k] = pack2(xa[k], xb[k]);
+    }
+    const ulonglong2 *sw2 = reinterpret_cast<const ulonglong2 *>(sw);
 #pragma unroll
     for (int i = 0; i < MLP_HID; ++i) {
-        float a = __half2float(sw[P_B1 + i]);
+        unsigned long long a = sw[P_B1 + i];
 #pragma unroll
-        for (int k = 0; k < MLP_IN; ++k) a = fmaf(__half2float(sw[P_W1 + i * MLP_IN + k]), xi[k], a);
-        h1[i] = fmaxf(a, 0.f);
+        for (int k = 0; k < MLP_IN; k += 2) {
+            const ulonglong2 w = sw2[(P_W1 + i * MLP_IN + k) / 2];
+            a = fma2(w.x, xi[k], a);
+            a = fma2(w.y, xi[k + 1], a);
+        }
+        h1[i] = relu2(a);
     }
-    float y0 = __half2float(sw[P_B3]), y1 = __half2float(sw[P_B3 + 1]);
+    unsigned long long y0 = sw[P_B3], y1 = sw[P_B3 + 1];
 #pragma unroll 1
     for (int i = 0; i < MLP_HID; ++i) {
-        float a = __half2float(sw[P_B2 + i]);
+        unsigned long long a = sw[P_B2 + i];
 #pragma unroll
-        for (int j = 0; j < MLP_HID; ++j) a = fmaf(__half2float(sw[P_W2 + i * MLP_HID + j]), h1[j], a);
-        const float h = fmaxf(a, 0.f);
-        y0 = fmaf(__half2float(sw[P_W3 + i]), h, y0);
-        y1 = fmaf(__half2float(sw[P_W3 + MLP_HID + i]), h, y1);
+        for (int j = 0; j < MLP_HID; j += 2) {
+            const ulonglong2 w = sw2[(P_W2 + i * MLP_HID + j) / 2];
+            a = fma2(w.x, h1[j], a);
+            a = fma2(w.y, h1[j + 1], a);
+        }
+        a = relu2(a);
+        y0 = fma2(sw[P_W3 + i], a, y0);
+        y1 = fma2(sw[P_W3 + MLP_HID + i], a, y1);
     }
-    y[s * MLP_OUT] = y0;
-    y[s * MLP_OUT + 1] = y1;
+    y[s0 * MLP_OUT] = lo2(y0);
+    y[s0 * MLP_OUT + 1] = lo2(y1);
+    if (s1 < n) {
+        y[s1 * MLP_OUT] = hi2(y0);
+        y[s1 * MLP_OUT + 1] = hi2(y1);
+    }
 }
 
 }  // namespace
@@ -189,7 +239,7 @@ void mlp_to_half(const float *w, __half *wh, cudaStream_t s) {
 
 void mlp_predict(const __half *wh, const float *x, int64_t n, float *y, cudaStream_t s) {
     if (n <= 0) return;
-    k_mlp_predict<<<(unsigned)ceil_div(n, 128), 128, 0, s>>>(wh, x, n, y);
+    k_mlp_predict<<<(unsigned)ceil_div(n, 2 * PT), PT, 0, s>>>(wh, x, n, y);
     CT_COUNT_LAUNCH();
     CT_LAUNCH_CHECK();
 }
