@@ -21,7 +21,6 @@
 #include <climits>
 #include <cmath>
 #include <cstring>
-#include <cuda.h>
 #include <mutex>
 #include <type_traits>
 
@@ -100,11 +99,10 @@ struct Views {
     QParams qp[kMaxClouds];
     int16_t item_len[kMaxClouds];  // candidate blocks per work item
     uint8_t use_tc[kMaxClouds];    // leaf kernel of the count pass: tensor-core tiles (1) or FP32 tiles (0)
-    // tensor-core filter rows: the fp16 rows, a TMA map of them, their squared norms, {s, s eps_up}
+    // tensor-core filter rows: the fp16 rows, their squared norms, {s, s eps_up}
     const uint4 *h16[kMaxClouds];
     const float *n16[kMaxClouds];
     const float *s16[kMaxClouds];
-    CUtensorMap tmap[kMaxClouds];  // (a 128-byte aligned type)
 };
 static_assert(sizeof(Views) <= 32000, "Views exceeds the kernel parameter space");
 __device__ __forceinline__ int cloud_of_group(const Views &V, int gg) {
@@ -756,12 +754,16 @@ __device__ __forceinline__ void cp_async16(void *smem, const void *gmem, bool va
     int n = valid ? 16 : 0;  // 0: the 16 bytes are zero-filled, nothing is read
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(sa), "l"(gmem), "r"(n));
 }
+__device__ __forceinline__ void cp_async16_at(uint32_t smem, const void *gmem) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem), "l"(gmem));
+}
 // 4-byte copy through L1 (cp.async.cg takes 16-byte copies only)
 __device__ __forceinline__ void cp_async4(void *smem, const void *gmem) {
     unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(gmem));
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N)); }
 
@@ -776,6 +778,22 @@ __device__ __forceinline__ unsigned long long f2_sqacc(unsigned long long d, uns
     unsigned long long r;
     asm("fma.rn.f32x2 %0, %1, %1, %2;" : "=l"(r) : "l"(d), "l"(acc));
     return r;
+}
+__device__ __forceinline__ unsigned long long f2_pack(float lo, float hi) {
+    unsigned long long d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+    return d;
+}
+__device__ __forceinline__ unsigned long long f2_add(unsigned long long a, unsigned long long b) {
+    unsigned long long d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ unsigned long long f2_fma(unsigned long long a, unsigned long long b,
+                                                     unsigned long long c) {
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
 }
 __device__ __forceinline__ float f2_sum(unsigned long long v) {
     return __uint_as_float((uint32_t)v) + __uint_as_float((uint32_t)(v >> 32));
@@ -960,10 +978,8 @@ struct Items {
 struct CapOut {
     const int64_t *off;      // n + 1 capacity offsets by original id
     int32_t *fill;           // entries produced per row (ends equal to the degree)
-    int32_t *col;
-    float *dist;             // capacity region
-    int32_t *ovf_row, *ovf_slot, *ovf_col;
-    float *ovf_dist;
+    uint2 *ent;              // capacity region: (col, distance bits)
+    uint4 *ovf;              // arena: (row, slot, col, distance bits)
     unsigned long long *ovf_n;
     int64_t ovf_cap;
     uint8_t *lost;
@@ -973,21 +989,13 @@ struct CapOut {
 __device__ __forceinline__ void cap_place(const CapOut &co, int o, int slot, int32_t c, float d) {
     const int64_t b = co.off[o];
     if (slot < co.off[o + 1] - b) {
-        co.col[b + slot] = c;
-        co.dist[b + slot] = d;
+        co.ent[b + slot] = make_uint2((uint32_t)c, __float_as_uint(d));
         return;
     }
     const unsigned long long k = atomicAdd(co.ovf_n, 1ull);
-    if ((int64_t)k < co.ovf_cap) {
-        co.ovf_row[k] = o;
-        co.ovf_slot[k] = slot;
-        co.ovf_col[k] = c;
-        co.ovf_dist[k] = d;
-    } else {
-        co.lost[o] = 1;
-    }
+    if ((int64_t)k < co.ovf_cap) co.ovf[k] = make_uint4((uint32_t)o, (uint32_t)slot, (uint32_t)c, __float_as_uint(d));
+    else co.lost[o] = 1;
 }
-
 __device__ __forceinline__ void cap_put(const CapOut &co, int o, int32_t c, float d) {
     cap_place(co, o, atomicAdd(&co.fill[o], 1), c, d);
 }
@@ -1655,55 +1663,36 @@ __global__ void k_cap_rows(int64_t n, const int64_t *__restrict__ row_ptr, const
 
 // Copies each kept row's capacity-region entries into the CSR (warp per row).
 __global__ void k_compact(int64_t n, const int64_t *__restrict__ row_ptr, const int64_t *__restrict__ off,
-                          const uint8_t *__restrict__ lost, const int32_t *__restrict__ ccol,
-                          const float *__restrict__ cdist, int32_t *__restrict__ col, float *__restrict__ dist) {
+                          const uint8_t *__restrict__ lost, const uint2 *__restrict__ ent, int32_t *__restrict__ col,
+                          float *__restrict__ dist) {
     const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (w >= n || lost[w]) return;
     const int64_t b = off[w], cap = off[w + 1] - b, d0 = row_ptr[w], deg = row_ptr[w + 1] - d0;
     const int64_t m = deg < cap ? deg : cap;
     for (int64_t j = lane; j < m; j += 32) {
-        col[d0 + j] = ccol[b + j];
-        dist[d0 + j] = cdist[b + j];
+        const uint2 e = ent[b + j];
+        col[d0 + j] = (int32_t)e.x;
+        dist[d0 + j] = __uint_as_float(e.y);
     }
 }
 
 // Places the overflow arena's entries of kept rows at their slots.
-__global__ void k_ovf_scatter(int64_t used, const int32_t *__restrict__ orow, const int32_t *__restrict__ oslot,
-                              const int32_t *__restrict__ ocol, const float *__restrict__ odist,
-                              const uint8_t *__restrict__ lost, const int64_t *__restrict__ row_ptr,
-                              int32_t *__restrict__ col, float *__restrict__ dist, int32_t *__restrict__ err) {
+__global__ void k_ovf_scatter(int64_t used, const uint4 *__restrict__ ovf, const uint8_t *__restrict__ lost,
+                              const int64_t *__restrict__ row_ptr, int32_t *__restrict__ col,
+                              float *__restrict__ dist, int32_t *__restrict__ err) {
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= used) return;
-    const int r = orow[k];
-    if (lost[r]) return;
-    const int64_t at = row_ptr[r] + oslot[k];
-    if (at >= row_ptr[r + 1]) {
+    const uint4 e = ovf[k];
+    if (lost[e.x]) return;
+    const int64_t at = row_ptr[e.x] + e.y;
+    if (at >= row_ptr[e.x + 1]) {
         atomicOr(err, 128);
         return;
     }
-    col[at] = ocol[k];
-    dist[at] = odist[k];
+    col[at] = (int32_t)e.z;
+    dist[at] = __uint_as_float(e.w);
 }
-
-// ---------------------------------------------------------------------------
-// Precision 1: tensor-core filter, FP32 recheck, FP64 guard band.
-//
-// Count pass per work item: the group's queries (B, N = 32) and 128-row tiles
-// of packed candidate points (A, M = 128), both as fp16 rows prepared once per
-// query (below), are multiplied by tcgen05 MMAs (K = 16 per instruction) into a
-// 128 x 32 fp32 accumulator in tensor memory.  The accumulator, the rows'
-// squared norms and a rigorous bound on the fp16 and fp32 rounding give a
-// filter that keeps every edge; kept pairs are decided like the FP32 path: the
-// canonical fp32 direct-difference sum of the original rows (decide32), the
-// pinned FP64 sum where that cannot decide.  The emit pass is the FP32 path's,
-// driven by the same per-block edge masks.
-constexpr int TC_ROWS = 128;
-constexpr int TC_NB = kItemTC;          // candidate blocks of one item
-constexpr uint32_t TC_WAIT = 1u << 22;  // mbarrier polls before a wait gives up
-constexpr uint32_t TC_HINT = 1u << 16;  // ns a suspended poll may sleep (woken by the phase)
-constexpr uint32_t TC_SLEEPS = 1u << 14;  // suspended polls before a wait gives up (about a second)
-constexpr int TC_KL = 1024;             // kept pairs rechecked per round
 
 // ---------------------------------------------------------------------------
 // FP16 rows for the tensor-core filter.  Each cloud's points are stored once
@@ -1855,479 +1844,7 @@ __global__ void __launch_bounds__(H16_T) k_to_h16(const __grid_constant__ Views 
     if (on && j == 0) out.n16[c][row] = sq;
 }
 
-constexpr int TC_T = 256;   // threads per CTA (two CTAs per SM)
-constexpr int TC_EB = 768;  // edge buffer entries (one-pass emit)
-constexpr int TC_ISSUER = TC_T - 32;  // lane 0 of the last warp: issues the tiles' MMAs, tracks the query rows' load
-struct __align__(1024) TcShared {
-    unsigned char A[2][2][TC_ROWS * 128];  // fp16 candidate rows: buffer, K half (64 halves), 128-byte swizzle
-    unsigned char B[2][32 * 128];          // fp16 query rows, the same layout
-    float pn[4][TC_ROWS];                  // squared norms of the rows, per map slot
-    int pos[4][TC_ROWS];                   // map slots of tiles t .. t + 3 (slot t & 3): tree positions
-    uint16_t li[4][TC_ROWS];               //   and candidate blocks
-    uint16_t kl[TC_KL];                    // kept pairs of the tile: (query << 7) | row
-    int ecol[TC_EB];
-    float edist[TC_EB];
-    uint16_t erank[TC_EB];
-    uint8_t eq[TC_EB];
-    float2 qhg[32];                        // per query: threshold terms (h_q, g_q) of the filter
-    int bbeg[TC_NB], bpre[TC_NB + 1];
-    uint32_t bem[TC_NB];
-    int qcnt[32], orig[32], qfill[32], qbase[32];
-    int wsum[TC_T / 32];
-    int kn[2], en;
-    uint32_t tslot;
-    uint64_t mbar[2], bbar;                // MMAs (per buffer), query rows
-};
-constexpr size_t kTcSmem = sizeof(TcShared) + 1024;
-static_assert(2 * (kTcSmem + 1024) <= 228 * 1024, "k_leaf_tc: two CTAs per SM");
-static_assert(TC_NB % TC_T == 0, "block prefix takes TC_NB / TC_T candidate blocks per thread");
-
-// Count pass (and one-pass emit) with the FP16 filter.  One CTA of 8 warps per
-// work item, two CTAs per SM (one's setup and drain overlap the other's
-// tiles).  Candidate rows arrive by 16-byte cp.async copies of every thread
-// (half a row each), written in the MMA's 128-byte swizzled operand layout,
-// two tiles ahead; the 32 query rows by TMA gathers.  One thread issues the
-// MMA of tile t + 1 (second accumulator) as the iteration of tile t begins, so
-// that it runs while tile t is filtered and rechecked.  Rechecks read the
-// original fp32 rows from global memory, eight lanes per pair.
-__global__ void __launch_bounds__(TC_T, 2) k_leaf_tc(const __grid_constant__ Views V, Items items,
-                                                     const uint32_t *__restrict__ cand, uint32_t *__restrict__ emask,
-                                                     int32_t *__restrict__ deg, unsigned long long *__restrict__ st,
-                                                     int32_t *__restrict__ err, CapOut co) {
-    extern __shared__ unsigned char tc_raw[];
-    TcShared &S = *reinterpret_cast<TcShared *>(((uintptr_t)tc_raw + 1023) & ~(uintptr_t)1023);
-    const int it = blockIdx.x;
-    if (it >= *items.count) return;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int gg = items.group[it];
-    const int cloud = cloud_of_group(V, gg);
-    const TreeView &tv = V.tv[cloud];
-    const QParams &qp = V.qp[cloud];
-    const void *tmap = &V.tmap[cloud];
-    const uint4 *h16 = V.h16[cloud];
-    const float *n16 = V.n16[cloud];
-    const int g = gg - V.gbase[cloud];
-    const int64_t rbase = V.rbase[cloud];  // CSR rows of this cloud start here
-    const int dp = tv.dp, dim = tv.dim, dp4 = dp >> 2;
-    const float4 *pts4 = reinterpret_cast<const float4 *>(tv.pts);
-    const int halves = (dp + 63) >> 6;               // 64-half K blocks of an fp16 row (1 or 2)
-    const int ksteps = 4 * halves;                   // MMA K steps of 16
-    const int kc = 8 * halves;                       // 16-byte chunks of an fp16 row
-    const uint32_t q_bytes = (uint32_t)(32 * 128 * halves);
-    const int qb = tv.group_begin[g], qn = tv.group_count[g];
-    const int qe = qb + qn;  // the group's positions; upper-triangle form: rows before qb are skipped, edges
-                             // with rows from qe on are mirrored into those rows
-    const int64_t c0 = items.begin[it];
-    const int nb = (int)(items.end[it] - c0);        // <= TC_NB
-    uint32_t pairs = 0, kept = 0, guard = 0, band = 0, rows_ld = 0;  // rows_ld, kept: thread 0
-    bool failed = false;
-    // next phase parity of each barrier (bit b: buffer b): mph in every thread
-    // (warp 0 waits), bph in the issuing thread (it waits), which also tracks
-    // what is in flight, for a clean exit after a failure
-    uint32_t mph = 0u, bph = 0u, mpend = 0u, bpend = 0u;
-    bool tok = true;  // the issuing thread (TC_ISSUER): its own waits succeeded
-
-    if (warp == 0) tc::tmem_alloc(&S.tslot, 64);
-    if (tid == 0) {
-        tc::mbar_init(&S.mbar[0], 1);
-        tc::mbar_init(&S.mbar[1], 1);
-        tc::mbar_init(&S.bbar, 1);
-        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-    }
-    // candidate blocks of the item and their row prefix (TC_NB / TC_T blocks per thread)
-    {
-        constexpr int BPT = TC_NB / TC_T;
-        int loc[BPT], sum = 0;
-#pragma unroll
-        for (int k = 0; k < BPT; ++k) {
-            const int i = BPT * tid + k;
-            int beg = 0, cnt = 0;
-            if (i < nb) {
-                const int v = (int)cand[c0 + i];
-                beg = tv.node_begin[v];
-                cnt = tv.node_count[v];
-            }
-            S.bbeg[i] = beg;
-            S.bem[i] = 0u;
-            loc[k] = cnt;
-            sum += cnt;
-        }
-        int incl = sum;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += y;
-        }
-        if (lane == 31) S.wsum[warp] = incl;
-        __syncthreads();
-        int base = 0;
-#pragma unroll
-        for (int w = 0; w < TC_T / 32; ++w)
-            if (w < warp) base += S.wsum[w];
-        int run = base + incl - sum;
-#pragma unroll
-        for (int k = 0; k < BPT; ++k) {
-            S.bpre[BPT * tid + k] = run;
-            run += loc[k];
-        }
-        if (tid == TC_T - 1) S.bpre[TC_NB] = run;
-    }
-    tc::fence_before_sync();
-    __syncthreads();
-    tc::fence_after_sync();
-    const uint32_t tmem = S.tslot;
-    const int T = S.bpre[TC_NB];
-    const int ntiles = (T + TC_ROWS - 1) / TC_ROWS;
-    const float s_eps = V.s16[cloud][1];  // s eps_up
-
-    // rows of tile t -> (position, block) in map slot t & 3 and the rows'
-    // norms (4-byte copies; each thread commits one copy group per call).
-    // Warp w in 1..4 maps rows 32 (w - 1) .. + 31 of the tile: the block b0
-    // holding the window's first row R0 comes from two 32-wide ballot
-    // searches over the block prefix (the largest b0 with bpre[b0] <= R0);
-    // blocks b0 + 1 .. b0 + 31 start inside the window or after it, and a
-    // row's block is b0 plus the number of block starts in (R0, R].
-    auto prep_map = [&](int t) {
-        const int wq = warp - 1, R0 = t * TC_ROWS + 32 * wq;
-        if (t < ntiles && wq >= 0 && wq < 4 && R0 < T) {  // warp-uniform
-            const unsigned mc = __ballot_sync(0xffffffffu, S.bpre[32 * lane] <= R0);  // bit 0 set: bpre[0] = 0
-            const int c = 31 - __clz(mc);
-            const unsigned mf = __ballot_sync(0xffffffffu, S.bpre[32 * c + lane] <= R0);
-            const int b0 = 32 * c + 31 - __clz(mf);
-            const int j = b0 + 1 + lane;
-            const int v = j <= TC_NB ? S.bpre[j] : INT_MAX;
-            const unsigned m = __reduce_or_sync(0xffffffffu, v < R0 + 32 ? 1u << (v - R0) : 0u);  // v > R0
-            const int R = R0 + lane;
-            if (R < T) {
-                const int blk = b0 + __popc(m & (0xffffffffu >> (31 - lane)));
-                const int pos = S.bbeg[blk] + (R - S.bpre[blk]);
-                const int r = 32 * wq + lane;
-                S.pos[t & 3][r] = pos;
-                S.li[t & 3][r] = (uint16_t)blk;
-                cp_async4(&S.pn[t & 3][r], n16 + pos);
-            }
-        }
-        cp_async_commit();
-    };
-    // every thread: rows of tile t (past the last row of a short tile: row 0
-    // again) into buffer t & 1 by 16-byte copies, consecutive threads taking
-    // consecutive chunks of a row (a warp's copy covers 2 or 4 whole rows), in
-    // the MMA's 128-byte swizzled K-major layout (chunk j of row r at chunk
-    // j ^ (r % 8) of the row's 128 bytes; 1024-byte atoms of 8 rows).
-    // Completed by the copy group wait, a proxy fence and the barrier at the
-    // top of the next iteration, before the MMA that reads them is issued.
-    auto load_tile = [&](int t) {
-        const int rows = min(TC_ROWS, T - t * TC_ROWS), sl = t & 3, bf = t & 1;
-        const int lkc = 2 + halves;  // log2 of kc (8 or 16 chunks per row)
-        for (int g = tid; g < TC_ROWS * kc; g += TC_T) {
-            const int r = g >> lkc, ch = g & (kc - 1), h = ch >> 3, j = ch & 7;
-            const int pos = S.pos[sl][r < rows ? r : 0];
-            cp_async16(S.A[bf][h] + r * 128 + ((j ^ (r & 7)) << 4), h16 + (size_t)pos * kc + ch, true);
-        }
-    };
-    // the issuing thread: tile t's MMA chain into accumulator columns 32 (t & 1)
-    auto mma_tile = [&](int t) {
-        const int bf = t & 1;
-        constexpr uint32_t idesc = tc::idesc_f16_f32(TC_ROWS, 32);
-        for (int ks = 0; ks < ksteps; ++ks) {
-            const int h = ks >> 2, j = ks & 3;  // K half, 16-half step inside it (32 bytes)
-            const uint64_t ad = tc::smem_desc_sw128(tc::smem_u32(S.A[bf][h]) + 32 * j);
-            const uint64_t bd = tc::smem_desc_sw128(tc::smem_u32(S.B[h]) + 32 * j);
-            tc::mma_f16(tmem + (uint32_t)(32 * bf), ad, bd, idesc, ks > 0);
-        }
-        tc::mma_commit(&S.mbar[bf]);
-        mpend |= 1u << bf;
-    };
-
-    for (int q0 = 0; q0 < qn && !failed; q0 += 32) {
-        const int nqr = min(32, qn - q0);
-        const int qfirst = qb + q0;
-        __syncthreads();
-        if (tid < 32) {
-            S.qcnt[tid] = 0;
-            S.qfill[tid] = 0;
-            S.orig[tid] = tid < nqr ? (int)(rbase + tv.perm[qfirst + tid]) : 0;
-            // filter test per query (see the filter)
-            const float qn2 = tid < nqr ? __ldg(n16 + qfirst + tid) : 0.f;
-            const float qa = sqrtf(qn2) * H16_NORM_UP;
-            const float E = fmaf(H16_REL, qa, s_eps) + H16_ABS;
-            const float h = 0.5f * (qn2 - fmaf(E, E, fmaf(H16_ABS2 * qa, qa, 0x1p-60f))) - 0x1p-20f * (E * E);
-            S.qhg[tid] = make_float2(h, -H16_REL * E);
-        }
-        for (int i = tid; i < nb; i += TC_T) S.bem[i] = 0u;
-        if (tid == 0) {
-            S.en = 0;
-            S.kn[0] = S.kn[1] = 0;
-        }
-        prep_map(0);
-        prep_map(1);
-        prep_map(2);
-        if (tid == TC_ISSUER) {  // the expectation before any gather of the query rows is issued
-            tc::mbar_arrive_expect_tx(&S.bbar, q_bytes);
-            bpend = 1u;
-        }
-        __syncthreads();
-        // query rows (past the group's queries: its last query again) and tiles 0, 1
-        if (warp == 0 && lane < 8) {
-            const int q = 4 * lane;
-            const int r0 = qfirst + min(q, nqr - 1), r1 = qfirst + min(q + 1, nqr - 1);
-            const int r2 = qfirst + min(q + 2, nqr - 1), r3 = qfirst + min(q + 3, nqr - 1);
-            for (int h = 0; h < halves; ++h) tc::tma_gather4(S.B[h] + q * 128, tmap, 64 * h, r0, r1, r2, r3, &S.bbar);
-        }
-        for (int t = 0; t < 2 && t < ntiles; ++t) load_tile(t);
-        cp_async_commit();
-        cp_async_wait<0>();
-        tc::fence_smem_to_async();
-        __syncthreads();
-        if (tid == TC_ISSUER) {  // the issuing thread alone tracks the query rows' barrier phase
-            const bool okb = tok && tc::mbar_wait_sleep(&S.bbar, bph, TC_SLEEPS, TC_HINT);
-            if (okb) {
-                bpend = 0u;
-                bph ^= 1u;
-                if (ntiles > 0) {
-                    tc::fence_after_sync();
-                    mma_tile(0);
-                }
-            }
-            tok = okb;
-        }
-
-        auto flush = [&]() {
-            if (tid < 32 && S.qfill[tid]) S.qbase[tid] = atomicAdd(&co.fill[S.orig[tid]], S.qfill[tid]);
-            __syncthreads();
-            const int n = min(S.en, TC_EB);
-            for (int i = tid; i < n; i += TC_T) {
-                const int q = S.eq[i];
-                if (q & 0x80)  // an edge mirrored into the row of tree position ecol (upper triangle)
-                    cap_put(co, (int)(rbase + tv.perm[S.ecol[i]]), tv.perm[qfirst + (q & 31)], S.edist[i]);
-                else
-                    cap_place(co, S.orig[q], S.qbase[q] + S.erank[i], tv.perm[S.ecol[i]], S.edist[i]);
-            }
-            __syncthreads();
-            if (tid < 32) S.qfill[tid] = 0;
-            if (tid == 0) S.en = 0;
-        };
-        // pair e = (query << 7) | row in map slot sl, by the eight lanes of an
-        // octet: lane j sums coordinate chunk j (16 floats of both original
-        // rows) in the canonical order, the chunk sums are added in ascending
-        // order -- the canonical fp32 sum; the octet's first lane decides (FP64
-        // where fp32 cannot) and records the edge
-        auto recheck8 = [&](int e, int sl) {
-            const int q = e >> 7, r = e & 127, sub = lane & 7;
-            const unsigned omask = 0xffu << (lane & 24);
-            const int ppos = S.pos[sl][r];
-            const float4 *prow = pts4 + (size_t)ppos * dp4;
-            const float4 *qrow = pts4 + (size_t)(qfirst + q) * dp4;
-            const int k0 = 4 * sub;
-            float lo = 0.f, hi = 0.f;
-            if (k0 < dp4) {
-                float4 a[4], b[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const bool in = k0 + u < dp4;
-                    a[u] = in ? qrow[k0 + u] : make_float4(0.f, 0.f, 0.f, 0.f);
-                    b[u] = in ? __ldg(prow + k0 + u) : make_float4(0.f, 0.f, 0.f, 0.f);
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-                    if (k0 + u < dp4) {
-                        const float dx = a[u].x - b[u].x, dy = a[u].y - b[u].y, dz = a[u].z - b[u].z,
-                                    dw = a[u].w - b[u].w;
-                        lo = fmaf(dx, dx, lo);
-                        hi = fmaf(dy, dy, hi);
-                        lo = fmaf(dz, dz, lo);
-                        hi = fmaf(dw, dw, hi);
-                    }
-            }
-            const float chunk = lo + hi;
-            const int nch = (dp4 + 3) >> 2;
-            float sv = __shfl_sync(omask, chunk, 0, 8);
-#pragma unroll
-            for (int j = 1; j < 8; ++j) {
-                const float cj = __shfl_sync(omask, chunk, j, 8);
-                if (j < nch) sv += cj;
-            }
-            if (sub) return;
-            unsigned long long in_band = 0;
-            const int edge = decide32(qp, sv, in_band);
-            band += (uint32_t)in_band;
-            bool is_edge;
-            float d;
-            if (edge < 0) {
-                ++guard;
-                note_guard_rows(S.orig[q], (int32_t)(rbase + tv.perm[ppos]));
-                const double s64 = sq_l2_exact4(qrow, prow, dim);
-                is_edge = s64 <= qp.eps2_64;
-                d = (float)sqrt(s64);
-            } else {
-                is_edge = edge != 0;
-                d = sqrtf(sv);
-            }
-            if (is_edge) {
-                if (qp.half && ppos >= qe) {
-                    const int64_t o = rbase + tv.perm[ppos];
-                    atomicAdd(&deg[o], 1);
-                    if (co.off) {  // its slot is taken at the flush, off the recheck's path
-                        const int slot = atomicAdd(&S.en, 1);
-                        if (slot < TC_EB) {
-                            S.eq[slot] = (uint8_t)(0x80 | q);
-                            S.ecol[slot] = ppos;
-                            S.edist[slot] = d;
-                        } else {
-                            cap_put(co, (int)o, tv.perm[qfirst + q], d);
-                        }
-                    }
-                }
-                atomicAdd(&S.qcnt[q], 1);
-                atomicOr(&S.bem[S.li[sl][r]], 1u << q);
-                if (co.off) {
-                    const int slot = atomicAdd(&S.en, 1);
-                    if (slot < TC_EB) {
-                        S.eq[slot] = (uint8_t)q;
-                        S.ecol[slot] = ppos;  // tree position; the original id is looked up at the flush
-                        S.edist[slot] = d;
-                        S.erank[slot] = (uint16_t)atomicAdd(&S.qfill[q], 1);
-                    } else {
-                        cap_put(co, S.orig[q], tv.perm[ppos], d);
-                    }
-                }
-            }
-        };
-
-        for (int t = 0; t < ntiles; ++t) {
-            const int sl = t & 3, bf = t & 1;
-            const int rows = min(TC_ROWS, T - t * TC_ROWS);
-            if (tid == 0) rows_ld += rows;
-            // tile t's MMA has completed (warp 0 waits); the rows of tile t + 1
-            // (copied an iteration ago) and the norms have landed
-            cp_async_wait<0>();
-            tc::fence_smem_to_async();
-            bool ok = tid != TC_ISSUER || tok;  // the issuing thread's own waits so far
-            if (warp == 0) ok = tc::mbar_wait_sleep(&S.mbar[bf], (mph >> bf) & 1u, TC_SLEEPS, TC_HINT);
-            if (!__syncthreads_and(ok)) {
-                if (tid == 0) atomicOr(err, 32);
-                failed = true;
-                break;
-            }
-            mph ^= 1u << bf;
-            if (tid == TC_ISSUER) mpend &= ~(1u << bf);
-            tc::fence_after_sync();
-            if (co.off && S.en >= TC_EB / 2) flush();  // tile t - 1's rechecks are done
-            // the issuing thread: tile t + 1's MMA into the other accumulator now,
-            // so that it runs while tile t is filtered and rechecked (its rows
-            // were copied an iteration ago; its columns were last read by tile
-            // t - 1's filter, before the barrier above)
-            if (t + 1 < ntiles && tid == TC_ISSUER && tok) mma_tile(t + 1);
-            if (t + 2 < ntiles) load_tile(t + 2);  // buffer bf: tile t's MMA has completed
-            prep_map(t + 3);                       // commits the group (tile t + 2's rows, t + 3's norms)
-            // epilogue, filter: warp w reads rows 32 (w % 4) .. + 31, queries
-            // 16 (w / 4) .. + 15; kept pairs go to the tile's list
-            uint32_t keepm = 0u;
-            int kb = 0;
-            {
-                const int quarter = warp & 3, qh = warp >> 2;
-                float dot[16];
-                tc::tmem_ld16(tmem + ((uint32_t)(32 * quarter) << 16) + (uint32_t)(32 * bf + 16 * qh), dot);
-                const int r = 32 * quarter + lane;
-                if (r < rows) {
-                    // kept iff d^2 = n^_q + n^_p - 2 dot <= (E_q + rel |p^|)^2 + abs2 (|q^|^2 + |p^|^2)
-                    // + 2^-60 with E_q = s eps + rel |q^| + 2^-20, i.e. iff dot >= h_q + g_q |p^| + w_p
-                    // with h_q = (n^_q - E_q^2 - abs2 |q^|^2 - 2^-60) / 2, g_q = -rel E_q,
-                    // w_p = (n^_p - (rel^2 + abs2) |p^|^2) / 2.  The rounding of this form stays
-                    // below 2^-21 (n^_q + n^_p + 2 E_q^2): the first part is inside the abs2
-                    // term's slack over the other fp32 errors, the second is covered by the
-                    // 2^-20 E_q^2 taken off h_q.  NaN keeps the pair.
-                    const int ppos = S.pos[sl][r];
-                    const float pn = S.pn[sl][r];
-                    const float pa = sqrtf(pn) * H16_NORM_UP;
-                    const float wp = 0.5f * fmaf(-(H16_REL * H16_REL + H16_ABS2) * pa, pa, pn);
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const float2 hg = S.qhg[16 * qh + j];
-                        if (!(dot[j] < fmaf(hg.y, pa, hg.x) + wp)) keepm |= 1u << j;
-                    }
-                    uint32_t validm = (nqr >= 16 * qh + 16 ? 0xffffu : (1u << max(nqr - 16 * qh, 0)) - 1u);
-                    const int self = ppos - qfirst - 16 * qh;
-                    if (!qp.include_self && (unsigned)self < 16u) validm &= ~(1u << self);
-                    if (qp.half && ppos < qb) validm = 0u;
-                    keepm &= validm;
-                    pairs += __popc(validm);
-                }
-                const int c = __popc(keepm);
-                int incl = c;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int y = __shfl_up_sync(0xffffffffu, incl, o);
-                    if (lane >= o) incl += y;
-                }
-                int base = 0;
-                if (lane == 31 && incl) base = atomicAdd(&S.kn[bf], incl);
-                kb = __shfl_sync(0xffffffffu, base, 31) + incl - c;
-                uint32_t m = keepm;
-                for (int idx = kb; m && idx < TC_KL; ++idx) {
-                    const int j = __ffs(m) - 1;
-                    m &= m - 1u;
-                    S.kl[idx] = (uint16_t)(((16 * qh + j) << 7) | r);
-                }
-            }
-            tc::fence_before_sync();
-            __syncthreads();
-            const int n = S.kn[bf];
-            if (tid == 0) {
-                kept += n;
-                S.kn[bf ^ 1] = 0;  // tile t + 1's list (filled after the next barrier)
-            }
-            // recheck: the kept pairs spread over the lane octets, one pair per
-            // octet, TC_KL at a time (pairs past the list are re-derived from
-            // the filter's masks)
-            for (int i = tid >> 3; i < min(n, TC_KL); i += TC_T / 8) recheck8(S.kl[i], sl);
-            for (int lo = TC_KL; lo < n; lo += TC_KL) {
-                __syncthreads();
-                uint32_t m = keepm;
-                const int qc = 16 * (warp >> 2), r = 32 * (warp & 3) + lane;
-                for (int idx = kb; m && idx < lo + TC_KL; ++idx) {
-                    const int j = __ffs(m) - 1;
-                    m &= m - 1u;
-                    if (idx >= lo) S.kl[idx - lo] = (uint16_t)(((qc + j) << 7) | r);
-                }
-                __syncthreads();
-                for (int i = tid >> 3; i < min(n - lo, TC_KL); i += TC_T / 8) recheck8(S.kl[i], sl);
-            }
-        }
-        if (failed) break;
-        __syncthreads();
-        if (co.off) flush();
-        __syncthreads();
-        if (tid < nqr && S.qcnt[tid]) atomicAdd(&deg[S.orig[tid]], S.qcnt[tid]);
-    }
-    if (!failed && emask)
-        for (int i = tid; i < nb; i += TC_T) emask[c0 + i] = qn <= 32 ? S.bem[i] : ~0u;
-    unsigned long long pairs64 = pairs, kept64 = kept, guard64 = guard, band64 = band;
-    for (int o = 16; o > 0; o >>= 1) {
-        pairs64 += __shfl_xor_sync(0xffffffffu, pairs64, o);
-        kept64 += __shfl_xor_sync(0xffffffffu, kept64, o);
-        guard64 += __shfl_xor_sync(0xffffffffu, guard64, o);
-        band64 += __shfl_xor_sync(0xffffffffu, band64, o);
-    }
-    if (lane == 0) {
-        stat_add(st, ST_PAIRS, pairs64);
-        stat_add(st, ST_RECHECK, kept64);
-        stat_add(st, ST_GUARD, guard64);
-        stat_add(st, ST_BAND, band64);
-        if (tid == 0) stat_add(st, ST_ROWS, rows_ld);
-    }
-    cp_async_wait<0>();  // no copy into this CTA's shared memory outlives it
-    if (tid == TC_ISSUER) {  // after a failure: let the query rows' gathers and MMAs in flight finish (bounded)
-        for (int b = 0; b < 2; ++b)
-            if (mpend >> b & 1u) tc::mbar_wait(&S.mbar[b], (mph >> b) & 1u, TC_WAIT);
-        if (bpend) tc::mbar_wait_sleep(&S.bbar, bph, TC_SLEEPS, TC_HINT);
-    }
-    tc::fence_before_sync();
-    __syncthreads();
-    tc::fence_after_sync();
-    if (warp == 0) tc::tmem_dealloc(tmem, 64);
-}
-
+#include "leaf_tc.cuh"
 
 // Dynamic shared memory of the L2 leaf kernel (set once per process).
 void leaf_l2_prepare() {
@@ -3527,29 +3044,6 @@ __global__ void k_rel_rows(int64_t n1, const int64_t *__restrict__ grow, int64_t
     if (i < n1) out[i] = grow[i] - grow[0];
 }
 
-// TMA map of n fp16 rows of kp halves (kp a multiple of 64): boxes of 64
-// halves x 1 row (gathered four rows at a time), 128-byte swizzle.
-typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
-                                  const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-void encode_rows_f16(CUtensorMap *m, const void *rows, int64_t n, int kp) {
-    static EncodeTiledFn fn = nullptr;
-    if (!fn) {
-        void *p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        CT_CHECK_CUDA(cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q));
-        if (q != cudaDriverEntryPointSuccess || !p) CT_FAIL(CT_ECUDA, "cuTensorMapEncodeTiled is not available");
-        fn = (EncodeTiledFn)p;
-    }
-    const cuuint64_t dims[2] = {(cuuint64_t)kp, (cuuint64_t)n};
-    const cuuint64_t strides[1] = {(cuuint64_t)kp * 2};
-    const cuuint32_t box[2] = {64, 1}, estr[2] = {1, 1};
-    const CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void *>(rows), dims, strides, box, estr,
-                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) CT_FAIL(CT_ECUDA, "cuTensorMapEncodeTiled failed (%d)", (int)r);
-}
-
 void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStream_t s, QueryOut *outs,
                  int precision, const ct_predictor *pred, Probe *probe) {
     if (C < 1 || C > kMaxClouds) CT_FAIL(CT_EINVAL, "between 1 and %d clouds per batch", kMaxClouds);
@@ -3611,7 +3105,6 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
             ho.n16[c] = ho.scal[c] + 4;
             rows += tc->n * (kp / 8);
             floats += dp + 4 + ceil_div(tc->n, 4) * 4;
-            encode_rows_f16(&V.tmap[c], ho.h16[c], tc->n, kp);
             V.h16[c] = ho.h16[c];
             V.n16[c] = ho.n16[c];
             V.s16[c] = ho.scal[c];
@@ -3798,7 +3291,7 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
     seg_group.reset();
     seg_count.reset();
     seg_begin.reset();
-    DBuf<uint32_t> emask(l2 ? (n_cand ? n_cand : 1) : 0, s);
+    DBuf<uint32_t> emask(l2 && any_fp ? (n_cand ? n_cand : 1) : 0, s);
     // work items: the groups' candidate ranges in slices of the clouds' item lengths
     const int64_t max_items = nseg + n_cand / min_len + 1;
     DBuf<int32_t> icnt(nseg + 1, s), igroup(max_items, s), nitems(1, s);
@@ -3850,26 +3343,22 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
     // one-pass emit: capacity region and overflow arena
     const bool capmode = pred && !probe && lp.one_pass;
     CapOut co{};
-    DBuf<int32_t> c_fill, c_col, o_row, o_slot, o_col;
-    DBuf<float> c_dist, o_dist;
+    DBuf<int32_t> c_fill;
+    DBuf<uint2> c_ent;
+    DBuf<uint4> o_ent;
     DBuf<unsigned long long> o_n;
     DBuf<uint8_t> lost;
     if (capmode) {
         const int64_t ct = lp.cap_total > 0 ? lp.cap_total : 1, oc = lp.arena > 0 ? lp.arena : 1;
         c_fill = DBuf<int32_t>(n + 1, s);
-        c_col = DBuf<int32_t>(ct, s);
-        c_dist = DBuf<float>(ct, s);
-        o_row = DBuf<int32_t>(oc, s);
-        o_slot = DBuf<int32_t>(oc, s);
-        o_col = DBuf<int32_t>(oc, s);
-        o_dist = DBuf<float>(oc, s);
+        c_ent = DBuf<uint2>(ct, s);
+        o_ent = DBuf<uint4>(oc, s);
         o_n = DBuf<unsigned long long>(3, s);
         lost = DBuf<uint8_t>(n + 1, s);
         CT_CHECK_CUDA(cudaMemsetAsync(c_fill.p, 0, (n + 1) * sizeof(int32_t), s));
         CT_CHECK_CUDA(cudaMemsetAsync(o_n.p, 0, 3 * sizeof(unsigned long long), s));
         CT_CHECK_CUDA(cudaMemsetAsync(lost.p, 0, n + 1, s));
-        co = CapOut{lp.cap_off.p, c_fill.p, c_col.p, c_dist.p, o_row.p, o_slot.p, o_col.p, o_dist.p,
-                    o_n.p, lp.arena > 0 ? lp.arena : 0, lost.p};
+        co = CapOut{lp.cap_off.p, c_fill.p, c_ent.p, o_ent.p, o_n.p, lp.arena > 0 ? lp.arena : 0, lost.p};
     }
 
     // 2. count pass
@@ -3909,30 +3398,17 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
         CT_COUNT_LAUNCH();
         CT_LAUNCH_CHECK();
     };
-    // each cloud's count kernel: tensor-core tiles (L2 rows of at most 128
-    // floats) or FP32 tiles -- the same output; a mixed batch splits its work
-    // items between the two launches
-    auto count_tc = [&](const Items &its) {
-        ProfScope ps("leaf_count_tc", s);
-        static bool tc_ready = false;
-        if (!tc_ready) {
-            CT_CHECK_CUDA(cudaFuncSetAttribute(k_leaf_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmem));
-            tc_ready = true;
-        }
-        if (G && nseg) {
-            k_leaf_tc<<<(unsigned)max_items, TC_T, kTcSmem, s>>>(V, its, cand_p, emask.p, deg.p, st.p, err, co);
-            CT_COUNT_LAUNCH();
-            CT_LAUNCH_CHECK();
-        }
-    };
-    if (!l2 || !any_tc) {
-        ProfScope ps("leaf_count", s);
-        leaf(false, nullptr, nullptr, nullptr, nullptr, items);
-    } else if (!any_fp) {
-        count_tc(items);
-    } else {
-        DBuf<int32_t> tg(max_items, s), fg(max_items, s), cnt2(2, s);
-        DBuf<int64_t> tb(max_items, s), te(max_items, s), fb(max_items, s), fe(max_items, s);
+    // each cloud's count kernel: the tensor-core filter and decisions (L2 rows
+    // of at most 128 floats) or FP32 tiles -- the same output; a mixed batch
+    // splits its work items
+    DBuf<int32_t> tg, fg, cnt2;
+    DBuf<int64_t> tb, te, fb, fe;
+    Items items_tc = items, items_fp = items;
+    if (l2 && any_tc && any_fp) {
+        tg = DBuf<int32_t>(max_items, s);
+        fg = DBuf<int32_t>(max_items, s);
+        cnt2 = DBuf<int32_t>(2, s);
+        for (DBuf<int64_t> *d : {&tb, &te, &fb, &fe}) *d = DBuf<int64_t>(max_items, s);
         CT_CHECK_CUDA(cudaMemsetAsync(cnt2.p, 0, 2 * sizeof(int32_t), s));
         if (nseg) {
             k_item_split<<<grid_for(max_items, 256), 256, 0, s>>>(V, items, tg.p, tb.p, te.p, cnt2.p, fg.p, fb.p, fe.p,
@@ -3940,10 +3416,148 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
             CT_COUNT_LAUNCH();
             CT_LAUNCH_CHECK();
         }
-        count_tc(Items{tg.p, tb.p, te.p, cnt2.p});
-        ProfScope ps("leaf_count", s);
-        leaf(false, nullptr, nullptr, nullptr, nullptr, Items{fg.p, fb.p, fe.p, cnt2.p + 1});
+        items_tc = Items{tg.p, tb.p, te.p, cnt2.p};
+        items_fp = Items{fg.p, fb.p, fe.p, cnt2.p + 1};
     }
+    // Tensor-core items in waves: a wave's kept pairs go to a list, which is
+    // decided before the next wave.  With many items a first wave of every
+    // 32nd gives the pairs per item; the rest is cut into interleaved parts
+    // (every part like the whole) whose lists fit pair_budget with a quarter
+    // to spare.  A list that runs out is sized again from what the filter
+    // counted, or its wave cut in two.  The two-pass form keeps its lists for
+    // the emit pass while they fit; else that filters again.
+    struct Wave {
+        FtWave wave;
+        int64_t n;         // entries reserved
+        DBuf<uint2> list;  // kept list (its first n entries), or empty
+    };
+    std::vector<Wave> waves;
+    unsigned long long tc_stats[3] = {0, 0, 0};
+    DBuf<unsigned long long> fctr(5, s);  // next item, entries, {valid pairs, kept pairs, rows}
+    bool lists_kept = !capmode && !probe;
+    int64_t filtered = 0;  // entries of the last filter
+    const int64_t pair_slack = (int64_t)num_sms() * FT_EWARPS * FT_CHUNK;  // partly filled chunks
+    int64_t pair_budget = 64ll << 20;  // one-pass: half a GB of pairs at a time
+    if (any_tc) {
+        size_t fr = 0, tot = 0;
+        if (cudaMemGetInfo(&fr, &tot) == cudaSuccess) {
+            const int64_t lim = (int64_t)(fr / 4 / sizeof(uint2));
+            // the two-pass form gains by one list (no second filter pass)
+            pair_budget = std::max<int64_t>(1 << 20, lists_kept ? lim : std::min(lim, pair_budget));
+        } else {
+            cudaGetLastError();
+        }
+        if (capacity_budget() > 0) pair_budget = std::max<int64_t>(1, capacity_budget() / (int64_t)sizeof(uint2));
+    }
+    // filters a wave's items into a list of at least `want` entries (grown to
+    // the need once that is known); false when the need exceeds `most`
+    auto tc_filter = [&](const FtWave &w, double want, DBuf<uint2> &list, bool stats, int64_t most) {
+        for (;;) {
+            const int64_t cap = ceil_div((int64_t)want, FT_CHUNK) * FT_CHUNK;
+            if ((int64_t)list.n < cap) {
+                list.reset();
+                list = DBuf<uint2>((size_t)cap, s);
+            }
+            CT_CHECK_CUDA(cudaMemsetAsync(fctr.p, 0, 5 * sizeof(unsigned long long), s));
+            const PairList pl{list.p, (int64_t)(list.n / FT_CHUNK * FT_CHUNK), fctr.p + 1, fctr.p + 2};
+            const int ctas = (int)std::min<int64_t>(num_sms(), max_items);
+            k_filter_tc<<<ctas, FT_T, kFtSmem, s>>>(V, items_tc, w, cand_p, pl, fctr.p, err);
+            CT_COUNT_LAUNCH();
+            CT_LAUNCH_CHECK();
+            unsigned long long h[4];
+            to_host(h, fctr.p + 1, 4, s);
+            filtered = (int64_t)h[0];
+            if (filtered <= pl.cap) {
+                if (stats)
+                    for (int k = 0; k < 3; ++k) tc_stats[k] += h[1 + k];
+                return true;
+            }
+            const int64_t need = filtered + pair_slack;  // the next run's chunks may be filled differently
+            if (need > most) return false;
+            want = (double)need;
+        }
+    };
+    auto tc_pairs = [&](int mode, uint2 *list, int64_t entries, const uint8_t *rowsel) {
+        if (!entries) return;
+        const PairList pl{list, entries, nullptr, nullptr};
+        const int blocks = (int)std::min<int64_t>(ceil_div(entries, 256), (int64_t)num_sms() * 16);
+        switch (mode) {
+#define CT_KP(M) case M: k_pairs<M><<<blocks, 256, 0, s>>>(V, pl, deg.p, co, all.row_ptr, rowcur.p, all.col, all.dist, rowsel, st.p, err); break;
+            CT_KP(PAIRS_COUNT) CT_KP(PAIRS_PLACE) CT_KP(PAIRS_EMIT)
+#undef CT_KP
+        }
+        CT_COUNT_LAUNCH();
+        CT_LAUNCH_CHECK();
+    };
+    auto count_tc = [&]() {
+        ProfScope ps("leaf_count_tc", s);
+        CT_CHECK_CUDA(cudaFuncSetAttribute(k_filter_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFtSmem));
+        if (!G || !nseg) return;
+        int64_t kept_entries = 0;
+        DBuf<uint2> list;
+        // waves still to run (a stack); a wave whose list would exceed the
+        // budget is cut in two interleaved halves
+        std::vector<FtWave> todo;
+        const bool sample = max_items > 32ll * num_sms();
+        todo.push_back(sample ? FtWave{1, 0, 1} : FtWave{0, 0, 1});
+        double want = (double)pair_slack + std::min(512.0 * (double)n, (double)(16 << 20));
+        bool sampled = !sample;
+        while (!todo.empty()) {
+            const FtWave w = todo.back();
+            todo.pop_back();
+            const bool can_cut = w.sampled != 1 && w.parts < (1 << 20);
+            if (!tc_filter(w, want, list, true, can_cut ? pair_budget + pair_slack : INT64_MAX)) {
+                todo.push_back(FtWave{w.sampled, w.part + w.parts, 2 * w.parts});
+                todo.push_back(FtWave{w.sampled, w.part, 2 * w.parts});
+                want = (double)(pair_budget + pair_slack);
+                continue;
+            }
+            tc_pairs(capmode ? PAIRS_PLACE : PAIRS_COUNT, list.p, filtered, nullptr);
+            waves.push_back(Wave{w, filtered, DBuf<uint2>()});
+            kept_entries += filtered;
+            if (lists_kept && kept_entries <= pair_budget + pair_slack) {
+                waves.back().list = std::move(list);
+            } else if (lists_kept) {
+                lists_kept = false;
+                for (auto &x : waves) x.list.reset();
+            }
+            if (!sampled) {  // the rest, from the sample's pairs
+                sampled = true;
+                const double total = 1.25 * (FT_SAMPLE - 1) * std::max(1.0, (double)tc_stats[1]);
+                const int parts = (int)std::min(65536.0, std::ceil(total / (double)pair_budget));
+                for (int k = parts - 1; k >= 0; --k) todo.push_back(FtWave{2, k, parts});
+                want = total / parts + (double)pair_slack;
+            }
+        }
+    };
+    if (!l2 || !any_tc) {
+        ProfScope ps("leaf_count", s);
+        leaf(false, nullptr, nullptr, nullptr, nullptr, items);
+    } else {
+        count_tc();
+        if (any_fp) {
+            ProfScope ps("leaf_count", s);
+            leaf(false, nullptr, nullptr, nullptr, nullptr, items_fp);
+        }
+        if (capmode)  // the entries placed are the degrees
+            for (int c = 0; c < C; ++c)
+                if (V.use_tc[c] && trees[c]->n)
+                    CT_CHECK_CUDA(cudaMemcpyAsync(deg.p + V.rbase[c], c_fill.p + V.rbase[c],
+                                                  (size_t)trees[c]->n * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
+    }
+    // emit pass (rowsel: of the selected rows)
+    auto emit = [&](const uint8_t *rowsel) {
+        if (!l2 || any_fp) leaf(true, all.row_ptr, all.col, all.dist, rowsel, items_fp);
+        DBuf<uint2> list;
+        for (auto &w : waves) {
+            if (lists_kept) {
+                tc_pairs(PAIRS_EMIT, w.list.p, w.n, rowsel);
+                continue;
+            }
+            tc_filter(w.wave, (double)(w.n + pair_slack), list, false, INT64_MAX);
+            tc_pairs(PAIRS_EMIT, list.p, filtered, rowsel);
+        }
+    };
 
     auto finish_stats = [&]() {
         unsigned long long hs[ST_N];
@@ -3953,11 +3567,11 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
             CT_FAIL(CT_ETIMEOUT, "a bounded wait of the tensor-core leaf kernel gave up (code %llu)", hs[ST_ERR]);
         if (hs[ST_ERR]) CT_FAIL(CT_ECUDA, "internal consistency check failed in the query (code %llu)", hs[ST_ERR]);
         all.stats.traversal_evals = (int64_t)hs[ST_TRAV];
-        all.stats.leaf_pairs = (int64_t)hs[ST_PAIRS];
+        all.stats.leaf_pairs = (int64_t)(hs[ST_PAIRS] + tc_stats[0]);
         all.stats.guard_fp64 = (int64_t)hs[ST_GUARD];
-        all.stats.recheck_fp32 = (int64_t)hs[ST_RECHECK];
+        all.stats.recheck_fp32 = (int64_t)(hs[ST_RECHECK] + tc_stats[1]);
         all.stats.emit_pairs = (int64_t)hs[ST_EMIT];
-        all.stats.leaf_rows = (int64_t)hs[ST_ROWS];
+        all.stats.leaf_rows = (int64_t)(hs[ST_ROWS] + tc_stats[2]);
         all.stats.guard_band = (int64_t)hs[ST_BAND];
         all.stats.lev_columns = (int64_t)hs[ST_COLS];
         all.stats.candidates = n_cand;
@@ -3987,35 +3601,34 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
             if (n) {
                 k_cap_rows<<<grid_for(n, 256), 256, 0, s>>>(n, row_ptr, lp.cap_off.p, c_fill.p, lost.p, o_n.p + 1, err);
                 CT_COUNT_LAUNCH();
-                k_compact<<<grid_for(n * 32, 256), 256, 0, s>>>(n, row_ptr, lp.cap_off.p, lost.p, c_col.p, c_dist.p,
-                                                                all.col, all.dist);
+                k_compact<<<grid_for(n * 32, 256), 256, 0, s>>>(n, row_ptr, lp.cap_off.p, lost.p, c_ent.p, all.col,
+                                                                all.dist);
                 CT_COUNT_LAUNCH();
                 CT_LAUNCH_CHECK();
             }
             to_host(hv, o_n.p, 3, s);
             const int64_t used = std::min<int64_t>((int64_t)hv[0], co.ovf_cap);
             if (used > 0) {
-                k_ovf_scatter<<<grid_for(used, 256), 256, 0, s>>>(used, o_row.p, o_slot.p, o_col.p, o_dist.p, lost.p,
-                                                                  row_ptr, all.col, all.dist, err);
+                k_ovf_scatter<<<grid_for(used, 256), 256, 0, s>>>(used, o_ent.p, lost.p, row_ptr, all.col, all.dist,
+                                                                  err);
                 CT_COUNT_LAUNCH();
                 CT_LAUNCH_CHECK();
             }
         }
         all.stats.overflow_rows = (int64_t)hv[1];
         all.stats.reemit_rows = (int64_t)hv[2];
-        c_col.reset();
-        c_dist.reset();
+        c_ent.reset();
         if (hv[2]) {
             ProfScope ps("reemit", s);
             CT_CHECK_CUDA(cudaMemsetAsync(rowcur.p, 0, (n + 1) * sizeof(int32_t), s));
-            leaf(true, row_ptr, all.col, all.dist, lost.p, items);
+            emit(lost.p);
             k_check_rows_sel<<<grid_for(n, 256), 256, 0, s>>>(n, row_ptr, rowcur.p, lost.p, err);
             CT_COUNT_LAUNCH();
         }
     } else if (nnz) {
         ProfScope ps("leaf_emit", s);
         CT_CHECK_CUDA(cudaMemsetAsync(rowcur.p, 0, (n + 1) * sizeof(int32_t), s));
-        leaf(true, row_ptr, all.col, all.dist, nullptr, items);
+        emit(nullptr);
         k_check_rows<<<grid_for(n, 256), 256, 0, s>>>(n, row_ptr, rowcur.p, err);
         CT_COUNT_LAUNCH();
     }

@@ -127,23 +127,15 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *mbar, uint32_t parity, uint3
     return false;
 }
 
-// One arrival on the mbarrier that also expects `bytes` of asynchronous
-// copies (TMA) to complete in the current phase.
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *mbar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_u32(mbar)), "r"(bytes)
-                 : "memory");
+// One arrival on the mbarrier (release).
+__device__ __forceinline__ void mbar_arrive(uint64_t *mbar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(mbar)) : "memory");
 }
 
-// TMA gather of four rows r0..r3 (columns col .. col + box - 1 of a 2-D tensor
-// map whose box is one row high) into consecutive rows at dst, completing
-// their bytes on mbar.  col * element size must be a multiple of 16 bytes.
-__device__ __forceinline__ void tma_gather4(void *dst, const void *tmap, int col, int r0, int r1, int r2, int r3,
-                                            uint64_t *mbar) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile::gather4.mbarrier::complete_tx::bytes "
-        "[%0], [%1, {%2, %3, %4, %5, %6}], [%7];\n" ::"r"(smem_u32(dst)),
-        "l"(tmap), "r"(col), "r"(r0), "r"(r1), "r"(r2), "r"(r3), "r"(smem_u32(mbar))
-        : "memory");
+// Arrives on the mbarrier once this thread's cp.async copies so far have
+// landed (counted in the barrier's expected arrivals).
+__device__ __forceinline__ void mbar_arrive_copies(uint64_t *mbar) {
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];\n" ::"r"(smem_u32(mbar)) : "memory");
 }
 
 // mbar_wait with the thread suspended between polls (up to `hint_ns` per poll,
