@@ -180,7 +180,7 @@ __device__ __forceinline__ void net_report(unsigned long long best, int cov, con
 // the distances its mask leaves, and the row is not read when none is left.
 // The test costs one 128-byte read per point, so it pays for rows longer than
 // that (dp > 16); shorter rows compute every distance.  root: the first pass
-// (D infinite) also reduces the farthest point of all into *root.
+// (D infinite) also reduces each hub's farthest point into root[hub].
 // Bound by the centres' shared-memory reads and the FP32 pipe where little is
 // pruned, by the latency of one chunk where the hub is small.
 // Build stage of 1M x 128 (mixture), 121k x 16 (uniform), 174k x 64 (mixture):
@@ -290,7 +290,7 @@ __global__ void __launch_bounds__(BT) k_net_update_l2(const float *__restrict__ 
             const unsigned long long v = __shfl_xor_sync(0xffffffffu, best, o);
             best = v > best ? v : best;
         }
-        if (lane == 0) atomicMax(root, best);
+        if (lane == 0) atomicMax(root + h, best);
     }
 }
 
@@ -605,7 +605,7 @@ __global__ void __launch_bounds__(BT) k_net_update_lev(Strings S, const int32_t 
         if (t % (LEV_P / NET_KEYS) == 0) {
             ch.keys[ck.z * NET_KEYS + t / (LEV_P / NET_KEYS)] = best;
             ch.cov[ck.z * NET_KEYS + t / (LEV_P / NET_KEYS)] = 0;  // no flat-split test for edit distance
-            if (root) atomicMax(root, best);
+            if (root) atomicMax(root + h, best);
         }
     }
 }
@@ -796,7 +796,7 @@ __global__ void __launch_bounds__(BT) k_net_update_ham(const uint32_t *__restric
             const unsigned long long k = __shfl_xor_sync(0xffffffffu, best, o);
             best = k > best ? k : best;
         }
-        if ((threadIdx.x & 31) == 0) atomicMax(root, best);
+        if ((threadIdx.x & 31) == 0) atomicMax(root + h, best);
     }
 }
 
@@ -1232,46 +1232,21 @@ __global__ void k_root_init(int64_t n, int root, int32_t *__restrict__ ids, floa
     lab[i] = 0;
 }
 
-// The root's first pass: hub 0 holds every point, its batch is position 0 with label 0.
-__global__ void k_root_hub(int64_t n, Hubs hb, int32_t *__restrict__ hslot, int32_t *__restrict__ bpos,
-                           int2 *__restrict__ hlist) {
-    hb.begin[0] = 0;
-    hb.count[0] = (int32_t)n;
-    hb.nc[0] = 1;
-    hb.m[0] = 1;
-    hb.done[0] = 0;
-    hb.thr[0] = 0.0f;
-    hb.key[0] = 0ull;
-    hslot[0] = 0;
-    bpos[0] = 0;
-    hlist[0] = make_int2(0, 0);
-}
-
-__global__ void k_root_node(int64_t n, int zeta, int metric, const unsigned long long *__restrict__ key,
-                            int32_t *__restrict__ node_begin, int32_t *__restrict__ node_count,
-                            int32_t *__restrict__ child_begin, int32_t *__restrict__ child_count,
-                            float *__restrict__ radius, int32_t *__restrict__ level, Hubs hb,
-                            int32_t *__restrict__ is_hub) {
-    float r = key_value(key[0]);
-    node_begin[0] = 0;
-    node_count[0] = (int32_t)n;
-    child_begin[0] = 0;
-    child_count[0] = 0;
-    radius[0] = round_radius_up(r, metric);
-    int l = r > 0.0f ? ceil_log2f(r) : INT_MIN;
-    level[0] = l;
-    int hub = (n > zeta && r > 0.0f) ? 1 : 0;
-    *is_hub = hub;
-    // the root hub for the first round
-    hb.begin[0] = 0;
-    hb.count[0] = (int32_t)n;
-    hb.node[0] = 0;
-    hb.nc[0] = 1;
-    hb.m[0] = 0;
-    hb.done[0] = 0;
-    hb.flat[0] = 0;
-    hb.level[0] = l;
-    hb.thr[0] = hub ? ldexpf(1.0f, l - 1) : 0.0f;
+// The roots' first pass: hub c holds every point of tree c, its batch is its
+// first position with label 0.
+__global__ void k_root_hubs(int R, const int32_t *__restrict__ rbegin, const int32_t *__restrict__ rcount, Hubs hb,
+                            int32_t *__restrict__ bpos, int2 *__restrict__ hlist) {
+    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    if (c >= R) return;
+    hb.begin[c] = rbegin[c];
+    hb.count[c] = rcount[c];
+    hb.nc[c] = 1;
+    hb.m[c] = 1;
+    hb.done[c] = 0;
+    hb.thr[c] = 0.0f;
+    hb.key[c] = 0ull;
+    bpos[(size_t)c * NET_M] = rbegin[c];
+    hlist[c] = make_int2(c, c);
 }
 
 // Rows already of dp = dim floats (dim a multiple of 4, 16-byte aligned
@@ -1489,12 +1464,29 @@ struct TreeGuard {
 };
 }  // namespace
 
-ct_tree *build_tree(const ct_points *pts, int zeta, int root, cudaStream_t s) {
+namespace {
+void finish_forest(const ct_tree &proto, const std::vector<int64_t> &off, int N, DBuf<int32_t> &ids, DBuf<float> &D,
+                   DBuf<int32_t> &nb, DBuf<int32_t> &ncnt, DBuf<int32_t> &cbeg, DBuf<int32_t> &ccnt,
+                   DBuf<int32_t> &lvl, DBuf<int32_t> &par, DBuf<float> &rad, const float *Xp, const uint32_t *Xb,
+                   std::vector<ct_tree *> &out, cudaStream_t s);
+
+// A tree of all points; or, with `off` (the first position of each tree, and
+// the end), a tree per range of points in `out`, all split together: their
+// levels share every launch.
+ct_tree *build_impl(const ct_points *pts, int zeta, int root, cudaStream_t s, const std::vector<int64_t> *off,
+                    std::vector<ct_tree *> *out) {
     const int64_t n = pts->n;
+    std::vector<int64_t> hroot;  // first position of each tree that has points
+    if (off) {
+        for (size_t c = 0; c + 1 < off->size(); ++c)
+            if ((*off)[c] < (*off)[c + 1]) hroot.push_back((*off)[c]);
+    } else if (n > 0) {
+        hroot.push_back(0);
+    }
     TreeGuard tg{new ct_tree()};
     ct_tree *t = tg.t;
     struct Flush { ~Flush() { prof_flush(); } } flush_at_exit;
-    ProfScope prof_all("build", s);
+    ProfScope prof_all("build", s, off ? (int64_t)off->size() - 1 : 1);
     t->metric = pts->metric;
     t->n = n;
     t->leaf_size = zeta;
@@ -1572,7 +1564,7 @@ ct_tree *build_tree(const ct_points *pts, int zeta, int root, cudaStream_t s) {
     }
 
     // tree arrays: a tree whose internal vertices have >= 2 children has < 2n vertices
-    const int64_t cap = 2 * n + 1;
+    const int64_t cap = 2 * n + 1 + (int64_t)hroot.size();
     DBuf<int32_t> nb(cap, s), ncnt(cap, s), cbeg(cap, s), ccnt(cap, s), lvl(cap, s), par(cap, s);
     CT_CHECK_CUDA(cudaMemsetAsync(par.p, 0xff, cap * sizeof(int32_t), s));
     DBuf<float> rad(cap, s);
@@ -1731,25 +1723,51 @@ ct_tree *build_tree(const ct_points *pts, int zeta, int root, cudaStream_t s) {
                 cov = DBuf<int32_t>(nchunks * NET_KEYS, s);
             }
         };
-        // the root's pass: a batch of one centre, position 0 (the memsets write zeros, k_root_hub the rest)
+        // the roots: vertices 0 .. R - 1, one hub each, with a batch of one centre (its first position)
+        const int R0 = (int)hroot.size();
+        DBuf<int32_t> rbegin(R0, s), rcount(R0, s);
+        {
+            std::vector<int32_t> hb(R0), hn(R0);
+            nchunks = 0;
+            for (int c = 0; c < R0; ++c) {
+                hb[c] = (int32_t)hroot[c];
+                hn[c] = (int32_t)((c + 1 < R0 ? hroot[c + 1] : n) - hroot[c]);
+                nchunks += ceil_div(hn[c], chunk_len);
+            }
+            CT_CHECK_CUDA(cudaMemcpyAsync(rbegin.p, hb.data(), R0 * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+            CT_CHECK_CUDA(cudaMemcpyAsync(rcount.p, hn.data(), R0 * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+            CT_CHECK_CUDA(cudaStreamSynchronize(s));  // the host arrays are on the stack
+        }
         DBuf<int64_t> i64tmp(4, s);
+        DBuf<int32_t> rhub(R0, s), rleafy(R0, s);
+        DBuf<int64_t> roff(R0, s);
+        if ((int64_t)bpos.n < (int64_t)R0 * NET_M) bpos = DBuf<int32_t>((size_t)R0 * NET_M, s);
         CT_CHECK_CUDA(cudaMemsetAsync(i64tmp.p, 0, 4 * sizeof(int64_t), s));
+        CT_CHECK_CUDA(cudaMemsetAsync(rleafy.p, 0, R0 * sizeof(int32_t), s));
         grow_chunks();
-        k_root_hub<<<1, 1, 0, s>>>(n, H, hslot.p, bpos.p, hl_a.p);
+        k_root_hubs<<<grid_for(R0), BT, 0, s>>>(R0, rbegin.p, rcount.p, H, bpos.p, hl_a.p);
         CT_COUNT_LAUNCH();
-        k_chunk_fill<<<grid_for(nchunks), BT, 0, s>>>(nchunks, 1, hl_a.p, H.begin, i64tmp.p, chunk_len, chunks_a.p);
+        k_chunk_counts<<<grid_for(R0), BT, 0, s>>>(R0, hl_a.p, H.count, chunk_len, rhub.p, hslot.p);
+        CT_COUNT_LAUNCH();
+        exclusive_scan_i32_to_i64(rhub.p, roff.p, R0, nullptr, s);
+        k_chunk_fill<<<grid_for(nchunks), BT, 0, s>>>(nchunks, R0, hl_a.p, H.begin, roff.p, chunk_len, chunks_a.p);
         CT_COUNT_LAUNCH();
         update(H, nchunks, chunks_a.p, Batch{bpos.p, cpos.p, dcc.p}, H.key);
-        DBuf<int32_t> is_root_hub(1, s);
-        k_root_node<<<1, 1, 0, s>>>(n, zeta, pts->metric, H.key, nb.p, ncnt.p, cbeg.p, ccnt.p, rad.p, lvl.p, H,
-                                    is_root_hub.p);
+        k_make_nodes<<<grid_for(R0), BT, 0, s>>>(R0, 0, zeta, pts->metric, rbegin.p, rcount.p, H.key, nb.p, ncnt.p,
+                                                 cbeg.p, ccnt.p, rad.p, lvl.p, rleafy.p, rhub.p);
+        CT_COUNT_LAUNCH();
+        exclusive_scan_i32_to_i64(rhub.p, roff.p, R0, i64tmp.p, s);
+        k_next_hubs<<<grid_for(R0), BT, 0, s>>>(R0, 0, rhub.p, roff.p, rbegin.p, rcount.p, H.key, lvl.p, H2, small_max,
+                                                chunk_len, hl_a.p, reinterpret_cast<int32_t *>(i64tmp.p + 1));
         CT_COUNT_LAUNCH();
         CT_LAUNCH_CHECK();
-        int32_t root_hub = 0;
-        to_host(&root_hub, is_root_hub.p, 1, s);
-        n_nodes = 1;
-        int64_t nh = root_hub ? 1 : 0;
-        int nl = root_hub && n > small_max ? 1 : 0;  // hubs of the level-wide passes
+        int64_t first[3] = {0, 0, 0};
+        to_host(first, i64tmp.p, 3, s);
+        std::swap(H, H2);
+        n_nodes = R0;
+        int64_t nh = first[0];
+        int nl = (int32_t)first[1];  // hubs of the level-wide passes
+        nchunks = (int32_t)first[2];
 
         // scratch for partitioning
         DBuf<uint32_t> pk(n, s), pv(n, s), tk(n, s), tv(n, s);
@@ -1877,6 +1895,10 @@ ct_tree *build_tree(const ct_points *pts, int zeta, int root, cudaStream_t s) {
     // ---- final layout
     t->n_nodes = n_nodes;
     t->depth = depth;
+    if (off) {
+        finish_forest(*t, *off, n_nodes, ids, D, nb, ncnt, cbeg, ccnt, lvl, par, rad, Xp.p, Xb.p, *out, s);
+        return nullptr;
+    }
     t->perm = ids.release();
     t->dcen = D.release();
     lab.reset();
@@ -2024,8 +2046,290 @@ ct_tree *build_tree(const ct_points *pts, int zeta, int root, cudaStream_t s) {
     return t;
 }
 
+// ---- Forests: trees built one after another cost their launches and
+// read-backs each (60 cells of 96820 x 64: 113 ms, 125 launches a tree); split
+// together they cost one tree's (5.2 ms).  The trees' vertices are created
+// level by level in one array;
+// a stable sort by tree gives each tree its own consecutive vertices (its root
+// first, siblings still consecutive), and every array is made relative to its
+// tree.
+
+// The tree (of R, by first position) that holds a position.
+__device__ __forceinline__ int tree_of(const int32_t *__restrict__ rbegin, int R, int pos) {
+    int lo = 0, hi = R;
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (__ldg(rbegin + mid) <= pos) lo = mid; else hi = mid;
+    }
+    return lo;
+}
+__global__ void k_tree_keys(int64_t n, const int32_t *__restrict__ pos, const uint32_t *__restrict__ order, int R,
+                            const int32_t *__restrict__ rbegin, uint32_t *__restrict__ keys,
+                            uint32_t *__restrict__ vals) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const uint32_t v = order ? order[i] : (uint32_t)i;
+    keys[i] = (uint32_t)tree_of(rbegin, R, pos[v]);
+    vals[i] = v;
+}
+// base[r] = first index of the (ascending) keys not below bound[r]; base[R] = n.
+__global__ void k_bounds(int R, int64_t n, const uint32_t *__restrict__ keys, const int32_t *__restrict__ bound,
+                         int32_t *__restrict__ base) {
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r > R) return;
+    const uint32_t want = r == R ? 0xffffffffu : bound ? (uint32_t)bound[r] : (uint32_t)r;
+    int64_t lo = 0, hi = n;
+    while (lo < hi) {
+        const int64_t mid = (lo + hi) >> 1;
+        if (r < R && keys[mid] >= want) hi = mid; else lo = mid + 1;
+    }
+    base[r] = (int32_t)lo;
+}
+__global__ void k_invert(int64_t n, const uint32_t *__restrict__ order, int32_t *__restrict__ inv) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) inv[order[i]] = (int32_t)i;
+}
+struct NodeArrays {
+    int32_t *begin, *count, *cbegin, *ccount, *level, *parent;
+    float *radius;
+};
+// Vertex j of the sorted order from its old record: indices in the sorted
+// order (children, parents; a root's parent becomes -2 - tree, so that
+// neighbouring trees' roots are no siblings).
+__global__ void k_forest_nodes(int64_t N, const uint32_t *__restrict__ order, const uint32_t *__restrict__ tree,
+                               const int32_t *__restrict__ inv, NodeArrays a, NodeArrays b) {
+    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= N) return;
+    const uint32_t v = order[j];
+    b.begin[j] = a.begin[v];
+    b.count[j] = a.count[v];
+    const int cc = a.ccount[v], p = a.parent[v];
+    b.ccount[j] = cc;
+    b.cbegin[j] = cc ? inv[a.cbegin[v]] : 0;
+    b.parent[j] = p >= 0 ? inv[p] : -2 - (int)tree[j];
+    b.level[j] = a.level[v];
+    b.radius[j] = a.radius[v];
+}
+// Everything relative to its tree.
+__global__ void k_forest_local(int64_t N, int64_t L, int64_t G, int64_t n, int R,
+                               const int32_t *__restrict__ rbegin, const int32_t *__restrict__ nbase,
+                               const int32_t *__restrict__ gbase, const uint32_t *__restrict__ ntree, NodeArrays b,
+                               const uint32_t *__restrict__ leaf_keys, const uint32_t *__restrict__ leaves,
+                               int32_t *__restrict__ leaf_ids, int32_t *__restrict__ group_begin,
+                               const uint32_t *__restrict__ gtree, const uint32_t *__restrict__ gsorted,
+                               int32_t *__restrict__ group_order, int32_t *__restrict__ perm) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < N) {
+        const int t = (int)ntree[i];
+        b.begin[i] -= rbegin[t];
+        if (b.ccount[i]) b.cbegin[i] -= nbase[t];
+        b.parent[i] = b.parent[i] >= 0 ? b.parent[i] - nbase[t] : -1;
+    }
+    if (i < L) leaf_ids[i] = (int32_t)leaves[i] - nbase[tree_of(rbegin, R, (int)leaf_keys[i])];
+    if (i < G) {
+        group_order[i] = (int32_t)gsorted[i] - gbase[gtree[i]];
+        group_begin[i] -= rbegin[tree_of(rbegin, R, group_begin[i])];
+    }
+    if (i < n) perm[i] -= rbegin[tree_of(rbegin, R, (int)i)];
+}
+
+void finish_forest(const ct_tree &proto, const std::vector<int64_t> &off, int N, DBuf<int32_t> &ids, DBuf<float> &D,
+                   DBuf<int32_t> &nb, DBuf<int32_t> &ncnt, DBuf<int32_t> &cbeg, DBuf<int32_t> &ccnt,
+                   DBuf<int32_t> &lvl, DBuf<int32_t> &par, DBuf<float> &rad, const float *Xp, const uint32_t *Xb,
+                   std::vector<ct_tree *> &out, cudaStream_t s) {
+    const int64_t n = proto.n;
+    const int C = (int)off.size() - 1, dp = proto.dp, wp = proto.wp;
+    const bool l2 = proto.metric == CT_L2_F32;
+    std::vector<int> tree_cell;  // the trees with points
+    std::vector<int32_t> hb;
+    for (int c = 0; c < C; ++c)
+        if (off[c] < off[c + 1]) {
+            tree_cell.push_back(c);
+            hb.push_back((int32_t)off[c]);
+        }
+    const int R = (int)hb.size();
+    // the arrays of all trees, released with the last tree
+    struct Blocks {
+        cudaStream_t s;
+        std::vector<void *> p;
+        ~Blocks() {
+            for (void *q : p) cudaFreeAsync(q, s);
+            cudaStreamSynchronize(s);
+        }
+    };
+    auto blocks = std::make_shared<Blocks>();
+    blocks->s = s;
+    auto take = [&](size_t bytes) {
+        void *q = dmalloc(bytes + 16, s);
+        blocks->p.push_back(q);
+        return q;
+    };
+    auto take_i = [&](int64_t k) { return (int32_t *)take((size_t)std::max<int64_t>(k, 1) * sizeof(int32_t)); };
+    DBuf<int32_t> rbegin(std::max(R, 1), s), nbase(R + 1, s), lbase(R + 1, s), gbase(R + 1, s);
+    if (R) CT_CHECK_CUDA(cudaMemcpyAsync(rbegin.p, hb.data(), R * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+    const int tbits = bits_for(R);
+    // vertices by tree
+    DBuf<uint32_t> nk(std::max(N, 1), s), nv(std::max(N, 1), s), tk(std::max(N, 1), s), tv(std::max(N, 1), s);
+    DBuf<int32_t> inv(std::max(N, 1), s);
+    NodeArrays a{nb.p, ncnt.p, cbeg.p, ccnt.p, lvl.p, par.p, rad.p}, b{};
+    b.begin = take_i(N);
+    b.count = take_i(N);
+    b.cbegin = take_i(N);
+    b.ccount = take_i(N);
+    b.level = take_i(N);
+    b.parent = take_i(N);
+    b.radius = (float *)take_i(N);
+    float *pts = nullptr, *ctr = nullptr;
+    uint32_t *bits = nullptr;
+    int32_t *perm = take_i(n);
+    float *dcen = (float *)take_i(n);
+    if (l2) {
+        pts = (float *)take((size_t)std::max<int64_t>(n, 1) * dp * sizeof(float));
+        ctr = (float *)take((size_t)std::max(N, 1) * dp * sizeof(float));
+    } else {
+        bits = (uint32_t *)take((size_t)std::max<int64_t>(n, 1) * wp * sizeof(uint32_t));
+    }
+    int32_t hc[2] = {0, 0};
+    DBuf<uint32_t> lk(std::max(N, 1), s), lv(std::max(N, 1), s);
+    DBuf<int32_t> cnts(2, s);
+    CT_CHECK_CUDA(cudaMemsetAsync(cnts.p, 0, 2 * sizeof(int32_t), s));
+    if (N) {
+        k_tree_keys<<<grid_for(N), BT, 0, s>>>(N, nb.p, nullptr, R, rbegin.p, nk.p, nv.p);
+        CT_COUNT_LAUNCH();
+        radix_sort_pairs(nk.p, nv.p, tk.p, tv.p, N, tbits, s);
+        k_bounds<<<grid_for(R + 1), BT, 0, s>>>(R, N, nk.p, nullptr, nbase.p);
+        CT_COUNT_LAUNCH();
+        k_invert<<<grid_for(N), BT, 0, s>>>(N, nv.p, inv.p);
+        CT_COUNT_LAUNCH();
+        k_forest_nodes<<<grid_for(N), BT, 0, s>>>(N, nv.p, nk.p, inv.p, a, b);
+        CT_COUNT_LAUNCH();
+        CT_CHECK_CUDA(cudaMemcpyAsync(perm, ids.p, n * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
+        CT_CHECK_CUDA(cudaMemcpyAsync(dcen, D.p, n * sizeof(float), cudaMemcpyDeviceToDevice, s));
+        if (l2) {
+            k_gather_rows<<<grid_for(n * (dp / 4)), BT, 0, s>>>(Xp, dp, perm, n, pts);
+            CT_COUNT_LAUNCH();
+            k_node_centres<<<grid_for((int64_t)N * (dp / 4)), BT, 0, s>>>(N, b.begin, pts, dp, ctr);
+        } else {
+            k_gather_bits<<<grid_for(n * (wp / 4)), BT, 0, s>>>(Xb, wp, perm, n, bits);
+        }
+        CT_COUNT_LAUNCH();
+        k_leaf_keys<<<grid_for(N), BT, 0, s>>>(N, b.ccount, b.begin, b.count, lk.p, lv.p, cnts.p, cnts.p + 1);
+        CT_COUNT_LAUNCH();
+        CT_LAUNCH_CHECK();
+    }
+    to_host(hc, cnts.p, 2, s);
+    const int L = hc[0];
+    // leaf blocks in position order, groups as in a single tree
+    int32_t *leaf_ids = take_i(L);
+    DBuf<int32_t> gstart(std::max(L, 1), s), gsize(std::max(L, 1), s), lcount(std::max(L, 1), s), lpar(std::max(L, 1), s);
+    DBuf<int64_t> gidx(std::max(L, 1), s), tot(2, s);
+    CT_CHECK_CUDA(cudaMemsetAsync(tot.p, 0, 2 * sizeof(int64_t), s));
+    if (L) {
+        radix_sort_pairs(lk.p, lv.p, tk.p, tv.p, L, bits_for(n), s);
+        k_bounds<<<grid_for(R + 1), BT, 0, s>>>(R, L, lk.p, rbegin.p, lbase.p);
+        CT_COUNT_LAUNCH();
+        const int32_t *leaves = reinterpret_cast<const int32_t *>(lv.p);
+        k_group_prep<<<grid_for(L), BT, 0, s>>>(L, leaves, b.count, b.parent, lcount.p, lpar.p);
+        CT_COUNT_LAUNCH();
+        k_group_marks<<<grid_for(L), BT, 0, s>>>(L, lcount.p, lpar.p, gstart.p, gsize.p,
+                                                 reinterpret_cast<unsigned long long *>(tot.p + 1));
+        CT_COUNT_LAUNCH();
+        exclusive_scan_i32_to_i64(gstart.p, gidx.p, L, tot.p, s);
+    }
+    int64_t gh[2] = {0, 0};
+    to_host(gh, tot.p, 2, s);
+    const int G = (int)gh[0];
+    int32_t *gbeg = take_i(G), *gcnt = take_i(G), *gord = take_i(G);
+    float *grad = (float *)take_i(G);
+    std::vector<int32_t> hn(R + 1, 0), hl(R + 1, 0), hg(R + 1, 0);
+    if (G) {
+        k_group_scatter<<<grid_for(L), BT, 0, s>>>(L, reinterpret_cast<const int32_t *>(lv.p), b.begin, gstart.p,
+                                                   gsize.p, gidx.p, gbeg, gcnt);
+        CT_COUNT_LAUNCH();
+        if (l2)
+            k_group_radius_l2<<<grid_for((int64_t)G * 32), BT, 0, s>>>(G, gbeg, gcnt, pts, dp, grad);
+        else
+            k_group_radius_ham<<<grid_for((int64_t)G * 32), BT, 0, s>>>(G, gbeg, gcnt, bits, wp, grad);
+        CT_COUNT_LAUNCH();
+        // walk order: by decreasing radius, then (stably) by tree
+        DBuf<uint32_t> ok(G, s), ov(G, s), ok2(G, s), ov2(G, s), sk(G, s), sv(G, s);
+        k_radius_desc_keys<<<grid_for(G), BT, 0, s>>>(G, grad, ok.p, ov.p);
+        CT_COUNT_LAUNCH();
+        radix_sort_pairs(ok.p, ov.p, sk.p, sv.p, G, 32, s);
+        k_tree_keys<<<grid_for(G), BT, 0, s>>>(G, gbeg, ov.p, R, rbegin.p, ok2.p, ov2.p);
+        CT_COUNT_LAUNCH();
+        radix_sort_pairs(ok2.p, ov2.p, sk.p, sv.p, G, tbits, s);
+        k_bounds<<<grid_for(R + 1), BT, 0, s>>>(R, G, ok2.p, nullptr, gbase.p);
+        CT_COUNT_LAUNCH();
+        const int64_t most = std::max<int64_t>(std::max<int64_t>(N, L), std::max<int64_t>(G, n));
+        k_forest_local<<<grid_for(most), BT, 0, s>>>(N, L, G, n, R, rbegin.p, nbase.p, gbase.p, nk.p, b, lk.p, lv.p,
+                                                     leaf_ids, gbeg, ok2.p, ov2.p, gord, perm);
+        CT_COUNT_LAUNCH();
+        CT_LAUNCH_CHECK();
+        to_host_async(hn.data(), nbase.p, R + 1, s);
+        to_host_async(hl.data(), lbase.p, R + 1, s);
+        to_host_async(hg.data(), gbase.p, R + 1, s);
+        CT_CHECK_CUDA(cudaStreamSynchronize(s));
+    }
+    // the trees: views of the arrays
+    std::vector<std::unique_ptr<ct_tree>> made;
+    for (int c = 0, r = 0; c < C; ++c) {
+        made.emplace_back(new ct_tree(proto));  // proto: metric, dimensions, leaf size, depth
+        ct_tree *t = made.back().get();
+        t->shared = blocks;
+        t->n = off[c + 1] - off[c];
+        const bool has = t->n > 0;
+        const int64_t p0 = has ? off[c] : 0, n0 = has ? hn[r] : 0, l0 = has ? hl[r] : 0, g0 = has ? hg[r] : 0;
+        t->n_nodes = has ? hn[r + 1] - hn[r] : 0;
+        t->n_leaves = has ? hl[r + 1] - hl[r] : 0;
+        t->n_groups = has ? hg[r + 1] - hg[r] : 0;
+        t->max_leaf_count = has ? hc[1] : 0;  // of the forest
+        t->max_group_count = has ? (int)gh[1] : 0;
+        t->perm = perm + p0;
+        t->dcen = dcen + p0;
+        if (l2) {
+            t->pts = pts + p0 * dp;
+            t->node_ctr = ctr + n0 * dp;
+        } else {
+            t->bits = bits + p0 * wp;
+        }
+        t->node_begin = b.begin + n0;
+        t->node_count = b.count + n0;
+        t->child_begin = b.cbegin + n0;
+        t->child_count = b.ccount + n0;
+        t->level = b.level + n0;
+        t->parent = b.parent + n0;
+        t->radius = b.radius + n0;
+        t->leaf_ids = leaf_ids + l0;
+        t->group_begin = gbeg + g0;
+        t->group_count = gcnt + g0;
+        t->group_radius = grad + g0;
+        t->group_order = gord + g0;
+        r += has ? 1 : 0;
+    }
+    for (auto &m : made) out.push_back(m.release());
+}
+
+}  // namespace
+
+ct_tree *build_tree(const ct_points *pts, int zeta, int root, cudaStream_t s) {
+    return build_impl(pts, zeta, root, s, nullptr, nullptr);
+}
+
+// A tree per consecutive range off[c] .. off[c + 1] - 1 of the points (the
+// root of each its first point); the trees share their device memory.
+std::vector<ct_tree *> build_forest(const ct_points *pts, const std::vector<int64_t> &off, int zeta, cudaStream_t s) {
+    std::vector<ct_tree *> out;
+    build_impl(pts, zeta, 0, s, &off, &out);
+    return out;
+}
+
 void free_tree(ct_tree *t) {
     if (!t) return;
+    if (t->shared) {  // a forest's memory goes with the last of its trees
+        delete t;
+        return;
+    }
     cudaStream_t s = t->stream;
     void *ptrs[] = {t->pts, t->bits, t->sdata, t->soff, t->perm, t->dcen, t->node_begin, t->node_count,
                     t->child_begin, t->child_count, t->radius, t->level, t->node_ctr, t->leaf_ids,

@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include <atomic>
+#include <memory>
 #include <string>
 #include <vector>
 
@@ -203,6 +204,9 @@ struct ct_tree {
     int32_t *group_count = nullptr;
     float *group_radius = nullptr;
     int32_t *group_order = nullptr;  // groups by decreasing radius (longest walks first)
+
+    // set for a tree of a forest: owns the memory its arrays are views into
+    std::shared_ptr<void> shared;
 };
 
 namespace ct {

@@ -5,7 +5,8 @@
 //   2. the ε-ghosts of every cell by Lemma 1: a point p outside cell k whose
 //      neighbours could lie in it, d(p, c_k) <= d(p, C) + 2 eps;
 //   3. one cover tree per cell over its points and ghosts (Algorithms 1-2),
-//      all cells queried in shared launches (the batched query);
+//      built together and queried together (a forest whose levels, and a batch
+//      whose stages, share their launches);
 //   4. every point's row taken from its own cell's CSR: by Lemma 1 each of
 //      its neighbours in another cell is a ghost of its own cell, so the row
 //      is complete there.
@@ -24,7 +25,7 @@
 
 namespace ct {
 
-ct_tree *build_tree(const ct_points *pts, int zeta, int root, cudaStream_t s);
+std::vector<ct_tree *> build_forest(const ct_points *pts, const std::vector<int64_t> &off, int zeta, cudaStream_t s);
 void free_tree(ct_tree *t);
 void query_batched(int n_clouds, const ct_tree *const *trees, const QParams *qps, const ct_query_opts *opts,
                    cudaStream_t s, QueryOut *outs);
@@ -274,14 +275,22 @@ void landmark_query(const ct_points *pts, const int64_t *centres_h, int m, doubl
     int64_t largest = 0;
     {
         ProfScope ps("landmark_build", s);
-        for (int k = 0; k < m; ++k) {
-            ct_points cp{};
-            cp.metric = pts->metric;
-            cp.dim = dim;
-            cp.n = hoff[k + 1] - hoff[k];
-            cp.data = l2 ? (const void *)(gx.p + hoff[k] * dim) : (const void *)(gb.p + hoff[k] * nb);
-            largest = std::max(largest, cp.n);
-            trees.t.push_back(build_tree(&cp, zeta, 0, s));
+        for (int k = 0; k < m; ++k) largest = std::max(largest, hoff[k + 1] - hoff[k]);
+        ct_points cp{};
+        cp.metric = pts->metric;
+        cp.dim = dim;
+        // forests of consecutive cells, within a bound on their points (scratch memory)
+        constexpr int64_t kForest = 1 << 24;
+        for (int k = 0; k < m;) {
+            int e = k + 1;
+            while (e < m && hoff[e + 1] - hoff[k] <= kForest) ++e;
+            ct_points fp = cp;
+            fp.n = hoff[e] - hoff[k];
+            fp.data = l2 ? (const void *)(gx.p + hoff[k] * dim) : (const void *)(gb.p + hoff[k] * nb);
+            std::vector<int64_t> off(hoff.begin() + k, hoff.begin() + e + 1);
+            for (int64_t &o : off) o -= hoff[k];
+            for (ct_tree *x : build_forest(&fp, off, zeta, s)) trees.t.push_back(x);
+            k = e;
         }
     }
     std::vector<QParams> qps((size_t)m, qp);

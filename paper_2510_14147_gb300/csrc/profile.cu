@@ -18,6 +18,7 @@ namespace {
 struct Pending {
     std::string name;
     cudaEvent_t a, b;
+    int64_t calls = 1;
     bool closed = false;  // its end event is recorded
     bool done = false;    // added to the table, events released
 };
@@ -34,10 +35,11 @@ std::vector<std::string> g_names;  // stable storage for returned names
 
 bool prof_on() { return g_on.load(std::memory_order_relaxed) != 0; }
 
-ProfScope::ProfScope(const char *name, cudaStream_t s) : s_(s), active_(prof_on()) {
+ProfScope::ProfScope(const char *name, cudaStream_t s, int64_t calls) : s_(s), active_(prof_on()) {
     if (!active_) return;
     Pending p;
     p.name = name;
+    p.calls = calls;
     cudaEventCreate(&p.a);
     cudaEventCreate(&p.b);
     cudaEventRecord(p.a, s);
@@ -68,7 +70,7 @@ void prof_flush() {
         if (cudaEventSynchronize(p.b) == cudaSuccess && cudaEventElapsedTime(&ms, p.a, p.b) == cudaSuccess) {
             Acc &a = g_acc[p.name];
             a.ms += ms;
-            a.calls += 1;
+            a.calls += p.calls;
         }
         cudaEventDestroy(p.a);
         cudaEventDestroy(p.b);

@@ -1,6 +1,7 @@
 // profile.cuh -- stage timing scopes (see profile.cu).
 #pragma once
 #include <cuda_runtime.h>
+#include <stdint.h>
 
 namespace ct {
 
@@ -10,7 +11,8 @@ void prof_flush();
 
 class ProfScope {
   public:
-    ProfScope(const char *name, cudaStream_t s);
+    // calls: what the stage counts as (a forest: one build per tree)
+    ProfScope(const char *name, cudaStream_t s, int64_t calls = 1);
     ~ProfScope();
     ProfScope(const ProfScope &) = delete;
     ProfScope &operator=(const ProfScope &) = delete;

@@ -65,3 +65,23 @@ def test_codes(bits, n):
     assert_csr_matches(csr.to_numpy(), oracle.brute_force(sp, bits // 8), integer_dist=True)
     code, msg = oracle.check_tree(sp, tree_from_export(tree), 0.0)
     assert code == 0, msg
+
+
+@pytest.mark.parametrize("metric", ["l2-dim7", "l2-dim16", "bits"])
+@pytest.mark.parametrize("centres", [[5], [0, 0, 1], [3, 700, 3, 12, 12, 900, 5]])
+def test_forest_with_empty_and_small_cells(metric, centres):
+    """The landmark form's trees are split together: repeated centres leave
+    cells without points, and some cells hold fewer points than a leaf."""
+    import torch
+    from paper_2510_14147_gb300 import ctgraph as cg
+    n = 1400
+    if metric == "bits":
+        rows = I.binary_codes(n, 96, n_centres=7, flip=0.06, seed=2)
+        args, eps, sp = {"bits": (torch.from_numpy(rows).cuda(), 96)}, 9, oracle.Space(bits=(rows, 96))
+    else:
+        x = I.gmm_embedded(n, dim=int(metric[6:]), intrinsic=4, n_centres=7, seed=3)
+        args, eps, sp = {"points": torch.from_numpy(x).cuda()}, 1.25, oracle.Space(points=x)
+    for kw in ({}, {"upper_triangle": True}):
+        csr, info = cg.eps_graph_query_landmark(centres, eps, **args, **kw)
+        assert info["cells"] == len(centres)
+        assert_csr_matches(csr.to_numpy(), oracle.brute_force(sp, eps), integer_dist=metric == "bits")
