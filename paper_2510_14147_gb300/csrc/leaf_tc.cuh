@@ -34,16 +34,6 @@ constexpr int FT_SCOUT = 4 * FT_PGROUPS, FT_MMA = FT_SCOUT + FT_ITEMS, FT_EPI = 
 constexpr int FT_EWARPS = 4 * FT_EGROUPS, FT_T = 32 * (FT_EPI + FT_EWARPS);
 static_assert(FT_EPI % 4 == 0, "an epilogue warp reads the tensor-memory lanes of its index mod 4");
 
-// A pair (global positions: the cloud's first row + tree position; the top
-// bit of y: a mirrored edge of the upper-triangle form).
-constexpr uint32_t PAIR_NONE = 0xffffffffu, PAIR_MIRROR = 0x80000000u;
-struct PairList {
-    uint2 *e;
-    int64_t cap;                // a multiple of FT_CHUNK
-    unsigned long long *n;      // entries reserved (may exceed cap: the rest was not stored)
-    unsigned long long *stat;   // valid pairs, kept pairs, rows
-};
-
 // The items of a wave, in increasing order: every FT_SAMPLE-th (the sample
 // that sizes the other waves), or part `part` of `parts` interleaved parts of
 // all items, or of those not in the sample.
@@ -534,13 +524,14 @@ __global__ void __launch_bounds__(256, 4) k_pairs(const __grid_constant__ Views 
                                                   const uint8_t *__restrict__ rowsel,
                                                   unsigned long long *__restrict__ st, int32_t *__restrict__ err) {
     const int lane = threadIdx.x & 31;
-    const int64_t total = list.cap;  // the entries, a multiple of 32
+    // the entries: all of cap, or the device's count of a list that did not run out
+    const int64_t total = !list.n ? list.cap : (int64_t)*list.n <= list.cap ? (int64_t)*list.n : 0;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
     unsigned long long guard = 0, band = 0;
     uint32_t done = 0;
     for (int64_t base = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32; base < total;
          base += warps * 32) {
-        const uint2 e = list.e[base + lane];
+        const uint2 e = base + lane < total ? list.e[base + lane] : make_uint2(PAIR_NONE, 0u);
         const bool valid = e.x != PAIR_NONE;
         const uint32_t gp = e.y & ~PAIR_MIRROR;
         int c = 0;

@@ -37,7 +37,10 @@ namespace {
 constexpr int TRAV_WARPS = 4;              // warps per traversal block
 constexpr int LEAF_T = 128;                // threads per leaf-tile block
 constexpr int KC = 128;                    // floats per K chunk of a tile
-constexpr int KS4 = KC / 4 + 1;            // padded row stride in float4
+// padded row stride of a tile in float4 (odd: rows 8 apart share no bank), for
+// rows of at most 64 floats and for longer ones (in chunks of KC)
+constexpr int KS_SHORT = 64 / 4 + 1, KS_LONG = KC / 4 + 1;
+constexpr bool short_rows(int dp) { return dp <= 64; }
 constexpr uint32_t FLAG = 0x80000000u;     // candidate produced an edge
 constexpr float PRUNE_REL = 1.0f + 0x1p-10f;
 constexpr float PRUNE_ABS = 0x1p-60f;
@@ -732,6 +735,7 @@ __device__ __forceinline__ void fill_tile(const TreeView &tv, const uint32_t *__
 // Loads rows (K chunk kc0 .. kc0 + 4 kq floats) into a padded shared tile;
 // row r comes from position pos[r] (or first + r when pos is null); rows
 // beyond `rows` are zero.
+template <int KS4>
 __device__ __forceinline__ void load_rows(float4 *__restrict__ tile, const float *__restrict__ pts, int dp,
                                           const int *pos, int first, int rows, int kc0, int kq) {
     for (int i = threadIdx.x; i < 32 * kq; i += LEAF_T) {
@@ -805,8 +809,10 @@ __device__ __forceinline__ float f2_sum(unsigned long long v) {
 // (FMA per term) and the chunk sums added into the total.  Contains barriers;
 // every thread of the block calls it.  On return the P tile is loaded and
 // every thread is past its last read of Qs/Ps for this call.
+template <int KS4>
 __device__ __forceinline__ void tile_accumulate(const float4 *Qs, const float4 *Ps, int kq, float (&tot)[2][4]);
 
+template <int KS4>
 __device__ __forceinline__ void tile_sqdist(const TreeView &tv, float4 *Qs, float4 *Ps, const int *prow, int npr,
                                             int qfirst, int nqr, int nkc, float (&tot)[2][4]) {
     const int dp = tv.dp;
@@ -818,10 +824,10 @@ __device__ __forceinline__ void tile_sqdist(const TreeView &tv, float4 *Qs, floa
         const int k0 = kc * KC;
         const int kq = min(KC, dp - k0) >> 2;
         if (kc > 0) __syncthreads();
-        if (nkc > 1) load_rows(Qs, tv.pts, dp, nullptr, qfirst, nqr, k0, kq);
-        load_rows(Ps, tv.pts, dp, prow, 0, npr, k0, kq);
+        if (nkc > 1) load_rows<KS4>(Qs, tv.pts, dp, nullptr, qfirst, nqr, k0, kq);
+        load_rows<KS4>(Ps, tv.pts, dp, prow, 0, npr, k0, kq);
         __syncthreads();
-        tile_accumulate(Qs, Ps, kq, tot);  // KC is a multiple of 16: chunks line up across K chunks
+        tile_accumulate<KS4>(Qs, Ps, kq, tot);  // KC is a multiple of 16: chunks line up across K chunks
     }
 }
 
@@ -830,6 +836,7 @@ __device__ __forceinline__ void tile_sqdist(const TreeView &tv, float4 *Qs, floa
 // and odd coordinates) are formed with FMA, added, and the chunk sum is added
 // into the running total: fp32 error of the squared distance <= ~19 u for
 // rows of 128 floats (u = 2^-24).
+template <int KS4>
 __device__ __forceinline__ void tile_accumulate(const float4 *Qs, const float4 *Ps, int kq, float (&tot)[2][4]) {
     const int tid = threadIdx.x, qi = tid >> 3, pj = tid & 7;
     const ulonglong2 *qa[2] = {reinterpret_cast<const ulonglong2 *>(Qs + qi * KS4),
@@ -886,12 +893,13 @@ __device__ __forceinline__ void tile_accumulate(const float4 *Qs, const float4 *
     }
 }
 
+template <int KS4>
 __device__ __forceinline__ void tile_sqdist_smem(const float4 *Qs, const float4 *Ps, int kq, float (&tot)[2][4]) {
 #pragma unroll
     for (int i = 0; i < 2; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) tot[i][j] = 0.f;
-    tile_accumulate(Qs, Ps, kq, tot);
+    tile_accumulate<KS4>(Qs, Ps, kq, tot);
 }
 
 // pair_sqdist with both rows in shared memory (plain loads).
@@ -926,6 +934,7 @@ __device__ __forceinline__ float pair_sqdist_smem(const float4 *x, const float4 
     return tot;
 }
 
+template <int KS4>
 struct LeafShared {
     float4 Qs[32 * KS4];
     float4 Ps[2][32 * KS4];
@@ -944,7 +953,9 @@ struct LeafShared {
     int64_t next_ci;
     int tpre[33];  // emit pass: pairs per row of the current tile (exclusive prefix)
 };
-constexpr size_t kLeafSmem = sizeof(LeafShared);
+constexpr size_t leaf_smem(bool shorts) {
+    return shorts ? sizeof(LeafShared<KS_SHORT>) : sizeof(LeafShared<KS_LONG>);
+}
 
 // One CTA per query group; queries in chunks of 32 (Q tile), candidate leaf
 // blocks in batches of NB.  Per batch:
@@ -1000,14 +1011,55 @@ __device__ __forceinline__ void cap_put(const CapOut &co, int o, int32_t c, floa
     cap_place(co, o, atomicAdd(&co.fill[o], 1), c, d);
 }
 
+// A pair (global positions: the cloud's first row + tree position; the top
+// bit of y: a mirrored edge of the upper-triangle form).
+constexpr uint32_t PAIR_NONE = 0xffffffffu, PAIR_MIRROR = 0x80000000u;
+struct PairList {
+    uint2 *e;
+    int64_t cap;
+    unsigned long long *n;      // entries reserved (may exceed cap: the rest was not stored)
+    unsigned long long *stat;   // tensor-core filter: valid pairs, kept pairs, rows
+};
+// A warp's part of the list: it reserves L2_CHUNK entries at a time and marks
+// what it leaves of the last ones.
+constexpr int L2_CHUNK = 128;
+struct PairCursor {
+    int64_t cur = 0, lim = 0;
+};
+// Appends n entries of the warp (each lane's from `at` of them on); room(i)
+// gives entry i's place.
+struct PairPlaces {
+    int64_t old, nxt;
+    int room;
+    __device__ __forceinline__ int64_t operator()(int i) const { return i < room ? old + i : nxt + (i - room); }
+};
+__device__ __forceinline__ PairPlaces pair_reserve(const PairList &pl, PairCursor &pc, int n) {
+    PairPlaces p{pc.cur, 0, (int)(pc.lim - pc.cur)};
+    if (n > p.room) {
+        const int more = ((n - p.room + L2_CHUNK - 1) / L2_CHUNK) * L2_CHUNK;
+        unsigned long long a = 0;
+        if ((threadIdx.x & 31) == 0) a = atomicAdd(pl.n, (unsigned long long)more);
+        p.nxt = (int64_t)__shfl_sync(0xffffffffu, a, 0);
+        pc.lim = p.nxt + more;
+        pc.cur = p.nxt + (n - p.room);
+    } else {
+        pc.cur += n;
+    }
+    return p;
+}
+__device__ __forceinline__ void pair_close(const PairList &pl, const PairCursor &pc) {
+    for (int64_t i = pc.cur + (threadIdx.x & 31); i < pc.lim && i < pl.cap; i += 32)
+        pl.e[i] = make_uint2(PAIR_NONE, 0u);
+}
+
 // One work item of the FP32 tiles (count or emit pass), by the whole CTA.
-template <bool EMIT>
+template <bool EMIT, int KS4>
 __device__ __forceinline__ void leaf_l2_item(
     const Views &V, const Items &items, const int it, const uint32_t *__restrict__ cand,
     uint32_t *__restrict__ emask, int32_t *__restrict__ deg, const int64_t *__restrict__ row_ptr,
     int32_t *__restrict__ rowcur, int32_t *__restrict__ col, float *__restrict__ dist,
     unsigned long long *__restrict__ st, int32_t *__restrict__ err, const CapOut &co,
-    const uint8_t *__restrict__ rowsel, LeafShared &S) {
+    const uint8_t *__restrict__ rowsel, const PairList &pl, PairCursor &pc, LeafShared<KS4> &S) {
     if (it >= *items.count) return;
     const int gg = items.group[it];
     const int cloud = cloud_of_group(V, gg);
@@ -1020,6 +1072,7 @@ __device__ __forceinline__ void leaf_l2_item(
     const int dp = tv.dp, dim = tv.dim;
     const int nkc = (dp + KC - 1) / KC;
     const int kq = dp >> 2;  // float4 per row when nkc == 1
+    const unsigned kq_inv = (65536u + kq - 1) / kq;  // i / kq = i * kq_inv >> 16: the excess stays below 1024 / 65536 < 1 / kq
     const bool fp32_dist_ok = dp <= 128;
     const int qb = tv.group_begin[g], qn = tv.group_count[g];
     const int qe = qb + qn;       // the group's positions: [qb, qe)
@@ -1051,6 +1104,10 @@ __device__ __forceinline__ void leaf_l2_item(
     for (int q0 = 0; q0 < qn; q0 += 32) {
         const int nqr = min(32, qn - q0);
         const int qfirst = qb + q0;
+        auto pair_of = [&](int q, int ppos) {
+            return make_uint2((uint32_t)(rbase + qfirst + q),
+                              (uint32_t)(rbase + ppos) | (half && ppos >= qe ? PAIR_MIRROR : 0u));
+        };
         __syncthreads();
         if (tid < 32) {
             S.qcnt[tid] = 0;
@@ -1070,7 +1127,7 @@ __device__ __forceinline__ void leaf_l2_item(
         }
         if (tid == 0) S.gn = 0;
         int cnt0 = 0, cnt1 = 0;
-        if (nkc == 1) load_rows(S.Qs, tv.pts, dp, nullptr, qfirst, nqr, 0, kq);
+        if (nkc == 1) load_rows<KS4>(S.Qs, tv.pts, dp, nullptr, qfirst, nqr, 0, kq);
 
         // decides the queued guard-band pairs; `all` drains everything, else
         // whole warps' worth and keeps the rest
@@ -1090,6 +1147,10 @@ __device__ __forceinline__ void leaf_l2_item(
                     if (!EMIT) {
                         atomicAdd(&S.qcnt[q], 1);
                         atomicOr(&S.bem[li], 1u << q);
+                        if (pl.e) {  // few: an entry of its own each
+                            const int64_t at = (int64_t)atomicAdd(pl.n, 1ull);
+                            if (at < pl.cap) pl.e[at] = pair_of(q, ppos);
+                        }
                         if (co.off) cap_put(co, S.cursor[q], tv.perm[ppos], (float)sqrt(s64));
                     } else if ((S.selm >> q) & 1u) {
                         int slot = atomicAdd(&rowcur[S.cursor[q]], 1);
@@ -1128,7 +1189,7 @@ __device__ __forceinline__ void leaf_l2_item(
             const int rows = min(32, nrows - r0);
             float4 *dst = S.Ps[buf];
             for (int i = tid; i < 32 * kq; i += LEAF_T) {
-                const int r = i / kq, k = i - r * kq;
+                const int r = (int)(((unsigned)i * kq_inv) >> 16), k = i - r * kq;  // i / kq (i < 1024, kq <= 32)
                 const bool valid = r < rows;
                 const int pos = valid ? rowsrc[r0 + r] : qfirst;
                 cp_async16(dst + r * KS4 + k, tv.pts + (size_t)pos * dp + 4 * k, valid);
@@ -1137,10 +1198,10 @@ __device__ __forceinline__ void leaf_l2_item(
         };
         auto compute = [&](int t, int buf, const int *rowsrc, int nrows, float (&tot)[2][4]) {
             if (nkc == 1) {
-                tile_sqdist_smem(S.Qs, S.Ps[buf], kq, tot);
+                tile_sqdist_smem<KS4>(S.Qs, S.Ps[buf], kq, tot);
             } else {
                 const int r0 = 32 * t;
-                tile_sqdist(tv, S.Qs, S.Ps[0], rowsrc + r0, min(32, nrows - r0), qfirst, nqr, nkc, tot);
+                tile_sqdist<KS4>(tv, S.Qs, S.Ps[0], rowsrc + r0, min(32, nrows - r0), qfirst, nqr, nkc, tot);
             }
         };
 
@@ -1449,6 +1510,23 @@ __device__ __forceinline__ void leaf_l2_item(
                             }
                         }
                     }
+                    if (!EMIT && pl.e && __any_sync(0xffffffffu, hitrow != 0u)) {  // the edges, for the emit pass
+                        const int c = __popc(hitrow);
+                        int incl = c;
+#pragma unroll
+                        for (int o = 1; o < 32; o <<= 1) {
+                            const int y = __shfl_up_sync(0xffffffffu, incl, o);
+                            if (lane >= o) incl += y;
+                        }
+                        const PairPlaces place = pair_reserve(pl, pc, __shfl_sync(0xffffffffu, incl, 31));
+                        uint32_t m = hitrow;
+                        for (int i = incl - c; m; ++i) {
+                            const int x = __ffs(m) - 1, j = x >> 2;
+                            m &= m - 1u;
+                            const int64_t at = place(i);
+                            if (at < pl.cap) pl.e[at] = pair_of(qi + 16 * (x & 1), S.rpos[32 * t + pj + 8 * j]);
+                        }
+                    }
                     if (!EMIT && hitrow) {
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {
@@ -1503,16 +1581,25 @@ __device__ __forceinline__ void leaf_l2_item(
     }
 }
 
-// One CTA per work item.
-template <bool EMIT>
-__global__ void __launch_bounds__(LEAF_T, 3) k_leaf_l2(
+// One CTA per work item.  Rows of at most 64 floats take a shorter tile stride
+// and fewer registers, so that five CTAs share an SM instead of three (a tile
+// is a chain of copy, barrier, arithmetic, barrier: more of them in flight).
+// 174k x 64 at 87 neighbours: count 16.3 -> 14.1 ms, bound by the shared-memory
+// reads of the micro-tiles (71 % of that pipe, four wavefronts per 16-byte
+// read whatever is broadcast) and the FP32 pipe (58 %).  The emit pass reads
+// the list of edges instead of the blocks' pairs: 4.8 -> 0.8 ms.
+template <bool EMIT, int KS4>
+__global__ void __launch_bounds__(LEAF_T, KS4 == KS_SHORT ? 5 : 3) k_leaf_l2(
     const __grid_constant__ Views V, Items items, const uint32_t *__restrict__ cand,
     uint32_t *__restrict__ emask, int32_t *__restrict__ deg, const int64_t *__restrict__ row_ptr,
     int32_t *__restrict__ rowcur, int32_t *__restrict__ col, float *__restrict__ dist,
-    unsigned long long *__restrict__ st, int32_t *__restrict__ err, CapOut co, const uint8_t *__restrict__ rowsel) {
+    unsigned long long *__restrict__ st, int32_t *__restrict__ err, CapOut co, const uint8_t *__restrict__ rowsel,
+    PairList pl) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    leaf_l2_item<EMIT>(V, items, blockIdx.x, cand, emask, deg, row_ptr, rowcur, col, dist, st, err, co, rowsel,
-                       *reinterpret_cast<LeafShared *>(smem_raw));
+    PairCursor pc;
+    leaf_l2_item<EMIT, KS4>(V, items, blockIdx.x, cand, emask, deg, row_ptr, rowcur, col, dist, st, err, co, rowsel,
+                            pl, pc, *reinterpret_cast<LeafShared<KS4> *>(smem_raw));
+    if (!EMIT && pl.e) pair_close(pl, pc);
 }
 
 // Work items: every pool segment split into slices of at most kItem blocks.
@@ -1846,12 +1933,17 @@ __global__ void __launch_bounds__(H16_T) k_to_h16(const __grid_constant__ Views 
 
 #include "leaf_tc.cuh"
 
-// Dynamic shared memory of the L2 leaf kernel (set once per process).
+// Dynamic shared memory of the L2 leaf kernels (set once per process).
 void leaf_l2_prepare() {
     static bool done = false;
     if (done) return;
-    CT_CHECK_CUDA(cudaFuncSetAttribute(k_leaf_l2<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLeafSmem));
-    CT_CHECK_CUDA(cudaFuncSetAttribute(k_leaf_l2<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLeafSmem));
+    auto allow = [](auto kern, bool shorts) {
+        CT_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)leaf_smem(shorts)));
+    };
+    allow(k_leaf_l2<true, KS_SHORT>, true);
+    allow(k_leaf_l2<false, KS_SHORT>, true);
+    allow(k_leaf_l2<true, KS_LONG>, false);
+    allow(k_leaf_l2<false, KS_LONG>, false);
     done = true;
 }
 
@@ -3054,7 +3146,7 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
     Views V;
     std::memset(&V, 0, sizeof(V));
     V.nc = C;
-    int max_dp = 4, max_depth = 0, max_len = 0, min_len = kItemTC;
+    int max_dp = 4, max_fp_dp = 4, max_depth = 0, max_len = 0, min_len = kItemTC;
     bool any_tc = false, any_fp = false, any_half = false;
     for (int c = 0; c < C; ++c) {
         const ct_tree *tc = trees[c];
@@ -3071,6 +3163,7 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
         V.gbase[c + 1] = V.gbase[c] + tc->n_groups;
         V.rbase[c + 1] = V.rbase[c] + tc->n;
         max_dp = std::max(max_dp, tc->dp);
+        if (!ch.use_tc) max_fp_dp = std::max(max_fp_dp, tc->dp);
         max_depth = std::max(max_depth, tc->depth);
         max_len = std::max(max_len, tc->max_len);
     }
@@ -3361,6 +3454,27 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
         co = CapOut{lp.cap_off.p, c_fill.p, c_ent.p, o_ent.p, o_n.p, lp.arena > 0 ? lp.arena : 0, lost.p};
     }
 
+    // FP32 tiles, two-pass form: the count pass lists its edges for the emit
+    // pass (8 bytes each; dp <= 128), which then decides only those again
+    // instead of every pair of an edge-bearing block and query.  The list holds
+    // 192 edges per point, within an eighth of the free memory; past that the
+    // emit pass takes the blocks' masks.
+    DBuf<uint2> fp_e;
+    DBuf<unsigned long long> fp_n(1, s);
+    PairList fp_list{};
+    if (l2 && any_fp && !capmode && !probe && max_fp_dp <= 128 && n > 0) {
+        size_t fr = 0, tot = 0;
+        int64_t cap = 192 * n + (int64_t)num_sms() * 5 * 4 * L2_CHUNK;
+        if (cudaMemGetInfo(&fr, &tot) == cudaSuccess) cap = std::min(cap, (int64_t)(fr / 8 / sizeof(uint2)));
+        else cudaGetLastError();
+        if (capacity_budget() > 0) cap = std::min<int64_t>(cap, capacity_budget() / (int64_t)sizeof(uint2));
+        fp_e = DBuf<uint2>((size_t)std::max<int64_t>(cap, 1), s);
+        CT_CHECK_CUDA(cudaMemsetAsync(fp_n.p, 0, sizeof(unsigned long long), s));
+        fp_list = PairList{fp_e.p, std::max<int64_t>(cap, 1), fp_n.p, nullptr};
+    }
+    bool fp_listed = false;  // the list holds every edge of the FP32 items
+    unsigned long long fp_entries = 0;
+
     // 2. count pass
     DBuf<int32_t> deg(n + 1, s);
     CT_CHECK_CUDA(cudaMemsetAsync(deg.p, 0, (n + 1) * sizeof(int32_t), s));
@@ -3370,10 +3484,14 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
         const CapOut cw = emit ? CapOut{} : co;
         if (l2) {
             leaf_l2_prepare();
-            if (emit)
-                k_leaf_l2<true><<<(unsigned)max_items, LEAF_T, kLeafSmem, s>>>(V, items, cand_p, emask.p, deg.p, row_ptr, rowcur.p, col, dist, st.p, err, cw, rowsel);
-            else
-                k_leaf_l2<false><<<(unsigned)max_items, LEAF_T, kLeafSmem, s>>>(V, items, cand_p, emask.p, deg.p, row_ptr, rowcur.p, col, dist, st.p, err, cw, rowsel);
+            const bool sh = short_rows(max_fp_dp);
+            auto go = [&](auto kern) {
+                kern<<<(unsigned)max_items, LEAF_T, leaf_smem(sh), s>>>(V, items, cand_p, emask.p, deg.p, row_ptr, rowcur.p, col, dist, st.p, err, cw, rowsel, emit ? PairList{} : fp_list);
+            };
+            if (emit && sh) go(k_leaf_l2<true, KS_SHORT>);
+            else if (emit) go(k_leaf_l2<true, KS_LONG>);
+            else if (sh) go(k_leaf_l2<false, KS_SHORT>);
+            else go(k_leaf_l2<false, KS_LONG>);
         } else if (ham) {
             const size_t hsm = (size_t)64 * (t->wp / 4) * sizeof(uint4);  // 32 query rows + 32 candidate rows
             if (emit)
@@ -3547,7 +3665,8 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
     }
     // emit pass (rowsel: of the selected rows)
     auto emit = [&](const uint8_t *rowsel) {
-        if (!l2 || any_fp) leaf(true, all.row_ptr, all.col, all.dist, rowsel, items_fp);
+        if (fp_listed) tc_pairs(PAIRS_EMIT, fp_e.p, (int64_t)fp_entries, rowsel);
+        else if (!l2 || any_fp) leaf(true, all.row_ptr, all.col, all.dist, rowsel, items_fp);
         DBuf<uint2> list;
         for (auto &w : waves) {
             if (lists_kept) {
@@ -3588,7 +3707,9 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
     all.row_ptr = row_ptr;
     exclusive_scan_i32_to_i64(deg.p, row_ptr, n + 1, nullptr, s);
     int64_t nnz = 0;
+    if (fp_list.e) to_host_async(&fp_entries, fp_n.p, 1, s);
     to_host(&nnz, row_ptr + n, 1, s);
+    fp_listed = fp_list.e && (int64_t)fp_entries <= fp_list.cap;
     all.nnz = nnz;
     all.col = (int32_t *)dmalloc((size_t)(nnz ? nnz : 1) * sizeof(int32_t), s);
     all.dist = (float *)dmalloc((size_t)(nnz ? nnz : 1) * sizeof(float), s);
@@ -3817,22 +3938,25 @@ __device__ __forceinline__ int queue_next(const Queue &Q, int32_t *err) {
 
 // The FP32 tiles as one persistent launch over the queue (count pass:
 // produce, then consume; emit pass: consume the complete queue again).
-template <bool EMIT>
-__global__ void __launch_bounds__(LEAF_T, 3) k_leaf_l2_queue(
+template <bool EMIT, int KS4>
+__global__ void __launch_bounds__(LEAF_T, KS4 == KS_SHORT ? 5 : 3) k_leaf_l2_queue(
     const __grid_constant__ Views V, Queue Q, const uint32_t *__restrict__ cand, uint32_t *__restrict__ emask,
     int32_t *__restrict__ deg, const int64_t *__restrict__ row_ptr, int32_t *__restrict__ rowcur,
     int32_t *__restrict__ col, float *__restrict__ dist, unsigned long long *__restrict__ st,
-    int32_t *__restrict__ err) {
+    int32_t *__restrict__ err, PairList pl) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    LeafShared &S = *reinterpret_cast<LeafShared *>(smem_raw);
+    LeafShared<KS4> &S = *reinterpret_cast<LeafShared<KS4> *>(smem_raw);
+    if (EMIT && pl.e && (int64_t)*pl.n <= pl.cap) return;  // the count pass listed every edge: k_pairs emits them
+    PairCursor pc;
     if (Q.produce) queue_produce(V, Q, err);
     const Items items{Q.group, Q.begin, Q.end, Q.tail};
     for (;;) {
         const int it = queue_next(Q, err);
         if (it < 0) break;
-        leaf_l2_item<EMIT>(V, items, it, cand, emask, deg, row_ptr, rowcur, col, dist, st, err, CapOut{}, nullptr,
-                           S);
+        leaf_l2_item<EMIT, KS4>(V, items, it, cand, emask, deg, row_ptr, rowcur, col, dist, st, err, CapOut{}, nullptr,
+                                EMIT ? PairList{} : pl, pc, S);
     }
+    if (!EMIT && pl.e) pair_close(pl, pc);
 }
 
 // Candidate ranges per group from the walk's segments (segment count read on
@@ -3957,6 +4081,8 @@ struct PlanImpl {
     DBuf<int32_t> seg_group, seg_count, col, sort_lists, sort_counts;
     DBuf<int64_t> seg_begin, gbegin, ibeg, iend, sums, row_ptr, rel;
     DBuf<float> dist, big_tmpd;
+    DBuf<uint2> pair_e;               // edges of the count pass, for the emit pass (rows of at most 128 floats)
+    DBuf<unsigned long long> pair_n;  // entries reserved
     DBuf<int64_t> big_lens, big_off;
     DBuf<uint64_t> big_k1, big_k2;
     DBuf<uint32_t> big_v1, big_v2;
@@ -4017,9 +4143,17 @@ void plan_enqueue(PlanImpl &p, cudaStream_t s) {
     CT_CHECK_CUDA(cudaMemsetAsync(p.deg.p, 0, (size_t)(n + 1) * sizeof(int32_t), s));
     Queue Q{p.qctr.p, p.qctr.p + 1, p.qctr.p + 2, p.qctr.p + 3, p.ready.p, p.igroup.p, p.ibeg.p, p.iend.p,
             p.order.p, p.gcount.p, p.gbegin.p, p.ctl.p, p.cand_cap, G, (int)p.item_cap, 1};
-    k_leaf_l2_queue<false><<<p.leaf_grid, LEAF_T, kLeafSmem, s>>>(V, Q, p.gcand.p, p.emask.p, p.deg.p, nullptr,
-                                                                  nullptr, nullptr, nullptr, st, err);
-    CT_COUNT_LAUNCH();
+    // (it lists the edges; the emit pass decides those again, or walks the queue when the list ran out)
+    const bool sh = short_rows(p.max_dp);
+    const PairList pl{p.pair_e.p, (int64_t)p.pair_e.n, p.pair_n.p, nullptr};
+    CT_CHECK_CUDA(cudaMemsetAsync(p.pair_n.p, 0, sizeof(unsigned long long), s));
+    auto leaf_queue = [&](auto kern, int64_t *rp) {
+        kern<<<p.leaf_grid, LEAF_T, leaf_smem(sh), s>>>(V, Q, p.gcand.p, p.emask.p, p.deg.p, rp, p.rowcur.p, p.col.p,
+                                                        p.dist.p, st, err, pl);
+        CT_COUNT_LAUNCH();
+    };
+    if (sh) leaf_queue(k_leaf_l2_queue<false, KS_SHORT>, nullptr);
+    else leaf_queue(k_leaf_l2_queue<false, KS_LONG>, nullptr);
     // 4. scan; a run above the plan's edge capacity empties every row
     exclusive_scan_i32_to_i64_into(p.deg.p, p.row_ptr.p, n + 1, nullptr, p.sums.p, s);
     k_plan_nnz_check<<<1, 1, 0, s>>>(p.row_ptr.p, n, p.nnz_cap, p.empty_flag.p, err);
@@ -4030,9 +4164,13 @@ void plan_enqueue(PlanImpl &p, cudaStream_t s) {
     CT_CHECK_CUDA(cudaMemsetAsync(p.qctr.p + 2, 0, sizeof(int32_t), s));
     CT_CHECK_CUDA(cudaMemsetAsync(p.rowcur.p, 0, (size_t)(n + 1) * sizeof(int32_t), s));
     Q.produce = 0;
-    k_leaf_l2_queue<true><<<p.leaf_grid, LEAF_T, kLeafSmem, s>>>(V, Q, p.gcand.p, p.emask.p, p.deg.p, p.row_ptr.p,
-                                                                 p.rowcur.p, p.col.p, p.dist.p, st, err);
-    CT_COUNT_LAUNCH();
+    if (sh) leaf_queue(k_leaf_l2_queue<true, KS_SHORT>, p.row_ptr.p);
+    else leaf_queue(k_leaf_l2_queue<true, KS_LONG>, p.row_ptr.p);
+    if (pl.e) {
+        k_pairs<PAIRS_EMIT><<<num_sms() * 8, 256, 0, s>>>(V, pl, p.deg.p, CapOut{}, p.row_ptr.p, p.rowcur.p, p.col.p,
+                                                          p.dist.p, nullptr, st, err);
+        CT_COUNT_LAUNCH();
+    }
     k_check_rows<<<grid_for(n, 256), 256, 0, s>>>(n, p.row_ptr.p, p.rowcur.p, err);
     CT_COUNT_LAUNCH();
     // 6. rows sorted in place (rows above the in-place sorts' length are reported)
@@ -4218,13 +4356,24 @@ PlanImpl *plan_create(int C, const ct_tree *const *trees, const QParams *qps, in
     leaf_l2_prepare();
     {
         int per_sm = 0;
-        CT_CHECK_CUDA(cudaFuncSetAttribute(k_leaf_l2_queue<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)kLeafSmem));
-        CT_CHECK_CUDA(cudaFuncSetAttribute(k_leaf_l2_queue<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)kLeafSmem));
-        CT_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_leaf_l2_queue<false>, LEAF_T,
-                                                                    kLeafSmem));
+        const bool sh = short_rows(p.max_dp);
+        auto resident = [&](auto kern) {
+            int b = 0;
+            CT_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)leaf_smem(sh)));
+            CT_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kern, LEAF_T, leaf_smem(sh)));
+            per_sm = per_sm ? std::min(per_sm, b) : b;
+        };
+        if (sh) {
+            resident(k_leaf_l2_queue<false, KS_SHORT>);
+            resident(k_leaf_l2_queue<true, KS_SHORT>);
+        } else {
+            resident(k_leaf_l2_queue<false, KS_LONG>);
+            resident(k_leaf_l2_queue<true, KS_LONG>);
+        }
         p.leaf_grid = std::max(1, num_sms() * std::max(per_sm, 1));
+        p.pair_n = DBuf<unsigned long long>(1, s);
+        if (p.max_dp <= 128)  // the edges, and what each warp leaves of its last entries
+            p.pair_e = DBuf<uint2>((size_t)(p.nnz_cap + (int64_t)p.leaf_grid * (LEAF_T / 32) * L2_CHUNK), s);
     }
     {
         const size_t tsm = (size_t)TRAV_WARPS * p.max_dp * sizeof(float);
@@ -4461,9 +4610,13 @@ void degrees_noalloc(const ct_tree *t, const QParams &qp, int32_t *degrees, cuda
         CT_COUNT_LAUNCH();
         Items items{igroup, ibeg, iend, nitems};
         leaf_l2_prepare();
-        k_leaf_l2<false><<<(unsigned)max_items, LEAF_T, kLeafSmem, s>>>(V, items, pool, nullptr, degrees, nullptr,
-                                                                          nullptr, nullptr, nullptr, st, err, CapOut{},
-                                                                          nullptr);
+        auto go = [&](auto kern, bool sh) {
+            kern<<<(unsigned)max_items, LEAF_T, leaf_smem(sh), s>>>(V, items, pool, nullptr, degrees, nullptr, nullptr,
+                                                                    nullptr, nullptr, st, err, CapOut{}, nullptr,
+                                                                    PairList{});
+        };
+        if (short_rows(t->dp)) go(k_leaf_l2<false, KS_SHORT>, true);
+        else go(k_leaf_l2<false, KS_LONG>, false);
         CT_COUNT_LAUNCH();
     }
     CT_LAUNCH_CHECK();
