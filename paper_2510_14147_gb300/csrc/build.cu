@@ -343,20 +343,48 @@ __device__ __forceinline__ int net_candidates(const Chunks &ch, int64_t first, i
     return total;
 }
 
-// The farthest of n candidates (lowest index among equals) as (distance bits,
-// ~index); every warp computes it for itself.
-__device__ __forceinline__ unsigned long long net_farthest(const float *cd, int n) {
-    unsigned long long best = 0ull;
-    for (int i = threadIdx.x & 31; i < n; i += 32) {
-        const unsigned long long k = pack_max_key(cd[i], (uint32_t)i);
-        best = k > best ? k : best;
-    }
+// The picks of one warp from n <= C candidates, farthest-first: each time the
+// candidate farthest from every centre so far (lowest index among equals),
+// while it lies beyond the threshold; pd(i, j): their mutual distances.  Two
+// warp reductions and a row of pd per pick.  Returns the number of picks.
+template <int C, class Pd>
+__device__ __forceinline__ int net_greedy(const float *cd, int n, float thr, int mcap, int *picks, Pd pd) {
+    const int lane = threadIdx.x & 31;
+    float d[C / 32];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long v = __shfl_xor_sync(0xffffffffu, best, o);
-        best = v > best ? v : best;
+    for (int k = 0; k < C / 32; ++k) d[k] = lane + 32 * k < n ? cd[lane + 32 * k] : 0.f;
+    int m = 0;
+    for (; m < mcap; ++m) {
+        float best = d[0];
+#pragma unroll
+        for (int k = 1; k < C / 32; ++k) best = fmaxf(best, d[k]);
+        // distances are not negative: their bits order as they do
+        const unsigned top = __reduce_max_sync(0xffffffffu, __float_as_uint(best));
+        if (!(__uint_as_float(top) > thr)) break;
+        unsigned at = 0xffffffffu;
+#pragma unroll
+        for (int k = C / 32 - 1; k >= 0; --k)
+            if (__float_as_uint(d[k]) == top) at = (unsigned)(lane + 32 * k);
+        const int pick = (int)__reduce_min_sync(0xffffffffu, at);
+        if (lane == 0) picks[m] = pick;
+#pragma unroll
+        for (int k = 0; k < C / 32; ++k)
+            if (lane + 32 * k < n) d[k] = fminf(d[k], pd(pick, lane + 32 * k));
     }
-    return best;
+    __syncwarp();
+    return m;
+}
+
+// Tile idx of the upper triangle (with its diagonal) of T x T tiles, rows
+// rp and T - 1 - rp folded into one row of T + 1; false: none.
+__device__ __forceinline__ bool upper_tile(int idx, int T, int &ti, int &tj) {
+    const int rp = idx / (T + 1), c = idx - rp * (T + 1);
+    ti = rp;
+    tj = rp + c;
+    if (c < T - rp) return true;
+    ti = T - 1 - rp;
+    tj = ti + (c - (T - rp));
+    return ti > rp;
 }
 
 // A hub's batch taken (thread 0): m centres after the nc it had, or done.
@@ -368,73 +396,96 @@ __device__ __forceinline__ void net_take(Hubs hb, int h, int m, bool flat, int32
     if (m) atomicAdd(active, 1);
 }
 
-// The next batch of a hub (one CTA per listed hub {hub, slot}).  The
-// candidates' rows are staged in shared memory where they fit.
-template <int TPD>
+// The next batch of a hub (one CTA per listed hub {hub, slot}): at most C
+// candidates, all their mutual distances at once (4 x 4 micro-tiles from rows
+// staged in shared memory; rows too long for it, TPD lanes per pair), then one
+// warp picks.  (Picking with a block-wide distance update per pick, two
+// barriers each, took 29 us at 121k x 16: 13 now; 15 at 100k x 64: 8.)
+// 128 candidates up to 32 floats per row, 64 above: the distances grow with both.
+template <int C, int TPD>
 __global__ void __launch_bounds__(BT) k_net_select_l2(const float *__restrict__ X, int dp,
                                                       const int32_t *__restrict__ ids, const int2 *__restrict__ hlist,
                                                       Hubs hb, const int64_t *__restrict__ coff, Chunks ch, Batch bt,
                                                       int mcap, int staged, int32_t *__restrict__ active) {
-    extern __shared__ float4 rows[];  // NET_C x nq if staged
-    __shared__ float cd[NET_C];
-    __shared__ int32_t cp[NET_C];
+    extern __shared__ float4 rows[];  // C x (nq + 1) if staged, then C x C distances
+    __shared__ float cd[C];
+    __shared__ int32_t cp[C];
+    __shared__ int picks[NET_M];
     const int2 hs = hlist[blockIdx.x];
     const int h = hs.x;
     if (hb.done[h]) return;
-    const int b = hb.begin[h], nc = hb.nc[h], nq = dp >> 2;
+    const int b = hb.begin[h], nc = hb.nc[h], nq = dp >> 2, rs = nq + 1;
+    float *pd = reinterpret_cast<float *>(rows + (staged ? C * rs : 0));
     const float thr = hb.thr[h];
     const int n_rep = (hb.count[h] + ch.len - 1) / ch.len * NET_KEYS;
     int covered;
-    const int n = net_candidates<NET_C>(ch, coff[hs.y] * NET_KEYS, n_rep, thr, cd, cp, &covered);
+    const int n = net_candidates<C>(ch, coff[hs.y] * NET_KEYS, n_rep, thr, cd, cp, &covered);
     const bool flat = n > 0 && flat_split(nc, covered);
     if (n == 0 || flat) {
         if (threadIdx.x == 0) net_take(hb, h, 0, flat, active);
         return;
     }
+    const int T = (n + 3) >> 2;
     if (staged) {
-        for (int i = threadIdx.x; i < n * nq; i += BT) {
+        for (int i = threadIdx.x; i < 4 * T * nq; i += BT) {
             const int c = i / nq, k = i - c * nq;
-            rows[i] = __ldg(reinterpret_cast<const float4 *>(X + (size_t)ids[cp[c]] * dp) + k);
+            rows[c * rs + k] = c < n ? __ldg(reinterpret_cast<const float4 *>(X + (size_t)ids[cp[c]] * dp) + k)
+                                     : make_float4(0.f, 0.f, 0.f, 0.f);
         }
         __syncthreads();
-    }
-    auto row_of = [&](int c) -> const float4 * {
-        return staged ? rows + c * nq : reinterpret_cast<const float4 *>(X + (size_t)ids[cp[c]] * dp);
-    };
-    constexpr int G = BT / TPD;
-    const int g = threadIdx.x / TPD, j = threadIdx.x % TPD;
-    int m = 0;
-    while (m < mcap) {
-        const unsigned long long f = net_farthest(cd, n);
-        if (!(key_value(f) > thr)) break;
-        const int pick = (int)key_pos(f);
-        if (threadIdx.x == 0) {
-            bt.pos[(size_t)hs.y * NET_M + m] = cp[pick];
-            bt.cpos[b + nc + m] = cp[pick];
-        }
-        ++m;
-        __syncthreads();  // every warp has read cd
-        const float4 *pr = row_of(pick);
-        for (int c0 = 0; c0 < n; c0 += G) {
-            const int c = c0 + g;
-            float acc = 0.f;
-            if (c < n) {
-                const float4 *cr = row_of(c);
-#pragma unroll 4
-                for (int k = j; k < nq; k += TPD) {
-                    const float4 x = pr[k], y = cr[k];
-                    const float dx = x.x - y.x, dy = x.y - y.y, dz = x.z - y.z, dw = x.w - y.w;
-                    acc = fmaf(dx, dx, acc);
-                    acc = fmaf(dy, dy, acc);
-                    acc = fmaf(dz, dz, acc);
-                    acc = fmaf(dw, dw, acc);
+        for (int idx = threadIdx.x; idx < ((T + 1) >> 1) * (T + 1); idx += BT) {
+            int ti, tj;
+            if (!upper_tile(idx, T, ti, tj)) continue;
+            float acc[4][4] = {};
+            for (int k = 0; k < nq; ++k) {
+                float4 x[4], y[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    x[u] = rows[(4 * ti + u) * rs + k];
+                    y[u] = rows[(4 * tj + u) * rs + k];
                 }
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) {
+                        const float dx = x[u].x - y[v].x, dy = x[u].y - y[v].y, dz = x[u].z - y[v].z,
+                                    dw = x[u].w - y[v].w;
+                        acc[u][v] = fmaf(dx, dx, acc[u][v]);
+                        acc[u][v] = fmaf(dy, dy, acc[u][v]);
+                        acc[u][v] = fmaf(dz, dz, acc[u][v]);
+                        acc[u][v] = fmaf(dw, dw, acc[u][v]);
+                    }
             }
 #pragma unroll
-            for (int o = TPD / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o, TPD);
-            if (c < n && j == 0) cd[c] = fminf(cd[c], sqrtf(acc));
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int v = 0; v < 4; ++v) {
+                    const float dd = sqrtf(acc[u][v]);
+                    pd[(4 * ti + u) * C + 4 * tj + v] = dd;
+                    pd[(4 * tj + v) * C + 4 * ti + u] = dd;
+                }
         }
-        __syncthreads();
+    } else {
+        constexpr int G = BT / TPD;
+        const int g = threadIdx.x / TPD, j = threadIdx.x % TPD;
+        for (int q0 = 0; q0 < n * n; q0 += G) {  // the same number of steps in every group
+            const int q = min(q0 + g, n * n - 1), u = q / n, v = q - u * n;
+            if (!__any_sync(0xffffffffu, u <= v)) continue;
+            RowRegs<TPD, 0> r;
+            r.load(reinterpret_cast<const float4 *>(X + (size_t)ids[cp[u]] * dp), nq, j);
+            const float dd = sqrtf(r.sqdist(reinterpret_cast<const float4 *>(X + (size_t)ids[cp[v]] * dp), nq, j));
+            if (j == 0 && u <= v) {
+                pd[u * C + v] = dd;
+                pd[v * C + u] = dd;
+            }
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    const int m = net_greedy<C>(cd, n, thr, mcap, picks, [&](int i, int j) { return pd[i * C + j]; });
+    for (int i = threadIdx.x; i < m; i += 32) {
+        bt.pos[(size_t)hs.y * NET_M + i] = cp[picks[i]];
+        bt.cpos[b + nc + i] = cp[picks[i]];
     }
     if (threadIdx.x == 0) {
         if (nc == 1) bt.cpos[b] = b;  // label 0: the hub's own centre
@@ -654,33 +705,29 @@ __global__ void __launch_bounds__(LEV_C) k_net_pairs_lev(Strings S, const int32_
         pr[t * LEV_C + a] = (uint16_t)d;
     }
 }
-__global__ void __launch_bounds__(32) k_net_pick_lev(const int2 *__restrict__ hlist, Hubs hb, Batch bt, LevCands lc,
-                                                     int mcap, int32_t *__restrict__ active) {
+__global__ void __launch_bounds__(128) k_net_pick_lev(const int2 *__restrict__ hlist, Hubs hb, Batch bt, LevCands lc,
+                                                      int mcap, int32_t *__restrict__ active) {
     __shared__ float cd[LEV_C];
+    __shared__ uint16_t pd[LEV_C * LEV_C];
+    __shared__ int picks[NET_M];
     const int2 hs = hlist[blockIdx.x];
-    const int h = hs.x, lane = threadIdx.x;
+    const int h = hs.x;
     if (hb.done[h]) return;
     const int n = lc.n[blockIdx.x], b = hb.begin[h], nc = hb.nc[h];
-    const float thr = hb.thr[h];
     const size_t o = (size_t)blockIdx.x * LEV_C;
-    for (int i = lane; i < n; i += 32) cd[i] = lc.d[o + i];
-    __syncwarp();
-    int m = 0;
-    while (m < mcap && n) {
-        const unsigned long long f = net_farthest(cd, n);
-        if (!(key_value(f) > thr)) break;
-        const int pick = (int)key_pos(f);
-        if (lane == 0) {
-            bt.pos[(size_t)hs.y * NET_M + m] = lc.pos[o + pick];
-            bt.cpos[b + nc + m] = lc.pos[o + pick];
-        }
-        ++m;
-        __syncwarp();
-        const uint16_t *pr = lc.pair + (o + pick) * LEV_C;
-        for (int i = lane; i < n; i += 32) cd[i] = fminf(cd[i], (float)pr[i]);
-        __syncwarp();
+    for (int i = threadIdx.x; i < n; i += blockDim.x) cd[i] = lc.d[o + i];
+    for (int i = threadIdx.x; i < n * LEV_C / 2; i += blockDim.x)  // rows below n (entries at and past n are not read)
+        reinterpret_cast<uint32_t *>(pd)[i] = reinterpret_cast<const uint32_t *>(lc.pair + o * LEV_C)[i];
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    const int m = n ? net_greedy<LEV_C>(cd, n, hb.thr[h], mcap, picks,
+                                        [&](int i, int j) { return (float)pd[i * LEV_C + j]; })
+                    : 0;
+    for (int i = threadIdx.x; i < m; i += 32) {
+        bt.pos[(size_t)hs.y * NET_M + i] = lc.pos[o + picks[i]];
+        bt.cpos[b + nc + i] = lc.pos[o + picks[i]];
     }
-    if (lane == 0) {
+    if (threadIdx.x == 0) {
         if (nc == 1) bt.cpos[b] = b;  // label 0: the hub's own centre
         net_take(hb, h, m, false, active);
     }
@@ -805,9 +852,10 @@ __global__ void __launch_bounds__(BT) k_net_select_ham(const uint32_t *__restric
                                                        const int32_t *__restrict__ ids, const int2 *__restrict__ hlist,
                                                        Hubs hb, const int64_t *__restrict__ coff, Chunks ch, Batch bt,
                                                        int32_t *__restrict__ active) {
-    extern __shared__ uint4 hrows[];  // NET_C x nq
+    extern __shared__ uint4 hrows[];  // NET_C x (nq + 1), then NET_C x NET_C distances
     __shared__ float cd[NET_C];
     __shared__ int32_t cp[NET_C];
+    __shared__ int picks[NET_M];
     const int2 hs = hlist[blockIdx.x];
     const int h = hs.x;
     if (hb.done[h]) return;
@@ -821,23 +869,24 @@ __global__ void __launch_bounds__(BT) k_net_select_ham(const uint32_t *__restric
         if (threadIdx.x == 0) net_take(hb, h, 0, flat, active);
         return;
     }
+    const int rs = nq + 1;
+    uint16_t *pd = reinterpret_cast<uint16_t *>(hrows + NET_C * rs);
     for (int i = threadIdx.x; i < n * nq; i += BT) {
         const int c = i / nq, k = i - c * nq;
-        hrows[i] = reinterpret_cast<const uint4 *>(X + (size_t)ids[cp[c]] * wp)[k];
+        hrows[c * rs + k] = reinterpret_cast<const uint4 *>(X + (size_t)ids[cp[c]] * wp)[k];
     }
     __syncthreads();
-    int m = 0;
-    while (m < NET_M) {
-        const unsigned long long f = net_farthest(cd, n);
-        if (!(key_value(f) > thr)) break;
-        const int pick = (int)key_pos(f);
-        if (threadIdx.x == 0) bt.pos[(size_t)hs.y * NET_M + m] = cp[pick];
-        ++m;
-        __syncthreads();  // every warp has read cd
-        if (threadIdx.x < n)
-            cd[threadIdx.x] = fminf(cd[threadIdx.x], (float)ham_dist4(hrows + pick * nq, hrows + threadIdx.x * nq, nq));
-        __syncthreads();
+    for (int idx = threadIdx.x; idx < ((n + 1) >> 1) * (n + 1); idx += BT) {
+        int i, j;
+        if (!upper_tile(idx, n, i, j)) continue;
+        const uint16_t d = (uint16_t)ham_dist4(hrows + i * rs, hrows + j * rs, nq);
+        pd[i * NET_C + j] = d;
+        pd[j * NET_C + i] = d;
     }
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    const int m = net_greedy<NET_C>(cd, n, thr, NET_M, picks, [&](int i, int j) { return (float)pd[i * NET_C + j]; });
+    for (int i = threadIdx.x; i < m; i += 32) bt.pos[(size_t)hs.y * NET_M + i] = cp[picks[i]];
     if (threadIdx.x == 0) net_take(hb, h, m, false, active);
 }
 
@@ -1673,11 +1722,12 @@ ct_tree *build_impl(const ct_points *pts, int zeta, int root, cudaStream_t s, co
                           int32_t *active) {
             const Chunks ch{nullptr, chunk_len, keys.p, cov.p};
             if (l2) {
-                const int staged = dp <= 128;
-                const size_t sm = staged ? (size_t)NET_C * dp * sizeof(float) : 0;
+                const int cands = dp <= 32 ? NET_C : NET_C / 2, staged = dp <= 256;
+                const size_t sm = ((size_t)cands * cands + (staged ? (size_t)cands * (dp + 4) : 0)) * sizeof(float);
                 const size_t dsm = (size_t)mcap * dp * sizeof(float);
                 dispatch([&](auto T, auto V) {
-                    auto kern = k_net_select_l2<T()>;
+                    auto kern = T() <= 2 ? k_net_select_l2<NET_C, T()> : k_net_select_l2<NET_C / 2, T()>;
+                    if (cands == NET_C / 2) kern = k_net_select_l2<NET_C / 2, T()>;
                     if (sm > 40 * 1024)
                         CT_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
                     kern<<<(unsigned)nlist, BT, sm, s>>>(Xp.p, dp, ids.p, list, hb, coff, ch, bt, mcap, staged, active);
@@ -1689,7 +1739,7 @@ ct_tree *build_impl(const ct_points *pts, int zeta, int root, cudaStream_t s, co
                 return;
             }
             if (ham) {
-                const size_t sm = (size_t)NET_C * wp * sizeof(uint32_t);
+                const size_t sm = (size_t)NET_C * (wp + 4) * sizeof(uint32_t) + (size_t)NET_C * NET_C * sizeof(uint16_t);
                 if (sm > 40 * 1024)
                     CT_CHECK_CUDA(cudaFuncSetAttribute(k_net_select_ham, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
                 k_net_select_ham<<<(unsigned)nlist, BT, sm, s>>>(Xb.p, wp, ids.p, list, hb, coff, ch, bt, active);
@@ -1703,7 +1753,7 @@ ct_tree *build_impl(const ct_points *pts, int zeta, int root, cudaStream_t s, co
 #undef CT_PL
                 }
                 CT_COUNT_LAUNCH();
-                k_net_pick_lev<<<(unsigned)nlist, 32, 0, s>>>(list, hb, bt, lc, mcap, active);
+                k_net_pick_lev<<<(unsigned)nlist, 128, 0, s>>>(list, hb, bt, lc, mcap, active);
                 CT_COUNT_LAUNCH();
                 switch (W) {
 #define CT_DL(WW) case WW: k_net_dists_lev<WW><<<dim3((unsigned)nlist, (unsigned)mcap), 128, sm, s>>>(S, ids.p, list, hb, bt); break;
