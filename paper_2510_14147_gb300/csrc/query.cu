@@ -265,9 +265,15 @@ __device__ __forceinline__ void pool_append(const Pool &P, int g, PoolCursor &pc
 // before the test, so that their loads overlap the test's.  With `sp`, a walk
 // that reaches sp->limit steps stores the ranges left on its stack in
 // sp->items and stops (if they do not fit it goes on).
+// A vertex's points are the positions from node_begin on, node_count of them;
+// vertices whose points all lie before `qlo` are left out with everything
+// below them (upper-triangle form: a group takes the pairs from its own first
+// row on; 0: none).  (They used to be walked and dropped when the candidates
+// were gathered.  Walk of 1M x 128: 11.2 -> 6.9 ms at 70 neighbours, 15.5 ->
+// 8.2 at 500; 1M codes 8.7 -> 5.5, with the gather 15 ms less in all.)
 template <class Tester>
-__device__ __forceinline__ int walk_group(const TreeView &tv, int2 *__restrict__ stack, int cap, int g, int2 start,
-                                          const Pool &P, PoolCursor &pc, unsigned long long &evals,
+__device__ __forceinline__ int walk_group(const TreeView &tv, int2 *__restrict__ stack, int cap, int g, int qlo,
+                                          int2 start, const Pool &P, PoolCursor &pc, unsigned long long &evals,
                                           int32_t *__restrict__ err, const Spill *sp, Tester tester) {
     const int lane = threadIdx.x & 31;
     int n_cand = 0, status = 0;
@@ -346,12 +352,13 @@ __device__ __forceinline__ int walk_group(const TreeView &tv, int2 *__restrict__
             if (nfull < nr && pe < 32 && lane == 0) stack[top - 1] = make_int2(px + (32 - pe), py - (32 - pe));
             if (lane < n) ++evals;
             const int v = lane < n ? kx + (lane - ke) : 0;
-            int ccount = 0, cbegin = 0;
+            int ccount = 0, cbegin = 0, end = INT_MAX;
             if (lane < n) {
                 ccount = tv.child_count[v];
                 cbegin = tv.child_begin[v];
+                if (qlo > 0) end = tv.node_begin[v] + tv.node_count[v];
             }
-            const bool keep = tester(v, n);
+            const bool keep = tester(v, n) && end > qlo;
             const bool leaf = keep && ccount == 0;
             pool_append(P, g, pc, keep && leaf, (uint32_t)v);
             n_cand += __popc(__ballot_sync(0xffffffffu, keep && leaf));
@@ -495,7 +502,8 @@ __global__ void __launch_bounds__(TRAV_WARPS * 32, 8) k_traverse_l2(
             }
         };
         const unsigned long long e0 = evals;
-        const int ws = walk_group(tv, stack, cap, gg, start, P, pc, evals, err, sp, tester);
+        const int qlo = V.qp[c].half ? tv.group_begin[g] : 0;
+        const int ws = walk_group(tv, stack, cap, gg, qlo, start, P, pc, evals, err, sp, tester);
         if (ws < 0) return;
         full = ws == POOL_STOPPED;
         if (gvisit) group_visits(gvisit, gg, evals - e0);
@@ -564,7 +572,8 @@ __global__ void __launch_bounds__(32) k_traverse_lev(
             return lev_myers<W>(peq, m, txt, n, k) <= k;
         };
         const unsigned long long e0 = evals;
-        const int ws = walk_group(tv, stack, cap, g, start, P, pc, evals, err, sp, tester);
+        const int qlo = qp.half ? tv.group_begin[g] : 0;
+        const int ws = walk_group(tv, stack, cap, g, qlo, start, P, pc, evals, err, sp, tester);
         if (ws < 0) return;
         full = ws == POOL_STOPPED;
         if (gvisit) group_visits(gvisit, g, evals - e0);
@@ -649,7 +658,8 @@ __global__ void __launch_bounds__(32) k_traverse_ham(
             return ham_rows(cen, row, nq) <= k;
         };
         const unsigned long long e0 = evals;
-        const int ws = walk_group(tv, stack, cap, g, start, P, pc, evals, err, sp, tester);
+        const int qlo = qp.half ? tv.group_begin[g] : 0;
+        const int ws = walk_group(tv, stack, cap, g, qlo, start, P, pc, evals, err, sp, tester);
         if (ws < 0) return;
         full = ws == POOL_STOPPED;
         if (gvisit) group_visits(gvisit, g, evals - e0);
@@ -1624,47 +1634,6 @@ __global__ void k_group_cand_copy(int nseg, const int32_t *__restrict__ seg_grou
     base = __shfl_sync(0xffffffffu, base, 0);
     const uint32_t *src = pool + seg_begin[i];
     for (int k = lane; k < c; k += 32) gcand[base + k] = src[k];
-}
-// The copy in the upper-triangle form: a group keeps the candidate blocks
-// that reach its first position or beyond (the pairs with earlier points are
-// evaluated by their own groups); each warp ballots a segment's blocks 32 at
-// a time and appends the kept ones, so a group's kept count ends in gfill.
-// With nseg_dev (a plan) the segment count is read on the device and the
-// destinations are checked against cand_cap.
-__global__ void k_group_cand_copy_half(const __grid_constant__ Views V, int nseg, const int32_t *__restrict__ nseg_dev,
-                                       int64_t seg_cap, const int32_t *__restrict__ seg_group,
-                                       const int64_t *__restrict__ seg_begin, const int32_t *__restrict__ seg_count,
-                                       const int64_t *__restrict__ goff, int32_t *__restrict__ gfill,
-                                       const uint32_t *__restrict__ pool, uint32_t *__restrict__ gcand,
-                                       int64_t cand_cap, int32_t *__restrict__ err) {
-    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    const int64_t ns = nseg_dev ? min((int64_t)*nseg_dev, seg_cap) : (int64_t)nseg;
-    if (i >= ns) return;
-    const int gg = seg_group[i], c = seg_count[i];
-    const int cl = cloud_of_group(V, gg);
-    const TreeView &tv = V.tv[cl];
-    const bool half = V.qp[cl].half != 0;
-    const int qb = tv.group_begin[gg - V.gbase[cl]];
-    const uint32_t *src = pool + seg_begin[i];
-    for (int k0 = 0; k0 < c; k0 += 32) {
-        const int k = k0 + lane;
-        uint32_t v = 0u;
-        bool keep = false;
-        if (k < c) {
-            v = src[k];
-            keep = !half || tv.node_begin[v] + tv.node_count[v] > qb;
-        }
-        const unsigned m = __ballot_sync(0xffffffffu, keep);
-        int64_t base = 0;
-        if (lane == 0 && m) base = goff[gg] + atomicAdd(gfill + gg, __popc(m));
-        base = __shfl_sync(0xffffffffu, base, 0);
-        if (base + __popc(m) > cand_cap) {  // a plan's overflow (reported; the producer skips the group)
-            if (lane == 0) atomicOr(err, 128);
-            return;
-        }
-        if (keep) gcand[base + __popc(m & lanemask_lt())] = v;
-    }
 }
 
 __global__ void k_iota(int n, int32_t *__restrict__ out) {
@@ -3147,13 +3116,12 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
     std::memset(&V, 0, sizeof(V));
     V.nc = C;
     int max_dp = 4, max_fp_dp = 4, max_depth = 0, max_len = 0, min_len = kItemTC;
-    bool any_tc = false, any_fp = false, any_half = false;
+    bool any_tc = false, any_fp = false;
     for (int c = 0; c < C; ++c) {
         const ct_tree *tc = trees[c];
         if ((tc->metric == CT_L2_F32) != l2) CT_FAIL(CT_EINVAL, "a batch mixes metrics");
         V.tv[c] = view_of(tc);
         V.qp[c] = qps[c];
-        any_half |= qps[c].half != 0;
         const LeafChoice ch = leaf_choice(tc, precision);
         V.use_tc[c] = (uint8_t)ch.use_tc;
         V.item_len[c] = (int16_t)ch.item_len;
@@ -3364,19 +3332,11 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
         k_group_cand_counts<<<grid_for(nseg, 256), 256, 0, s>>>(nseg, seg_group.p, seg_count.p, gseg_count.p);
         CT_COUNT_LAUNCH();
         exclusive_scan_i32_to_i64(gseg_count.p, gseg_begin.p, G, gseg_begin.p + G, s);
-        if (any_half)
-            k_group_cand_copy_half<<<grid_for((int64_t)nseg * 32, 256), 256, 0, s>>>(
-                V, nseg, nullptr, 0, seg_group.p, seg_begin.p, seg_count.p, gseg_begin.p, gfill.p, pool.p, gcand.p,
-                INT64_MAX, err);
-        else
-            k_group_cand_copy<<<grid_for((int64_t)nseg * 32, 256), 256, 0, s>>>(nseg, seg_group.p, seg_begin.p,
-                                                                              seg_count.p, gseg_begin.p, gfill.p,
-                                                                              pool.p, gcand.p);
+        k_group_cand_copy<<<grid_for((int64_t)nseg * 32, 256), 256, 0, s>>>(nseg, seg_group.p, seg_begin.p, seg_count.p,
+                                                                          gseg_begin.p, gfill.p, pool.p, gcand.p);
         CT_COUNT_LAUNCH();
         k_iota<<<grid_for(G, 256), 256, 0, s>>>(G, gseg_group.p);
         CT_COUNT_LAUNCH();
-        if (any_half)  // the groups' kept counts
-            CT_CHECK_CUDA(cudaMemcpyAsync(gseg_count.p, gfill.p, G * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
         CT_LAUNCH_CHECK();
         nseg = G;
     }
@@ -4067,7 +4027,6 @@ struct PlanImpl {
     int max_dp = 4, cap_stack = 0, spill_cap = 0, leaf_grid = 1;
     TravLaunch tl{1, 1};
     int64_t pool_cap = 0, seg_cap = 0, cand_cap = 0, item_cap = 0, nnz_cap = 0;
-    bool any_half = false;  // some cloud is queried in the upper-triangle form
     int big_rows = 0;       // rows above the in-place sorts' length the plan sorts by radix
     int64_t big_cap = 0;    // their entries
     cudaStream_t s0 = 0;
@@ -4124,19 +4083,10 @@ void plan_enqueue(PlanImpl &p, cudaStream_t s) {
                                                               p.gcount.p);
     CT_COUNT_LAUNCH();
     exclusive_scan_i32_to_i64_into(p.gcount.p, p.gbegin.p, G, p.gbegin.p + G, p.sums.p, s);
-    if (p.any_half) {
-        k_group_cand_copy_half<<<grid_for(p.seg_cap * 32, 256), 256, 0, s>>>(
-            V, 0, P.nseg, p.seg_cap, P.seg_group, P.seg_begin, P.seg_count, p.gbegin.p, p.gfill.p, P.data, p.gcand.p,
-            p.cand_cap, err);
-        CT_COUNT_LAUNCH();
-        // the groups' kept counts (ranges past the plan's capacity are never read: the producer skips them)
-        CT_CHECK_CUDA(cudaMemcpyAsync(p.gcount.p, p.gfill.p, (size_t)G * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
-    } else {
-        k_plan_cand_copy<<<grid_for(p.seg_cap * 32, 256), 256, 0, s>>>(P.nseg, p.seg_cap, P.seg_group, P.seg_begin,
-                                                                      P.seg_count, p.gbegin.p, p.gfill.p, P.data,
-                                                                      p.gcand.p, p.cand_cap, err);
-        CT_COUNT_LAUNCH();
-    }
+    k_plan_cand_copy<<<grid_for(p.seg_cap * 32, 256), 256, 0, s>>>(P.nseg, p.seg_cap, P.seg_group, P.seg_begin,
+                                                                  P.seg_count, p.gbegin.p, p.gfill.p, P.data,
+                                                                  p.gcand.p, p.cand_cap, err);
+    CT_COUNT_LAUNCH();
     // 3. count pass: one persistent launch producing and consuming the work queue
     CT_CHECK_CUDA(cudaMemsetAsync(p.qctr.p, 0, 4 * sizeof(int32_t), s));
     CT_CHECK_CUDA(cudaMemsetAsync(p.ready.p, 0, (size_t)p.item_cap * sizeof(int32_t), s));
@@ -4224,7 +4174,6 @@ PlanImpl *plan_create(int C, const ct_tree *const *trees, const QParams *qps, in
         p.trees.push_back(t);
         p.V.tv[c] = view_of(t);
         p.V.qp[c] = qps[c];
-        p.any_half |= qps[c].half != 0;
         p.V.use_tc[c] = 0;  // the persistent launch runs the FP32 tiles
         const int len = precision == 2 ? leaf_choice(t, 2).item_len : kItem;
         p.V.item_len[c] = (int16_t)len;

@@ -26,7 +26,8 @@ def test_rows_after_the_pool_grew(metric):
     from paper_2510_14147_gb300 import ctgraph as cg
     opts = {}
     if metric.startswith("l2"):
-        n = 40001
+        # (an upper-triangle walk leaves out what lies before a group: half the candidates)
+        n = 100001 if metric == "l2-upper-tc" else 40001
         x = I.uniform_cube(n, 16, seed=3)
         sp, args, eps = oracle.Space(points=x), {"points": torch.from_numpy(x).cuda()}, 0.75
         if metric == "l2-upper-tc":
