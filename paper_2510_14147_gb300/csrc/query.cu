@@ -672,18 +672,16 @@ __global__ void __launch_bounds__(32) k_traverse_ham(
 
 // ------------------------------------------------------------ leaf tiles
 
-// Packs the next run of candidate points into a tile of up to 32 rows.  The
-// candidates of a group are leaf blocks of a few points each; rows of
-// consecutive candidates are concatenated so that every tile is full.
-// Called by warp 0; (s_ci, s_off) is the cursor: candidate index and the number
-// of its points already consumed.  In the emit pass, candidates without the
-// "produced an edge" flag are skipped.
-__device__ __forceinline__ void fill_tile(const TreeView &tv, const uint32_t *__restrict__ cand, int64_t c1,
-                                          bool flagged_only, int64_t *s_ci, int *s_off, int *s_rows,
-                                          int *tpos, int64_t *tcand) {
+// Packs the next run of candidate points into a tile of up to 32 rows, with one
+// warp.  The candidates of a group are leaf blocks of a few points each; rows
+// of consecutive candidates are concatenated so that every tile is full.
+// (ci, off) is the cursor: candidate index and the number of its points already
+// consumed.  Returns the rows; lane r < rows gets row r's position and
+// candidate.  In the emit pass, candidates without the "produced an edge" flag
+// are skipped.
+__device__ __forceinline__ int tile_rows(const TreeView &tv, const uint32_t *__restrict__ cand, int64_t c1,
+                                         bool flagged_only, int64_t &ci, int &off, int &pos, int64_t &pcand) {
     const int lane = threadIdx.x & 31;
-    const int64_t ci = *s_ci;
-    const int off = *s_off;
     const int64_t c = ci + lane;
     int beg = 0, cnt = 0;
     if (c < c1) {
@@ -716,28 +714,43 @@ __device__ __forceinline__ void fill_tile(const TreeView &tv, const uint32_t *__
     }
     const int bl = __shfl_sync(0xffffffffu, beg, L);
     const int el = __shfl_sync(0xffffffffu, excl, L);
-    if (lane < rows) {
-        tpos[lane] = bl + (lane - el);
-        tcand[lane] = ci + L;
-    }
+    pos = bl + (lane - el);
+    pcand = ci + L;
     const int L31 = __shfl_sync(0xffffffffu, L, 31);
     const int e31 = __shfl_sync(0xffffffffu, excl, L31);
     const int n31 = __shfl_sync(0xffffffffu, cnt, L31);
-    if (lane == 0) {
-        if (total <= 32) {
-            int64_t nx = ci + 32;
-            *s_ci = nx < c1 ? nx : c1;
-            *s_off = 0;
+    if (total <= 32) {
+        ci = ci + 32 < c1 ? ci + 32 : c1;
+        off = 0;
+    } else {
+        const int used = 32 - e31;
+        if (used == n31) {
+            ci += L31 + 1;
+            off = 0;
         } else {
-            int used = 32 - e31;
-            if (used == n31) {
-                *s_ci = ci + L31 + 1;
-                *s_off = 0;
-            } else {
-                *s_ci = ci + L31;
-                *s_off = (L31 == 0 ? off : 0) + used;
-            }
+            off = (L31 == 0 ? off : 0) + used;
+            ci += L31;
         }
+    }
+    return rows;
+}
+
+// The same by warp 0 for a block: the cursor and the tile in shared memory.
+__device__ __forceinline__ void fill_tile(const TreeView &tv, const uint32_t *__restrict__ cand, int64_t c1,
+                                          bool flagged_only, int64_t *s_ci, int *s_off, int *s_rows,
+                                          int *tpos, int64_t *tcand) {
+    const int lane = threadIdx.x & 31;
+    int64_t ci = *s_ci, pc;
+    int off = *s_off, pos;
+    __syncwarp();
+    const int rows = tile_rows(tv, cand, c1, flagged_only, ci, off, pos, pc);
+    if (lane < rows) {
+        tpos[lane] = pos;
+        tcand[lane] = pc;
+    }
+    if (lane == 0) {
+        *s_ci = ci;
+        *s_off = off;
         *s_rows = rows;
     }
 }
@@ -2114,104 +2127,167 @@ __global__ void __launch_bounds__(LEAF_T) k_leaf_lev(
     }
 }
 
-// Hamming leaf stage: one CTA per work item; the group's query rows and each
-// tile of up to 32 candidate rows in shared memory; thread t takes pairs
-// t, t + LEAF_T, ... of the tile (query-major), integer distances.
-template <bool EMIT>
+// Set bits of eight words: four full adders leave the ones in two words and the
+// twos and fours in one each, so four population counts instead of eight.
+__device__ __forceinline__ int popc8(const uint4 x, const uint4 y) {
+    const uint32_t s1 = x.x ^ x.y ^ x.z, c1 = (x.x & x.y) | (x.x & x.z) | (x.y & x.z);
+    const uint32_t s2 = x.w ^ y.x ^ y.y, c2 = (x.w & y.x) | (x.w & y.y) | (y.x & y.y);
+    const uint32_t s3 = s1 ^ s2 ^ y.z, c3 = (s1 & s2) | (s1 & y.z) | (s2 & y.z);
+    const uint32_t t = c1 ^ c2 ^ c3, u = (c1 & c2) | (c1 & c3) | (c2 & c3);
+    return (__popc(s3) + __popc(y.w)) + 2 * __popc(t) + 4 * __popc(u);
+}
+__device__ __forceinline__ int popc4(const uint4 x) {
+    const uint32_t s1 = x.x ^ x.y ^ x.z, c1 = (x.x & x.y) | (x.x & x.z) | (x.y & x.z);
+    return (__popc(s1) + __popc(x.w)) + 2 * __popc(c1);
+}
+__device__ __forceinline__ uint4 xor4(const uint4 a, const uint4 b) {
+    return make_uint4(a.x ^ b.x, a.y ^ b.y, a.z ^ b.z, a.w ^ b.w);
+}
+
+// Hamming leaf stage, integer distances: one CTA per work item, the group's
+// query rows (zero padded to nch x NQ uint4) in shared memory.  Each warp takes
+// a quarter of the item's candidates by itself (handing out 32 at a time to the
+// four was slower: 16.1 against 14.7 ms) and packs 32 rows at a time: lane p keeps
+// row p in registers (NQ uint4; longer rows in nch chunks, eight queries at a
+// time) and the queries are read as broadcasts, so a pair costs no shared
+// bandwidth and the tiles no barriers.  The hits of a lane are a mask over the
+// queries; they are written after the tile, two rounds or so for all lanes
+// together instead of a divergent branch per hit.
+// Bound by the population counts (16 per clock and SM) and the logic before
+// them: 6.6e9 pairs of 256 bits took 23.4 ms as 32 x 32 tiles of two shared rows per
+// pair and a count per word, 14.7 ms now.
+template <bool EMIT, int NQ>
 __global__ void __launch_bounds__(LEAF_T) k_leaf_ham(
     TreeView tv, QParams qp, Items items, uint32_t *__restrict__ cand, int32_t *__restrict__ deg,
     const int64_t *__restrict__ row_ptr, int32_t *__restrict__ rowcur, int32_t *__restrict__ col,
     float *__restrict__ dist, unsigned long long *__restrict__ st, int32_t *__restrict__ err, CapOut co,
     const uint8_t *__restrict__ rowsel) {
-    extern __shared__ uint4 hsm[];  // 32 query rows, then 32 candidate rows (wp / 4 uint4 each)
-    __shared__ int cnt[32], cursor[32], sel[32];
+    constexpr int QB = 8;
+    extern __shared__ uint4 Qs[];  // 32 query rows
+    __shared__ int cnt[32], cursor[32];
     __shared__ int64_t rowb[32], rowe[32];
-    __shared__ int tpos[32];
-    __shared__ int64_t tcand[32];
-    __shared__ int64_t s_ci;
-    __shared__ int s_off, s_rows;
-    __shared__ unsigned s_hit;
-    const int tid = threadIdx.x;
+    __shared__ unsigned s_sel;
+    const int tid = threadIdx.x, lane = tid & 31;
     const int it = blockIdx.x;
     if (it >= *items.count) return;
     const int g = items.group[it];
     const int qb = tv.group_begin[g], qn = tv.group_count[g], qe = qb + qn;  // at most 32 queries
-    const int64_t c0 = items.begin[it], c1 = items.end[it];
-    const int k = qp.lev_k, nq = tv.wp >> 2;
-    uint4 *Qs = hsm, *Ps = hsm + 32 * nq;
-    unsigned long long pairs = 0;
+    const int k = qp.lev_k, nq = tv.wp >> 2, nch = (nq + NQ - 1) / NQ, qs = nch * NQ;
+    const uint4 *rows = reinterpret_cast<const uint4 *>(tv.bits);
     if (tid < 32) {
         cnt[tid] = 0;
+        bool sel = false;
         if (tid < qn) {
             const int o = tv.perm[qb + tid];
             cursor[tid] = o;
-            sel[tid] = rowsel == nullptr || rowsel[o] != 0;
+            sel = rowsel == nullptr || rowsel[o] != 0;
             if (EMIT) {
                 rowb[tid] = row_ptr[o];
                 rowe[tid] = row_ptr[o + 1];
             }
         }
+        const unsigned m = __ballot_sync(0xffffffffu, sel);
+        if (tid == 0) s_sel = m;
     }
-    for (int i = tid; i < qn * nq; i += LEAF_T)
-        Qs[i] = reinterpret_cast<const uint4 *>(tv.bits)[(size_t)(qb + i / nq) * nq + i % nq];
-    if (tid == 0) {
-        s_ci = c0;
-        s_off = 0;
-        s_hit = 0u;
-    }
-    for (;;) {
-        __syncthreads();
-        if (tid < 32) fill_tile(tv, cand, c1, EMIT, &s_ci, &s_off, &s_rows, tpos, tcand);
-        __syncthreads();
-        const int npr = s_rows;
-        const bool last = s_ci >= c1;
-        for (int i = tid; i < npr * nq; i += LEAF_T)
-            Ps[i] = reinterpret_cast<const uint4 *>(tv.bits)[(size_t)tpos[i / nq] * nq + i % nq];
-        __syncthreads();
-        if (npr > 0) {
-            unsigned hit = 0u;
-            for (int t = tid; t < qn * npr; t += LEAF_T) {
-                const int q = t / npr, p = t - q * npr;
-                const int qpos = qb + q, ppos = tpos[p];
-                if (qpos == ppos && !qp.include_self) continue;
-                if (qp.half && ppos < qb) continue;
-                const bool mir = qp.half && ppos >= qe;
-                if (EMIT && !sel[q] && !(mir && rowsel)) continue;
-                if (!EMIT) ++pairs;
-                const int d = ham_rows_smem(Qs + q * nq, Ps + p * nq, nq);
-                if (d > k) continue;
-                if (mir) mirror_int(tv, deg, row_ptr, rowcur, col, dist, err, co, rowsel, EMIT, qpos, ppos, d);
-                if (!EMIT) {
-                    hit |= 1u << p;
-                    atomicAdd(&cnt[q], 1);
-                    if (co.off) cap_put(co, cursor[q], tv.perm[ppos], (float)d);
-                } else if (sel[q]) {
-                    const int slot = atomicAdd(&rowcur[cursor[q]], 1);
-                    const int64_t at = rowb[q] + slot;
-                    if (at < rowe[q]) {
-                        col[at] = tv.perm[ppos];
-                        dist[at] = (float)d;
-                    } else {
-                        atomicOr(err, 4);
-                    }
-                }
-            }
-            if (!EMIT) {
-                if (hit) atomicOr(&s_hit, hit);
-                __syncthreads();
-                if (tid < npr && ((s_hit >> tid) & 1u)) atomicOr(&cand[tcand[tid]], FLAG);
-                __syncthreads();
-                if (tid == 0) s_hit = 0u;
-            }
-        }
-        if (last) break;
+    for (int i = tid; i < 32 * qs; i += LEAF_T) {
+        const int q = i / qs, j = i - q * qs;
+        Qs[i] = q < qn && j < nq ? rows[(size_t)(qb + q) * nq + j] : make_uint4(0u, 0u, 0u, 0u);
     }
     __syncthreads();
-    if (!EMIT && tid < qn && cnt[tid]) atomicAdd(&deg[cursor[tid]], cnt[tid]);
-    if (!EMIT) {
-        for (int o = 16; o > 0; o >>= 1) pairs += __shfl_xor_sync(0xffffffffu, pairs, o);
-        if ((tid & 31) == 0) stat_add(st, ST_PAIRS, pairs);
+    const unsigned selm = s_sel, qmask = 0xffffffffu >> (32 - qn);
+    // the warp's part: whole steps of 32 candidates
+    const int64_t c0 = items.begin[it], c1 = items.end[it];
+    const int64_t part = ((c1 - c0 + LEAF_T - 1) / LEAF_T) * 32;
+    int64_t ci = c0 + (tid >> 5) * part;
+    const int64_t ce = min(ci + part, c1);
+    int off = 0;
+    unsigned long long pairs = 0;
+    while (ci < ce) {
+        int pos;
+        int64_t pcand;
+        const int npr = tile_rows(tv, cand, ce, EMIT, ci, off, pos, pcand);
+        if (npr == 0) continue;
+        const int ppos = lane < npr ? pos : qb;
+        const bool mir = qp.half && ppos >= qe;
+        // the queries this row is paired with
+        unsigned want = lane < npr && !(qp.half && ppos < qb) ? qmask : 0u;
+        if (!qp.include_self && ppos >= qb && ppos < qe) want &= ~(1u << (ppos - qb));
+        if (EMIT && !(mir && rowsel)) want &= selm;
+        if (!EMIT) pairs += __popc(want);
+        const uint4 *prow = rows + (size_t)ppos * nq;
+        uint4 x[NQ];
+        unsigned hits = 0u;
+        for (int q0 = 0; q0 < qn; q0 += QB) {
+            int acc[QB];
+#pragma unroll
+            for (int j = 0; j < QB; ++j) acc[j] = 0;
+            for (int c = 0; c < nch; ++c) {
+                if (q0 == 0 || nch > 1) {
+#pragma unroll
+                    for (int i = 0; i < NQ; ++i)
+                        x[i] = c * NQ + i < nq ? __ldg(prow + c * NQ + i) : make_uint4(0u, 0u, 0u, 0u);
+                }
+#pragma unroll
+                for (int j = 0; j < QB; ++j) {
+                    const uint4 *a = Qs + (q0 + j) * qs + c * NQ;
+                    if (NQ == 1) acc[j] += popc4(xor4(a[0], x[0]));
+#pragma unroll
+                    for (int i = 0; i + 1 < NQ; i += 2) acc[j] += popc8(xor4(a[i], x[i]), xor4(a[i + 1], x[i + 1]));
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < QB; ++j) hits |= (acc[j] <= k ? 1u : 0u) << (q0 + j);
+        }
+        hits &= want;
+        const int o = hits ? tv.perm[ppos] : 0;
+        if (!EMIT && hits) atomicOr(&cand[pcand], FLAG);
+        int mslot = 0;  // the lane's first entry of its own (mirrored) row
+        if (!EMIT && mir && hits) {
+            atomicAdd(&deg[o], __popc(hits));
+            if (co.off) mslot = atomicAdd(&co.fill[o], __popc(hits));
+        }
+        const bool mrow = EMIT && mir && hits && (!rowsel || rowsel[o]);
+        const int64_t mb = mrow ? row_ptr[o] : 0, me = mrow ? row_ptr[o + 1] : 0;
+        if (mrow) mslot = atomicAdd(&rowcur[o], __popc(hits));
+        for (; hits; hits &= hits - 1u) {
+            const int q = __ffs(hits) - 1, oq = cursor[q];
+            int di = 0;
+            if (EMIT || co.off) di = ham_rows_smem(Qs + q * qs, prow, nq);
+            const float d = (float)di;
+            if (!EMIT) {
+                atomicAdd(&cnt[q], 1);
+                if (co.off) {
+                    cap_put(co, oq, o, d);
+                    if (mir) cap_place(co, o, mslot++, oq, d);
+                }
+                continue;
+            }
+            if (mrow) {
+                const int64_t at = mb + mslot++;
+                if (at < me) {
+                    col[at] = oq;
+                    dist[at] = d;
+                } else {
+                    atomicOr(err, 4);
+                }
+            }
+            if ((selm >> q) & 1u) {
+                const int64_t at = rowb[q] + atomicAdd(&rowcur[oq], 1);
+                if (at < rowe[q]) {
+                    col[at] = o;
+                    dist[at] = d;
+                } else {
+                    atomicOr(err, 4);
+                }
+            }
+        }
+        __syncwarp();
     }
+    if (EMIT) return;
+    __syncthreads();
+    if (tid < qn && cnt[tid]) atomicAdd(&deg[cursor[tid]], cnt[tid]);
+    for (int o = 16; o > 0; o >>= 1) pairs += __shfl_xor_sync(0xffffffffu, pairs, o);
+    if (lane == 0) stat_add(st, ST_PAIRS, pairs);
 }
 
 __global__ void k_alphabet(const uint8_t *__restrict__ s, int64_t nbytes, int32_t *__restrict__ present) {
@@ -3453,11 +3529,14 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
             else if (sh) go(k_leaf_l2<false, KS_SHORT>);
             else go(k_leaf_l2<false, KS_LONG>);
         } else if (ham) {
-            const size_t hsm = (size_t)64 * (t->wp / 4) * sizeof(uint4);  // 32 query rows + 32 candidate rows
-            if (emit)
-                k_leaf_ham<true><<<(unsigned)max_items, LEAF_T, hsm, s>>>(V.tv[0], V.qp[0], items, cand_p, deg.p, row_ptr, rowcur.p, col, dist, st.p, err, cw, rowsel);
-            else
-                k_leaf_ham<false><<<(unsigned)max_items, LEAF_T, hsm, s>>>(V.tv[0], V.qp[0], items, cand_p, deg.p, row_ptr, rowcur.p, col, dist, st.p, err, cw, rowsel);
+            const int nq = t->wp / 4;
+            auto go = [&](auto kern, int qreg) {  // qreg: uint4 of a row in registers
+                const size_t hsm = (size_t)32 * ((nq + qreg - 1) / qreg * qreg) * sizeof(uint4);
+                kern<<<(unsigned)max_items, LEAF_T, hsm, s>>>(V.tv[0], V.qp[0], items, cand_p, deg.p, row_ptr, rowcur.p, col, dist, st.p, err, cw, rowsel);
+            };
+            if (nq <= 1) emit ? go(k_leaf_ham<true, 1>, 1) : go(k_leaf_ham<false, 1>, 1);
+            else if (nq <= 2) emit ? go(k_leaf_ham<true, 2>, 2) : go(k_leaf_ham<false, 2>, 2);
+            else emit ? go(k_leaf_ham<true, 4>, 4) : go(k_leaf_ham<false, 4>, 4);
         } else {
             switch (W) {
 #define CT_LL(WW)                                                                                                      \
