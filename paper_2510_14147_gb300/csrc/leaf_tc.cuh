@@ -506,16 +506,30 @@ __device__ __forceinline__ void ld_f8(const float4 *p, bool al, float4 &a, float
     }
 }
 
+__device__ __forceinline__ float4 f4_sub(float4 a, float4 b) {
+    return make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w);
+}
+// A warp's batch of 32 pairs: positions, clouds, the pairs' eight chunk sums.
+struct PairShared {
+    float sum[32 * 8];
+    uint2 pos[32];
+    int cloud[32];
+};
+
 // Decides a list's pairs.  A warp takes 32 entries at a time: the eight lanes
 // of an octet read both fp32 rows of a pair, lane j eight floats of every 64
 // (contiguous 256-byte reads; a lane per 16-float chunk would touch four times
 // the lines per load), and form the canonical sum (l2dist.cuh) in its order --
 // a chunk of 16 coordinates lies in two neighbouring lanes, and its two FMA
-// chains pass from the even to the odd one; the octet's first odd lane adds
-// the chunks up.  Rows of at most 16 floats take one lane per pair.  Then lane
-// i decides and writes pair i.  Bound by the L1 data path: 1 KB of rows per
-// pair at 128 floats, and the shuffles, which share it: 39 M pairs of 128
-// floats placed in 3.4 ms (85 % of the data path's rate, ncu).
+// chains pass from one to the other: in the first 64 coordinates from the even
+// lane to the odd one, in the second the other way round, so one exchange
+// serves both and every lane ends with one chunk sum.  The chunk sums of the 32
+// pairs go through shared memory, lane i adds up pair i's, decides and writes
+// it.  Rows of at most 16 floats take one lane per pair.  Bound by the L1 data
+// path: 1 KB of rows per pair at 128 floats, and the shuffles, which share it
+// (13 per four pairs when the sums were gathered by shuffles too, 2 now).
+// 256 M pairs of 128 floats and their 478 M entries placed in 17.7 ms (19.0
+// before), 39 M in 3.2.
 template <int MODE>
 __global__ void __launch_bounds__(256, 4) k_pairs(const __grid_constant__ Views V, PairList list,
                                                   int32_t *__restrict__ deg, CapOut co,
@@ -527,6 +541,8 @@ __global__ void __launch_bounds__(256, 4) k_pairs(const __grid_constant__ Views 
     // the entries: all of cap, or the device's count of a list that did not run out
     const int64_t total = !list.n ? list.cap : (int64_t)*list.n <= list.cap ? (int64_t)*list.n : 0;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    __shared__ PairShared shared[8];  // one per warp
+    PairShared &sh = shared[threadIdx.x >> 5];
     unsigned long long guard = 0, band = 0;
     uint32_t done = 0;
     for (int64_t base = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32; base < total;
@@ -553,22 +569,27 @@ __global__ void __launch_bounds__(256, 4) k_pairs(const __grid_constant__ Views 
         const unsigned wide = __ballot_sync(0xffffffffu, valid && dp4 > 4);
         if (wide) {
             const int j = lane & 7;
+            const bool odd = lane & 1;
             const int nu = (int)__reduce_max_sync(0xffffffffu, valid ? (unsigned)((dp4 + 15) >> 4) : 0u);
+            __syncwarp();  // the last batch's sums are read
+            sh.pos[lane] = make_uint2(e.x, gp);
+            if (V.nc > 1) sh.cloud[lane] = c;
+            __syncwarp();
             for (int r = 0; r < 8; ++r) {
                 if (!((wide >> (4 * r)) & 0xfu)) continue;
                 const int src = 4 * r + (lane >> 3);
                 const bool on = (wide >> src) & 1u;
-                const uint32_t qs = __shfl_sync(0xffffffffu, e.x, src), ps = __shfl_sync(0xffffffffu, gp, src);
-                const int cs = V.nc > 1 ? __shfl_sync(0xffffffffu, c, src) : 0;
+                const uint2 sp = sh.pos[src];
+                const int cs = V.nc > 1 ? sh.cloud[src] : 0;
                 const int n4 = V.tv[cs].dp >> 2;
                 const float4 *pts = reinterpret_cast<const float4 *>(V.tv[cs].pts);
-                const float4 *x = pts + (int64_t)(qs - (uint32_t)V.rbase[cs]) * n4;
-                const float4 *y = pts + (int64_t)(ps - (uint32_t)V.rbase[cs]) * n4;
+                const float4 *x = pts + (int64_t)(sp.x - (uint32_t)V.rbase[cs]) * n4;
+                const float4 *y = pts + (int64_t)(sp.y - (uint32_t)V.rbase[cs]) * n4;
                 const bool al = ((n4 & 1) | (int)(reinterpret_cast<uintptr_t>(pts) & 31)) == 0;
                 float4 a[2][2], d[2][2];
 #pragma unroll
                 for (int u = 0; u < 2; ++u) {  // dp <= 128: at most two times eight floats per lane
-                    const int f = 16 * u + 2 * j;  // float4s f and f + 1
+                    const int f = 16 * u + 2 * (j ^ u);  // float4s f and f + 1
                     a[u][0] = a[u][1] = d[u][0] = d[u][1] = make_float4(0.f, 0.f, 0.f, 0.f);
                     if (on && f + 1 < n4) {
                         ld_f8(x + f, al, a[u][0], a[u][1]);
@@ -578,29 +599,39 @@ __global__ void __launch_bounds__(256, 4) k_pairs(const __grid_constant__ Views 
                         d[u][0] = __ldg(y + f);
                     }
                 }
-                float ssum = 0.f;
+                // the chains of a chunk's first eight floats (u = 0: even lanes, 1: odd lanes) go to
+                // the neighbour, which has its last eight
+                float lo[2], hi[2];
 #pragma unroll
                 for (int u = 0; u < 2; ++u) {
-                    if (u >= nu) break;  // warp-uniform
-                    const float dx = a[u][0].x - d[u][0].x, dy = a[u][0].y - d[u][0].y, dz = a[u][0].z - d[u][0].z,
-                                dw = a[u][0].w - d[u][0].w;
-                    const float ex = a[u][1].x - d[u][1].x, ey = a[u][1].y - d[u][1].y, ez = a[u][1].z - d[u][1].z,
-                                ew = a[u][1].w - d[u][1].w;
-                    // the chains of an even lane's eight floats, then of the odd lane's after them
-                    float lo = fmaf(ez, ez, fmaf(ex, ex, fmaf(dz, dz, dx * dx)));
-                    float hi = fmaf(ew, ew, fmaf(ey, ey, fmaf(dw, dw, dy * dy)));
-                    lo = __shfl_up_sync(0xffffffffu, lo, 1);
-                    hi = __shfl_up_sync(0xffffffffu, hi, 1);
-                    lo = fmaf(ez, ez, fmaf(ex, ex, fmaf(dz, dz, fmaf(dx, dx, lo))));
-                    hi = fmaf(ew, ew, fmaf(ey, ey, fmaf(dw, dw, fmaf(dy, dy, hi))));
-                    const float chunk = lo + hi;  // chunk 4 u + j / 2, in odd lanes
-                    ssum += chunk;                // lane 1: chunk 4 u
-                    ssum += __shfl_down_sync(0xffffffffu, chunk, 2);
-                    ssum += __shfl_down_sync(0xffffffffu, chunk, 4);
-                    ssum += __shfl_down_sync(0xffffffffu, chunk, 6);
+                    a[u][0] = f4_sub(a[u][0], d[u][0]);
+                    a[u][1] = f4_sub(a[u][1], d[u][1]);
+                    const float4 p = a[u][0], q = a[u][1];
+                    lo[u] = fmaf(q.z, q.z, fmaf(q.x, q.x, fmaf(p.z, p.z, p.x * p.x)));
+                    hi[u] = fmaf(q.w, q.w, fmaf(q.y, q.y, fmaf(p.w, p.w, p.y * p.y)));
                 }
-                const float v = __shfl_sync(0xffffffffu, ssum, ((lane & 3) << 3) + 1);
-                if ((lane >> 2) == r && ((wide >> lane) & 1u)) sv = v;
+                const float lo_in = __shfl_xor_sync(0xffffffffu, odd ? lo[1] : lo[0], 1);
+                const float hi_in = __shfl_xor_sync(0xffffffffu, odd ? hi[1] : hi[0], 1);
+                float chunk[2];
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const float4 p = a[u][0], q = a[u][1];
+                    chunk[u] = fmaf(q.z, q.z, fmaf(q.x, q.x, fmaf(p.z, p.z, fmaf(p.x, p.x, lo_in)))) +
+                               fmaf(q.w, q.w, fmaf(q.y, q.y, fmaf(p.w, p.w, fmaf(p.y, p.y, hi_in))));
+                }
+                // chunk j / 2 in odd lanes, 4 + j / 2 in even ones; odd rounds swap the halves (banks)
+                sh.sum[8 * src + ((odd ? j >> 1 : 4 + (j >> 1)) ^ ((r & 1) << 2))] = odd ? chunk[0] : chunk[1];
+            }
+            __syncwarp();
+            if ((wide >> lane) & 1u) {
+                const float4 *ss = reinterpret_cast<const float4 *>(sh.sum + 8 * lane);
+                const int sw = (lane >> 2) & 1;
+                const float4 s0 = ss[sw];
+                sv = ((s0.x + s0.y) + s0.z) + s0.w;
+                if (nu > 1) {
+                    const float4 s1 = ss[1 - sw];
+                    sv = (((sv + s1.x) + s1.y) + s1.z) + s1.w;
+                }
             }
         }
         if (!valid) continue;
