@@ -164,6 +164,38 @@ constexpr int TRAV_LIMIT = 128;    // step limit of the next rounds
 // L2 steps, so its walks stop much sooner
 constexpr int TRAV_LIMIT0_LEV = 8, TRAV_LIMIT_LEV = 8;
 
+// Packed fp32 pairs (sm_100+ f32x2 instructions): two independent IEEE
+// round-to-nearest operations per instruction.
+__device__ __forceinline__ unsigned long long f2_sub(unsigned long long a, unsigned long long b) {
+    unsigned long long d;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ unsigned long long f2_sqacc(unsigned long long d, unsigned long long acc) {
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %1, %2;" : "=l"(r) : "l"(d), "l"(acc));
+    return r;
+}
+__device__ __forceinline__ unsigned long long f2_pack(float lo, float hi) {
+    unsigned long long d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+    return d;
+}
+__device__ __forceinline__ unsigned long long f2_add(unsigned long long a, unsigned long long b) {
+    unsigned long long d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ unsigned long long f2_fma(unsigned long long a, unsigned long long b,
+                                                     unsigned long long c) {
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ float f2_sum(unsigned long long v) {
+    return __uint_as_float((uint32_t)v) + __uint_as_float((uint32_t)(v >> 32));
+}
+
 // Warp-uniform write cursor: current chunk, its fill, the open segment.
 struct PoolCursor {
     int64_t cur;
@@ -390,10 +422,12 @@ __device__ __forceinline__ void group_visits(int32_t *gvisit, int g, unsigned lo
     if ((threadIdx.x & 31) == 0) atomicAdd(gvisit + g, (int32_t)(v < 0x7fffffffull ? v : 0x7fffffffull));
 }
 
-// L2 test of `take` consecutive vertices against the group centre (shared
+// L2 test of `take` vertices (lane i's: vid) against the group centre (shared
 // memory): TPD lanes share one vertex and read its centre row in coalesced
-// 16-byte pieces; the partial sums are reduced by shuffles and lane i gets
-// vertex i's squared distance.  Keep v unless d > (r(v) + eps + r_g)(1 + 2^-10).
+// 16-byte pieces.  The TPD rounds' partial sums are reduced together -- each
+// exchange halves the sums a lane holds, 7 shuffles instead of 8 x 4 at 8 lanes
+// a vertex -- and lane i gets vertex i's squared distance.  Keep v unless
+// d > (r(v) + eps + r_g)(1 + 2^-10).
 template <int TPD>
 __device__ __forceinline__ bool l2_keep(const TreeView &tv, const float4 *cen, int nq4, int vid, int take,
                                         float add) {
@@ -406,33 +440,31 @@ __device__ __forceinline__ bool l2_keep(const TreeView &tv, const float4 *cen, i
     for (int u = 0; u < TPD; ++u) {
         const int i = u * NPR + sub;
         const int vi = __shfl_sync(0xffffffffu, vid, i);  // vertex of lane i
-        float acc = 0.f;
+        unsigned long long acc = 0ull;
         if (u * NPR < take && i < take) {
-            const float4 *row = reinterpret_cast<const float4 *>(tv.node_ctr) + (size_t)vi * nq4;
+            const ulonglong2 *row = reinterpret_cast<const ulonglong2 *>(tv.node_ctr) + (size_t)vi * nq4;
+            const ulonglong2 *c = reinterpret_cast<const ulonglong2 *>(cen);
 #pragma unroll 4
             for (int k = j; k < nq4; k += TPD) {
-                const float4 a = cen[k], b = __ldg(row + k);
-                const float dx = a.x - b.x, dy = a.y - b.y, dz = a.z - b.z, dw = a.w - b.w;
-                acc = fmaf(dx, dx, acc);
-                acc = fmaf(dy, dy, acc);
-                acc = fmaf(dz, dz, acc);
-                acc = fmaf(dw, dw, acc);
+                const ulonglong2 a = c[k], b = __ldg(row + k);
+                const unsigned long long dx = f2_sub(a.x, b.x), dy = f2_sub(a.y, b.y);
+                acc = f2_sqacc(dx, acc);
+                acc = f2_sqacc(dy, acc);
             }
         }
-        part[u] = acc;
+        part[u] = f2_sum(acc);
     }
-    float mine = 0.f;
 #pragma unroll
-    for (int u = 0; u < TPD; ++u) {
-        if (u * NPR >= take) break;  // warp-uniform
-        float acc = part[u];
+    for (int o = TPD / 2; o > 0; o >>= 1) {  // lane j keeps the sums of the rounds u with bit o of j
+        const bool upper = (j & o) != 0;
 #pragma unroll
-        for (int o = TPD / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        const int r0 = u * NPR;
-        const int src = ((lane - r0) & (NPR - 1)) * TPD;
-        const float v = __shfl_sync(0xffffffffu, acc, src);
-        if (lane >= r0 && lane < r0 + NPR) mine = v;
+        for (int i = 0; i < o; ++i) {
+            const float send = upper ? part[i] : part[i + o], own = upper ? part[i + o] : part[i];
+            part[i] = own + __shfl_xor_sync(0xffffffffu, send, o);
+        }
     }
+    // lane (sub, j) holds vertex j NPR + sub
+    const float mine = __shfl_sync(0xffffffffu, part[0], (lane & (NPR - 1)) * TPD + lane / NPR);
     if (lane >= take) return false;
     const float bound = fmaf(rad + add, PRUNE_REL, PRUNE_ABS);
     return !(sqrtf(mine) > bound);
@@ -793,38 +825,6 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N)); }
-
-// Packed fp32 pairs (sm_100+ f32x2 instructions): two independent IEEE
-// round-to-nearest operations per instruction.
-__device__ __forceinline__ unsigned long long f2_sub(unsigned long long a, unsigned long long b) {
-    unsigned long long d;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ unsigned long long f2_sqacc(unsigned long long d, unsigned long long acc) {
-    unsigned long long r;
-    asm("fma.rn.f32x2 %0, %1, %1, %2;" : "=l"(r) : "l"(d), "l"(acc));
-    return r;
-}
-__device__ __forceinline__ unsigned long long f2_pack(float lo, float hi) {
-    unsigned long long d;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
-    return d;
-}
-__device__ __forceinline__ unsigned long long f2_add(unsigned long long a, unsigned long long b) {
-    unsigned long long d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ unsigned long long f2_fma(unsigned long long a, unsigned long long b,
-                                                     unsigned long long c) {
-    unsigned long long d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ float f2_sum(unsigned long long v) {
-    return __uint_as_float((uint32_t)v) + __uint_as_float((uint32_t)(v >> 32));
-}
 
 // Squared distances of the 2 x 4 pairs owned by this thread: queries qi and
 // qi + 16 of the Q tile against rows pj, pj+8, pj+16, pj+24 of the P tile,
