@@ -34,27 +34,6 @@ namespace {
 
 constexpr int LM_T = 256;
 
-// Distances of the Voronoi step: fp32 direct differences (L2; the ghost test
-// below carries a margin far above their error) or exact popcounts (Hamming).
-__device__ __forceinline__ float lm_dist_l2(const float *__restrict__ x, const float *__restrict__ c, int dim) {
-    float acc = 0.f;
-    for (int k = 0; k < dim; ++k) {
-        const float d = x[k] - c[k];
-        acc = fmaf(d, d, acc);
-    }
-    return sqrtf(acc);
-}
-__device__ __forceinline__ int lm_dist_ham(const uint8_t *__restrict__ a, const uint8_t *__restrict__ b, int dim) {
-    const int nb = (dim + 7) >> 3;
-    int d = 0;
-    for (int i = 0; i < nb; ++i) {
-        uint32_t x = (uint32_t)(a[i] ^ b[i]);
-        if (8 * i + 8 > dim) x &= (1u << (dim - 8 * i)) - 1u;  // bits past dim are not part of the row
-        d += __popc(x);
-    }
-    return d;
-}
-
 struct LmInput {
     int metric, dim;
     const float *X;      // L2: n x dim
@@ -62,13 +41,6 @@ struct LmInput {
     const int64_t *cid;  // m centre ids
     int m;
 };
-
-__device__ __forceinline__ float lm_dist(const LmInput &in, int64_t p, int k) {
-    const int64_t c = in.cid[k];
-    if (in.metric == CT_L2_F32) return lm_dist_l2(in.X + p * in.dim, in.X + c * in.dim, in.dim);
-    const int nb = (in.dim + 7) >> 3;
-    return (float)lm_dist_ham(in.B + p * nb, in.B + c * nb, in.dim);
-}
 
 // Lemma 1's ghost test of point p (nearest-centre distance dmin) for cell k:
 // exact for Hamming (integers); for L2 with a relative margin of 2^-10 over
@@ -78,45 +50,159 @@ __device__ __forceinline__ bool lm_ghost(const LmInput &in, float d, float dmin,
     return d <= fmaf(dmin + eps_up, 1.0f + 0x1p-10f, eps_up) + 0x1p-60f;
 }
 
-__global__ void k_lm_nearest(LmInput in, int64_t n, int32_t *__restrict__ cell, float *__restrict__ dmin) {
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= n) return;
-    int best = 0;
-    float bd = lm_dist(in, p, 0);
-    for (int k = 1; k < in.m; ++k) {
-        const float d = lm_dist(in, p, k);
-        if (d < bd) {
-            bd = d;
-            best = k;
+// Distances of LM_P points to LM_C centres at a time: fp32 direct differences,
+// a term after the other (L2; the ghost test carries a margin far above their
+// error), or exact popcounts (Hamming).  A block has LM_P points; the rows of
+// both sides go through shared memory in chunks of 32 words, coalesced, and
+// every thread forms 4 x 4 of the distances.
+// k_lm_cells<false>: nearest centre and distance of each point, then its number
+// of memberships (its own cell and the cells it is a ghost of); a single tile
+// of centres is evaluated once for both.  k_lm_cells<true>: the membership keys
+// (cell << 32 | p) at moff[p], in increasing cell.
+// Bound by the shared-memory reads (8 words per 16 terms).  97k x 64 against 60
+// centres: both kernels together took 4.5 ms with a thread per point that read
+// its row and the centres' a word at a time, 0.1 ms now.
+constexpr int LM_P = 64, LM_C = 64, LM_KC = 32;
+
+struct LmTile {
+    uint32_t x[LM_P][LM_KC + 1], c[LM_C][LM_KC + 1];
+    float d[LM_P][LM_C + 1];
+};
+
+// Word w of a row: a float's bits, or 32 bits of a code (bits past dim cleared).
+__device__ __forceinline__ uint32_t lm_word(const LmInput &in, int64_t p, int w) {
+    if (in.metric == CT_L2_F32) return __float_as_uint(in.X[p * in.dim + w]);
+    const int nb = (in.dim + 7) >> 3;
+    const uint8_t *r = in.B + p * nb;
+    uint32_t v = 0u;
+    for (int i = 0; i < 4; ++i)
+        if (4 * w + i < nb) v |= (uint32_t)r[4 * w + i] << (8 * i);
+    const int bits = in.dim - 32 * w;
+    return bits < 32 ? v & ((1u << bits) - 1u) : v;
+}
+
+// S.d[i][j] = distance of point p0 + i and centre k0 + j (i < np, j < nc).
+__device__ __forceinline__ void lm_tile(const LmInput &in, LmTile &S, int64_t p0, int np, int k0, int nc) {
+    const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+    const bool l2 = in.metric == CT_L2_F32;
+    const int words = l2 ? in.dim : (in.dim + 31) >> 5;
+    float acc[4][4] = {};
+    int bits[4][4] = {};
+    for (int w0 = 0; w0 < words; w0 += LM_KC) {
+        const int kn = min(LM_KC, words - w0);
+        __syncthreads();
+        for (int i = tid; i < (LM_P + LM_C) * LM_KC; i += LM_T) {
+            const int r = i / LM_KC, w = i % LM_KC;
+            if (w >= kn) continue;
+            if (r < LM_P) S.x[r][w] = r < np ? lm_word(in, p0 + r, w0 + w) : 0u;
+            else S.c[r - LM_P][w] = r - LM_P < nc ? lm_word(in, in.cid[k0 + r - LM_P], w0 + w) : 0u;
+        }
+        __syncthreads();
+        if (l2) {
+            for (int w = 0; w < kn; ++w) {
+                float c[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) c[j] = __uint_as_float(S.c[tx + 16 * j][w]);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float x = __uint_as_float(S.x[ty + 16 * i][w]);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float t = x - c[j];
+                        acc[i][j] = fmaf(t, t, acc[i][j]);
+                    }
+                }
+            }
+        } else {
+            for (int w = 0; w < kn; ++w)
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) bits[i][j] += __popc(S.x[ty + 16 * i][w] ^ S.c[tx + 16 * j][w]);
         }
     }
-    cell[p] = best;
-    dmin[p] = bd;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) S.d[ty + 16 * i][tx + 16 * j] = l2 ? sqrtf(acc[i][j]) : (float)bits[i][j];
+    __syncthreads();
 }
 
-// Memberships of point p: its own cell and the cells it is a ghost of
-// (count pass: keys == nullptr; fill pass: keys (cell << 32 | p) at moff[p]).
-__global__ void k_lm_members(LmInput in, int64_t n, const int32_t *__restrict__ cell, const float *__restrict__ dmin,
-                             float eps_up, int lev_k, int32_t *__restrict__ mcount, const int64_t *__restrict__ moff,
-                             uint64_t *__restrict__ keys) {
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= n) return;
-    const int own = cell[p];
-    const float dm = dmin[p];
-    int64_t at = keys ? moff[p] : 0;
-    int c = 0;
-    for (int k = 0; k < in.m; ++k) {
-        const bool mem = k == own || lm_ghost(in, lm_dist(in, p, k), dm, eps_up, lev_k);
-        if (!mem) continue;
-        if (keys) keys[at++] = ((uint64_t)k << 32) | (uint64_t)p;
-        ++c;
+template <bool FILL>
+__global__ void __launch_bounds__(LM_T) k_lm_cells(LmInput in, int64_t n, float eps_up, int lev_k,
+                                                   int32_t *__restrict__ cell, float *__restrict__ dmin,
+                                                   int32_t *__restrict__ mcount, const int64_t *__restrict__ moff,
+                                                   uint64_t *__restrict__ keys) {
+    static_assert(LM_T == 4 * LM_P, "four threads per point");
+    __shared__ LmTile S;
+    __shared__ int s_cell[LM_P];
+    __shared__ float s_dmin[LM_P];
+    const int tid = threadIdx.x;
+    const int64_t p0 = (int64_t)blockIdx.x * LM_P;
+    const int np = (int)min((int64_t)LM_P, n - p0);
+    if (tid < np && FILL) {
+        s_cell[tid] = cell[p0 + tid];
+        s_dmin[tid] = dmin[p0 + tid];
     }
-    if (!keys) mcount[p] = c;
+    if (!FILL) {
+        int best = 0;
+        float bd = 0.f;
+        for (int k0 = 0; k0 < in.m; k0 += LM_C) {
+            const int nc = min(LM_C, in.m - k0);
+            __syncthreads();
+            lm_tile(in, S, p0, np, k0, nc);
+            if (tid < np) {
+                for (int j = 0; j < nc; ++j) {
+                    const float d = S.d[tid][j];
+                    if (d < bd || k0 + j == 0) {  // the lowest index among equals
+                        bd = d;
+                        best = k0 + j;
+                    }
+                }
+            }
+        }
+        if (tid < np) {
+            cell[p0 + tid] = s_cell[tid] = best;
+            dmin[p0 + tid] = s_dmin[tid] = bd;
+        }
+    }
+    // memberships: four threads per point, 16 centres of a tile each
+    const int r = tid >> 2, part = tid & 3;
+    int64_t at = FILL && r < np ? moff[p0 + r] : 0;
+    for (int k0 = 0; k0 < in.m; k0 += LM_C) {
+        const int nc = min(LM_C, in.m - k0);
+        __syncthreads();
+        if (FILL || in.m > LM_C) lm_tile(in, S, p0, np, k0, nc);
+        uint32_t mem = 0u;
+        if (r < np) {
+            const int own = s_cell[r];
+            const float dm = s_dmin[r];
+            for (int j = 16 * part; j < min(16 * part + 16, nc); ++j)
+                if (k0 + j == own || lm_ghost(in, S.d[r][j], dm, eps_up, lev_k)) mem |= 1u << (j & 15);
+        }
+        const int c = __popc(mem);
+        const int c1 = __shfl_up_sync(0xffffffffu, c, 1, 4), c2 = __shfl_up_sync(0xffffffffu, c, 2, 4),
+                  c3 = __shfl_up_sync(0xffffffffu, c, 3, 4);
+        const int before = (part > 0 ? c1 : 0) + (part > 1 ? c2 : 0) + (part > 2 ? c3 : 0);
+        if (FILL) {
+            for (int64_t a = at + before; mem; mem &= mem - 1u)
+                keys[a++] = ((uint64_t)(k0 + 16 * part + __ffs(mem) - 1) << 32) | (uint64_t)(p0 + r);
+        }
+        at += __shfl_sync(0xffffffffu, before + c, 3, 4);
+    }
+    if (!FILL && r < np && part == 0) mcount[p0 + r] = (int32_t)at;
 }
 
-__global__ void k_lm_cell_counts(const uint64_t *__restrict__ keys, int64_t M, int32_t *__restrict__ cnt) {
-    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (j < M) atomicAdd(&cnt[(int)(keys[j] >> 32)], 1);
+// First member of each cell in the sorted keys (k in [0, m]).
+__global__ void k_lm_cell_offsets(const uint64_t *__restrict__ keys, int64_t M, int m, int64_t *__restrict__ off) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k > m) return;
+    int64_t lo = 0, hi = M;
+    while (lo < hi) {
+        const int64_t mid = (lo + hi) >> 1;
+        if ((int64_t)(keys[mid] >> 32) < k) lo = mid + 1; else hi = mid;
+    }
+    off[k] = lo;
 }
 
 // Rows of the members, cell by cell, in member order.
@@ -212,19 +298,17 @@ void landmark_query(const ct_points *pts, const int64_t *centres_h, int m, doubl
     DBuf<int32_t> cell(n, s), mcount(n + 1, s);
     DBuf<float> dmin(n, s);
     DBuf<int64_t> moff(n + 1, s);
-    k_lm_nearest<<<grid_of(n, LM_T), LM_T, 0, s>>>(in, n, cell.p, dmin.p);
-    CT_COUNT_LAUNCH();
     CT_CHECK_CUDA(cudaMemsetAsync(mcount.p + n, 0, sizeof(int32_t), s));
-    k_lm_members<<<grid_of(n, LM_T), LM_T, 0, s>>>(in, n, cell.p, dmin.p, qp.eps_up, qp.lev_k, mcount.p, nullptr,
-                                                   nullptr);
+    k_lm_cells<false><<<grid_of(n, LM_P), LM_T, 0, s>>>(in, n, qp.eps_up, qp.lev_k, cell.p, dmin.p, mcount.p, nullptr,
+                                                        nullptr);
     CT_COUNT_LAUNCH();
     exclusive_scan_i32_to_i64(mcount.p, moff.p, n + 1, nullptr, s);
     int64_t M = 0;
     to_host(&M, moff.p + n, 1, s);
     DBuf<uint64_t> keys(M, s), tk(M, s);
     DBuf<uint32_t> vals(M, s), tv(M, s);
-    k_lm_members<<<grid_of(n, LM_T), LM_T, 0, s>>>(in, n, cell.p, dmin.p, qp.eps_up, qp.lev_k, mcount.p, moff.p,
-                                                   keys.p);
+    k_lm_cells<true><<<grid_of(n, LM_P), LM_T, 0, s>>>(in, n, qp.eps_up, qp.lev_k, cell.p, dmin.p, mcount.p, moff.p,
+                                                       keys.p);
     CT_COUNT_LAUNCH();
     CT_CHECK_CUDA(cudaMemsetAsync(vals.p, 0, (size_t)M * sizeof(uint32_t), s));
     int bits = 32;
@@ -233,12 +317,9 @@ void landmark_query(const ct_points *pts, const int64_t *centres_h, int m, doubl
     tk.reset();
     tv.reset();
     vals.reset();
-    DBuf<int32_t> ccnt(m + 1, s);
     DBuf<int64_t> coff(m + 1, s);
-    CT_CHECK_CUDA(cudaMemsetAsync(ccnt.p, 0, (size_t)(m + 1) * sizeof(int32_t), s));
-    k_lm_cell_counts<<<grid_of(M, LM_T), LM_T, 0, s>>>(keys.p, M, ccnt.p);
+    k_lm_cell_offsets<<<grid_of(m + 1, LM_T), LM_T, 0, s>>>(keys.p, M, m, coff.p);
     CT_COUNT_LAUNCH();
-    exclusive_scan_i32_to_i64(ccnt.p, coff.p, m + 1, nullptr, s);
     std::vector<int64_t> hoff(m + 1);
     to_host(hoff.data(), coff.p, m + 1, s);
     // 3. member rows gathered cell by cell; a tree per cell
