@@ -6,6 +6,19 @@
 //
 // lev_myers returns the distance when it is <= k and some value > k
 // otherwise; it stops early once the bottom-row value can no longer fall to k.
+//
+// lev_band is the form for a bound below the word length (Hyyrö 2003): a path
+// of cost <= k from (0, 0) to (m, n) stays within floor((k - |m - n|) / 2)
+// diagonals of the two that these lie on, at most k + 1 diagonals in all, so
+// one word holds a column's part of that band whatever the pattern's length.
+// The word slides down a row per column.  Cells outside count as one more than
+// their diagonal predecessor, so every value is the cost of some path and the
+// ones on a path of cost <= k are exact.  Rows above the table (bits below row
+// 0) hold the column number, which makes row 0 grow by one per column.  The
+// value on the diagonal of (m, n) never falls: the form stops at the first
+// one above k.  Against four 32-bit words of a whole column of 96 symbols, a
+// column of the band is one: the leaf stage of 50k
+// reads of 96 symbols (18.7 M pairs within 13) takes 2.0 ms instead of 9.0.
 #pragma once
 
 #include <stdint.h>
@@ -34,6 +47,67 @@ __device__ __forceinline__ void lev_build_peq(uint64_t *peq, const uint8_t *pat,
         atomicOr((unsigned long long *)&peq[pat[j] * W + (j >> 6)], 1ull << (j & 63));
 }
 
+// Word i of a symbol's match mask, from the 64-bit words (zero outside).
+template <int W>
+CT_HD uint32_t lev_word(const uint64_t *eq, int i, uint32_t) {
+    return (unsigned)i < 2u * W ? (uint32_t)(eq[i >> 1] >> (32 * (i & 1))) : 0u;
+}
+template <int W>
+CT_HD uint64_t lev_word(const uint64_t *eq, int i, uint64_t) {
+    return (unsigned)i < (unsigned)W ? eq[i] : 0ull;
+}
+CT_HD uint32_t lev_window(uint32_t lo, uint32_t hi, int sh) {
+#ifdef __CUDA_ARCH__
+    return __funnelshift_r(lo, hi, sh);
+#else
+    return sh ? (lo >> sh) | (hi << (32 - sh)) : lo;
+#endif
+}
+CT_HD uint64_t lev_window(uint64_t lo, uint64_t hi, int sh) { return sh ? (lo >> sh) | (hi << (64 - sh)) : lo; }
+
+// The distance if it is <= k, else k + 1; m, n >= 1, |m - n| <= k < bits of T.
+// sym(character) is the character's row in peq; cols: columns evaluated.
+template <class T, int W, class Sym>
+CT_HD int lev_band(const uint64_t *peq, Sym sym, int m, const uint8_t *txt, int n, int k, int &cols) {
+    constexpr int B = 8 * sizeof(T), LB = sizeof(T) == 8 ? 6 : 5;
+    const int dl = m - n;
+    const int c = ((k - (dl < 0 ? -dl : dl)) >> 1) + (dl < 0 ? -dl : 0);  // bit 0: diagonal -c
+    const int bf = dl + c;                                                // the bit of (m, n)'s diagonal
+    T VP = ~(T)0 << c, VN = 0;
+    int score = dl > 0 ? dl : 0;
+    constexpr int LEV_PF = 8;  // as in lev_myers
+    int nxt[LEV_PF];
+#pragma unroll
+    for (int u = 0; u < LEV_PF; ++u) nxt[u] = u < n ? (int)txt[u] : 0;
+    for (int j0 = 0; j0 < n; j0 += LEV_PF) {
+        int blk[LEV_PF];
+#pragma unroll
+        for (int u = 0; u < LEV_PF; ++u) {
+            blk[u] = nxt[u];
+            nxt[u] = j0 + LEV_PF + u < n ? (int)txt[j0 + LEV_PF + u] : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < LEV_PF; ++u) {
+            const int j = j0 + u;
+            if (j >= n) break;
+            const uint64_t *eqr = peq + sym(blk[u]) * W;
+            const int base = j - c, wi = base >> LB;  // pattern index of bit 0 (rows are 1-based)
+            const T Eq = lev_window(lev_word<W>(eqr, wi, T()), lev_word<W>(eqr, wi + 1, T()), base & (B - 1));
+            const T D0 = (((Eq & VP) + VP) ^ VP) | Eq | VN;
+            const T HP = VN | ~(D0 | VP), HN = D0 & VP;
+            score += (int)((D0 >> bf) & 1) ^ 1;
+            if (score > k) {
+                cols = j + 1;
+                return k + 1;
+            }
+            VP = HN | ~((D0 >> 1) | HP);
+            VN = (D0 >> 1) & HP;
+        }
+    }
+    cols = n;
+    return score;
+}
+
 template <int W>
 CT_HD int lev_myers(const uint64_t *peq, int m, const uint8_t *txt, int n, int k) {
     if (k < 0) return 0 == m && 0 == n ? 0 : k + 1;
@@ -41,6 +115,12 @@ CT_HD int lev_myers(const uint64_t *peq, int m, const uint8_t *txt, int n, int k
     if (dl > k) return k + 1;
     if (m == 0) return n;
     if (n == 0) return m;
+    if (W > 1 && k < 64) {
+        int cols;
+        auto same = [](int s) { return s; };
+        return k < 32 ? lev_band<uint32_t, W>(peq, same, m, txt, n, k, cols)
+                      : lev_band<uint64_t, W>(peq, same, m, txt, n, k, cols);
+    }
     const int nw = (m + 63) >> 6;
     const int hw = (m - 1) >> 6;
     const uint64_t hbit = 1ull << ((m - 1) & 63);

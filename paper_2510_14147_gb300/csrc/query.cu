@@ -1963,6 +1963,14 @@ __device__ __forceinline__ int lev_mapped(const uint64_t *__restrict__ pq, const
     if ((m > n ? m - n : n - m) > k) return k + 1;
     if (m == 0) return n;
     if (n == 0) return m;
+    if (W > 1 && k < 64) {
+        int done;
+        auto sym = [amap](int s) { return (int)amap[s]; };
+        const int d = k < 32 ? lev_band<uint32_t, W>(pq, sym, m, txt, n, k, done)
+                             : lev_band<uint64_t, W>(pq, sym, m, txt, n, k, done);
+        cols += (unsigned)done;
+        return d;
+    }
     const int nw = (m + 63) >> 6, hw = (m - 1) >> 6;
     const uint64_t hbit = 1ull << ((m - 1) & 63);
     uint64_t Pv[W], Mv[W];
