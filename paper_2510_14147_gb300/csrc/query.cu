@@ -157,7 +157,13 @@ struct Spill {
     int cap;
     int limit;       // steps before a walk stops
 };
-constexpr int TRAV_ROUNDS = 4;     // rounds after the groups' round; the last one has no step limit
+// Rounds after the groups' round; the last one has no step limit, and walks
+// that are long when it begins set its time.  L2 walks are done by the third
+// or fourth.  Of edit-distance walks, whose vertices can have thousands of
+// children, 6.0 of 7.3 ms were spent in the last of 4 rounds (50k reads of 96);
+// with long ranges cut up they are done by the fourth, 1.5 ms in all, and two
+// spare rounds stand against other data.  A round that finds no work takes 6 us.
+constexpr int TRAV_ROUNDS = 4, TRAV_ROUNDS_LEV = 6;
 constexpr int TRAV_LIMIT0 = 256;   // step limit of the groups' round
 constexpr int TRAV_LIMIT = 128;    // step limit of the next rounds
 // edit distance: a step (32 bit-parallel recurrences) costs about a hundred
@@ -326,13 +332,29 @@ __device__ __forceinline__ int walk_group(const TreeView &tv, int2 *__restrict__
         int limit = sp ? sp->limit : INT_MAX;
         for (int steps = 0; top > 0; ++steps) {
             if (steps >= limit) {
+                // long ranges are stored in pieces that a quarter of the limit walks: a
+                // vertex can have tens of thousands of children
+                const int piece = max(32, 8 * sp->limit);
+                int total = 0;
+                for (int i = lane; i < top; i += 32) total += (stack[i].y + piece - 1) / piece;
+                total = (int)__reduce_add_sync(0xffffffffu, (unsigned)total);
                 int base = 0;
-                if (lane == 0) base = atomicAdd(sp->count, top);
+                if (lane == 0) base = atomicAdd(sp->count, total);
                 base = __shfl_sync(0xffffffffu, base, 0);
-                if (base + top <= sp->cap) {
-                    for (int i = lane; i < top; i += 32) {
-                        const int2 r = stack[i];
-                        sp->items[base + i] = make_int4(g, r.x, r.y, 0);
+                if (base + total <= sp->cap) {
+                    for (int i0 = 0; i0 < top; i0 += 32) {
+                        const int2 r = i0 + lane < top ? stack[i0 + lane] : make_int2(0, 0);
+                        const int c = (r.y + piece - 1) / piece;
+                        int incl = c;
+#pragma unroll
+                        for (int o = 1; o < 32; o <<= 1) {
+                            const int y = __shfl_up_sync(0xffffffffu, incl, o);
+                            if (lane >= o) incl += y;
+                        }
+                        for (int j = 0; j < c; ++j)
+                            sp->items[base + incl - c + j] =
+                                make_int4(g, r.x + j * piece, min(piece, r.y - j * piece), 0);
+                        base += __shfl_sync(0xffffffffu, incl, 31);
                     }
                     break;
                 }
@@ -3113,12 +3135,13 @@ void launch_traversal(const Views &V, int64_t G, int max_dp, int max_len, bool l
         tv.group_order = order;
         const bool ham = tv.wp != 0;
         CT_CHECK_CUDA(cudaMemsetAsync(spill_cnt, 0, 2 * sizeof(int32_t), s));
-        for (int r = 0; r <= TRAV_ROUNDS; ++r) {
+        const int rounds = ham ? TRAV_ROUNDS : TRAV_ROUNDS_LEV;
+        for (int r = 0; r <= rounds; ++r) {
             const int4 *in = r ? spill[(r - 1) & 1] : resumed;
             const int32_t *in_cnt = r ? spill_cnt + ((r - 1) & 1) : n_resumed;
             const int in_cap = r ? spill_cap : resumed_cap;
             Spill out{nullptr, spill_cnt + (r & 1), spill_cap, INT_MAX};
-            if (r < TRAV_ROUNDS) {
+            if (r < rounds) {
                 out.items = spill[r & 1];
                 out.limit = ham ? (r ? TRAV_LIMIT : TRAV_LIMIT0) : (r ? TRAV_LIMIT_LEV : TRAV_LIMIT0_LEV);
             }
@@ -3341,7 +3364,7 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
     for (int pass = 0;; ++pass) {
         // a segment per walk (groups, stored ranges) and per chunk a walk crosses
         const int64_t old_seg = seg_cap, nseg0 = pass ? (int64_t)(uint32_t)hc[1] : 0;
-        seg_cap = old_seg + G + (int64_t)TRAV_ROUNDS * spill_cap + pool_cap / POOL_CHUNK + tl.warps + 16 +
+        seg_cap = old_seg + G + (int64_t)(l2 || ham ? TRAV_ROUNDS : TRAV_ROUNDS_LEV) * spill_cap + pool_cap / POOL_CHUNK + tl.warps + 16 +
                   (pass ? resume_cap : 0);
         auto grown = [&](auto &buf, int64_t cap_new, int64_t used) {  // a larger copy
             std::decay_t<decltype(buf)> b((size_t)cap_new, s);
