@@ -394,10 +394,10 @@ def roofline(prof: dict, st: dict, wl: dict, workload: str, peaks: dict, dim: in
         flops = st["leaf_pairs"] * 2.0 * dim
         peak = peaks.get("bf16_tflops_sustained", 1700.0)
         ach = flops / t / 1e12
-        traffic = profile_value("k_leaf_tc", workload, "dram_bytes_per_launch")
+        traffic = profile_value("k_filter_tc", workload, "dram_bytes_per_launch")
         kp = 64 * ((((dim + 3) // 4) * 4 + 63) // 64)
         nbytes = st["leaf_rows"] * (2.0 * kp + 4.0) + st["recheck_fp32"] * 4.0 * dim
-        return {"kernel": "k_leaf_tc", "bound": "tensor", "achieved": ach, "peak": peak, "unit": "TFLOP/s",
+        return {"kernel": "k_filter_tc + k_pairs", "bound": "tensor", "achieved": ach, "peak": peak, "unit": "TFLOP/s",
                 "frac": ach / peak, "traffic": traffic,
                 "peak_note": ("measured cuBLAS bf16 sustained (MEASURED_PEAKS.json); fp16 operands run at the "
                               "same dense rate" if peaks else "fallback 1.7 PFLOP/s sustained"),
@@ -443,8 +443,9 @@ def roofline(prof: dict, st: dict, wl: dict, workload: str, peaks: dict, dim: in
                 "traffic": profile_value("k_leaf_lev_count", workload, "dram_bytes_per_launch"),
                 "peak_note": "derived: 152 SMs x 64 INT32 lanes x %.0f MHz / 2 (a 64-bit word operation is "
                              "two 32-bit ones)" % sm_max,
-                "ops_rule": "lev_columns (text characters processed x pattern words, counted by the kernel: "
-                            "pairs that stop early count what they ran) x 17 word-ops per column",
+                "ops_rule": "lev_columns (text characters processed x words, counted by the kernel: one word in the "
+                            "band form, the pattern's in the full form; pairs that stop early count what "
+                            "they ran) x 17 word-ops per column",
                 "full_recurrence_ops_per_launch": st["leaf_pairs"] * 17.0 * math.ceil(mean_len / 64.0) * mean_len,
                 "ops_per_launch": ops, "ms_per_launch": t * 1e3, "dominant_stage": dom}
     return None

@@ -98,7 +98,10 @@ typedef struct {
  *                     ct_autotune measured fastest for its row length (before
  *                     tuning: tensor-core tiles from 32 floats per row up).
  *                 All give the same edge set and distances.
- *  use_predictor: 0 = two-pass count -> scan -> emit;
+ *  use_predictor: 0 = two-pass count -> scan -> emit (for L2 points the count
+ *                     pass lists its edges, 8 bytes each, within an eighth
+ *                     of the free memory, and the emit pass decides those
+ *                     again; without room it decides its blocks' pairs);
  *                 1 = one-pass emit into row capacities predicted by
  *                     `predictor` (a fitted ct_predictor on the tree's
  *                     device); entries past a row's capacity go to an
@@ -137,11 +140,12 @@ typedef struct {
 
 /* Counters of one query, read back with ct_csr_stats. */
 typedef struct {
-    int64_t traversal_evals;  /* distance evaluations in the tree walk (count pass) */
+    int64_t traversal_evals;  /* distance evaluations in the tree walk (count pass); the upper-
+                                 triangle form leaves out what lies before a group */
     int64_t leaf_pairs;       /* (query, candidate point) pairs decided (count pass) */
     int64_t guard_fp64;       /* pairs decided by the pinned FP64 sum */
     int64_t recheck_fp32;     /* pairs re-evaluated in FP32 after the tensor-core filter */
-    int64_t candidates;       /* (group, candidate leaf block) entries */
+    int64_t candidates;       /* (group, candidate leaf block) entries of the walk */
     int64_t overflow_rows;    /* learned form: rows whose degree exceeded the predicted capacity */
     int64_t kernel_launches;  /* kernels this library launched for the query */
     int64_t emit_pairs;       /* pairs evaluated again by the emit pass */
@@ -151,7 +155,8 @@ typedef struct {
                                  these, only those the fp32 error bound cannot place on one side
                                  of eps go to FP64 */
     int64_t lev_columns;      /* edit distance, count pass: text characters the bit-parallel
-                                 recurrence processed, times the pattern's 64-bit words */
+                                 recurrence processed, times its words: one where a word holds
+                                 the band of floor(eps) edits, else the pattern's 64-bit words */
 } ct_query_stats;
 
 typedef struct ct_tree ct_tree;           /* opaque, device-resident */
@@ -197,8 +202,9 @@ ct_status eps_graph_query_batched(int32_t n_clouds, const ct_tree *const *trees,
  * chunk of groups into a device work queue (groups in the walk order; item
  * lengths per row-length class from ct_autotune with precision 2), then
  * takes queue slots, waiting for a slot's producer with a bounded number of
- * polls -- then the scan, the emit pass (the same persistent launch over the
- * complete queue) and the row sorts (rows above 4096 entries by one radix
+ * polls -- then the scan, the emit pass (over the list of edges that the count
+ * pass left; rows above 128 floats: the same persistent launch over the complete
+ * queue) and the row sorts (rows above 4096 entries by one radix
  * sort over a capacity sized like the others).  With use_graph the run is
  * captured once into a CUDA graph and every launch replays it.  A plan's leaf
  * tiles are the FP32 ones (precision 1 is taken as 0); use_predictor orders
@@ -509,7 +515,9 @@ ct_status ct_debug_pool_used(uint64_t *bytes);
  * default.  Predicted capacities that need more are scaled down to the budget
  * (entries past a row's capacity go to the arena, rows past the arena are
  * emitted again exactly); a budget below the arena's minimum takes the
- * two-pass emit.  Errors: CT_EINVAL (bytes < 0). */
+ * two-pass emit.  A budget also bounds the lists of pairs and edges (in place
+ * of their share of the free memory): pairs are then decided in waves, and
+ * edges that do not fit are found again from their blocks.  Errors: CT_EINVAL (bytes < 0). */
 ct_status ct_debug_capacity_budget(int64_t bytes);
 
 /* Thread-local message for the last non-OK status of this thread. */

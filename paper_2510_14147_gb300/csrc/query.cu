@@ -1,21 +1,22 @@
 // query.cu -- the batched ε query (Algorithm 3 with the batching of Sec. IV-B)
-// as a two-pass count -> scan -> emit pipeline, plus the CSR row sort.
+// as a count -> scan -> emit pipeline, plus the CSR row sort.
 //
-// Query groups are the tree's leaf blocks (<= zeta points, contiguous in tree
-// order, centre c_g, radius r_g).  Stages:
+// Query groups are runs of sibling leaf blocks (at most 32 points, contiguous
+// in tree order, centre c_g, radius r_g).  Stages:
 //   1. traversal (k_traverse_*): one warp per group walks the tree from the
 //      root with a stack of sibling ranges; 32 vertices are tested at a time,
 //      one per lane.  A vertex v survives iff d(c_g, v) <= r(v) + eps + r_g
 //      (every query q of the group has d(q, c_g) <= r_g, so no descendant of a
 //      pruned v is within eps of any q: triangle inequality).  Survivors are
 //      compacted with ballots: leaf blocks are candidates, internal vertices
-//      push their child range.  Run twice: count, then fill a CSR of
-//      candidates per group.
-//   2. leaf tiles (k_leaf_*): one CTA per group evaluates every (query,
-//      candidate point) pair and decides d(q, p) <= eps exactly (see QParams).
-//      Count pass: per-query degree, and a flag on every candidate block that
-//      produced an edge.  Emit pass: flagged blocks only; writes col/dist at
-//      the row offsets.
+//      push their child range.  One pass into a pool that grows when it runs
+//      out, then one range of candidates per group.
+//   2. leaf stage: slices of a group's candidates (work items) decide d(q, p) <=
+//      eps exactly (see QParams) for every (query, candidate point) pair.  Count
+//      pass: per-query degrees and, for L2 points, a list of the edges (or, from
+//      the tensor-core filter, of the pairs that may be edges); the learned form
+//      places the edges right away.  Emit pass: the list's entries, or the
+//      blocks flagged by the count pass; writes col/dist at the row offsets.
 //   3. scan of degrees to row_ptr (int64), then a per-row sort by column.
 #include <cfloat>
 #include <climits>
