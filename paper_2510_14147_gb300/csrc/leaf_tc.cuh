@@ -17,8 +17,8 @@
 // 16 warps to hide it, and a tile without any cost 2500.  As two kernels each
 // has its own bound: the filter the 16-byte copies of its operands and the
 // issue slots of its epilogue, the decisions the L1 reads of both rows.
-// Count stage, 1M x 128 at 70 / 500 neighbours: 27.5 / 78.0 -> 10.9 / 30.5 ms;
-// two-pass count + emit of 20 clouds (3 to 64 floats per row): 35.8 -> 9.5 ms.
+// Count stage, 1M x 128 at 70 / 500 neighbours: 27.5 / 78.0 -> 10.8 / 28.7 ms;
+// two-pass count + emit of 20 clouds (3 to 64 floats per row): 35.8 -> 10.3 ms.
 
 constexpr int TC_ROWS = 128;
 constexpr int TC_NB = kItemTC;            // candidate blocks of one item

@@ -450,7 +450,9 @@ __device__ __forceinline__ void group_visits(int32_t *gvisit, int g, unsigned lo
 // 16-byte pieces.  The TPD rounds' partial sums are reduced together -- each
 // exchange halves the sums a lane holds, 7 shuffles instead of 8 x 4 at 8 lanes
 // a vertex -- and lane i gets vertex i's squared distance.  Keep v unless
-// d > (r(v) + eps + r_g)(1 + 2^-10).
+// d > (r(v) + eps + r_g)(1 + 2^-10).  Bound by the latency of a step's loads
+// (L2 hits) and its issue slots: walk of 1M x 128 6.85 -> 6.4 ms with the packed
+// arithmetic and the joint reduction.
 template <int TPD>
 __device__ __forceinline__ bool l2_keep(const TreeView &tv, const float4 *cen, int nq4, int vid, int take,
                                         float add) {
