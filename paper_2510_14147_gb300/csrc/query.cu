@@ -28,6 +28,7 @@
 #include "lev.cuh"
 #include "profile.cuh"
 #include "query.cuh"
+#include "reserve.cuh"
 #include "tc.cuh"
 #include "l2dist.cuh"
 
@@ -154,7 +155,7 @@ constexpr int POOL_STOPPED = 1;
 // (global group, first vertex, count, -) that the next round walks.
 struct Spill {
     int4 *items;
-    int32_t *count;  // may exceed cap: ranges past cap were not stored
+    int32_t *count;  // never above cap (list_reserve)
     int cap;
     int limit;       // steps before a walk stops
 };
@@ -340,9 +341,11 @@ __device__ __forceinline__ int walk_group(const TreeView &tv, int2 *__restrict__
                 for (int i = lane; i < top; i += 32) total += (stack[i].y + piece - 1) / piece;
                 total = (int)__reduce_add_sync(0xffffffffu, (unsigned)total);
                 int base = 0;
-                if (lane == 0) base = atomicAdd(sp->count, total);
+                if (lane == 0)
+                    base = list_reserve(*(volatile int32_t *)sp->count, total, sp->cap,
+                                        [&](int seen, int want) { return atomicCAS(sp->count, seen, want); });
                 base = __shfl_sync(0xffffffffu, base, 0);
-                if (base + total <= sp->cap) {
+                if (base >= 0) {
                     for (int i0 = 0; i0 < top; i0 += 32) {
                         const int2 r = i0 + lane < top ? stack[i0 + lane] : make_int2(0, 0);
                         const int c = (r.y + piece - 1) / piece;
@@ -359,10 +362,7 @@ __device__ __forceinline__ int walk_group(const TreeView &tv, int2 *__restrict__
                     }
                     break;
                 }
-                // no room: the slots reserved below the end hold empty ranges
-                // (count 0, skipped), and the walk is finished here
-                for (int i = base + lane; i < sp->cap; i += 32) sp->items[i] = make_int4(g, 0, 0, 0);
-                limit = INT_MAX;
+                limit = INT_MAX;  // no room: the walk is finished here
             }
             // resumable walks have room for every vertex of a step before it begins
             if (P.resume && pc.fill > POOL_CHUNK - 32 && !pool_more(P, g, pc)) {
@@ -531,7 +531,6 @@ __global__ void __launch_bounds__(TRAV_WARPS * 32, 8) k_traverse_l2(
         int2 start = make_int2(0, 0);
         if (in_items) {
             const int4 w = in_items[gi];
-            if (w.z == 0) continue;  // an empty range (a stop that did not fit)
             gg = w.x;
             if (w.z > 0) start = make_int2(w.y, w.z);
         } else {
@@ -603,7 +602,6 @@ __global__ void __launch_bounds__(32) k_traverse_lev(
         int2 start = make_int2(0, 0);
         if (in_items) {
             const int4 w = in_items[gi];
-            if (w.z == 0) continue;  // an empty range (a stop that did not fit)
             g = w.x;
             if (w.z > 0) start = make_int2(w.y, w.z);
         } else {
@@ -693,7 +691,6 @@ __global__ void __launch_bounds__(32) k_traverse_ham(
         int2 start = make_int2(0, 0);
         if (in_items) {
             const int4 w = in_items[gi];
-            if (w.z == 0) continue;  // an empty range (a stop that did not fit)
             g = w.x;
             if (w.z > 0) start = make_int2(w.y, w.z);
         } else {
