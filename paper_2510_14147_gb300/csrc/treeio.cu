@@ -7,6 +7,7 @@
 // 64-bit FNV-1a checksum of everything before it.  A file whose magic,
 // version, sizes or checksum do not match is rejected with CT_EINVAL.
 #include <algorithm>
+#include <climits>
 #include <cstdio>
 #include <cstring>
 #include <memory>
@@ -84,14 +85,16 @@ size_t alloc_bytes(size_t bytes) { return (bytes ? bytes : 8) + 16; }
 
 // Index ranges of a loaded tree: every vertex, leaf, group and permutation
 // entry must point inside the arrays it indexes (a file from another writer
-// must not send a kernel out of bounds).
+// must not send a kernel out of bounds).  max_group: points a group may hold
+// (k_leaf_ham keeps its queries in arrays of kGroupSize; the other leaf stages
+// take a larger group in chunks).
 __global__ void k_check_loaded(int64_t n, int N, int L, int G, const int32_t *__restrict__ perm,
                                const int32_t *__restrict__ nb, const int32_t *__restrict__ ncnt,
                                const int32_t *__restrict__ cb, const int32_t *__restrict__ cc,
                                const int32_t *__restrict__ leaf_ids, const int32_t *__restrict__ par,
                                const int32_t *__restrict__ gb, const int32_t *__restrict__ gc,
                                const int32_t *__restrict__ go, const int64_t *__restrict__ soff, int64_t sbytes,
-                               int max_len, int32_t *__restrict__ bad) {
+                               int max_len, int max_group, int32_t *__restrict__ bad) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     int b = 0;
     if (soff && i < n) {
@@ -106,7 +109,7 @@ __global__ void k_check_loaded(int64_t n, int N, int L, int G, const int32_t *__
     }
     if (i < L) b |= leaf_ids[i] < 0 || leaf_ids[i] >= N;
     if (i < G) {
-        b |= gb[i] < 0 || gc[i] < 1 || (int64_t)gb[i] + gc[i] > n;
+        b |= gb[i] < 0 || gc[i] < 1 || gc[i] > max_group || (int64_t)gb[i] + gc[i] > n;
         b |= go[i] < 0 || go[i] >= G;
     }
     if (b) atomicOr(bad, 1);
@@ -215,7 +218,7 @@ ct_tree *load_tree(const char *path, cudaStream_t s) {
         k_check_loaded<<<(unsigned)ceil_div(span, 256), 256, 0, s>>>(
             t->n, t->n_nodes, t->n_leaves, t->n_groups, t->perm, t->node_begin, t->node_count, t->child_begin,
             t->child_count, t->leaf_ids, t->parent, t->group_begin, t->group_count, t->group_order, t->soff,
-            t->sbytes, t->max_len, bad.p);
+            t->sbytes, t->max_len, ham ? kGroupSize : INT_MAX, bad.p);
         CT_COUNT_LAUNCH();
         CT_LAUNCH_CHECK();
     }
