@@ -506,6 +506,11 @@ __global__ void __launch_bounds__(BT) k_net_select_l2(const float *__restrict__ 
     }
 }
 
+// its dynamic shared memory (dp: 0 where the rows are not staged)
+constexpr size_t net_select_smem(int cands, int dp) {
+    return ((size_t)cands * cands + (dp ? (size_t)cands * (dp + 4) : 0)) * sizeof(float);
+}
+
 // Distances of a hub's centres (labels below nc) to its new batch: blocks
 // (hub, y) over the labels, TPD lanes per label.
 template <int TPD, int NV>
@@ -901,6 +906,10 @@ __global__ void __launch_bounds__(BT) k_net_select_ham(const uint32_t *__restric
     const int m = net_greedy<NET_C>(cd, n, thr, NET_M, picks, [&](int i, int j) { return (float)pd[i * NET_C + j]; });
     for (int i = threadIdx.x; i < m; i += 32) bt.pos[(size_t)hs.y * NET_M + i] = cp[picks[i]];
     if (threadIdx.x == 0) net_take(hb, h, m, false, active);
+}
+
+constexpr size_t net_select_ham_smem(int wp) {
+    return (size_t)NET_C * (wp + 4) * sizeof(uint32_t) + (size_t)NET_C * NET_C * sizeof(uint16_t);
 }
 
 __global__ void k_gather_bits(const uint32_t *__restrict__ Xb, int wp, const int32_t *__restrict__ perm, int64_t n,
@@ -1736,13 +1745,13 @@ ct_tree *build_impl(const ct_points *pts, int zeta, int root, cudaStream_t s, co
             const Chunks ch{nullptr, chunk_len, keys.p, cov.p};
             if (l2) {
                 const int cands = dp <= 32 ? NET_C : NET_C / 2, staged = dp <= 256;
-                const size_t sm = ((size_t)cands * cands + (staged ? (size_t)cands * (dp + 4) : 0)) * sizeof(float);
+                const size_t sm = net_select_smem(cands, staged ? dp : 0);
                 const size_t dsm = (size_t)mcap * dp * sizeof(float);
                 dispatch([&](auto T, auto V) {
                     auto kern = T() <= 2 ? k_net_select_l2<NET_C, T()> : k_net_select_l2<NET_C / 2, T()>;
                     if (cands == NET_C / 2) kern = k_net_select_l2<NET_C / 2, T()>;
                     if (sm > 40 * 1024)
-                        CT_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+                        allow_smem(kern, cands == NET_C ? net_select_smem(NET_C, 32) : net_select_smem(NET_C / 2, 256));
                     kern<<<(unsigned)nlist, BT, sm, s>>>(Xp.p, dp, ids.p, list, hb, coff, ch, bt, mcap, staged, active);
                     if (prune) {
                         CT_COUNT_LAUNCH();
@@ -1752,9 +1761,8 @@ ct_tree *build_impl(const ct_points *pts, int zeta, int root, cudaStream_t s, co
                 return;
             }
             if (ham) {
-                const size_t sm = (size_t)NET_C * (wp + 4) * sizeof(uint32_t) + (size_t)NET_C * NET_C * sizeof(uint16_t);
-                if (sm > 40 * 1024)
-                    CT_CHECK_CUDA(cudaFuncSetAttribute(k_net_select_ham, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+                const size_t sm = net_select_ham_smem(wp);
+                if (sm > 40 * 1024) allow_smem(k_net_select_ham, net_select_ham_smem(128));  // 4096 bits
                 k_net_select_ham<<<(unsigned)nlist, BT, sm, s>>>(Xb.p, wp, ids.p, list, hb, coff, ch, bt, active);
             } else {
                 const size_t sm = (size_t)A * W * sizeof(uint64_t);

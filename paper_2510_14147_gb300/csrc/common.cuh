@@ -100,6 +100,15 @@ inline void to_host_async(T *h, const T *d, size_t count, cudaStream_t s) {
 }
 
 int num_sms();
+
+// Allows a kernel's launches `most` bytes of dynamic shared memory: the most
+// any call asks for, not what this one needs, since calls of other threads may
+// set the limit again between here and the launch.
+template <class K>
+inline void allow_smem(K *kern, size_t most) {
+    CT_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most));
+}
+
 inline int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
 // Counts kernel launches made by the library on this thread (reported with

@@ -37,6 +37,8 @@ namespace ct {
 namespace {
 
 constexpr int TRAV_WARPS = 4;              // warps per traversal block
+constexpr size_t kTravSmemMost = TRAV_WARPS * 4096 * sizeof(float);  // the group centres at the longest rows
+constexpr size_t kLevSmemMost = 96 * 1024;                           // match masks of an edit-distance leaf block
 constexpr int LEAF_T = 128;                // threads per leaf-tile block
 constexpr int KC = 128;                    // floats per K chunk of a tile
 // padded row stride of a tile in float4 (odd: rows 8 apart share no bank), for
@@ -3108,8 +3110,7 @@ void launch_traversal(const Views &V, int64_t G, int max_dp, int max_len, bool l
     if (G == 0) return;
     if (l2) {
         const size_t tsm = (size_t)TRAV_WARPS * max_dp * sizeof(float);
-        if (tsm > 48 * 1024)
-            CT_CHECK_CUDA(cudaFuncSetAttribute(k_traverse_l2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tsm));
+        if (tsm > 48 * 1024) allow_smem(k_traverse_l2, kTravSmemMost);
         CT_CHECK_CUDA(cudaMemsetAsync(spill_cnt, 0, 2 * sizeof(int32_t), s));
         for (int r = 0; r <= TRAV_ROUNDS; ++r) {
             const int4 *in = r ? spill[(r - 1) & 1] : resumed;
@@ -3496,7 +3497,7 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
         CT_CHECK_CUDA(cudaMemcpyAsync(amap.p, hm, 256, cudaMemcpyHostToDevice, s));
         CT_CHECK_CUDA(cudaStreamSynchronize(s));
         size_t per_q = (size_t)A * W * sizeof(uint64_t);
-        qchunk = (int)std::max<size_t>(1, std::min<size_t>(32, (96 * 1024) / per_q));
+        qchunk = (int)std::max<size_t>(1, std::min<size_t>(32, kLevSmemMost / per_q));
     }
     size_t lsm = l2 || ham ? 0 : (size_t)qchunk * A * W * sizeof(uint64_t);
 
@@ -3573,8 +3574,8 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
 #define CT_LL(WW)                                                                                                      \
     case WW:                                                                                                           \
         if (lsm > 48 * 1024) {                                                                                         \
-            CT_CHECK_CUDA(cudaFuncSetAttribute(k_leaf_lev<true, WW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lsm)); \
-            CT_CHECK_CUDA(cudaFuncSetAttribute(k_leaf_lev<false, WW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lsm)); \
+            allow_smem(k_leaf_lev<true, WW>, kLevSmemMost);                                                            \
+            allow_smem(k_leaf_lev<false, WW>, kLevSmemMost);                                                           \
         }                                                                                                              \
         if (emit) k_leaf_lev<true, WW><<<(unsigned)max_items, LEAF_T, lsm, s>>>(V.tv[0], V.qp[0], amap.p, A, qchunk, items, cand_p, deg.p, row_ptr, rowcur.p, col, dist, st.p, err, cw, rowsel); \
         else k_leaf_lev<false, WW><<<(unsigned)max_items, LEAF_T, lsm, s>>>(V.tv[0], V.qp[0], amap.p, A, qchunk, items, cand_p, deg.p, row_ptr, rowcur.p, col, dist, st.p, err, cw, rowsel);    \
@@ -4436,8 +4437,7 @@ PlanImpl *plan_create(int C, const ct_tree *const *trees, const QParams *qps, in
     }
     {
         const size_t tsm = (size_t)TRAV_WARPS * p.max_dp * sizeof(float);
-        if (tsm > 48 * 1024)
-            CT_CHECK_CUDA(cudaFuncSetAttribute(k_traverse_l2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tsm));
+        if (tsm > 48 * 1024) allow_smem(k_traverse_l2, kTravSmemMost);
         sort_grids();  // row-sort attributes set outside the capture
     }
     CT_CHECK_CUDA(cudaStreamSynchronize(s));
