@@ -356,10 +356,29 @@ __device__ __forceinline__ int net_candidates(const Chunks &ch, int64_t first, i
     return total;
 }
 
+// The candidate farthest from every centre so far (lowest index among equals;
+// lane l of the warp holds candidates l, l + 32, ...), or -1: none lies beyond
+// the threshold.
+template <int C>
+__device__ __forceinline__ int net_farthest(const float (&d)[C / 32], float thr) {
+    const int lane = threadIdx.x & 31;
+    float best = d[0];
+#pragma unroll
+    for (int k = 1; k < C / 32; ++k) best = fmaxf(best, d[k]);
+    // distances are not negative: their bits order as they do
+    const unsigned top = __reduce_max_sync(0xffffffffu, __float_as_uint(best));
+    if (!(__uint_as_float(top) > thr)) return -1;
+    unsigned at = 0xffffffffu;
+#pragma unroll
+    for (int k = C / 32 - 1; k >= 0; --k)
+        if (__float_as_uint(d[k]) == top) at = (unsigned)(lane + 32 * k);
+    return (int)__reduce_min_sync(0xffffffffu, at);
+}
+
 // The picks of one warp from n <= C candidates, farthest-first: each time the
-// candidate farthest from every centre so far (lowest index among equals),
-// while it lies beyond the threshold; pd(i, j): their mutual distances.  Two
-// warp reductions and a row of pd per pick.  Returns the number of picks.
+// candidate farthest from every centre so far, while it lies beyond the
+// threshold; pd(i, j): their mutual distances.  Two warp reductions and a row
+// of pd per pick.  Returns the number of picks.
 template <int C, class Pd>
 __device__ __forceinline__ int net_greedy(const float *cd, int n, float thr, int mcap, int *picks, Pd pd) {
     const int lane = threadIdx.x & 31;
@@ -368,17 +387,8 @@ __device__ __forceinline__ int net_greedy(const float *cd, int n, float thr, int
     for (int k = 0; k < C / 32; ++k) d[k] = lane + 32 * k < n ? cd[lane + 32 * k] : 0.f;
     int m = 0;
     for (; m < mcap; ++m) {
-        float best = d[0];
-#pragma unroll
-        for (int k = 1; k < C / 32; ++k) best = fmaxf(best, d[k]);
-        // distances are not negative: their bits order as they do
-        const unsigned top = __reduce_max_sync(0xffffffffu, __float_as_uint(best));
-        if (!(__uint_as_float(top) > thr)) break;
-        unsigned at = 0xffffffffu;
-#pragma unroll
-        for (int k = C / 32 - 1; k >= 0; --k)
-            if (__float_as_uint(d[k]) == top) at = (unsigned)(lane + 32 * k);
-        const int pick = (int)__reduce_min_sync(0xffffffffu, at);
+        const int pick = net_farthest<C>(d, thr);
+        if (pick < 0) break;
         if (lane == 0) picks[m] = pick;
 #pragma unroll
         for (int k = 0; k < C / 32; ++k)
@@ -409,18 +419,75 @@ __device__ __forceinline__ void net_take(Hubs hb, int h, int m, bool flat, int32
     if (m) atomicAdd(active, 1);
 }
 
+// Picks from candidates whose rows are too long to stage: after each pick its
+// distances alone, TPD lanes per candidate, a group's candidates together (so
+// that their loads overlap).  A batch of such rows has few centres (3 at 4096
+// floats), so that m n distances are far fewer than the n^2 / 2 of all pairs:
+// build of 20000 x 4096 27.8 -> 7.8 ms (9.3 to 11.2 with a launch per centre).
+template <int C, int TPD>
+__device__ __forceinline__ int net_pick_long(const float *__restrict__ X, int dp, const int32_t *__restrict__ ids,
+                                             float *cd, const int32_t *cp, int n, float thr, int mcap, int *picks) {
+    constexpr int G = BT / TPD, U = C / G;  // groups; candidates of a group
+    __shared__ int s_pick;
+    const int lane = threadIdx.x & 31, g = threadIdx.x / TPD, j = threadIdx.x % TPD, nq = dp >> 2;
+    int m = 0;
+    for (; m < mcap; ++m) {
+        if (threadIdx.x < 32) {
+            float d[C / 32];
+#pragma unroll
+            for (int k = 0; k < C / 32; ++k) d[k] = lane + 32 * k < n ? cd[lane + 32 * k] : 0.f;
+            const int p = net_farthest<C>(d, thr);
+            if (lane == 0) s_pick = picks[m] = p;
+        }
+        __syncthreads();
+        const int p = s_pick;
+        if (p < 0) break;
+        if (m + 1 < mcap) {
+            const float4 *x = reinterpret_cast<const float4 *>(X + (size_t)ids[cp[p]] * dp);
+            const float4 *y[U];
+            float acc[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                y[u] = reinterpret_cast<const float4 *>(X + (size_t)ids[cp[min(g + u * G, n - 1)]] * dp);
+                acc[u] = 0.f;
+            }
+            for (int k = j; k < nq; k += TPD) {
+                const float4 a = __ldg(x + k);
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const float4 b = __ldg(y[u] + k);
+                    const float dx = a.x - b.x, dy = a.y - b.y, dz = a.z - b.z, dw = a.w - b.w;
+                    acc[u] = fmaf(dx, dx, acc[u]);
+                    acc[u] = fmaf(dy, dy, acc[u]);
+                    acc[u] = fmaf(dz, dz, acc[u]);
+                    acc[u] = fmaf(dw, dw, acc[u]);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+#pragma unroll
+                for (int o = TPD / 2; o > 0; o >>= 1) acc[u] += __shfl_xor_sync(0xffffffffu, acc[u], o, TPD);
+                const int c = g + u * G;
+                if (j == 0 && c < n) cd[c] = fminf(cd[c], sqrtf(acc[u]));
+            }
+        }
+        __syncthreads();  // the distances; s_pick has been read
+    }
+    return m;
+}
+
 // The next batch of a hub (one CTA per listed hub {hub, slot}): at most C
 // candidates, all their mutual distances at once (4 x 4 micro-tiles from rows
-// staged in shared memory; rows too long for it, TPD lanes per pair), then one
-// warp picks.  (Picking with a block-wide distance update per pick, two
-// barriers each, took 29 us at 121k x 16: 13 now; 15 at 100k x 64: 8.)
+// staged in shared memory), then one warp picks.  (Picking with a block-wide
+// distance update per pick, two barriers each, took 29 us at 121k x 16: 13 now;
+// 15 at 100k x 64: 8.)  Rows too long to stage: net_pick_long.
 // 128 candidates up to 32 floats per row, 64 above: the distances grow with both.
 template <int C, int TPD>
 __global__ void __launch_bounds__(BT) k_net_select_l2(const float *__restrict__ X, int dp,
                                                       const int32_t *__restrict__ ids, const int2 *__restrict__ hlist,
                                                       Hubs hb, const int64_t *__restrict__ coff, Chunks ch, Batch bt,
                                                       int mcap, int staged, int32_t *__restrict__ active) {
-    extern __shared__ float4 rows[];  // C x (nq + 1) if staged, then C x C distances
+    extern __shared__ float4 rows[];  // staged: C x (nq + 1), then C x C distances
     __shared__ float cd[C];
     __shared__ int32_t cp[C];
     __shared__ int picks[NET_M];
@@ -428,7 +495,7 @@ __global__ void __launch_bounds__(BT) k_net_select_l2(const float *__restrict__ 
     const int h = hs.x;
     if (hb.done[h]) return;
     const int b = hb.begin[h], nc = hb.nc[h], nq = dp >> 2, rs = nq + 1;
-    float *pd = reinterpret_cast<float *>(rows + (staged ? C * rs : 0));
+    float *pd = reinterpret_cast<float *>(rows + C * rs);
     const float thr = hb.thr[h];
     const int n_rep = (hb.count[h] + ch.len - 1) / ch.len * NET_KEYS;
     int covered;
@@ -478,24 +545,14 @@ __global__ void __launch_bounds__(BT) k_net_select_l2(const float *__restrict__ 
                     pd[(4 * tj + v) * C + 4 * ti + u] = dd;
                 }
         }
-    } else {
-        constexpr int G = BT / TPD;
-        const int g = threadIdx.x / TPD, j = threadIdx.x % TPD;
-        for (int q0 = 0; q0 < n * n; q0 += G) {  // the same number of steps in every group
-            const int q = min(q0 + g, n * n - 1), u = q / n, v = q - u * n;
-            if (!__any_sync(0xffffffffu, u <= v)) continue;
-            RowRegs<TPD, 0> r;
-            r.load(reinterpret_cast<const float4 *>(X + (size_t)ids[cp[u]] * dp), nq, j);
-            const float dd = sqrtf(r.sqdist(reinterpret_cast<const float4 *>(X + (size_t)ids[cp[v]] * dp), nq, j));
-            if (j == 0 && u <= v) {
-                pd[u * C + v] = dd;
-                pd[v * C + u] = dd;
-            }
-        }
+    }
+    int m;
+    if constexpr (TPD >= 16) {  // staged up to 256 floats: shorter rows have fewer lanes
+        if (!staged) m = net_pick_long<C, TPD>(X, dp, ids, cd, cp, n, thr, mcap, picks);
     }
     __syncthreads();
     if (threadIdx.x >= 32) return;
-    const int m = net_greedy<C>(cd, n, thr, mcap, picks, [&](int i, int j) { return pd[i * C + j]; });
+    if (staged) m = net_greedy<C>(cd, n, thr, mcap, picks, [&](int i, int j) { return pd[i * C + j]; });
     for (int i = threadIdx.x; i < m; i += 32) {
         bt.pos[(size_t)hs.y * NET_M + i] = cp[picks[i]];
         bt.cpos[b + nc + i] = cp[picks[i]];
@@ -506,9 +563,9 @@ __global__ void __launch_bounds__(BT) k_net_select_l2(const float *__restrict__ 
     }
 }
 
-// its dynamic shared memory (dp: 0 where the rows are not staged)
+// its dynamic shared memory where the rows are staged
 constexpr size_t net_select_smem(int cands, int dp) {
-    return ((size_t)cands * cands + (dp ? (size_t)cands * (dp + 4) : 0)) * sizeof(float);
+    return ((size_t)cands * cands + (size_t)cands * (dp + 4)) * sizeof(float);
 }
 
 // Distances of a hub's centres (labels below nc) to its new batch: blocks
@@ -1745,7 +1802,7 @@ ct_tree *build_impl(const ct_points *pts, int zeta, int root, cudaStream_t s, co
             const Chunks ch{nullptr, chunk_len, keys.p, cov.p};
             if (l2) {
                 const int cands = dp <= 32 ? NET_C : NET_C / 2, staged = dp <= 256;
-                const size_t sm = net_select_smem(cands, staged ? dp : 0);
+                const size_t sm = staged ? net_select_smem(cands, dp) : 0;
                 const size_t dsm = (size_t)mcap * dp * sizeof(float);
                 dispatch([&](auto T, auto V) {
                     auto kern = T() <= 2 ? k_net_select_l2<NET_C, T()> : k_net_select_l2<NET_C / 2, T()>;
