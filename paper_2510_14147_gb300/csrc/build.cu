@@ -606,6 +606,15 @@ __global__ void __launch_bounds__(BT) k_net_dists_l2(const float *__restrict__ X
 // threads run the recurrence on full warps.
 constexpr int LEV_P = 64;     // points per chunk
 constexpr int LEV_C = 64;     // candidates of a selection
+// Long strings of many symbols (masks above 10 KB a centre, so that 40 KB hold
+// fewer than four): a pass lasts as long as the full recurrences that follow one
+// another in it, however few centres it takes.  It takes six centres and chunks
+// of 42 points (a pair per thread), and compares them all: two recurrences, not
+// the three of a pass that prunes (update, pairs, distances to the centres so
+// far).  5000 / 20000 strings of 1000 symbols out of 256 (32 KB a centre), ms:
+// 276 / 532 with a launch per centre, 625 / - pruned with a centre per pass,
+// 148 / 490 this way.
+constexpr int LEV_WIDE_M = 6, LEV_WIDE_P = BT / LEV_WIDE_M;
 
 __global__ void k_present(const uint8_t *__restrict__ s, int64_t nbytes, int32_t *__restrict__ present) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1729,13 +1738,15 @@ ct_tree *build_impl(const ct_points *pts, int zeta, int root, cudaStream_t s, co
         while (l2 && tpd < 32 && 2 * tpd * 16 <= dp) tpd *= 2;
         const int nv = (dp / 4 + tpd - 1) / tpd;  // float4s per lane
         const int passes = tpd == 1 ? net_passes<1>() : tpd == 2 ? net_passes<2>() : net_passes<4>();
-        const int chunk_len = l2 ? passes * (BT / tpd) : ham ? BT : LEV_P;
+        const int mask_bytes = A * W * (int)sizeof(uint64_t);  // of a centre (edit distance)
+        const bool wide = lev && 40960 / mask_bytes < 4;
+        const int chunk_len = l2 ? passes * (BT / tpd) : ham ? BT : wide ? LEV_WIDE_P : LEV_P;
         // hubs of at most small_max points are split whole in one CTA each
         const int small_max = l2 && dp <= 128 ? SPLIT_SMALL : 0;
         // centres of a batch: what 48 KB of shared memory hold
         const int mcap = l2 ? std::max(1, std::min(NET_M, 12288 / std::max(dp, 1)))
-                       : lev ? std::max(1, std::min(NET_M, 40960 / (A * W * 8))) : NET_M;
-        const bool prune = lev || (l2 && dp > 16);
+                       : wide ? LEV_WIDE_M : lev ? std::min(NET_M, 40960 / mask_bytes) : NET_M;
+        const bool prune = l2 ? dp > 16 : lev && !wide;
         const Strings S{scode.p - sspan[0], pts->offsets, A};
         DBuf<int32_t> cpos(l2 || lev ? n : 1, s);
         DBuf<float> dcc(prune ? (size_t)n * NET_M : 1, s);
@@ -1786,9 +1797,9 @@ ct_tree *build_impl(const ct_points *pts, int zeta, int root, cudaStream_t s, co
 #undef CT_UH
                 }
             } else {
-                const size_t sm = (size_t)mcap * A * W * sizeof(uint64_t);
+                const size_t sm = (size_t)mcap * mask_bytes;
                 switch (W) {
-#define CT_UL(WW) case WW: k_net_update_lev<WW><<<(unsigned)nck, BT, sm, s>>>(S, ids.p, D.p, lab.p, ch, hb, bt, hslot.p, root ? 0 : 1, root); break;
+#define CT_UL(WW) case WW: if (wide) allow_smem(k_net_update_lev<WW>, (size_t)LEV_WIDE_M * 256 * WW * sizeof(uint64_t)); k_net_update_lev<WW><<<(unsigned)nck, BT, sm, s>>>(S, ids.p, D.p, lab.p, ch, hb, bt, hslot.p, prune && !root, root); break;
                     CT_UL(1) CT_UL(2) CT_UL(4) CT_UL(8) CT_UL(16)
 #undef CT_UL
                 }
@@ -1822,7 +1833,7 @@ ct_tree *build_impl(const ct_points *pts, int zeta, int root, cudaStream_t s, co
                 if (sm > 40 * 1024) allow_smem(k_net_select_ham, net_select_ham_smem(128));  // 4096 bits
                 k_net_select_ham<<<(unsigned)nlist, BT, sm, s>>>(Xb.p, wp, ids.p, list, hb, coff, ch, bt, active);
             } else {
-                const size_t sm = (size_t)A * W * sizeof(uint64_t);
+                const size_t sm = mask_bytes;
                 k_net_cands_lev<<<(unsigned)nlist, BT, 0, s>>>(list, hb, coff, ch, lc);
                 CT_COUNT_LAUNCH();
                 switch (W) {
@@ -1832,8 +1843,8 @@ ct_tree *build_impl(const ct_points *pts, int zeta, int root, cudaStream_t s, co
                 }
                 CT_COUNT_LAUNCH();
                 k_net_pick_lev<<<(unsigned)nlist, 128, 0, s>>>(list, hb, bt, lc, mcap, active);
-                CT_COUNT_LAUNCH();
-                switch (W) {
+                if (prune) CT_COUNT_LAUNCH();
+                if (prune) switch (W) {
 #define CT_DL(WW) case WW: k_net_dists_lev<WW><<<dim3((unsigned)nlist, (unsigned)mcap), 128, sm, s>>>(S, ids.p, list, hb, bt); break;
                     CT_DL(1) CT_DL(2) CT_DL(4) CT_DL(8) CT_DL(16)
 #undef CT_DL
