@@ -91,6 +91,7 @@ struct RowRegs {
                 if (k < nq) add(v[u], other[k]);
             }
         } else if (row) {
+#pragma unroll 4
             for (int k = j; k < nq; k += TPD) add(__ldg(row + k), other[k]);
         }
 #pragma unroll
@@ -150,11 +151,29 @@ struct Chunks {
     unsigned long long *keys;    // NET_KEYS per chunk: (distance, position) of a part's farthest point
     int32_t *cov;                // NET_KEYS per chunk: points of the part within the threshold
 };
-// The hub's batch: positions of its centres; their labels are nc - m ...
+// A hub's batch.  The arrays are laid out by position, so that a hub's part
+// grows with its points: it has at most as many centres.
 struct Batch {
-    int32_t *pos;     // NET_M per listed hub
-    int32_t *cpos;    // centre positions by hub label (begin + label)
-    float *dcc;       // (begin + label) x NET_M: distance of the label's centre to the batch's centres
+    int32_t *pos;     // begin + i: position of the batch's centre i (label nc - m + i)
+    int32_t *cpos;    // begin + label: position of the label's centre
+    float *dcc;       // DCC_PP floats per point, see Dcc
+};
+// Distances of a hub's labels to its batch, a row per label: 32 columns (8 to 24
+// in hubs of one to three chunks: a batch has at most NET_KEYS centres a chunk)
+// and the rows that fit 8 floats a point.  Labels past them, where more than a
+// quarter of a hub's points are centres, are not pruned.  (A row of 32 for every
+// point is as much memory as a row of 32 floats, and builds no faster.)
+constexpr int DCC_PP = NET_KEYS;
+struct Dcc {
+    float *p;
+    int rows, cols;
+    __device__ __forceinline__ Dcc(const Batch &bt, int begin, int count, int chunk_len) {
+        const int c = min(NET_M / NET_KEYS, (count + chunk_len - 1) / chunk_len);
+        p = bt.dcc + (size_t)begin * DCC_PP;
+        cols = c * NET_KEYS;
+        rows = count / c;
+    }
+    __device__ __forceinline__ float *row(int label) const { return p + (size_t)label * cols; }
 };
 
 template <int TPD>
@@ -190,7 +209,6 @@ template <int TPD, int NV, bool PRUNE>
 __global__ void __launch_bounds__(BT) k_net_update_l2(const float *__restrict__ X, int dp,
                                                       const int32_t *__restrict__ ids, float *__restrict__ D,
                                                       int32_t *__restrict__ lab, Chunks ch, Hubs hb, Batch bt,
-                                                      const int32_t *__restrict__ hslot,
                                                       unsigned long long *__restrict__ root) {
     extern __shared__ float4 cen[];  // m x nq
     constexpr int P = net_passes<TPD>(), G = BT / TPD;
@@ -200,7 +218,7 @@ __global__ void __launch_bounds__(BT) k_net_update_l2(const float *__restrict__ 
     const int hbeg = hb.begin[h], m = hb.m[h], lbl0 = hb.nc[h] - m, nq = dp >> 2;
     const int end = min(start + ch.len, hbeg + hb.count[h]);
     const float thr = hb.thr[h];
-    const int32_t *bpos = bt.pos + (size_t)hslot[h] * NET_M;
+    const int32_t *bpos = bt.pos + hbeg;
     for (int i = threadIdx.x; i < m * nq; i += BT) {
         const int c = i / nq, k = i - c * nq;
         cen[i] = __ldg(reinterpret_cast<const float4 *>(X + (size_t)ids[bpos[c]] * dp) + k);
@@ -219,11 +237,12 @@ __global__ void __launch_bounds__(BT) k_net_update_l2(const float *__restrict__ 
         mask[p] = valid && m ? 0xffffffffu >> (32 - m) : 0u;
     }
     if (PRUNE && m && !root) {
+        const Dcc dcc(bt, hbeg, hb.count[h], ch.len);
 #pragma unroll
         for (int p = 0; p < P; ++p) {
-            if (!mask[p]) continue;
+            if (!mask[p] || lb[p] >= dcc.rows) continue;
             const float lim = 2.0f * cur[p] * (1.0f + 0x1p-12f) + 0x1p-60f;
-            const float4 *row = reinterpret_cast<const float4 *>(bt.dcc + (size_t)(hbeg + lb[p]) * NET_M);
+            const float4 *row = reinterpret_cast<const float4 *>(dcc.row(lb[p]));
             unsigned near = 0u;
             for (int q = j; 4 * q < m; q += TPD) {  // entries at and past m are masked out
                 const float4 d = row[q];
@@ -423,7 +442,7 @@ __device__ __forceinline__ void net_take(Hubs hb, int h, int m, bool flat, int32
 // distances alone, TPD lanes per candidate, a group's candidates together (so
 // that their loads overlap).  A batch of such rows has few centres (3 at 4096
 // floats), so that m n distances are far fewer than the n^2 / 2 of all pairs:
-// build of 20000 x 4096 27.8 -> 7.8 ms (9.3 to 11.2 with a launch per centre).
+// build of 20000 x 4096 27.8 -> 8.1 ms (9.3 to 11.2 with a launch per centre).
 template <int C, int TPD>
 __device__ __forceinline__ int net_pick_long(const float *__restrict__ X, int dp, const int32_t *__restrict__ ids,
                                              float *cd, const int32_t *cp, int n, float thr, int mcap, int *picks) {
@@ -554,7 +573,7 @@ __global__ void __launch_bounds__(BT) k_net_select_l2(const float *__restrict__ 
     if (threadIdx.x >= 32) return;
     if (staged) m = net_greedy<C>(cd, n, thr, mcap, picks, [&](int i, int j) { return pd[i * C + j]; });
     for (int i = threadIdx.x; i < m; i += 32) {
-        bt.pos[(size_t)hs.y * NET_M + i] = cp[picks[i]];
+        bt.pos[b + i] = cp[picks[i]];
         bt.cpos[b + nc + i] = cp[picks[i]];
     }
     if (threadIdx.x == 0) {
@@ -573,15 +592,16 @@ constexpr size_t net_select_smem(int cands, int dp) {
 template <int TPD, int NV>
 __global__ void __launch_bounds__(BT) k_net_dists_l2(const float *__restrict__ X, int dp,
                                                      const int32_t *__restrict__ ids, const int2 *__restrict__ hlist,
-                                                     Hubs hb, Batch bt) {
+                                                     Hubs hb, Batch bt, int chunk_len) {
     extern __shared__ float4 cen[];  // m x nq
-    const int2 hs = hlist[blockIdx.x];
-    const int h = hs.x;
+    const int h = hlist[blockIdx.x].x;
     if (hb.done[h]) return;
-    const int b = hb.begin[h], nc = hb.nc[h], m = hb.m[h], nq = dp >> 2;
+    const int b = hb.begin[h], m = hb.m[h], nq = dp >> 2;
+    const Dcc dcc(bt, b, hb.count[h], chunk_len);
+    const int nc = min(hb.nc[h], dcc.rows);
     constexpr int G = BT / TPD;
     if ((int)blockIdx.y * G >= nc) return;
-    const int32_t *bpos = bt.pos + (size_t)hs.y * NET_M;
+    const int32_t *bpos = bt.pos + b;
     for (int i = threadIdx.x; i < m * nq; i += BT) {
         const int c = i / nq, k = i - c * nq;
         cen[i] = __ldg(reinterpret_cast<const float4 *>(X + (size_t)ids[bpos[c]] * dp) + k);
@@ -592,7 +612,7 @@ __global__ void __launch_bounds__(BT) k_net_dists_l2(const float *__restrict__ X
         const int L = L0 + g;
         RowRegs<TPD, NV> r;
         r.load(reinterpret_cast<const float4 *>(X + (size_t)ids[bt.cpos[b + min(L, nc - 1)]] * dp), nq, j);
-        float *out = bt.dcc + (size_t)(b + L) * NET_M;
+        float *out = dcc.row(L);
         for (int i = 0; i < m; ++i) {
             const float s = r.sqdist(cen + i * nq, nq, j);
             if (L < nc && j == 0) out[i] = sqrtf(s);
@@ -661,7 +681,7 @@ __device__ __forceinline__ void lev_masks(uint64_t *peq, const uint8_t *pat, int
 template <int W>
 __global__ void __launch_bounds__(BT) k_net_update_lev(Strings S, const int32_t *__restrict__ ids,
                                                        float *__restrict__ D, int32_t *__restrict__ lab, Chunks ch,
-                                                       Hubs hb, Batch bt, const int32_t *__restrict__ hslot, int prune,
+                                                       Hubs hb, Batch bt, int prune,
                                                        unsigned long long *__restrict__ root) {
     extern __shared__ uint64_t speq[];  // m x A x W
     __shared__ int sd[LEV_P], sid[LEV_P], clen[NET_M];
@@ -673,7 +693,7 @@ __global__ void __launch_bounds__(BT) k_net_update_lev(Strings S, const int32_t 
     if (hb.done[h]) return;
     const int hbeg = hb.begin[h], m = hb.m[h], lbl0 = hb.nc[h] - m;
     const int np = min(ch.len, hbeg + hb.count[h] - start);
-    const int32_t *bpos = bt.pos + (size_t)hslot[h] * NET_M;
+    const int32_t *bpos = bt.pos + hbeg;
     const int t = threadIdx.x;
     for (int i = t; i < m * S.A * W; i += BT) speq[i] = 0ull;
     float cur = 0.f;
@@ -697,11 +717,14 @@ __global__ void __launch_bounds__(BT) k_net_update_lev(Strings S, const int32_t 
             atomicOr((unsigned long long *)&speq[((size_t)c * S.A + pat[i]) * W + (i >> 6)], 1ull << (i & 63));
     }
     // the pairs left by the triangle inequality: d(c, p) >= d(c, centre of p) - D(p)
+    const Dcc dcc(bt, hbeg, hb.count[h], ch.len);
     for (int i0 = 0; i0 < m * LEV_P; i0 += BT) {
         const int i = i0 + t, c = i / LEV_P, p = i % LEV_P;
         bool keep = c < m && p < np;
-        if (keep && prune)
-            keep = bt.dcc[(size_t)(hbeg + lab[start + p]) * NET_M + c] < 2.0f * (float)sd[p];
+        if (keep && prune) {
+            const int L = lab[start + p];
+            keep = L >= dcc.rows || dcc.row(L)[c] < 2.0f * (float)sd[p];
+        }
         const unsigned bal = __ballot_sync(0xffffffffu, keep);
         int base = 0;
         if ((t & 31) == 0 && bal) base = atomicAdd(&s_n, __popc(bal));
@@ -748,12 +771,22 @@ __global__ void __launch_bounds__(BT) k_net_update_lev(Strings S, const int32_t 
 // Selection in three launches: the candidates, all their mutual distances
 // (one block per candidate: a distance takes tens of microseconds, so they
 // are not left to the picks' chain), and the picks.
+// Laid out by position, as the batches.
 struct LevCands {
     int32_t *n;          // per listed hub
-    float *d;            // LEV_C per listed hub
+    float *d;            // begin + i
     int32_t *pos;
-    uint16_t *pair;      // LEV_C x LEV_C per listed hub
+    uint16_t *pair;      // LEV_PAIR_PP per point: K x K, K = lev_most_cands
 };
+// Candidates of a hub at most: its chunks' reports (one per eight points, or
+// part of eight, of a chunk).  K^2 <= 10 count for chunks of 64 and 42 points.
+// (64 x 64 pairs for every hub took 8 KB a hub, and with a leaf size of 1 there
+// is a hub for every few strings.)
+constexpr int LEV_PAIR_PP = 10;
+__device__ __forceinline__ int lev_most_cands(int count, int chunk_len) {
+    constexpr int pts = LEV_P / NET_KEYS;  // of a report
+    return min(min(count, LEV_C), (count + chunk_len - 1) / chunk_len * ((chunk_len + pts - 1) / pts));
+}
 __global__ void __launch_bounds__(BT) k_net_cands_lev(const int2 *__restrict__ hlist, Hubs hb,
                                                       const int64_t *__restrict__ coff, Chunks ch, LevCands lc) {
     __shared__ float cd[LEV_C];
@@ -764,52 +797,52 @@ __global__ void __launch_bounds__(BT) k_net_cands_lev(const int2 *__restrict__ h
     int covered;
     const int n = net_candidates<LEV_C>(ch, coff[hs.y] * NET_KEYS, n_rep, hb.thr[hs.x], cd, cp, &covered);
     if (threadIdx.x < n) {
-        lc.d[(size_t)blockIdx.x * LEV_C + threadIdx.x] = cd[threadIdx.x];
-        lc.pos[(size_t)blockIdx.x * LEV_C + threadIdx.x] = cp[threadIdx.x];
+        lc.d[hb.begin[hs.x] + threadIdx.x] = cd[threadIdx.x];
+        lc.pos[hb.begin[hs.x] + threadIdx.x] = cp[threadIdx.x];
     }
     if (threadIdx.x == 0) lc.n[blockIdx.x] = n;
 }
 template <int W>
 __global__ void __launch_bounds__(LEV_C) k_net_pairs_lev(Strings S, const int32_t *__restrict__ ids,
-                                                         const int2 *__restrict__ hlist, Hubs hb, LevCands lc) {
+                                                         const int2 *__restrict__ hlist, Hubs hb, LevCands lc,
+                                                         int chunk_len) {
     extern __shared__ uint64_t speq[];  // A x W
-    const int i = blockIdx.x, a = blockIdx.y, t = threadIdx.x;
-    if (hb.done[hlist[i].x]) return;
-    const int n = lc.n[i];
+    const int i = blockIdx.x, a = blockIdx.y, t = threadIdx.x, h = hlist[i].x;
+    if (hb.done[h]) return;
+    const int n = lc.n[i], b = hb.begin[h], K = lev_most_cands(hb.count[h], chunk_len);
     if (a >= n) return;
-    const int32_t *pos = lc.pos + (size_t)i * LEV_C;
+    const int32_t *pos = lc.pos + b;
     const int ia = ids[pos[a]];
     const int la = (int)(S.off[ia + 1] - S.off[ia]);
     lev_masks<W>(speq, S.s + S.off[ia], la, S.A);
     if (t < n && t >= a) {
         const int ib = ids[pos[t]];
         const int d = t == a ? 0 : lev_myers<W>(speq, la, S.s + S.off[ib], (int)(S.off[ib + 1] - S.off[ib]), INT_MAX / 2);
-        uint16_t *pr = lc.pair + (size_t)i * LEV_C * LEV_C;
-        pr[a * LEV_C + t] = (uint16_t)d;
-        pr[t * LEV_C + a] = (uint16_t)d;
+        uint16_t *pr = lc.pair + (size_t)b * LEV_PAIR_PP;
+        pr[a * K + t] = (uint16_t)d;
+        pr[t * K + a] = (uint16_t)d;
     }
 }
 __global__ void __launch_bounds__(128) k_net_pick_lev(const int2 *__restrict__ hlist, Hubs hb, Batch bt, LevCands lc,
-                                                      int mcap, int32_t *__restrict__ active) {
+                                                      int mcap, int chunk_len, int32_t *__restrict__ active) {
     __shared__ float cd[LEV_C];
     __shared__ uint16_t pd[LEV_C * LEV_C];
     __shared__ int picks[NET_M];
     const int2 hs = hlist[blockIdx.x];
     const int h = hs.x;
     if (hb.done[h]) return;
-    const int n = lc.n[blockIdx.x], b = hb.begin[h], nc = hb.nc[h];
-    const size_t o = (size_t)blockIdx.x * LEV_C;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) cd[i] = lc.d[o + i];
-    for (int i = threadIdx.x; i < n * LEV_C / 2; i += blockDim.x)  // rows below n (entries at and past n are not read)
-        reinterpret_cast<uint32_t *>(pd)[i] = reinterpret_cast<const uint32_t *>(lc.pair + o * LEV_C)[i];
+    const int n = lc.n[blockIdx.x], b = hb.begin[h], nc = hb.nc[h], K = lev_most_cands(hb.count[h], chunk_len);
+    for (int i = threadIdx.x; i < n; i += blockDim.x) cd[i] = lc.d[b + i];
+    for (int i = threadIdx.x; i < n * K; i += blockDim.x)  // rows below n (entries at and past n are not read)
+        pd[i] = lc.pair[(size_t)b * LEV_PAIR_PP + i];
     __syncthreads();
     if (threadIdx.x >= 32) return;
     const int m = n ? net_greedy<LEV_C>(cd, n, hb.thr[h], mcap, picks,
-                                        [&](int i, int j) { return (float)pd[i * LEV_C + j]; })
+                                        [&](int i, int j) { return (float)pd[i * K + j]; })
                     : 0;
     for (int i = threadIdx.x; i < m; i += 32) {
-        bt.pos[(size_t)hs.y * NET_M + i] = lc.pos[o + picks[i]];
-        bt.cpos[b + nc + i] = lc.pos[o + picks[i]];
+        bt.pos[b + i] = lc.pos[b + picks[i]];
+        bt.cpos[b + nc + i] = lc.pos[b + picks[i]];
     }
     if (threadIdx.x == 0) {
         if (nc == 1) bt.cpos[b] = b;  // label 0: the hub's own centre
@@ -819,18 +852,20 @@ __global__ void __launch_bounds__(128) k_net_pick_lev(const int2 *__restrict__ h
 // Distances of a hub's centres to its new batch: block (hub, batch centre).
 template <int W>
 __global__ void __launch_bounds__(128) k_net_dists_lev(Strings S, const int32_t *__restrict__ ids,
-                                                       const int2 *__restrict__ hlist, Hubs hb, Batch bt) {
+                                                       const int2 *__restrict__ hlist, Hubs hb, Batch bt,
+                                                       int chunk_len) {
     extern __shared__ uint64_t speq[];  // A x W
-    const int2 hs = hlist[blockIdx.x];
-    const int h = hs.x, c = blockIdx.y;
+    const int h = hlist[blockIdx.x].x, c = blockIdx.y;
     if (hb.done[h] || c >= hb.m[h]) return;
-    const int b = hb.begin[h], nc = hb.nc[h];
-    const int id = ids[bt.pos[(size_t)hs.y * NET_M + c]];
+    const int b = hb.begin[h];
+    const Dcc dcc(bt, b, hb.count[h], chunk_len);
+    const int nc = min(hb.nc[h], dcc.rows);
+    const int id = ids[bt.pos[b + c]];
     const int m = (int)(S.off[id + 1] - S.off[id]);
     lev_masks<W>(speq, S.s + S.off[id], m, S.A);
     for (int L = threadIdx.x; L < nc; L += blockDim.x) {
         const int il = ids[bt.cpos[b + L]];
-        bt.dcc[(size_t)(b + L) * NET_M + c] =
+        dcc.row(L)[c] =
             (float)lev_myers<W>(speq, m, S.s + S.off[il], (int)(S.off[il + 1] - S.off[il]), INT_MAX / 2);
     }
 }
@@ -872,7 +907,6 @@ template <int NQ>
 __global__ void __launch_bounds__(BT) k_net_update_ham(const uint32_t *__restrict__ X, int wp,
                                                        const int32_t *__restrict__ ids, float *__restrict__ D,
                                                        int32_t *__restrict__ lab, Chunks ch, Hubs hb, Batch bt,
-                                                       const int32_t *__restrict__ hslot,
                                                        unsigned long long *__restrict__ root) {
     extern __shared__ uint4 hcen[];  // m x nq
     const int4 ck = ch.list[blockIdx.x];
@@ -880,7 +914,7 @@ __global__ void __launch_bounds__(BT) k_net_update_ham(const uint32_t *__restric
     if (hb.done[h]) return;
     const int hbeg = hb.begin[h], m = hb.m[h], lbl0 = hb.nc[h] - m, nq = NQ ? NQ : wp >> 2;
     const int end = min(start + ch.len, hbeg + hb.count[h]);
-    const int32_t *bpos = bt.pos + (size_t)hslot[h] * NET_M;
+    const int32_t *bpos = bt.pos + hbeg;
     for (int i = threadIdx.x; i < m * nq; i += BT) {
         const int c = i / nq, k = i - c * nq;
         hcen[i] = reinterpret_cast<const uint4 *>(X + (size_t)ids[bpos[c]] * wp)[k];
@@ -943,7 +977,7 @@ __global__ void __launch_bounds__(BT) k_net_select_ham(const uint32_t *__restric
     const int2 hs = hlist[blockIdx.x];
     const int h = hs.x;
     if (hb.done[h]) return;
-    const int nc = hb.nc[h], nq = wp >> 2;
+    const int b = hb.begin[h], nc = hb.nc[h], nq = wp >> 2;
     const float thr = hb.thr[h];
     const int n_rep = (hb.count[h] + ch.len - 1) / ch.len * NET_KEYS;
     int covered;
@@ -970,7 +1004,7 @@ __global__ void __launch_bounds__(BT) k_net_select_ham(const uint32_t *__restric
     __syncthreads();
     if (threadIdx.x >= 32) return;
     const int m = net_greedy<NET_C>(cd, n, thr, NET_M, picks, [&](int i, int j) { return (float)pd[i * NET_C + j]; });
-    for (int i = threadIdx.x; i < m; i += 32) bt.pos[(size_t)hs.y * NET_M + i] = cp[picks[i]];
+    for (int i = threadIdx.x; i < m; i += 32) bt.pos[b + i] = cp[picks[i]];
     if (threadIdx.x == 0) net_take(hb, h, m, false, active);
 }
 
@@ -1002,14 +1036,12 @@ __global__ void k_group_radius_ham(int ng, const int32_t *__restrict__ gbeg, con
     if (lane == 0) grad[g] = (float)r;
 }
 
-// Chunks per listed hub, and the listed hubs' slots (their index in the list).
+// Chunks per listed hub.
 __global__ void k_chunk_counts(int nl, const int2 *__restrict__ hlist, const int32_t *__restrict__ count,
-                               int chunk_len, int32_t *__restrict__ out, int32_t *__restrict__ hslot) {
+                               int chunk_len, int32_t *__restrict__ out) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= nl) return;
-    const int h = hlist[i].x;
-    out[i] = (count[h] + chunk_len - 1) / chunk_len;
-    hslot[h] = i;
+    out[i] = (count[hlist[i].x] + chunk_len - 1) / chunk_len;
 }
 
 // The whole split of one small hub (at most SPLIT_SMALL points) in one CTA,
@@ -1382,7 +1414,7 @@ __global__ void k_root_hubs(int R, const int32_t *__restrict__ rbegin, const int
     hb.done[c] = 0;
     hb.thr[c] = 0.0f;
     hb.key[c] = 0ull;
-    bpos[(size_t)c * NET_M] = rbegin[c];
+    bpos[rbegin[c]] = rbegin[c];
     hlist[c] = make_int2(c, c);
 }
 
@@ -1749,16 +1781,16 @@ ct_tree *build_impl(const ct_points *pts, int zeta, int root, cudaStream_t s, co
         const bool prune = l2 ? dp > 16 : lev && !wide;
         const Strings S{scode.p - sspan[0], pts->offsets, A};
         DBuf<int32_t> cpos(l2 || lev ? n : 1, s);
-        DBuf<float> dcc(prune ? (size_t)n * NET_M : 1, s);
-        DBuf<int32_t> hslot(cap_h + 1, s), bpos(NET_M, s);
+        DBuf<float> dcc(prune ? (size_t)n * DCC_PP : 1, s);
+        DBuf<int32_t> bpos(n, s);
         DBuf<int4> chunks_a, chunks_b;
         DBuf<int2> hl_a(cap_h + 1, s), hl_b(cap_h + 1, s);
         DBuf<unsigned long long> keys;
         DBuf<int32_t> cov;
-        LevCands lc{};
-        DBuf<int32_t> lcn, lcpos;
-        DBuf<float> lcd;
-        DBuf<uint16_t> lcpair;
+        DBuf<int32_t> lcn, lcpos(lev ? n : 0, s);
+        DBuf<float> lcd(lev ? n : 0, s);
+        DBuf<uint16_t> lcpair(lev ? (size_t)n * LEV_PAIR_PP : 0, s);
+        LevCands lc{nullptr, lcd.p, lcpos.p, lcpair.p};
         auto dispatch = [&](auto f) {  // f(lanes per distance, float4s per lane) as compile-time constants
 #define CT_TN(T, V) f(std::integral_constant<int, T>(), std::integral_constant<int, V>())
 #define CT_T48(T) case T: if (nv <= 4) CT_TN(T, 4); else CT_TN(T, 8); break;
@@ -1779,16 +1811,16 @@ ct_tree *build_impl(const ct_points *pts, int zeta, int root, cudaStream_t s, co
                 const size_t sm = (size_t)mcap * dp * sizeof(float);
                 dispatch([&](auto T, auto V) {
                     if (prune)
-                        k_net_update_l2<T(), V(), true><<<(unsigned)nck, BT, sm, s>>>(Xp.p, dp, ids.p, D.p, lab.p, ch, hb, bt, hslot.p, root);
+                        k_net_update_l2<T(), V(), true><<<(unsigned)nck, BT, sm, s>>>(Xp.p, dp, ids.p, D.p, lab.p, ch, hb, bt, root);
                     else
-                        k_net_update_l2<T(), V(), false><<<(unsigned)nck, BT, sm, s>>>(Xp.p, dp, ids.p, D.p, lab.p, ch, hb, bt, hslot.p, root);
+                        k_net_update_l2<T(), V(), false><<<(unsigned)nck, BT, sm, s>>>(Xp.p, dp, ids.p, D.p, lab.p, ch, hb, bt, root);
                 });
                 return;
             }
             if (ham) {
                 const size_t sm = (size_t)NET_M * wp * sizeof(uint32_t);
                 switch (wp / 4) {
-#define CT_UH(Q) k_net_update_ham<Q><<<(unsigned)nck, BT, sm, s>>>(Xb.p, wp, ids.p, D.p, lab.p, ch, hb, bt, hslot.p, root)
+#define CT_UH(Q) k_net_update_ham<Q><<<(unsigned)nck, BT, sm, s>>>(Xb.p, wp, ids.p, D.p, lab.p, ch, hb, bt, root)
                     case 1: CT_UH(1); break;
                     case 2: CT_UH(2); break;
                     case 3: CT_UH(3); break;
@@ -1799,7 +1831,7 @@ ct_tree *build_impl(const ct_points *pts, int zeta, int root, cudaStream_t s, co
             } else {
                 const size_t sm = (size_t)mcap * mask_bytes;
                 switch (W) {
-#define CT_UL(WW) case WW: if (wide) allow_smem(k_net_update_lev<WW>, (size_t)LEV_WIDE_M * 256 * WW * sizeof(uint64_t)); k_net_update_lev<WW><<<(unsigned)nck, BT, sm, s>>>(S, ids.p, D.p, lab.p, ch, hb, bt, hslot.p, prune && !root, root); break;
+#define CT_UL(WW) case WW: if (wide) allow_smem(k_net_update_lev<WW>, (size_t)LEV_WIDE_M * 256 * WW * sizeof(uint64_t)); k_net_update_lev<WW><<<(unsigned)nck, BT, sm, s>>>(S, ids.p, D.p, lab.p, ch, hb, bt, prune && !root, root); break;
                     CT_UL(1) CT_UL(2) CT_UL(4) CT_UL(8) CT_UL(16)
 #undef CT_UL
                 }
@@ -1823,7 +1855,7 @@ ct_tree *build_impl(const ct_points *pts, int zeta, int root, cudaStream_t s, co
                     kern<<<(unsigned)nlist, BT, sm, s>>>(Xp.p, dp, ids.p, list, hb, coff, ch, bt, mcap, staged, active);
                     if (prune) {
                         CT_COUNT_LAUNCH();
-                        k_net_dists_l2<T(), V()><<<dim3((unsigned)nlist, nlist >= 64 ? 4 : 32), BT, dsm, s>>>(Xp.p, dp, ids.p, list, hb, bt);
+                        k_net_dists_l2<T(), V()><<<dim3((unsigned)nlist, nlist >= 64 ? 4 : 32), BT, dsm, s>>>(Xp.p, dp, ids.p, list, hb, bt, chunk_len);
                     }
                 });
                 return;
@@ -1837,15 +1869,15 @@ ct_tree *build_impl(const ct_points *pts, int zeta, int root, cudaStream_t s, co
                 k_net_cands_lev<<<(unsigned)nlist, BT, 0, s>>>(list, hb, coff, ch, lc);
                 CT_COUNT_LAUNCH();
                 switch (W) {
-#define CT_PL(WW) case WW: k_net_pairs_lev<WW><<<dim3((unsigned)nlist, LEV_C), LEV_C, sm, s>>>(S, ids.p, list, hb, lc); break;
+#define CT_PL(WW) case WW: k_net_pairs_lev<WW><<<dim3((unsigned)nlist, LEV_C), LEV_C, sm, s>>>(S, ids.p, list, hb, lc, chunk_len); break;
                     CT_PL(1) CT_PL(2) CT_PL(4) CT_PL(8) CT_PL(16)
 #undef CT_PL
                 }
                 CT_COUNT_LAUNCH();
-                k_net_pick_lev<<<(unsigned)nlist, 128, 0, s>>>(list, hb, bt, lc, mcap, active);
+                k_net_pick_lev<<<(unsigned)nlist, 128, 0, s>>>(list, hb, bt, lc, mcap, chunk_len, active);
                 if (prune) CT_COUNT_LAUNCH();
                 if (prune) switch (W) {
-#define CT_DL(WW) case WW: k_net_dists_lev<WW><<<dim3((unsigned)nlist, (unsigned)mcap), 128, sm, s>>>(S, ids.p, list, hb, bt); break;
+#define CT_DL(WW) case WW: k_net_dists_lev<WW><<<dim3((unsigned)nlist, (unsigned)mcap), 128, sm, s>>>(S, ids.p, list, hb, bt, chunk_len); break;
                     CT_DL(1) CT_DL(2) CT_DL(4) CT_DL(8) CT_DL(16)
 #undef CT_DL
                 }
@@ -1880,13 +1912,12 @@ ct_tree *build_impl(const ct_points *pts, int zeta, int root, cudaStream_t s, co
         DBuf<int64_t> i64tmp(4, s);
         DBuf<int32_t> rhub(R0, s), rleafy(R0, s);
         DBuf<int64_t> roff(R0, s);
-        if ((int64_t)bpos.n < (int64_t)R0 * NET_M) bpos = DBuf<int32_t>((size_t)R0 * NET_M, s);
         CT_CHECK_CUDA(cudaMemsetAsync(i64tmp.p, 0, 4 * sizeof(int64_t), s));
         CT_CHECK_CUDA(cudaMemsetAsync(rleafy.p, 0, R0 * sizeof(int32_t), s));
         grow_chunks();
         k_root_hubs<<<grid_for(R0), BT, 0, s>>>(R0, rbegin.p, rcount.p, H, bpos.p, hl_a.p);
         CT_COUNT_LAUNCH();
-        k_chunk_counts<<<grid_for(R0), BT, 0, s>>>(R0, hl_a.p, H.count, chunk_len, rhub.p, hslot.p);
+        k_chunk_counts<<<grid_for(R0), BT, 0, s>>>(R0, hl_a.p, H.count, chunk_len, rhub.p);
         CT_COUNT_LAUNCH();
         exclusive_scan_i32_to_i64(rhub.p, roff.p, R0, nullptr, s);
         k_chunk_fill<<<grid_for(nchunks), BT, 0, s>>>(nchunks, R0, hl_a.p, H.begin, roff.p, chunk_len, chunks_a.p);
@@ -1929,15 +1960,9 @@ ct_tree *build_impl(const ct_points *pts, int zeta, int root, cudaStream_t s, co
                     DBuf<int32_t> ccounts(nl, s);
                     DBuf<int64_t> coff(nl, s);
                     grow_chunks();
-                    if ((int64_t)bpos.n < (int64_t)nl * NET_M) bpos = DBuf<int32_t>((size_t)nl * NET_M, s);
-                    if (lev && (int64_t)lcn.n < nl) {
-                        lcn = DBuf<int32_t>(nl, s);
-                        lcpos = DBuf<int32_t>((size_t)nl * LEV_C, s);
-                        lcd = DBuf<float>((size_t)nl * LEV_C, s);
-                        lcpair = DBuf<uint16_t>((size_t)nl * LEV_C * LEV_C, s);
-                        lc = LevCands{lcn.p, lcd.p, lcpos.p, lcpair.p};
-                    }
-                    k_chunk_counts<<<grid_for(nl), BT, 0, s>>>(nl, hl_a.p, H.count, chunk_len, ccounts.p, hslot.p);
+                    if (lev && (int64_t)lcn.n < nl) lcn = DBuf<int32_t>(nl, s);
+                    lc.n = lcn.p;
+                    k_chunk_counts<<<grid_for(nl), BT, 0, s>>>(nl, hl_a.p, H.count, chunk_len, ccounts.p);
                     CT_COUNT_LAUNCH();
                     exclusive_scan_i32_to_i64(ccounts.p, coff.p, nl, nullptr, s);
                     k_chunk_fill<<<grid_for(nchunks), BT, 0, s>>>(nchunks, nl, hl_a.p, H.begin, coff.p, chunk_len,
