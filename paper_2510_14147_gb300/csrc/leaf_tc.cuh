@@ -34,20 +34,6 @@ constexpr int FT_SCOUT = 4 * FT_PGROUPS, FT_MMA = FT_SCOUT + FT_ITEMS, FT_EPI = 
 constexpr int FT_EWARPS = 4 * FT_EGROUPS, FT_T = 32 * (FT_EPI + FT_EWARPS);
 static_assert(FT_EPI % 4 == 0, "an epilogue warp reads the tensor-memory lanes of its index mod 4");
 
-// The items of a wave, in increasing order: every FT_SAMPLE-th (the sample
-// that sizes the other waves), or part `part` of `parts` interleaved parts of
-// all items, or of those not in the sample.
-constexpr int FT_SAMPLE = 32;
-struct FtWave {
-    int sampled;  // 0: of all items; 1: the sample; 2: of the rest
-    int part, parts;
-    __host__ __device__ int64_t item(int64_t i) const {
-        if (sampled == 1) return i * FT_SAMPLE;
-        const int64_t j = i * parts + part;
-        return sampled == 2 ? j + j / (FT_SAMPLE - 1) + 1 : j;
-    }
-};
-
 struct FtItem {
     int ntiles;   // -1: no more items in this buffer
     int T, qfirst, nqr, qb, qe, cloud, rbase;
@@ -107,7 +93,7 @@ __device__ __forceinline__ bool ft_wait(FtShared &S, uint64_t *bar, uint32_t par
 // tile and SM, of which the epilogue's warps are busy 650 and the producers'
 // 800; 292 M rows of 16 floats: 6.3 ms.
 __global__ void __launch_bounds__(FT_T, 1) k_filter_tc(const __grid_constant__ Views V, Items items,
-                                                       FtWave wave, const uint32_t *__restrict__ cand, PairList out,
+                                                       ItemWave wave, const uint32_t *__restrict__ cand, PairList out,
                                                        unsigned long long *__restrict__ next,
                                                        int32_t *__restrict__ err) {
     extern __shared__ unsigned char ft_raw[];

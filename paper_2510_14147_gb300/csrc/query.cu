@@ -1028,6 +1028,20 @@ struct Items {
     const int32_t *count;  // device: number of items
 };
 
+// The items of a wave, in increasing order: every WAVE_SAMPLE-th (the sample
+// that sizes the other waves), or part `part` of `parts` interleaved parts of
+// all items, or of those not in the sample.
+constexpr int WAVE_SAMPLE = 32;
+struct ItemWave {
+    int sampled;  // 0: of all items; 1: the sample; 2: of the rest
+    int part, parts;
+    __host__ __device__ int64_t item(int64_t i) const {
+        if (sampled == 1) return i * WAVE_SAMPLE;
+        const int64_t j = i * parts + part;
+        return sampled == 2 ? j + j / (WAVE_SAMPLE - 1) + 1 : j;
+    }
+};
+
 // One-pass emit (learned form): the count pass also writes every edge into a
 // per-row capacity region sized from the predicted degree.  A row's entries
 // past its capacity go to an overflow arena as (row, slot, col, dist); once
@@ -1628,24 +1642,39 @@ __device__ __forceinline__ void leaf_l2_item(
     }
 }
 
-// One CTA per work item.  Rows of at most 64 floats take a shorter tile stride
-// and fewer registers, so that five CTAs share an SM instead of three (a tile
-// is a chain of copy, barrier, arithmetic, barrier: more of them in flight).
+// The wave's items, taken dynamically by a grid of resident CTAs (leaf_l2_ctas):
+// a warp's place in the edge list outlives an item.  (With a CTA per item every
+// warp that found an edge left up to 127 entries of its own behind: 240
+// thousand warps of 121k x 16 uniform points asked for 31 M entries to list 2.5
+// M edges, more than the list had.)
+// Rows of at most 64 floats take a shorter tile stride and fewer registers, so
+// that five CTAs share an SM instead of three (a tile is a chain of copy,
+// barrier, arithmetic, barrier: more of them in flight).
 // 174k x 64 at 87 neighbours: count 16.3 -> 14.1 ms, bound by the shared-memory
 // reads of the micro-tiles (71 % of that pipe, four wavefronts per 16-byte
 // read whatever is broadcast) and the FP32 pipe (58 %).  The emit pass reads
 // the list of edges instead of the blocks' pairs: 4.8 -> 0.8 ms.
+constexpr int leaf_l2_ctas(bool shorts) { return shorts ? 5 : 3; }  // of an SM
 template <bool EMIT, int KS4>
-__global__ void __launch_bounds__(LEAF_T, KS4 == KS_SHORT ? 5 : 3) k_leaf_l2(
-    const __grid_constant__ Views V, Items items, const uint32_t *__restrict__ cand,
+__global__ void __launch_bounds__(LEAF_T, leaf_l2_ctas(KS4 == KS_SHORT)) k_leaf_l2(
+    const __grid_constant__ Views V, Items items, ItemWave wave, unsigned long long *__restrict__ next,
+    const uint32_t *__restrict__ cand,
     uint32_t *__restrict__ emask, int32_t *__restrict__ deg, const int64_t *__restrict__ row_ptr,
     int32_t *__restrict__ rowcur, int32_t *__restrict__ col, float *__restrict__ dist,
     unsigned long long *__restrict__ st, int32_t *__restrict__ err, CapOut co, const uint8_t *__restrict__ rowsel,
     PairList pl) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ int64_t s_it;
     PairCursor pc;
-    leaf_l2_item<EMIT, KS4>(V, items, blockIdx.x, cand, emask, deg, row_ptr, rowcur, col, dist, st, err, co, rowsel,
-                            pl, pc, *reinterpret_cast<LeafShared<KS4> *>(smem_raw));
+    for (;;) {
+        __syncthreads();  // the last item is done
+        if (threadIdx.x == 0) s_it = wave.item((int64_t)atomicAdd(next, 1ull));
+        __syncthreads();
+        const int64_t it = s_it;
+        if (it >= *items.count) break;
+        leaf_l2_item<EMIT, KS4>(V, items, (int)it, cand, emask, deg, row_ptr, rowcur, col, dist, st, err, co, rowsel,
+                                pl, pc, *reinterpret_cast<LeafShared<KS4> *>(smem_raw));
+    }
     if (!EMIT && pl.e) pair_close(pl, pc);
 }
 
@@ -3522,24 +3551,13 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
         co = CapOut{lp.cap_off.p, c_fill.p, c_ent.p, o_ent.p, o_n.p, lp.arena > 0 ? lp.arena : 0, lost.p};
     }
 
-    // FP32 tiles, two-pass form: the count pass lists its edges for the emit
-    // pass (8 bytes each; dp <= 128), which then decides only those again
-    // instead of every pair of an edge-bearing block and query.  The list holds
-    // 192 edges per point, within an eighth of the free memory; past that the
-    // emit pass takes the blocks' masks.
+    // counters of the FP32 leaf launches, each used once (count: one or two; emit; rows emitted again)
+    DBuf<unsigned long long> fp_ctr(8, s);
+    if (l2) CT_CHECK_CUDA(cudaMemsetAsync(fp_ctr.p, 0, 8 * sizeof(unsigned long long), s));
+    int fp_launches = 0;
+    unsigned long long *const fp_n = fp_ctr.p + 7;  // entries of the edge list
     DBuf<uint2> fp_e;
-    DBuf<unsigned long long> fp_n(1, s);
     PairList fp_list{};
-    if (l2 && any_fp && !capmode && !probe && max_fp_dp <= 128 && n > 0) {
-        size_t fr = 0, tot = 0;
-        int64_t cap = 192 * n + (int64_t)num_sms() * 5 * 4 * L2_CHUNK;
-        if (cudaMemGetInfo(&fr, &tot) == cudaSuccess) cap = std::min(cap, (int64_t)(fr / 8 / sizeof(uint2)));
-        else cudaGetLastError();
-        if (capacity_budget() > 0) cap = std::min<int64_t>(cap, capacity_budget() / (int64_t)sizeof(uint2));
-        fp_e = DBuf<uint2>((size_t)std::max<int64_t>(cap, 1), s);
-        CT_CHECK_CUDA(cudaMemsetAsync(fp_n.p, 0, sizeof(unsigned long long), s));
-        fp_list = PairList{fp_e.p, std::max<int64_t>(cap, 1), fp_n.p, nullptr};
-    }
     bool fp_listed = false;  // the list holds every edge of the FP32 items
     unsigned long long fp_entries = 0;
 
@@ -3547,14 +3565,16 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
     DBuf<int32_t> deg(n + 1, s);
     CT_CHECK_CUDA(cudaMemsetAsync(deg.p, 0, (n + 1) * sizeof(int32_t), s));
     auto leaf = [&](bool emit, int64_t *row_ptr, int32_t *col, float *dist, const uint8_t *rowsel,
-                    const Items &items) {
+                    const Items &items, const ItemWave &wave) {
         if (G == 0 || nseg == 0) return;
         const CapOut cw = emit ? CapOut{} : co;
         if (l2) {
             leaf_l2_prepare();
             const bool sh = short_rows(max_fp_dp);
+            const int ctas = (int)std::min<int64_t>(max_items, (int64_t)num_sms() * leaf_l2_ctas(sh));
+            unsigned long long *const next = fp_ctr.p + fp_launches++;
             auto go = [&](auto kern) {
-                kern<<<(unsigned)max_items, LEAF_T, leaf_smem(sh), s>>>(V, items, cand_p, emask.p, deg.p, row_ptr, rowcur.p, col, dist, st.p, err, cw, rowsel, emit ? PairList{} : fp_list);
+                kern<<<ctas, LEAF_T, leaf_smem(sh), s>>>(V, items, wave, next, cand_p, emask.p, deg.p, row_ptr, rowcur.p, col, dist, st.p, err, cw, rowsel, emit ? PairList{} : fp_list);
             };
             if (emit && sh) go(k_leaf_l2<true, KS_SHORT>);
             else if (emit) go(k_leaf_l2<true, KS_LONG>);
@@ -3616,7 +3636,7 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
     // counted, or its wave cut in two.  The two-pass form keeps its lists for
     // the emit pass while they fit; else that filters again.
     struct Wave {
-        FtWave wave;
+        ItemWave wave;
         int64_t n;         // entries reserved
         DBuf<uint2> list;  // kept list (its first n entries), or empty
     };
@@ -3640,7 +3660,7 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
     }
     // filters a wave's items into a list of at least `want` entries (grown to
     // the need once that is known); false when the need exceeds `most`
-    auto tc_filter = [&](const FtWave &w, double want, DBuf<uint2> &list, bool stats, int64_t most) {
+    auto tc_filter = [&](const ItemWave &w, double want, DBuf<uint2> &list, bool stats, int64_t most) {
         for (;;) {
             const int64_t cap = ceil_div((int64_t)want, FT_CHUNK) * FT_CHUNK;
             if ((int64_t)list.n < cap) {
@@ -3686,18 +3706,18 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
         DBuf<uint2> list;
         // waves still to run (a stack); a wave whose list would exceed the
         // budget is cut in two interleaved halves
-        std::vector<FtWave> todo;
+        std::vector<ItemWave> todo;
         const bool sample = max_items > 32ll * num_sms();
-        todo.push_back(sample ? FtWave{1, 0, 1} : FtWave{0, 0, 1});
+        todo.push_back(sample ? ItemWave{1, 0, 1} : ItemWave{0, 0, 1});
         double want = (double)pair_slack + std::min(512.0 * (double)n, (double)(16 << 20));
         bool sampled = !sample;
         while (!todo.empty()) {
-            const FtWave w = todo.back();
+            const ItemWave w = todo.back();
             todo.pop_back();
             const bool can_cut = w.sampled != 1 && w.parts < (1 << 20);
             if (!tc_filter(w, want, list, true, can_cut ? pair_budget + pair_slack : INT64_MAX)) {
-                todo.push_back(FtWave{w.sampled, w.part + w.parts, 2 * w.parts});
-                todo.push_back(FtWave{w.sampled, w.part, 2 * w.parts});
+                todo.push_back(ItemWave{w.sampled, w.part + w.parts, 2 * w.parts});
+                todo.push_back(ItemWave{w.sampled, w.part, 2 * w.parts});
                 want = (double)(pair_budget + pair_slack);
                 continue;
             }
@@ -3712,22 +3732,41 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
             }
             if (!sampled) {  // the rest, from the sample's pairs
                 sampled = true;
-                const double total = 1.25 * (FT_SAMPLE - 1) * std::max(1.0, (double)tc_stats[1]);
+                const double total = 1.25 * (WAVE_SAMPLE - 1) * std::max(1.0, (double)tc_stats[1]);
                 const int parts = (int)std::min(65536.0, std::ceil(total / (double)pair_budget));
-                for (int k = parts - 1; k >= 0; --k) todo.push_back(FtWave{2, k, parts});
+                for (int k = parts - 1; k >= 0; --k) todo.push_back(ItemWave{2, k, parts});
                 want = total / parts + (double)pair_slack;
             }
         }
     };
-    if (!l2 || !any_tc) {
+    // Count pass of the other kernels.  FP32 tiles of the two-pass form list
+    // their edges for the emit pass (8 bytes each; dp <= 128), which then decides
+    // only those again instead of every pair of an edge-bearing block and query.
+    // The list holds 192 edges per point, within an eighth of the free memory; past
+    // that the emit pass takes the blocks' masks.
+    auto count_other = [&](const Items &items) {
         ProfScope ps("leaf_count", s);
-        leaf(false, nullptr, nullptr, nullptr, nullptr, items);
+        const ItemWave every{0, 0, 1};
+        auto count = [&](const ItemWave &w) { leaf(false, nullptr, nullptr, nullptr, nullptr, items, w); };
+        if (!l2 || capmode || probe || max_fp_dp > 128 || n == 0) return count(every);
+        // entries that the warps leave unused
+        const int64_t slack =
+            std::min<int64_t>(max_items, (int64_t)num_sms() * leaf_l2_ctas(short_rows(max_fp_dp))) * (LEAF_T / 32) * L2_CHUNK;
+        int64_t most = 192 * n + slack;
+        size_t fr = 0, tot = 0;
+        if (cudaMemGetInfo(&fr, &tot) == cudaSuccess) most = std::min(most, (int64_t)(fr / 8 / sizeof(uint2)));
+        else cudaGetLastError();
+        if (capacity_budget() > 0) most = std::min<int64_t>(most, capacity_budget() / (int64_t)sizeof(uint2));
+        most = std::max<int64_t>(most, 1);
+        fp_e = DBuf<uint2>((size_t)most, s);
+        fp_list = PairList{fp_e.p, most, fp_n, nullptr};
+        count(every);
+    };
+    if (!l2 || !any_tc) {
+        count_other(items);
     } else {
         count_tc();
-        if (any_fp) {
-            ProfScope ps("leaf_count", s);
-            leaf(false, nullptr, nullptr, nullptr, nullptr, items_fp);
-        }
+        if (any_fp) count_other(items_fp);
         if (capmode)  // the entries placed are the degrees
             for (int c = 0; c < C; ++c)
                 if (V.use_tc[c] && trees[c]->n)
@@ -3737,7 +3776,7 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
     // emit pass (rowsel: of the selected rows)
     auto emit = [&](const uint8_t *rowsel) {
         if (fp_listed) tc_pairs(PAIRS_EMIT, fp_e.p, (int64_t)fp_entries, rowsel);
-        else if (!l2 || any_fp) leaf(true, all.row_ptr, all.col, all.dist, rowsel, items_fp);
+        else if (!l2 || any_fp) leaf(true, all.row_ptr, all.col, all.dist, rowsel, items_fp, ItemWave{0, 0, 1});
         DBuf<uint2> list;
         for (auto &w : waves) {
             if (lists_kept) {
@@ -3778,7 +3817,7 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
     all.row_ptr = row_ptr;
     exclusive_scan_i32_to_i64(deg.p, row_ptr, n + 1, nullptr, s);
     int64_t nnz = 0;
-    if (fp_list.e) to_host_async(&fp_entries, fp_n.p, 1, s);
+    if (fp_list.e) to_host_async(&fp_entries, fp_n, 1, s);
     to_host(&nnz, row_ptr + n, 1, s);
     fp_listed = fp_list.e && (int64_t)fp_entries <= fp_list.cap;
     all.nnz = nnz;
@@ -4010,7 +4049,7 @@ __device__ __forceinline__ int queue_next(const Queue &Q, int32_t *err) {
 // The FP32 tiles as one persistent launch over the queue (count pass:
 // produce, then consume; emit pass: consume the complete queue again).
 template <bool EMIT, int KS4>
-__global__ void __launch_bounds__(LEAF_T, KS4 == KS_SHORT ? 5 : 3) k_leaf_l2_queue(
+__global__ void __launch_bounds__(LEAF_T, leaf_l2_ctas(KS4 == KS_SHORT)) k_leaf_l2_queue(
     const __grid_constant__ Views V, Queue Q, const uint32_t *__restrict__ cand, uint32_t *__restrict__ emask,
     int32_t *__restrict__ deg, const int64_t *__restrict__ row_ptr, int32_t *__restrict__ rowcur,
     int32_t *__restrict__ col, float *__restrict__ dist, unsigned long long *__restrict__ st,
@@ -4669,10 +4708,12 @@ void degrees_noalloc(const ct_tree *t, const QParams &qp, int32_t *degrees, cuda
         CT_COUNT_LAUNCH();
         Items items{igroup, ibeg, iend, nitems};
         leaf_l2_prepare();
+        CT_CHECK_CUDA(cudaMemsetAsync(ctr, 0, sizeof(unsigned long long), s));  // the walk's counters have been read
         auto go = [&](auto kern, bool sh) {
-            kern<<<(unsigned)max_items, LEAF_T, leaf_smem(sh), s>>>(V, items, pool, nullptr, degrees, nullptr, nullptr,
-                                                                    nullptr, nullptr, st, err, CapOut{}, nullptr,
-                                                                    PairList{});
+            const int ctas = (int)std::min<int64_t>(max_items, (int64_t)num_sms() * leaf_l2_ctas(sh));
+            kern<<<ctas, LEAF_T, leaf_smem(sh), s>>>(V, items, ItemWave{0, 0, 1}, ctr, pool, nullptr, degrees, nullptr,
+                                                     nullptr, nullptr, nullptr, st, err, CapOut{}, nullptr,
+                                                     PairList{});
         };
         if (short_rows(t->dp)) go(k_leaf_l2<false, KS_SHORT>, true);
         else go(k_leaf_l2<false, KS_LONG>, false);
