@@ -99,9 +99,10 @@ typedef struct {
  *                     tuning: tensor-core tiles from 32 floats per row up).
  *                 All give the same edge set and distances.
  *  use_predictor: 0 = two-pass count -> scan -> emit (for L2 points the count
- *                     pass lists its edges, 8 bytes each, within an eighth
- *                     of the free memory, and the emit pass decides those
- *                     again; without room it decides its blocks' pairs);
+ *                     pass lists its edges, 8 bytes each, at most 192 a
+ *                     point and an eighth of the free memory, and the emit
+ *                     pass decides those again; without room it decides its
+ *                     blocks' pairs);
  *                 1 = one-pass emit into row capacities predicted by
  *                     `predictor` (a fitted ct_predictor on the tree's
  *                     device); entries past a row's capacity go to an

@@ -3742,25 +3742,55 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
     // Count pass of the other kernels.  FP32 tiles of the two-pass form list
     // their edges for the emit pass (8 bytes each; dp <= 128), which then decides
     // only those again instead of every pair of an edge-bearing block and query.
-    // The list holds 192 edges per point, within an eighth of the free memory; past
-    // that the emit pass takes the blocks' masks.
+    // The list holds 192 edges per point at most, within an eighth of the free
+    // memory (a denser graph's emit pass takes the blocks' masks).  Where that is
+    // more than 1 GB (700 thousand points), every 32nd item is counted first and
+    // its edges size the list, with half as much again to spare; a sample of
+    // fewer points does not fill the chip (130k x 3 at 64 MB: 3.00 -> 3.19 ms).
+    // The list is no condition: without the memory for it, or when it runs out,
+    // the emit pass takes the masks.
     auto count_other = [&](const Items &items) {
         ProfScope ps("leaf_count", s);
         const ItemWave every{0, 0, 1};
         auto count = [&](const ItemWave &w) { leaf(false, nullptr, nullptr, nullptr, nullptr, items, w); };
         if (!l2 || capmode || probe || max_fp_dp > 128 || n == 0) return count(every);
-        // entries that the warps leave unused
+        // entries that the warps of two launches leave unused
         const int64_t slack =
-            std::min<int64_t>(max_items, (int64_t)num_sms() * leaf_l2_ctas(short_rows(max_fp_dp))) * (LEAF_T / 32) * L2_CHUNK;
+            2 * std::min<int64_t>(max_items, (int64_t)num_sms() * leaf_l2_ctas(short_rows(max_fp_dp))) * (LEAF_T / 32) * L2_CHUNK;
         int64_t most = 192 * n + slack;
         size_t fr = 0, tot = 0;
         if (cudaMemGetInfo(&fr, &tot) == cudaSuccess) most = std::min(most, (int64_t)(fr / 8 / sizeof(uint2)));
         else cudaGetLastError();
         if (capacity_budget() > 0) most = std::min<int64_t>(most, capacity_budget() / (int64_t)sizeof(uint2));
         most = std::max<int64_t>(most, 1);
-        fp_e = DBuf<uint2>((size_t)most, s);
-        fp_list = PairList{fp_e.p, most, fp_n, nullptr};
-        count(every);
+        auto room = [&](int64_t cap, int64_t used) {  // a list of cap entries with the first `used` of the last one
+            DBuf<uint2> e;
+            try {
+                e = DBuf<uint2>((size_t)cap, s);
+            } catch (const Error &x) {
+                if (x.st != CT_ENOMEM) throw;
+            }
+            if (e.p && used) CT_CHECK_CUDA(cudaMemcpyAsync(e.p, fp_e.p, (size_t)used * sizeof(uint2), cudaMemcpyDeviceToDevice, s));
+            fp_e = std::move(e);
+            fp_list = fp_e.p ? PairList{fp_e.p, cap, fp_n, nullptr} : PairList{};
+        };
+        if (most <= (1ll << 30) / (int64_t)sizeof(uint2)) {
+            room(most, 0);
+            return count(every);
+        }
+        room(std::min(most, 192 * n / WAVE_SAMPLE + slack), 0);
+        count(ItemWave{1, 0, 1});
+        if (fp_list.e) {
+            to_host(&fp_entries, fp_n, 1, s);
+            const int64_t used = (int64_t)fp_entries, all = WAVE_SAMPLE * used + slack;
+            if (used <= fp_list.cap && all <= most) {
+                room(std::min(most, all + all / 2), used);
+            } else {
+                fp_e.reset();
+                fp_list = PairList{};
+            }
+        }
+        count(ItemWave{2, 0, 1});
     };
     if (!l2 || !any_tc) {
         count_other(items);
@@ -4471,8 +4501,13 @@ PlanImpl *plan_create(int C, const ct_tree *const *trees, const QParams *qps, in
         }
         p.leaf_grid = std::max(1, num_sms() * std::max(per_sm, 1));
         p.pair_n = DBuf<unsigned long long>(1, s);
-        if (p.max_dp <= 128)  // the edges, and what each warp leaves of its last entries
-            p.pair_e = DBuf<uint2>((size_t)(p.nnz_cap + (int64_t)p.leaf_grid * (LEAF_T / 32) * L2_CHUNK), s);
+        if (p.max_dp <= 128) {  // the edges, and what each warp leaves of its last entries; without room, none
+            try {
+                p.pair_e = DBuf<uint2>((size_t)(p.nnz_cap + (int64_t)p.leaf_grid * (LEAF_T / 32) * L2_CHUNK), s);
+            } catch (const Error &x) {
+                if (x.st != CT_ENOMEM) throw;
+            }
+        }
     }
     {
         const size_t tsm = (size_t)TRAV_WARPS * p.max_dp * sizeof(float);

@@ -76,3 +76,19 @@ t = cg.ct_build(strings=a, leaf_size=1)
 print(a[1].numel() - 1, before - free())
 """)
     assert grown <= 800 * n + (33 << 20)
+
+
+def test_query_of_low_degree():
+    # the candidate pool (256 entries of 4 bytes a point), a copy of the candidates in use (at
+    # most a quarter of it), the walk's lists and the CSR's arrays (under 200): 1500; a list of
+    # 192 edges a point whatever the degree would add 1536
+    n, grown = _numbers("""
+cg.eps_graph_query(cg.ct_build(points=torch.rand(5000, 3, generator=g, device="cuda")), 0.01).free()
+t = cg.ct_build(points=torch.rand(2000000, 3, generator=g, device="cuda"))
+torch.cuda.empty_cache()
+before = free()
+c = cg.eps_graph_query(t, 0.008)
+assert c.stats()["emit_pairs"] == c.nnz and 2 < c.nnz / 2e6 < 8
+print(2000000, before - free())
+""")
+    assert grown <= 1500 * n + (200 << 20)
