@@ -517,8 +517,10 @@ ct_status ct_debug_pool_used(uint64_t *bytes);
  * (entries past a row's capacity go to the arena, rows past the arena are
  * emitted again exactly); a budget below the arena's minimum takes the
  * two-pass emit.  A budget also bounds the lists of pairs and edges (in place
- * of their share of the free memory): pairs are then decided in waves, and
- * edges that do not fit are found again from their blocks.  Errors: CT_EINVAL (bytes < 0). */
+ * of their share of the free memory; beyond it, a list of pairs has the 15 MB
+ * that the filter's warps may leave unused): pairs are then decided in waves,
+ * and edges that do not fit are found again from their blocks.  Errors:
+ * CT_EINVAL (bytes < 0). */
 ct_status ct_debug_capacity_budget(int64_t bytes);
 
 /* Thread-local message for the last non-OK status of this thread. */

@@ -1028,16 +1028,16 @@ struct Items {
     const int32_t *count;  // device: number of items
 };
 
-// The items of a wave, in increasing order: every WAVE_SAMPLE-th (the sample
-// that sizes the other waves), or part `part` of `parts` interleaved parts of
-// all items, or of those not in the sample.
+// The items of a wave, in increasing order: part `part` of `parts` interleaved
+// parts of all items, of every WAVE_SAMPLE-th (the sample that sizes the other
+// waves), or of those not in the sample.
 constexpr int WAVE_SAMPLE = 32;
 struct ItemWave {
     int sampled;  // 0: of all items; 1: the sample; 2: of the rest
     int part, parts;
     __host__ __device__ int64_t item(int64_t i) const {
-        if (sampled == 1) return i * WAVE_SAMPLE;
         const int64_t j = i * parts + part;
+        if (sampled == 1) return j * WAVE_SAMPLE;
         return sampled == 2 ? j + j / (WAVE_SAMPLE - 1) + 1 : j;
     }
 };
@@ -3709,28 +3709,29 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
         std::vector<ItemWave> todo;
         const bool sample = max_items > 32ll * num_sms();
         todo.push_back(sample ? ItemWave{1, 0, 1} : ItemWave{0, 0, 1});
-        double want = (double)pair_slack + std::min(512.0 * (double)n, (double)(16 << 20));
+        const int64_t most = pair_budget + pair_slack;
+        double want = std::min((double)most, (double)pair_slack + std::min(512.0 * (double)n, (double)(16 << 20)));
         bool sampled = !sample;
         while (!todo.empty()) {
             const ItemWave w = todo.back();
             todo.pop_back();
-            const bool can_cut = w.sampled != 1 && w.parts < (1 << 20);
-            if (!tc_filter(w, want, list, true, can_cut ? pair_budget + pair_slack : INT64_MAX)) {
+            const bool can_cut = w.parts < (1 << 20);
+            if (!tc_filter(w, want, list, true, can_cut ? most : INT64_MAX)) {
                 todo.push_back(ItemWave{w.sampled, w.part + w.parts, 2 * w.parts});
                 todo.push_back(ItemWave{w.sampled, w.part, 2 * w.parts});
-                want = (double)(pair_budget + pair_slack);
+                want = (double)most;
                 continue;
             }
             tc_pairs(capmode ? PAIRS_PLACE : PAIRS_COUNT, list.p, filtered, nullptr);
             waves.push_back(Wave{w, filtered, DBuf<uint2>()});
             kept_entries += filtered;
-            if (lists_kept && kept_entries <= pair_budget + pair_slack) {
+            if (lists_kept && kept_entries <= most) {
                 waves.back().list = std::move(list);
             } else if (lists_kept) {
                 lists_kept = false;
                 for (auto &x : waves) x.list.reset();
             }
-            if (!sampled) {  // the rest, from the sample's pairs
+            if (!sampled && todo.empty()) {  // the rest, from the sample's pairs
                 sampled = true;
                 const double total = 1.25 * (WAVE_SAMPLE - 1) * std::max(1.0, (double)tc_stats[1]);
                 const int parts = (int)std::min(65536.0, std::ceil(total / (double)pair_budget));
