@@ -3366,7 +3366,7 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
     int32_t *gvisit = probe ? probe->gvisit : nullptr;
 
     const int W = l2 || ham ? 1 : lev_words_for(t->max_len);
-    // 1. traversal: one pass into the candidate pool (rerun once if it overflows)
+    // 1. traversal into the candidate pool, which grows when it runs out
     const int cap = 32 * (max_depth + 2);
     TravLaunch tl = trav_launch_config(l2, G);
     DBuf<int2> stacks((size_t)tl.warps * cap, s);
@@ -3380,7 +3380,10 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
     DBuf<longlong2> cursors(tl.warps, s);
     // a pool of whole chunks; work left when it runs out goes to a resume list
     // (at most every group, a full spill buffer a round and the stacks of the
-    // warps; a list that is too short restarts the pass with a larger pool)
+    // warps; a list that is too short restarts the walk with a larger pool).
+    // Every pass at least doubles the pool while half of the free memory allows
+    // it; passes that go on and those that restart are counted together.
+    constexpr int kPoolPasses = 16;
     int64_t pool_cap = ceil_div(pool_capacity_guess(n, G, tl), POOL_CHUNK) * POOL_CHUNK;
     const int resume_cap = (int)std::min<int64_t>(G + 2LL * spill_cap + 65536, 1 << 26);
     DBuf<uint32_t> pool;
@@ -3391,7 +3394,7 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
     unsigned long long hc[4] = {0, 0, 0, 0};
     int64_t seg_cap = 0;
     Pool P{};
-    for (int pass = 0;; ++pass) {
+    for (int pass = 0, passes = 1;; ++pass, ++passes) {
         // a segment per walk (groups, stored ranges) and per chunk a walk crosses
         const int64_t old_seg = seg_cap, nseg0 = pass ? (int64_t)(uint32_t)hc[1] : 0;
         seg_cap = old_seg + G + (int64_t)(l2 || ham ? TRAV_ROUNDS : TRAV_ROUNDS_LEV) * spill_cap + pool_cap / POOL_CHUNK + tl.warps + 16 +
@@ -3421,7 +3424,7 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
         to_host(hc, ctr.p, 4, s);
         const uint32_t full = (uint32_t)hc[3];
         if (!full) break;
-        if (pass >= 16) CT_FAIL(CT_ECUDA, "the candidate pool overflowed %d times", pass);
+        if (passes > kPoolPasses) CT_FAIL(CT_ECUDA, "the candidate pool overflowed %d times", passes);
         // the size the walked groups ask for (the longest walks come first), at
         // least double, within half of the free memory if that is still larger
         int32_t whole = 0;
