@@ -530,7 +530,7 @@ __global__ void __launch_bounds__(256, 4) k_pairs(const __grid_constant__ Views 
     __shared__ PairShared shared[8];  // one per warp
     PairShared &sh = shared[threadIdx.x >> 5];
     unsigned long long guard = 0, band = 0;
-    uint32_t done = 0;
+    uint32_t done = 0;  // emit: pairs decided; one-pass: entries of the edges found
     for (int64_t base = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32; base < total;
          base += warps * 32) {
         const uint2 e = base + lane < total ? list.e[base + lane] : make_uint2(PAIR_NONE, 0u);
@@ -622,7 +622,7 @@ __global__ void __launch_bounds__(256, 4) k_pairs(const __grid_constant__ Views 
         }
         if (!valid) continue;
         const QParams &qp = V.qp[c];
-        if (MODE != PAIRS_COUNT) ++done;
+        if (MODE == PAIRS_EMIT) ++done;
         const int edge = decide32(qp, sv, band);
         bool is_edge = edge > 0;
         float d = sqrtf(sv);
@@ -645,6 +645,7 @@ __global__ void __launch_bounds__(256, 4) k_pairs(const __grid_constant__ Views 
             atomicAdd(&deg[o], 1);
             if (mir) atomicAdd(&deg[p], 1);
         } else if (MODE == PAIRS_PLACE) {
+            done += mir ? 2u : 1u;
             cap_put(co, (int)o, (int)(p - rb), d);
             if (mir) cap_put(co, (int)p, (int)(o - rb), d);
         } else {
@@ -674,6 +675,7 @@ __global__ void __launch_bounds__(256, 4) k_pairs(const __grid_constant__ Views 
         } else {
             stat_add(st, ST_GUARD, guard);
             stat_add(st, ST_BAND, band);
+            if (MODE == PAIRS_PLACE) stat_add(st, ST_PLACED, done64);
         }
     }
 }

@@ -1762,9 +1762,10 @@ __global__ void k_check_rows_sel(int64_t n, const int64_t *__restrict__ row_ptr,
     if (i < n && rowsel[i] && row_ptr[i] + rowcur[i] != row_ptr[i + 1]) atomicOr(err, 8);
 }
 
-// One-pass emit, after the count pass: every row's produced entries must
-// equal its degree; counts rows past their capacity (cnt[0]) and lost rows
-// (cnt[1]).
+// One-pass emit, after the count pass: every row's produced entries must equal
+// its degree (tensor-core clouds have no degrees of their own: the entries are
+// the degrees, and their total is compared with the edges that k_pairs found);
+// counts rows past their capacity (cnt[0]) and lost rows (cnt[1]).
 __global__ void k_cap_rows(int64_t n, const int64_t *__restrict__ row_ptr, const int64_t *__restrict__ off,
                            const int32_t *__restrict__ fill, const uint8_t *__restrict__ lost,
                            unsigned long long *__restrict__ cnt, int32_t *__restrict__ err) {
@@ -3822,6 +3823,7 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
         }
     };
 
+    unsigned long long tc_placed = 0;  // one-pass form: entries of the tensor-core clouds' rows
     auto finish_stats = [&]() {
         unsigned long long hs[ST_N];
         to_host(hs, st.p, ST_N, s);
@@ -3829,10 +3831,12 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
         if (hs[ST_ERR] & 32)
             CT_FAIL(CT_ETIMEOUT, "a bounded wait of the tensor-core leaf kernel gave up (code %llu)", hs[ST_ERR]);
         if (hs[ST_ERR]) CT_FAIL(CT_ECUDA, "internal consistency check failed in the query (code %llu)", hs[ST_ERR]);
+        if (hs[ST_PLACED] != tc_placed)
+            CT_FAIL(CT_ECUDA, "internal consistency check failed in the query (%llu entries of %llu found)", tc_placed, hs[ST_PLACED]);
         all.stats.traversal_evals = (int64_t)hs[ST_TRAV];
         all.stats.leaf_pairs = (int64_t)(hs[ST_PAIRS] + tc_stats[0]);
         all.stats.guard_fp64 = (int64_t)hs[ST_GUARD];
-        all.stats.recheck_fp32 = (int64_t)(hs[ST_RECHECK] + tc_stats[1]);
+        all.stats.recheck_fp32 = (int64_t)tc_stats[1];
         all.stats.emit_pairs = (int64_t)hs[ST_EMIT];
         all.stats.leaf_rows = (int64_t)(hs[ST_ROWS] + tc_stats[2]);
         all.stats.guard_band = (int64_t)hs[ST_BAND];
@@ -3872,6 +3876,15 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
                 CT_LAUNCH_CHECK();
             }
             to_host(hv, o_n.p, 3, s);
+            if (any_tc && any_fp) {
+                std::vector<int64_t> first(C + 1);  // the clouds' first entries
+                for (int c = 0; c <= C; ++c) to_host_async(&first[c], row_ptr + V.rbase[c], 1, s);
+                CT_CHECK_CUDA(cudaStreamSynchronize(s));
+                for (int c = 0; c < C; ++c)
+                    if (V.use_tc[c]) tc_placed += (unsigned long long)(first[c + 1] - first[c]);
+            } else if (any_tc) {
+                tc_placed = (unsigned long long)nnz;
+            }
             const int64_t used = std::min<int64_t>((int64_t)hv[0], co.ovf_cap);
             if (used > 0) {
                 k_ovf_scatter<<<grid_for(used, 256), 256, 0, s>>>(used, o_ent.p, lost.p, row_ptr, all.col, all.dist,

@@ -111,6 +111,6 @@ void sort_rows(const int64_t *row_ptr, int64_t n, int64_t ncols, int32_t *col, f
                cudaStream_t s);
 
 // Stats slots accumulated on the device.
-enum { ST_TRAV = 0, ST_PAIRS, ST_GUARD, ST_RECHECK, ST_CAND, ST_OVERFLOW, ST_ERR, ST_EMIT, ST_ROWS, ST_BAND, ST_COLS, ST_N };
+enum { ST_TRAV = 0, ST_PAIRS, ST_GUARD, ST_PLACED, ST_CAND, ST_OVERFLOW, ST_ERR, ST_EMIT, ST_ROWS, ST_BAND, ST_COLS, ST_N };
 
 }  // namespace ct
