@@ -1392,10 +1392,15 @@ __global__ void k_next_hubs(int64_t T, int node_base, const int32_t *__restrict_
     nh.thr[h] = ldexpf(1.0f, l - 1);
 }
 
+// rbegin, rcount: the range of the only tree, or null.
 __global__ void k_root_init(int64_t n, int root, int32_t *__restrict__ ids, float *__restrict__ D,
-                            int32_t *__restrict__ lab) {
+                            int32_t *__restrict__ lab, int32_t *__restrict__ rbegin, int32_t *__restrict__ rcount) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
+    if (i == 0 && rbegin) {
+        *rbegin = 0;
+        *rcount = (int32_t)n;
+    }
     ids[i] = i == 0 ? root : (i <= root ? (int32_t)i - 1 : (int32_t)i);
     D[i] = INFINITY;
     lab[i] = 0;
@@ -1762,7 +1767,9 @@ ct_tree *build_impl(const ct_points *pts, int zeta, int root, cudaStream_t s, co
         };
         Hubs H = make_hubs(hbuf, hthr, hkey), H2 = make_hubs(hbuf2, hthr2, hkey2);
 
-        k_root_init<<<grid_for(n), BT, 0, s>>>(n, root, ids.p, D.p, lab.p);
+        const int R0 = (int)hroot.size();
+        DBuf<int32_t> rbegin(R0, s), rcount(R0, s);
+        k_root_init<<<grid_for(n), BT, 0, s>>>(n, root, ids.p, D.p, lab.p, R0 == 1 ? rbegin.p : nullptr, rcount.p);
         CT_COUNT_LAUNCH();
         // lanes per distance: four 16-byte loads each (at most eight for row
         // lengths between two powers of two, more above 1024 floats)
@@ -1895,9 +1902,7 @@ ct_tree *build_impl(const ct_points *pts, int zeta, int root, cudaStream_t s, co
             }
         };
         // the roots: vertices 0 .. R - 1, one hub each, with a batch of one centre (its first position)
-        const int R0 = (int)hroot.size();
-        DBuf<int32_t> rbegin(R0, s), rcount(R0, s);
-        {
+        if (R0 > 1) {
             std::vector<int32_t> hb(R0), hn(R0);
             nchunks = 0;
             for (int c = 0; c < R0; ++c) {
