@@ -104,7 +104,6 @@ struct Hubs {
     int32_t *begin, *count, *node, *nc, *m, *done, *level;
     int32_t *flat;  // 1: the split stopped early and every child is a leaf block
     float *thr;
-    unsigned long long *key;
 };
 
 // A split that has taken FLAT_MIN_CENTRES centres while they cover on average
@@ -636,10 +635,6 @@ constexpr int LEV_C = 64;     // candidates of a selection
 // 148 / 490 this way.
 constexpr int LEV_WIDE_M = 6, LEV_WIDE_P = BT / LEV_WIDE_M;
 
-__global__ void k_present(const uint8_t *__restrict__ s, int64_t nbytes, int32_t *__restrict__ present) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < nbytes) present[s[i]] = 1;
-}
 // code[byte] = its rank among the bytes that occur; *A = their number.
 __global__ void k_codes(const int32_t *__restrict__ present, uint8_t *__restrict__ code, int32_t *__restrict__ A) {
     __shared__ int s_w[8];
@@ -1366,8 +1361,7 @@ __global__ void k_make_nodes(int64_t T, int node_base, int zeta, int metric,
 // hubs, their chunks).
 __global__ void k_next_hubs(int64_t T, int node_base, const int32_t *__restrict__ is_hub,
                             const int64_t *__restrict__ hub_off, const int32_t *__restrict__ cbegin,
-                            const int32_t *__restrict__ ccount, const unsigned long long *__restrict__ ckey,
-                            const int32_t *__restrict__ level, Hubs nh, int small_max, int chunk_len,
+                            const int32_t *__restrict__ ccount, const int32_t *__restrict__ level, Hubs nh, int small_max, int chunk_len,
                             int2 *__restrict__ hlist, int32_t *__restrict__ cnt) {
     int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const bool hub = c < T && is_hub[c];
@@ -1386,7 +1380,6 @@ __global__ void k_next_hubs(int64_t T, int node_base, const int32_t *__restrict_
     nh.m[h] = 0;
     nh.done[h] = 0;
     nh.flat[h] = 0;
-    nh.key[h] = ckey[c];
     int l = level[v];
     nh.level[h] = l;
     nh.thr[h] = ldexpf(1.0f, l - 1);
@@ -1409,7 +1402,8 @@ __global__ void k_root_init(int64_t n, int root, int32_t *__restrict__ ids, floa
 // The roots' first pass: hub c holds every point of tree c, its batch is its
 // first position with label 0.
 __global__ void k_root_hubs(int R, const int32_t *__restrict__ rbegin, const int32_t *__restrict__ rcount, Hubs hb,
-                            int32_t *__restrict__ bpos, int2 *__restrict__ hlist) {
+                            int32_t *__restrict__ bpos, int2 *__restrict__ hlist,
+                            unsigned long long *__restrict__ rkey) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= R) return;
     hb.begin[c] = rbegin[c];
@@ -1418,7 +1412,7 @@ __global__ void k_root_hubs(int R, const int32_t *__restrict__ rbegin, const int
     hb.m[c] = 1;
     hb.done[c] = 0;
     hb.thr[c] = 0.0f;
-    hb.key[c] = 0ull;
+    rkey[c] = 0ull;
     bpos[rbegin[c]] = rbegin[c];
     hlist[c] = make_int2(c, c);
 }
@@ -1724,8 +1718,7 @@ ct_tree *build_impl(const ct_points *pts, int zeta, int root, cudaStream_t s, co
         scode = DBuf<uint8_t>(bytes > 0 ? bytes : 1, s);
         const uint8_t *src = (const uint8_t *)pts->data + sspan[0];
         if (bytes > 0) {
-            k_present<<<grid_for(bytes), BT, 0, s>>>(src, bytes, present.p);
-            CT_COUNT_LAUNCH();
+            mark_bytes(src, bytes, present.p, s);
             k_codes<<<1, 256, 0, s>>>(present.p, codes.p, present.p + 256);
             CT_COUNT_LAUNCH();
             k_recode<<<grid_for(bytes), BT, 0, s>>>(src, bytes, codes.p, scode.p);
@@ -1752,20 +1745,18 @@ ct_tree *build_impl(const ct_points *pts, int zeta, int root, cudaStream_t s, co
         const int64_t cap_h = n;  // hubs per round never exceed n / (zeta+1) + 1
         DBuf<int32_t> hbuf(8 * (cap_h + 1), s);
         DBuf<float> hthr(cap_h + 1, s);
-        DBuf<unsigned long long> hkey(cap_h + 1, s);
         DBuf<int32_t> hbuf2(8 * (cap_h + 1), s);
         DBuf<float> hthr2(cap_h + 1, s);
-        DBuf<unsigned long long> hkey2(cap_h + 1, s);
-        auto make_hubs = [&](DBuf<int32_t> &b, DBuf<float> &th, DBuf<unsigned long long> &k) {
+        auto make_hubs = [&](DBuf<int32_t> &b, DBuf<float> &th) {
             Hubs h;
             int64_t st = cap_h + 1;
             h.begin = b.p; h.count = b.p + st; h.node = b.p + 2 * st; h.nc = b.p + 3 * st;
             h.m = b.p + 4 * st; h.done = b.p + 5 * st; h.level = b.p + 6 * st;
             h.flat = b.p + 7 * st;
-            h.thr = th.p; h.key = k.p;
+            h.thr = th.p;
             return h;
         };
-        Hubs H = make_hubs(hbuf, hthr, hkey), H2 = make_hubs(hbuf2, hthr2, hkey2);
+        Hubs H = make_hubs(hbuf, hthr), H2 = make_hubs(hbuf2, hthr2);
 
         const int R0 = (int)hroot.size();
         DBuf<int32_t> rbegin(R0, s), rcount(R0, s);
@@ -1917,22 +1908,23 @@ ct_tree *build_impl(const ct_points *pts, int zeta, int root, cudaStream_t s, co
         DBuf<int64_t> i64tmp(4, s);
         DBuf<int32_t> rhub(R0, s), rleafy(R0, s);
         DBuf<int64_t> roff(R0, s);
+        DBuf<unsigned long long> rkey(R0, s);  // each root's farthest point
         CT_CHECK_CUDA(cudaMemsetAsync(i64tmp.p, 0, 4 * sizeof(int64_t), s));
         CT_CHECK_CUDA(cudaMemsetAsync(rleafy.p, 0, R0 * sizeof(int32_t), s));
         grow_chunks();
-        k_root_hubs<<<grid_for(R0), BT, 0, s>>>(R0, rbegin.p, rcount.p, H, bpos.p, hl_a.p);
+        k_root_hubs<<<grid_for(R0), BT, 0, s>>>(R0, rbegin.p, rcount.p, H, bpos.p, hl_a.p, rkey.p);
         CT_COUNT_LAUNCH();
         k_chunk_counts<<<grid_for(R0), BT, 0, s>>>(R0, hl_a.p, H.count, chunk_len, rhub.p);
         CT_COUNT_LAUNCH();
         exclusive_scan_i32_to_i64(rhub.p, roff.p, R0, nullptr, s);
         k_chunk_fill<<<grid_for(nchunks), BT, 0, s>>>(nchunks, R0, hl_a.p, H.begin, roff.p, chunk_len, chunks_a.p);
         CT_COUNT_LAUNCH();
-        update(H, nchunks, chunks_a.p, Batch{bpos.p, cpos.p, dcc.p}, H.key);
-        k_make_nodes<<<grid_for(R0), BT, 0, s>>>(R0, 0, zeta, pts->metric, rbegin.p, rcount.p, H.key, nb.p, ncnt.p,
+        update(H, nchunks, chunks_a.p, Batch{bpos.p, cpos.p, dcc.p}, rkey.p);
+        k_make_nodes<<<grid_for(R0), BT, 0, s>>>(R0, 0, zeta, pts->metric, rbegin.p, rcount.p, rkey.p, nb.p, ncnt.p,
                                                  cbeg.p, ccnt.p, rad.p, lvl.p, rleafy.p, rhub.p);
         CT_COUNT_LAUNCH();
         exclusive_scan_i32_to_i64(rhub.p, roff.p, R0, i64tmp.p, s);
-        k_next_hubs<<<grid_for(R0), BT, 0, s>>>(R0, 0, rhub.p, roff.p, rbegin.p, rcount.p, H.key, lvl.p, H2, small_max,
+        k_next_hubs<<<grid_for(R0), BT, 0, s>>>(R0, 0, rhub.p, roff.p, rbegin.p, rcount.p, lvl.p, H2, small_max,
                                                 chunk_len, hl_a.p, reinterpret_cast<int32_t *>(i64tmp.p + 1));
         CT_COUNT_LAUNCH();
         CT_LAUNCH_CHECK();
@@ -2043,7 +2035,7 @@ ct_tree *build_impl(const ct_points *pts, int zeta, int root, cudaStream_t s, co
             CT_CHECK_CUDA(cudaMemsetAsync(i64tmp.p + 1, 0, 2 * sizeof(int64_t), s));
             exclusive_scan_i32_to_i64(is_hub.p, hub_off.p, T, i64tmp.p, s);
             // a hub has more than zeta points: at most n / (zeta + 1) of them, within cap_h
-            k_next_hubs<<<grid_for(T), BT, 0, s>>>(T, n_nodes, is_hub.p, hub_off.p, cbegin.p, ccount.p, ckey.p, lvl.p,
+            k_next_hubs<<<grid_for(T), BT, 0, s>>>(T, n_nodes, is_hub.p, hub_off.p, cbegin.p, ccount.p, lvl.p,
                                                    H2, small_max, chunk_len, hl_a.p,
                                                    reinterpret_cast<int32_t *>(i64tmp.p + 1));
             CT_COUNT_LAUNCH();

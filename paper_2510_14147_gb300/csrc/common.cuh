@@ -119,8 +119,8 @@ extern std::atomic<int64_t> g_total_launches;
 
 // ------------------------------------------------------------- scans
 
-// Exclusive prefix sums (reduce-then-scan, three launches).  `out` may alias
-// `in`.  Writes the total to *total_dev when given (device int64).
+// Exclusive prefix sums (one block up to 16384 values, else reduce-then-scan in
+// three launches).  `out` may alias an int64 `in`.  Writes the total to *total_dev when given (device int64).
 void exclusive_scan_i32_to_i64(const int32_t *in, int64_t *out, int64_t n, int64_t *total_dev,
                                cudaStream_t s);
 void exclusive_scan_i64(const int64_t *in, int64_t *out, int64_t n, int64_t *total_dev,
@@ -129,6 +129,9 @@ void exclusive_scan_i64(const int64_t *in, int64_t *out, int64_t n, int64_t *tot
 int64_t scan_scratch_entries(int64_t n);
 void exclusive_scan_i32_to_i64_into(const int32_t *in, int64_t *out, int64_t n, int64_t *total_dev,
                                     int64_t *tile_sums, cudaStream_t s);
+
+// present[b] = 1 for every byte value b that occurs (entries of others are left).
+void mark_bytes(const uint8_t *bytes, int64_t n, int32_t *present, cudaStream_t s);
 
 // Stable LSD radix sort of (key, value) pairs by the low `key_bits` bits of
 // the key.  Sorted output returned in keys/vals (tmp buffers of n entries).

@@ -1,6 +1,7 @@
 // mlp.cu -- forward, backward and Adam kernels of the degree/work predictor
 // (16 -> 64 -> 64 -> 2, ReLU, mean squared error).  The paper has no learned
 // component; this predictor sizes the one-pass emit and orders work.
+#include "f32x2.cuh"
 #include "mlp.cuh"
 
 namespace ct {
@@ -125,21 +126,8 @@ __global__ void k_to_half(const float *__restrict__ w, __half *__restrict__ wh) 
     if (e < MLP_NPARAMS) wh[e] = __float2half_rn(w[e]);
 }
 
-// Packed fp32 pairs: two independent IEEE round-to-nearest operations.
-__device__ __forceinline__ unsigned long long pack2(float lo, float hi) {
-    unsigned long long d;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
-    return d;
-}
-__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
-    unsigned long long d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ float lo2(unsigned long long v) { return __uint_as_float((uint32_t)v); }
-__device__ __forceinline__ float hi2(unsigned long long v) { return __uint_as_float((uint32_t)(v >> 32)); }
 __device__ __forceinline__ unsigned long long relu2(unsigned long long v) {
-    return pack2(fmaxf(lo2(v), 0.f), fmaxf(hi2(v), 0.f));
+    return f2_pack(fmaxf(f2_lo(v), 0.f), fmaxf(f2_hi(v), 0.f));
 }
 
 // Inference with fp16-rounded weights and fp32 sums: two samples per thread
@@ -153,7 +141,7 @@ __global__ void __launch_bounds__(PT) k_mlp_predict(const __half *__restrict__ w
     __shared__ __align__(16) unsigned long long sw[MLP_NPARAMS];
     for (int e = threadIdx.x; e < MLP_NPARAMS; e += PT) {
         const float w = __half2float(wh[e]);
-        sw[e] = pack2(w, w);
+        sw[e] = f2_pack(w, w);
     }
     __syncthreads();
     const int64_t s0 = (int64_t)blockIdx.x * 2 * PT + threadIdx.x, s1 = s0 + PT;
@@ -164,14 +152,14 @@ __global__ void __launch_bounds__(PT) k_mlp_predict(const __half *__restrict__ w
 #pragma unroll
         for (int k = 0; k < MLP_IN; k += 4) {
             const float4 a = *reinterpret_cast<const float4 *>(xa + k), b = *reinterpret_cast<const float4 *>(xb + k);
-            xi[k] = pack2(a.x, b.x);
-            xi[k + 1] = pack2(a.y, b.y);
-            xi[k + 2] = pack2(a.z, b.z);
-            xi[k + 3] = pack2(a.w, b.w);
+            xi[k] = f2_pack(a.x, b.x);
+            xi[k + 1] = f2_pack(a.y, b.y);
+            xi[k + 2] = f2_pack(a.z, b.z);
+            xi[k + 3] = f2_pack(a.w, b.w);
         }
     } else {  // a caller's rows at any float
 #pragma unroll
-        for (int k = 0; k < MLP_IN; ++k) xi[k] = pack2(xa[k], xb[k]);
+        for (int k = 0; k < MLP_IN; ++k) xi[k] = f2_pack(xa[k], xb[k]);
     }
     const ulonglong2 *sw2 = reinterpret_cast<const ulonglong2 *>(sw);
 #pragma unroll
@@ -180,8 +168,8 @@ __global__ void __launch_bounds__(PT) k_mlp_predict(const __half *__restrict__ w
 #pragma unroll
         for (int k = 0; k < MLP_IN; k += 2) {
             const ulonglong2 w = sw2[(P_W1 + i * MLP_IN + k) / 2];
-            a = fma2(w.x, xi[k], a);
-            a = fma2(w.y, xi[k + 1], a);
+            a = f2_fma(w.x, xi[k], a);
+            a = f2_fma(w.y, xi[k + 1], a);
         }
         h1[i] = relu2(a);
     }
@@ -192,18 +180,18 @@ __global__ void __launch_bounds__(PT) k_mlp_predict(const __half *__restrict__ w
 #pragma unroll
         for (int j = 0; j < MLP_HID; j += 2) {
             const ulonglong2 w = sw2[(P_W2 + i * MLP_HID + j) / 2];
-            a = fma2(w.x, h1[j], a);
-            a = fma2(w.y, h1[j + 1], a);
+            a = f2_fma(w.x, h1[j], a);
+            a = f2_fma(w.y, h1[j + 1], a);
         }
         a = relu2(a);
-        y0 = fma2(sw[P_W3 + i], a, y0);
-        y1 = fma2(sw[P_W3 + MLP_HID + i], a, y1);
+        y0 = f2_fma(sw[P_W3 + i], a, y0);
+        y1 = f2_fma(sw[P_W3 + MLP_HID + i], a, y1);
     }
-    y[s0 * MLP_OUT] = lo2(y0);
-    y[s0 * MLP_OUT + 1] = lo2(y1);
+    y[s0 * MLP_OUT] = f2_lo(y0);
+    y[s0 * MLP_OUT + 1] = f2_lo(y1);
     if (s1 < n) {
-        y[s1 * MLP_OUT] = hi2(y0);
-        y[s1 * MLP_OUT + 1] = hi2(y1);
+        y[s1 * MLP_OUT] = f2_hi(y0);
+        y[s1 * MLP_OUT + 1] = f2_hi(y1);
     }
 }
 

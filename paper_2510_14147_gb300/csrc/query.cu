@@ -25,6 +25,7 @@
 #include <mutex>
 #include <type_traits>
 
+#include "f32x2.cuh"
 #include "lev.cuh"
 #include "profile.cuh"
 #include "query.cuh"
@@ -173,38 +174,6 @@ constexpr int TRAV_LIMIT = 128;    // step limit of the next rounds
 // edit distance: a step (32 bit-parallel recurrences) costs about a hundred
 // L2 steps, so its walks stop much sooner
 constexpr int TRAV_LIMIT0_LEV = 8, TRAV_LIMIT_LEV = 8;
-
-// Packed fp32 pairs (sm_100+ f32x2 instructions): two independent IEEE
-// round-to-nearest operations per instruction.
-__device__ __forceinline__ unsigned long long f2_sub(unsigned long long a, unsigned long long b) {
-    unsigned long long d;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ unsigned long long f2_sqacc(unsigned long long d, unsigned long long acc) {
-    unsigned long long r;
-    asm("fma.rn.f32x2 %0, %1, %1, %2;" : "=l"(r) : "l"(d), "l"(acc));
-    return r;
-}
-__device__ __forceinline__ unsigned long long f2_pack(float lo, float hi) {
-    unsigned long long d;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
-    return d;
-}
-__device__ __forceinline__ unsigned long long f2_add(unsigned long long a, unsigned long long b) {
-    unsigned long long d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ unsigned long long f2_fma(unsigned long long a, unsigned long long b,
-                                                     unsigned long long c) {
-    unsigned long long d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ float f2_sum(unsigned long long v) {
-    return __uint_as_float((uint32_t)v) + __uint_as_float((uint32_t)(v >> 32));
-}
 
 // Warp-uniform write cursor: current chunk, its fill, the open segment.
 struct PoolCursor {
@@ -501,7 +470,8 @@ __device__ __forceinline__ bool l2_keep(const TreeView &tv, const float4 *cen, i
 // (global group ids), or -- in the later rounds -- per stored range of a
 // walk that reached the step limit; the lanes per vertex test follow the
 // cloud's row length.  Walks stop at out.limit steps (no limit without
-// out.items) and store the rest of their stack in `out`.
+// out.items) and store the rest of their stack in `out`.  (Eight blocks an SM
+// leave 64 registers a thread; -Xptxas -v: 4 bytes of them spilled.)
 __global__ void __launch_bounds__(TRAV_WARPS * 32, 8) k_traverse_l2(
     const __grid_constant__ Views V, const int32_t *__restrict__ order, int n_order,
     const int4 *__restrict__ in_items, const int32_t *__restrict__ in_count, int in_cap, Spill out, Pool P,
@@ -1649,7 +1619,8 @@ __device__ __forceinline__ void leaf_l2_item(
 // M edges, more than the list had.)
 // Rows of at most 64 floats take a shorter tile stride and fewer registers, so
 // that five CTAs share an SM instead of three (a tile is a chain of copy,
-// barrier, arithmetic, barrier: more of them in flight).
+// barrier, arithmetic, barrier: more of them in flight; -Xptxas -v: 96
+// registers, the count form spills 32 bytes of them and reads 28 back).
 // 174k x 64 at 87 neighbours: count 16.3 -> 14.1 ms, bound by the shared-memory
 // reads of the micro-tiles (71 % of that pipe, four wavefronts per 16-byte
 // read whatever is broadcast) and the FP32 pipe (58 %).  The emit pass reads
@@ -2350,11 +2321,6 @@ __global__ void __launch_bounds__(LEAF_T) k_leaf_ham(
     if (tid < qn && cnt[tid]) atomicAdd(&deg[cursor[tid]], cnt[tid]);
     for (int o = 16; o > 0; o >>= 1) pairs += __shfl_xor_sync(0xffffffffu, pairs, o);
     if (lane == 0) stat_add(st, ST_PAIRS, pairs);
-}
-
-__global__ void k_alphabet(const uint8_t *__restrict__ s, int64_t nbytes, int32_t *__restrict__ present) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < nbytes) present[s[i]] = 1;
 }
 
 // ------------------------------------------------------------- row sort
@@ -3511,8 +3477,7 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
         DBuf<int32_t> present(256, s);
         CT_CHECK_CUDA(cudaMemsetAsync(present.p, 0, 256 * sizeof(int32_t), s));
         if (t->sbytes) {
-            k_alphabet<<<grid_for(t->sbytes, 256), 256, 0, s>>>(t->sdata, t->sbytes, present.p);
-            CT_COUNT_LAUNCH();
+            mark_bytes(t->sdata, t->sbytes, present.p, s);
         }
         int32_t hp[256];
         to_host(hp, present.p, 256, s);

@@ -72,6 +72,17 @@ int num_sms() {
     return sms[dev];
 }
 
+__global__ void k_mark_bytes(const uint8_t *__restrict__ bytes, int64_t n, int32_t *__restrict__ present) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) present[bytes[i]] = 1;
+}
+void mark_bytes(const uint8_t *bytes, int64_t n, int32_t *present, cudaStream_t s) {
+    if (n <= 0) return;
+    k_mark_bytes<<<(unsigned)ceil_div(n, 256), 256, 0, s>>>(bytes, n, present);
+    CT_COUNT_LAUNCH();
+    CT_LAUNCH_CHECK();
+}
+
 // ------------------------------------------------------------------ scans
 
 constexpr int SCAN_THREADS = 512;
