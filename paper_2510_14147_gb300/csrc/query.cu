@@ -148,7 +148,7 @@ struct Pool {
     // work left when the pool ran out, as items (group, first vertex, count or
     // -1: the whole group); null: walks go on, counting without writing
     int4 *resume = nullptr;
-    int32_t *n_resume = nullptr;
+    unsigned long long *n_resume = nullptr;
     int32_t *n_whole = nullptr;  // whole groups among them
     int resume_cap = 0;
 };
@@ -158,7 +158,7 @@ constexpr int POOL_STOPPED = 1;
 // (global group, first vertex, count, -) that the next round walks.
 struct Spill {
     int4 *items;
-    int32_t *count;  // never above cap (list_reserve)
+    unsigned long long *count;  // entries asked for: may exceed cap (see reserve.cuh)
     int cap;
     int limit;       // steps before a walk stops
 };
@@ -219,15 +219,15 @@ __device__ __forceinline__ bool pool_more(const Pool &P, int g, PoolCursor &pc) 
     pc.seg_begin = pc.cur;
     return true;
 }
-__device__ __forceinline__ void resume_put(const Pool &P, int at, int4 item) {
-    if (at < P.resume_cap) P.resume[at] = item;
+__device__ __forceinline__ void resume_put(const Pool &P, unsigned long long at, int4 item) {
+    if (at < (unsigned long long)P.resume_cap) P.resume[at] = item;
     else atomicOr(P.overflow, 2);
 }
 // Leaves one work item (group, range; count 0: the whole group) for the next pass.
 __device__ __forceinline__ void resume_item(const Pool &P, int g, int2 start) {
     if ((threadIdx.x & 31) == 0) {
         if (start.y == 0) atomicAdd(P.n_whole, 1);
-        resume_put(P, atomicAdd(P.n_resume, 1), make_int4(g, start.x, start.y ? start.y : -1, 0));
+        resume_put(P, atomicAdd(P.n_resume, 1ull), make_int4(g, start.x, start.y ? start.y : -1, 0));
     }
 }
 
@@ -311,12 +311,11 @@ __device__ __forceinline__ int walk_group(const TreeView &tv, int2 *__restrict__
                 int total = 0;
                 for (int i = lane; i < top; i += 32) total += (stack[i].y + piece - 1) / piece;
                 total = (int)__reduce_add_sync(0xffffffffu, (unsigned)total);
-                int base = 0;
-                if (lane == 0)
-                    base = list_reserve(*(volatile int32_t *)sp->count, total, sp->cap,
-                                        [&](int seen, int want) { return atomicCAS(sp->count, seen, want); });
-                base = __shfl_sync(0xffffffffu, base, 0);
-                if (base >= 0) {
+                unsigned long long first = 0;
+                if (lane == 0) first = atomicAdd(sp->count, (unsigned long long)total);
+                const ListRoom room = list_room(__shfl_sync(0xffffffffu, first, 0), total, sp->cap);
+                if (room.fits) {
+                    int base = room.begin;
                     for (int i0 = 0; i0 < top; i0 += 32) {
                         const int2 r = i0 + lane < top ? stack[i0 + lane] : make_int2(0, 0);
                         const int c = (r.y + piece - 1) / piece;
@@ -333,12 +332,15 @@ __device__ __forceinline__ int walk_group(const TreeView &tv, int2 *__restrict__
                     }
                     break;
                 }
-                limit = INT_MAX;  // no room: the walk is finished here
+                // no room: what was asked for below the end holds empty ranges (count 0,
+                // skipped), and the walk is finished here
+                for (int i = room.begin + lane; i < sp->cap; i += 32) sp->items[i] = make_int4(g, 0, 0, 0);
+                limit = INT_MAX;
             }
             // resumable walks have room for every vertex of a step before it begins
             if (P.resume && pc.fill > POOL_CHUNK - 32 && !pool_more(P, g, pc)) {
-                int base = 0;
-                if (lane == 0) base = atomicAdd(P.n_resume, top);
+                unsigned long long base = 0;
+                if (lane == 0) base = atomicAdd(P.n_resume, (unsigned long long)top);
                 base = __shfl_sync(0xffffffffu, base, 0);
                 for (int i = lane; i < top; i += 32) {
                     const int2 r = stack[i];
@@ -474,7 +476,7 @@ __device__ __forceinline__ bool l2_keep(const TreeView &tv, const float4 *cen, i
 // leave 64 registers a thread; -Xptxas -v: 4 bytes of them spilled.)
 __global__ void __launch_bounds__(TRAV_WARPS * 32, 8) k_traverse_l2(
     const __grid_constant__ Views V, const int32_t *__restrict__ order, int n_order,
-    const int4 *__restrict__ in_items, const int32_t *__restrict__ in_count, int in_cap, Spill out, Pool P,
+    const int4 *__restrict__ in_items, const unsigned long long *__restrict__ in_count, int in_cap, Spill out, Pool P,
     longlong2 *__restrict__ cursors, int2 *__restrict__ stacks, int cap, unsigned long long *__restrict__ st,
     int32_t *__restrict__ err, int32_t *__restrict__ next_group, int32_t *__restrict__ gvisit, int max_nq4) {
     extern __shared__ float4 sc[];  // TRAV_WARPS x (largest dp / 4)
@@ -490,7 +492,7 @@ __global__ void __launch_bounds__(TRAV_WARPS * 32, 8) k_traverse_l2(
         pc.cur = c.x;
         pc.fill = (int)c.y;
     }
-    const int n_work = in_items ? min(*in_count, in_cap) : n_order;
+    const int n_work = in_items ? list_length(*in_count, in_cap) : n_order;
     const Spill *sp = out.items ? &out : nullptr;
     bool full = false;  // the pool had no chunk for this warp
     for (;;) {
@@ -503,6 +505,7 @@ __global__ void __launch_bounds__(TRAV_WARPS * 32, 8) k_traverse_l2(
         int2 start = make_int2(0, 0);
         if (in_items) {
             const int4 w = in_items[gi];
+            if (w.z == 0) continue;  // an empty range (a stop that did not fit)
             gg = w.x;
             if (w.z > 0) start = make_int2(w.y, w.z);
         } else {
@@ -547,7 +550,7 @@ __global__ void __launch_bounds__(TRAV_WARPS * 32, 8) k_traverse_l2(
 // in shared memory.
 template <int W>
 __global__ void __launch_bounds__(32) k_traverse_lev(
-    TreeView tv, QParams qp, const int4 *__restrict__ in_items, const int32_t *__restrict__ in_count, int in_cap,
+    TreeView tv, QParams qp, const int4 *__restrict__ in_items, const unsigned long long *__restrict__ in_count, int in_cap,
     Spill out, Pool P, longlong2 *__restrict__ cursors, int2 *__restrict__ stacks, int cap,
     unsigned long long *__restrict__ st, int32_t *__restrict__ err, int32_t *__restrict__ next_group,
     int32_t *__restrict__ gvisit) {
@@ -562,7 +565,7 @@ __global__ void __launch_bounds__(32) k_traverse_lev(
         pc.cur = c.x;
         pc.fill = (int)c.y;
     }
-    const int n_work = in_items ? min(*in_count, in_cap) : tv.n_groups;
+    const int n_work = in_items ? list_length(*in_count, in_cap) : tv.n_groups;
     const Spill *sp = out.items ? &out : nullptr;
     bool full = false;  // the pool had no chunk for this warp
     for (;;) {
@@ -574,6 +577,7 @@ __global__ void __launch_bounds__(32) k_traverse_lev(
         int2 start = make_int2(0, 0);
         if (in_items) {
             const int4 w = in_items[gi];
+            if (w.z == 0) continue;  // an empty range (a stop that did not fit)
             g = w.x;
             if (w.z > 0) start = make_int2(w.y, w.z);
         } else {
@@ -635,7 +639,7 @@ __device__ __forceinline__ int ham_rows_smem(const uint4 *a, const uint4 *b, int
 }
 
 __global__ void __launch_bounds__(32) k_traverse_ham(
-    TreeView tv, QParams qp, const int4 *__restrict__ in_items, const int32_t *__restrict__ in_count, int in_cap,
+    TreeView tv, QParams qp, const int4 *__restrict__ in_items, const unsigned long long *__restrict__ in_count, int in_cap,
     Spill out, Pool P, longlong2 *__restrict__ cursors, int2 *__restrict__ stacks, int cap,
     unsigned long long *__restrict__ st, int32_t *__restrict__ err, int32_t *__restrict__ next_group,
     int32_t *__restrict__ gvisit) {
@@ -651,7 +655,7 @@ __global__ void __launch_bounds__(32) k_traverse_ham(
         pc.cur = c.x;
         pc.fill = (int)c.y;
     }
-    const int n_work = in_items ? min(*in_count, in_cap) : tv.n_groups;
+    const int n_work = in_items ? list_length(*in_count, in_cap) : tv.n_groups;
     const Spill *sp = out.items ? &out : nullptr;
     bool full = false;  // the pool had no chunk for this warp
     for (;;) {
@@ -663,6 +667,7 @@ __global__ void __launch_bounds__(32) k_traverse_ham(
         int2 start = make_int2(0, 0);
         if (in_items) {
             const int4 w = in_items[gi];
+            if (w.z == 0) continue;  // an empty range (a stop that did not fit)
             g = w.x;
             if (w.z > 0) start = make_int2(w.y, w.z);
         } else {
@@ -3093,9 +3098,9 @@ int64_t pool_capacity_guess(int64_t n, int64_t G, const TravLaunch &tl) {
 // warp per block; edit-distance walks stop sooner: their steps cost more).
 void launch_traversal(const Views &V, int64_t G, int max_dp, int max_len, bool l2, const int32_t *order,
                       const Pool &P, int2 *stacks, int cap, const TravLaunch &tl, unsigned long long *st,
-                      int32_t *err, int32_t *next_group, int4 *const spill[2], int32_t *spill_cnt, int spill_cap,
+                      int32_t *err, int32_t *next_group, int4 *const spill[2], unsigned long long *spill_cnt, int spill_cap,
                       longlong2 *cursors, cudaStream_t s, int32_t *gvisit = nullptr, const int4 *resumed = nullptr,
-                      const int32_t *n_resumed = nullptr, int resumed_cap = 0) {
+                      const unsigned long long *n_resumed = nullptr, int resumed_cap = 0) {
     // P.next .. P.overflow are the four 64-bit words of one counter block
     // (kept when a resume list is walked on, as are gvisit and the cursors)
     CT_CHECK_CUDA(cudaMemsetAsync(next_group, 0, sizeof(int32_t), s));
@@ -3107,10 +3112,10 @@ void launch_traversal(const Views &V, int64_t G, int max_dp, int max_len, bool l
     if (l2) {
         const size_t tsm = (size_t)TRAV_WARPS * max_dp * sizeof(float);
         if (tsm > 48 * 1024) allow_smem(k_traverse_l2, kTravSmemMost);
-        CT_CHECK_CUDA(cudaMemsetAsync(spill_cnt, 0, 2 * sizeof(int32_t), s));
+        CT_CHECK_CUDA(cudaMemsetAsync(spill_cnt, 0, 2 * sizeof(unsigned long long), s));
         for (int r = 0; r <= TRAV_ROUNDS; ++r) {
             const int4 *in = r ? spill[(r - 1) & 1] : resumed;
-            const int32_t *in_cnt = r ? spill_cnt + ((r - 1) & 1) : n_resumed;
+            const unsigned long long *in_cnt = r ? spill_cnt + ((r - 1) & 1) : n_resumed;
             const int in_cap = r ? spill_cap : resumed_cap;
             Spill out{nullptr, spill_cnt + (r & 1), spill_cap, INT_MAX};
             if (r < TRAV_ROUNDS) {
@@ -3119,7 +3124,7 @@ void launch_traversal(const Views &V, int64_t G, int max_dp, int max_len, bool l
             }
             if (r) {
                 CT_CHECK_CUDA(cudaMemsetAsync(next_group, 0, sizeof(int32_t), s));
-                CT_CHECK_CUDA(cudaMemsetAsync(spill_cnt + (r & 1), 0, sizeof(int32_t), s));
+                CT_CHECK_CUDA(cudaMemsetAsync(spill_cnt + (r & 1), 0, sizeof(unsigned long long), s));
             }
             k_traverse_l2<<<tl.blocks, TRAV_WARPS * 32, tsm, s>>>(V, order, (int)G, in, in_cnt, in_cap, out, P,
                                                                    cursors, stacks, cap, st, err, next_group,
@@ -3131,11 +3136,11 @@ void launch_traversal(const Views &V, int64_t G, int max_dp, int max_len, bool l
         TreeView tv = V.tv[0];
         tv.group_order = order;
         const bool ham = tv.wp != 0;
-        CT_CHECK_CUDA(cudaMemsetAsync(spill_cnt, 0, 2 * sizeof(int32_t), s));
+        CT_CHECK_CUDA(cudaMemsetAsync(spill_cnt, 0, 2 * sizeof(unsigned long long), s));
         const int rounds = ham ? TRAV_ROUNDS : TRAV_ROUNDS_LEV;
         for (int r = 0; r <= rounds; ++r) {
             const int4 *in = r ? spill[(r - 1) & 1] : resumed;
-            const int32_t *in_cnt = r ? spill_cnt + ((r - 1) & 1) : n_resumed;
+            const unsigned long long *in_cnt = r ? spill_cnt + ((r - 1) & 1) : n_resumed;
             const int in_cap = r ? spill_cap : resumed_cap;
             Spill out{nullptr, spill_cnt + (r & 1), spill_cap, INT_MAX};
             if (r < rounds) {
@@ -3144,7 +3149,7 @@ void launch_traversal(const Views &V, int64_t G, int max_dp, int max_len, bool l
             }
             if (r) {
                 CT_CHECK_CUDA(cudaMemsetAsync(next_group, 0, sizeof(int32_t), s));
-                CT_CHECK_CUDA(cudaMemsetAsync(spill_cnt + (r & 1), 0, sizeof(int32_t), s));
+                CT_CHECK_CUDA(cudaMemsetAsync(spill_cnt + (r & 1), 0, sizeof(unsigned long long), s));
             }
             if (ham) {
                 k_traverse_ham<<<tl.blocks, 32, 0, s>>>(tv, V.qp[0], in, in_cnt, in_cap, out, P, cursors, stacks,
@@ -3342,7 +3347,7 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
     // ranges of step-limited walks: two buffers and their counters
     const int spill_cap = (int)std::min<int64_t>(std::max<int64_t>(4 * G, 1 << 16), 1 << 20);
     DBuf<int4> spill_a(spill_cap, s), spill_b(spill_cap, s);
-    DBuf<int32_t> spill_cnt(2, s);
+    DBuf<unsigned long long> spill_cnt(2, s);
     int4 *const spills[2] = {spill_a.p, spill_b.p};
     DBuf<longlong2> cursors(tl.warps, s);
     // a pool of whole chunks; work left when it runs out goes to a resume list
@@ -3355,7 +3360,7 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
     const int resume_cap = (int)std::min<int64_t>(G + 2LL * spill_cap + 65536, 1 << 26);
     DBuf<uint32_t> pool;
     DBuf<int4> resume[2];
-    DBuf<int32_t> rctr(3, s);  // entries of the two lists, whole groups
+    DBuf<unsigned long long> rctr(3, s);  // entries of the two lists, whole groups
     DBuf<int32_t> seg_group, seg_count;
     DBuf<int64_t> seg_begin;
     unsigned long long hc[4] = {0, 0, 0, 0};
@@ -3377,11 +3382,11 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
         grown(seg_begin, seg_cap, nseg0);
         const int cur = pass & 1;  // this pass writes list cur and reads the other
         if (!resume[cur].p) resume[cur] = DBuf<int4>(resume_cap, s);
-        CT_CHECK_CUDA(cudaMemsetAsync(rctr.p + cur, 0, sizeof(int32_t), s));
-        CT_CHECK_CUDA(cudaMemsetAsync(rctr.p + 2, 0, sizeof(int32_t), s));
+        CT_CHECK_CUDA(cudaMemsetAsync(rctr.p + cur, 0, sizeof(unsigned long long), s));
+        CT_CHECK_CUDA(cudaMemsetAsync(rctr.p + 2, 0, sizeof(unsigned long long), s));
         P = Pool{pool.p, pool_cap, ctr.p, seg_group.p, seg_count.p, seg_begin.p,
                  reinterpret_cast<int32_t *>(ctr.p + 1), seg_cap, ctr.p + 2, reinterpret_cast<int32_t *>(ctr.p + 3),
-                 resume[cur].p, rctr.p + cur, rctr.p + 2, resume_cap};
+                 resume[cur].p, rctr.p + cur, reinterpret_cast<int32_t *>(rctr.p + 2), resume_cap};
         {
             ProfScope ps("traverse", s);
             launch_traversal(V, G, max_dp, max_len, l2, order, P, stacks.p, cap, tl, st.p, err, next_group.p, spills,
@@ -3395,7 +3400,7 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
         // the size the walked groups ask for (the longest walks come first), at
         // least double, within half of the free memory if that is still larger
         int32_t whole = 0;
-        to_host(&whole, rctr.p + 2, 1, s);
+        to_host(&whole, reinterpret_cast<int32_t *>(rctr.p + 2), 1, s);
         const double walked = std::max(1.0, (double)(G - whole));
         double want = std::max(2.0 * (double)pool_cap,
                                1.1 * (double)hc[2] * (double)G / walked + 2.0 * (double)tl.warps * POOL_CHUNK);
@@ -4194,7 +4199,7 @@ struct PlanImpl {
     cudaStream_t s0 = 0;
     DBuf<int32_t> order;
     DBuf<unsigned long long> st, ctr;
-    DBuf<int32_t> next_group, spill_cnt, ctl, qctr, ready, igroup, gcount, gfill, deg, rowcur, empty_flag;
+    DBuf<int32_t> next_group, ctl, qctr, ready, igroup, gcount, gfill, deg, rowcur, empty_flag;
     DBuf<int2> stacks;
     DBuf<int4> spill_a, spill_b;
     DBuf<longlong2> cursors;
@@ -4203,6 +4208,7 @@ struct PlanImpl {
     DBuf<int64_t> seg_begin, gbegin, ibeg, iend, sums, row_ptr, rel;
     DBuf<float> dist, big_tmpd;
     DBuf<uint2> pair_e;               // edges of the count pass, for the emit pass (rows of at most 128 floats)
+    DBuf<unsigned long long> spill_cnt;
     DBuf<unsigned long long> pair_n;  // entries reserved
     DBuf<int64_t> big_lens, big_off;
     DBuf<uint64_t> big_k1, big_k2;
@@ -4423,7 +4429,7 @@ PlanImpl *plan_create(int C, const ct_tree *const *trees, const QParams *qps, in
     p.st = DBuf<unsigned long long>(ST_N, s);
     p.ctr = DBuf<unsigned long long>(4, s);
     p.next_group = DBuf<int32_t>(1, s);
-    p.spill_cnt = DBuf<int32_t>(2, s);
+    p.spill_cnt = DBuf<unsigned long long>(2, s);
     p.ctl = DBuf<int32_t>(2, s);
     p.qctr = DBuf<int32_t>(4, s);
     p.empty_flag = DBuf<int32_t>(1, s);
@@ -4647,7 +4653,7 @@ void degrees_noalloc(const ct_tree *t, const QParams &qp, int32_t *degrees, cuda
     int32_t *next_group = (int32_t *)take(sizeof(int32_t));
     int32_t *nitems = (int32_t *)take(sizeof(int32_t));
     constexpr int kSpillCap = 1 << 15;  // ranges of step-limited walks per round (a full buffer only ends the limit)
-    int32_t *spill_cnt = (int32_t *)take(2 * sizeof(int32_t));
+    unsigned long long *spill_cnt = (unsigned long long *)take(2 * sizeof(unsigned long long));
     int4 *const spills[2] = {(int4 *)take(kSpillCap * sizeof(int4)), (int4 *)take(kSpillCap * sizeof(int4))};
     TravLaunch tl = trav_launch_config(true, t->n_groups);
     const size_t stack_per_block = (size_t)TRAV_WARPS * cap * sizeof(int2);

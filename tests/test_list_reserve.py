@@ -1,7 +1,7 @@
 """Room in a list that many warps fill (reserve.cuh), compiled for the host:
-requests whose sum passes 2^31 and other warps that take room in between never
-bring the count past the list's end, and every request that fits is granted.
-CPU only."""
+requests whose sum passes 2^32 are granted while they fit, never point outside
+the list, and leave every entry below its length either stored or marked empty,
+once.  CPU only."""
 import os
 import subprocess
 
@@ -11,41 +11,39 @@ PROGRAM = r"""
 #define CT_HD inline
 #include "reserve.cuh"
 #include <cstdio>
+#include <vector>
 int main() {
-    const int cap = 1 << 20;
-    int count = 0;
-    unsigned long long asked = 0;
-    unsigned r = 12345u;
-    for (int i = 0; i < 300000; ++i) {
-        r = r * 1664525u + 1013904223u;
-        const int n = i % 3 == 0 ? 16384 : (int)(r >> 18);   // 0 .. 16383
-        const int seen = i % 5 ? count : 0;                  // a count read long ago
-        int others = (int)((r >> 8) & 3u);                   // other warps take an entry each first
-        const int before = count;
-        int taken = 0;
-        const int at = ct::list_reserve(seen, n, cap, [&](int expected, int desired) {
-            if (others > 0 && count < cap) { --others; ++count; ++taken; }
-            const int found = count;
-            if (found == expected) count = desired;
-            return found;
-        });
-        asked += (unsigned)n;
-        if (at >= 0 && (at != before + taken || count != at + n)) return 1;
-        if (at < 0 && n <= cap - count) return 2;
-        if (count < 0 || count > cap) return 3;
+    for (int cap : {1, 1000, 1 << 20}) {
+        std::vector<unsigned char> written(cap, 0);
+        unsigned long long count = 0;
+        unsigned r = 12345u;
+        for (int i = 0; i < 600000; ++i) {
+            r = r * 1664525u + 1013904223u;
+            const int n = i % 3 == 0 ? 16384 : (int)(r >> (i % 5 == 1 ? 30 : 18));
+            const ct::ListRoom room = ct::list_room(count, n, cap);
+            if (room.fits != (count + n <= (unsigned long long)cap)) return 1;
+            count += n;
+            if (room.begin < 0 || room.begin > cap) return 2;
+            const int end = room.fits ? room.begin + n : cap;
+            if (end > cap) return 3;
+            for (int k = room.begin; k < end; ++k)
+                if (written[k]++) return 4;
+        }
+        if (count < (1ull << 32)) return 5;
+        if (ct::list_length(count, cap) != cap || ct::list_length(cap - 1, cap) != cap - 1) return 6;
+        for (int k = 0; k < cap; ++k)
+            if (!written[k]) return 7;
     }
-    if (asked < (1ull << 31)) return 4;
-    printf("%d\n", count);
+    puts("ok");
     return 0;
 }
 """
 
 
-def test_count_never_passes_the_end(tmp_path):
+def test_counts_past_32_bits(tmp_path):
     src, exe = tmp_path / "reserve.cpp", tmp_path / "reserve"
     src.write_text(PROGRAM)
     subprocess.run(["g++", "-std=c++17", "-O1", "-I", os.path.join(ROOT, "paper_2510_14147_gb300", "csrc"),
                     "-o", str(exe), str(src)], check=True)
     out = subprocess.run([str(exe)], stdout=subprocess.PIPE)
-    assert out.returncode == 0
-    assert 0 < int(out.stdout) <= 1 << 20
+    assert out.returncode == 0 and out.stdout == b"ok\n"
