@@ -473,7 +473,8 @@ __device__ __forceinline__ bool l2_keep(const TreeView &tv, const float4 *cen, i
 // walk that reached the step limit; the lanes per vertex test follow the
 // cloud's row length.  Walks stop at out.limit steps (no limit without
 // out.items) and store the rest of their stack in `out`.  (Eight blocks an SM
-// leave 64 registers a thread; -Xptxas -v: 4 bytes of them spilled.)
+// leave 64 registers a thread; -Xptxas -v: 124 bytes of them spilled, 100 read
+// back.)
 __global__ void __launch_bounds__(TRAV_WARPS * 32, 8) k_traverse_l2(
     const __grid_constant__ Views V, const int32_t *__restrict__ order, int n_order,
     const int4 *__restrict__ in_items, const unsigned long long *__restrict__ in_count, int in_cap, Spill out, Pool P,
@@ -1056,9 +1057,9 @@ struct PairList {
     unsigned long long *n;      // entries reserved (may exceed cap: the rest was not stored)
     unsigned long long *stat;   // tensor-core filter: valid pairs, kept pairs, rows
 };
-// A warp's part of the list: it reserves L2_CHUNK entries at a time and marks
-// what it leaves of the last ones.
-constexpr int L2_CHUNK = 128;
+// A warp's part of the list: it reserves l2_chunk entries at a time and marks
+// what it leaves of the last ones (k_leaf_l2).
+constexpr int l2_chunk(bool shorts) { return shorts ? 128 : 32; }
 struct PairCursor {
     int64_t cur = 0, lim = 0;
 };
@@ -1069,10 +1070,11 @@ struct PairPlaces {
     int room;
     __device__ __forceinline__ int64_t operator()(int i) const { return i < room ? old + i : nxt + (i - room); }
 };
+template <int CHUNK>
 __device__ __forceinline__ PairPlaces pair_reserve(const PairList &pl, PairCursor &pc, int n) {
     PairPlaces p{pc.cur, 0, (int)(pc.lim - pc.cur)};
     if (n > p.room) {
-        const int more = ((n - p.room + L2_CHUNK - 1) / L2_CHUNK) * L2_CHUNK;
+        const int more = ((n - p.room + CHUNK - 1) / CHUNK) * CHUNK;
         unsigned long long a = 0;
         if ((threadIdx.x & 31) == 0) a = atomicAdd(pl.n, (unsigned long long)more);
         p.nxt = (int64_t)__shfl_sync(0xffffffffu, a, 0);
@@ -1554,7 +1556,8 @@ __device__ __forceinline__ void leaf_l2_item(
                             const int y = __shfl_up_sync(0xffffffffu, incl, o);
                             if (lane >= o) incl += y;
                         }
-                        const PairPlaces place = pair_reserve(pl, pc, __shfl_sync(0xffffffffu, incl, 31));
+                        const PairPlaces place =
+                            pair_reserve<l2_chunk(KS4 == KS_SHORT)>(pl, pc, __shfl_sync(0xffffffffu, incl, 31));
                         uint32_t m = hitrow;
                         for (int i = incl - c; m; ++i) {
                             const int x = __ffs(m) - 1, j = x >> 2;
@@ -1617,11 +1620,14 @@ __device__ __forceinline__ void leaf_l2_item(
     }
 }
 
-// The wave's items, taken dynamically by a grid of resident CTAs (leaf_l2_ctas):
-// a warp's place in the edge list outlives an item.  (With a CTA per item every
-// warp that found an edge left up to 127 entries of its own behind: 240
-// thousand warps of 121k x 16 uniform points asked for 31 M entries to list 2.5
-// M edges, more than the list had.)
+// The wave's items.  Rows of at most 64 floats: taken dynamically by a grid of
+// resident CTAs (leaf_l2_ctas), so that a warp's place in the edge list outlives
+// an item.  (With a CTA per item every warp that found an edge left up to 127
+// entries of its own behind: 240 thousand warps of 121k x 16 uniform points asked
+// for 31 M entries to list 2.5 M edges, more than the list had.)  Longer rows,
+// whose items take longer: a CTA per item, which the hardware schedules better
+// (1M x 128, upper triangle: 91.5 ms, 93.9 with resident CTAs), and reservations
+// of 32 entries (l2_chunk), whose leavings the list has room for.
 // Rows of at most 64 floats take a shorter tile stride and fewer registers, so
 // that five CTAs share an SM instead of three (a tile is a chain of copy,
 // barrier, arithmetic, barrier: more of them in flight; -Xptxas -v: 96
@@ -1631,6 +1637,14 @@ __device__ __forceinline__ void leaf_l2_item(
 // read whatever is broadcast) and the FP32 pipe (58 %).  The emit pass reads
 // the list of edges instead of the blocks' pairs: 4.8 -> 0.8 ms.
 constexpr int leaf_l2_ctas(bool shorts) { return shorts ? 5 : 3; }  // of an SM
+// CTAs of a launch over a wave of at most max_items items, and the list entries
+// that the warps of all waves of a call (two at most) may leave unused.
+int64_t leaf_l2_grid(bool shorts, int64_t max_items) {
+    return shorts ? std::min<int64_t>(max_items, (int64_t)num_sms() * leaf_l2_ctas(true)) : max_items;
+}
+int64_t leaf_l2_slack(bool shorts, int64_t max_items) {
+    return (shorts ? 2 : 1) * leaf_l2_grid(shorts, max_items) * (LEAF_T / 32) * l2_chunk(shorts);
+}
 template <bool EMIT, int KS4>
 __global__ void __launch_bounds__(LEAF_T, leaf_l2_ctas(KS4 == KS_SHORT)) k_leaf_l2(
     const __grid_constant__ Views V, Items items, ItemWave wave, unsigned long long *__restrict__ next,
@@ -1640,16 +1654,26 @@ __global__ void __launch_bounds__(LEAF_T, leaf_l2_ctas(KS4 == KS_SHORT)) k_leaf_
     unsigned long long *__restrict__ st, int32_t *__restrict__ err, CapOut co, const uint8_t *__restrict__ rowsel,
     PairList pl) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int64_t s_it;
+    LeafShared<KS4> &S = *reinterpret_cast<LeafShared<KS4> *>(smem_raw);
     PairCursor pc;
-    for (;;) {
-        __syncthreads();  // the last item is done
-        if (threadIdx.x == 0) s_it = wave.item((int64_t)atomicAdd(next, 1ull));
-        __syncthreads();
-        const int64_t it = s_it;
-        if (it >= *items.count) break;
-        leaf_l2_item<EMIT, KS4>(V, items, (int)it, cand, emask, deg, row_ptr, rowcur, col, dist, st, err, co, rowsel,
-                                pl, pc, *reinterpret_cast<LeafShared<KS4> *>(smem_raw));
+    if constexpr (KS4 == KS_LONG) {
+        // the wave's items from the block index alone (uniform registers): a CTA for every
+        // 32nd item, or for every item but those, which leave at once
+        const int it = (int)blockIdx.x * (wave.sampled == 1 ? WAVE_SAMPLE : 1);
+        if (wave.sampled == 2 && it % WAVE_SAMPLE == 0) return;
+        leaf_l2_item<EMIT, KS4>(V, items, it, cand, emask, deg, row_ptr, rowcur, col, dist, st, err, co, rowsel, pl,
+                                pc, S);
+    } else {
+        __shared__ int64_t s_it;
+        for (;;) {
+            __syncthreads();  // the last item is done
+            if (threadIdx.x == 0) s_it = wave.item((int64_t)atomicAdd(next, 1ull));
+            __syncthreads();
+            const int64_t it = s_it;
+            if (it >= *items.count) break;
+            leaf_l2_item<EMIT, KS4>(V, items, (int)it, cand, emask, deg, row_ptr, rowcur, col, dist, st, err, co,
+                                    rowsel, pl, pc, S);
+        }
     }
     if (!EMIT && pl.e) pair_close(pl, pc);
 }
@@ -3545,7 +3569,7 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
         if (l2) {
             leaf_l2_prepare();
             const bool sh = short_rows(max_fp_dp);
-            const int ctas = (int)std::min<int64_t>(max_items, (int64_t)num_sms() * leaf_l2_ctas(sh));
+            const unsigned ctas = (unsigned)leaf_l2_grid(sh, wave.sampled == 1 ? ceil_div(max_items, WAVE_SAMPLE) : max_items);
             unsigned long long *const next = fp_ctr.p + fp_launches++;
             auto go = [&](auto kern) {
                 kern<<<ctas, LEAF_T, leaf_smem(sh), s>>>(V, items, wave, next, cand_p, emask.p, deg.p, row_ptr, rowcur.p, col, dist, st.p, err, cw, rowsel, emit ? PairList{} : fp_list);
@@ -3719,9 +3743,10 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
     // only those again instead of every pair of an edge-bearing block and query.
     // The list holds 192 edges per point at most, within an eighth of the free
     // memory (a denser graph's emit pass takes the blocks' masks).  Where that is
-    // more than 1 GB (700 thousand points), every 32nd item is counted first and
+    // more than 2 GB (1.4 million points), every 32nd item is counted first and
     // its edges size the list, with half as much again to spare; a sample of
-    // fewer points does not fill the chip (130k x 3 at 64 MB: 3.00 -> 3.19 ms).
+    // fewer points does not fill the chip (with a line at 64 MB, 130k x 3: 3.00 ->
+    // 3.19 ms; at 1 GB, 1M x 128: 91.3 -> 92.2).
     // The list is no condition: without the memory for it, or when it runs out,
     // the emit pass takes the masks.
     auto count_other = [&](const Items &items) {
@@ -3729,9 +3754,7 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
         const ItemWave every{0, 0, 1};
         auto count = [&](const ItemWave &w) { leaf(false, nullptr, nullptr, nullptr, nullptr, items, w); };
         if (!l2 || capmode || probe || max_fp_dp > 128 || n == 0) return count(every);
-        // entries that the warps of two launches leave unused
-        const int64_t slack =
-            2 * std::min<int64_t>(max_items, (int64_t)num_sms() * leaf_l2_ctas(short_rows(max_fp_dp))) * (LEAF_T / 32) * L2_CHUNK;
+        const int64_t slack = leaf_l2_slack(short_rows(max_fp_dp), max_items);
         int64_t most = 192 * n + slack;
         size_t fr = 0, tot = 0;
         if (cudaMemGetInfo(&fr, &tot) == cudaSuccess) most = std::min(most, (int64_t)(fr / 8 / sizeof(uint2)));
@@ -3749,7 +3772,7 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
             fp_e = std::move(e);
             fp_list = fp_e.p ? PairList{fp_e.p, cap, fp_n, nullptr} : PairList{};
         };
-        if (most <= (1ll << 30) / (int64_t)sizeof(uint2)) {
+        if (most <= (2ll << 30) / (int64_t)sizeof(uint2)) {
             room(most, 0);
             return count(every);
         }
@@ -4491,7 +4514,7 @@ PlanImpl *plan_create(int C, const ct_tree *const *trees, const QParams *qps, in
         p.pair_n = DBuf<unsigned long long>(1, s);
         if (p.max_dp <= 128) {  // the edges, and what each warp leaves of its last entries; without room, none
             try {
-                p.pair_e = DBuf<uint2>((size_t)(p.nnz_cap + (int64_t)p.leaf_grid * (LEAF_T / 32) * L2_CHUNK), s);
+                p.pair_e = DBuf<uint2>((size_t)(p.nnz_cap + (int64_t)p.leaf_grid * (LEAF_T / 32) * l2_chunk(sh)), s);
             } catch (const Error &x) {
                 if (x.st != CT_ENOMEM) throw;
             }
@@ -4733,7 +4756,7 @@ void degrees_noalloc(const ct_tree *t, const QParams &qp, int32_t *degrees, cuda
         leaf_l2_prepare();
         CT_CHECK_CUDA(cudaMemsetAsync(ctr, 0, sizeof(unsigned long long), s));  // the walk's counters have been read
         auto go = [&](auto kern, bool sh) {
-            const int ctas = (int)std::min<int64_t>(max_items, (int64_t)num_sms() * leaf_l2_ctas(sh));
+            const unsigned ctas = (unsigned)leaf_l2_grid(sh, max_items);
             kern<<<ctas, LEAF_T, leaf_smem(sh), s>>>(V, items, ItemWave{0, 0, 1}, ctr, pool, nullptr, degrees, nullptr,
                                                      nullptr, nullptr, nullptr, st, err, CapOut{}, nullptr,
                                                      PairList{});

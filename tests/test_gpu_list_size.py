@@ -1,4 +1,4 @@
-"""The FP32 edge list where it is sized from a sample (above 700 thousand points), where
+"""The FP32 edge list where it is sized from a sample (above 1.4 million points), where
 there are many work items of few edges each, and where there is no memory for
 it: the list is used (the emit pass decides its entries alone) or the block
 masks are, and the graph is the same."""
@@ -48,7 +48,7 @@ def _both(t, eps, **kw):
     return got.nnz, got.stats()["emit_pairs"]
 
 
-@pytest.mark.parametrize("n,dim,degree", [(720001, 3, 30), (710001, 64, 12), (705001, 100, 8)])
+@pytest.mark.parametrize("n,dim,degree", [(1420001, 3, 20), (1410001, 61, 8), (1405001, 66, 6)])
 @pytest.mark.parametrize("upper", [False, True])
 def test_list_sized_from_a_sample(n, dim, degree, upper):
     x = I.gmm_embedded(n, dim=dim, intrinsic=min(dim, 5), n_centres=60, seed=n)
@@ -61,19 +61,21 @@ def test_list_sized_from_a_sample(n, dim, degree, upper):
 
 def test_list_of_a_dense_graph():
     # more than 192 edges a point (as a sample sees, or as the count pass finds): masks
-    for n in (60001, 720001):
+    for n in (60001, 1420001):
         x = I.uniform_cube(n, 3, seed=n)
         nnz, emitted = _both(_tree(x), float((270 / n / 4.18879) ** (1 / 3)))
         assert nnz > 200 * n and emitted > nnz
 
 
-def test_many_items_with_few_edges():
-    x = I.uniform_cube(100001, 16, seed=3)
+@pytest.mark.parametrize("dim", [16, 68])
+def test_many_items_with_few_edges(dim):
+    x = np.zeros((100001, dim), np.float32)  # 16 coordinates: the same items for both kernels
+    x[:, :16] = I.uniform_cube(100001, 16, seed=3)
     nnz, emitted = _both(_tree(x), 0.75)
     assert emitted == nnz
 
 
-@pytest.mark.parametrize("n", [3000, 720001])
+@pytest.mark.parametrize("n", [3000, 1420001])
 def test_without_memory_for_the_list(n):
     """Each allocation of the call fails in turn: the call either fails with
     CT_ENOMEM or, when the list's failed, gives the graph without it."""
