@@ -107,7 +107,10 @@ typedef struct {
  *                     `predictor` (a fitted ct_predictor on the tree's
  *                     device); entries past a row's capacity go to an
  *                     overflow arena, rows that overflow the arena too are
- *                     emitted again exactly.  Same output.
+ *                     emitted again exactly.  Same output.  It saves the
+ *                     second decision of the tensor-core form's kept pairs;
+ *                     with precision 0 it is the faster one at hundreds of
+ *                     neighbours only.
  *  include_self:  1 adds the pair (i, i) to every row (d(p, p) = 0 <= eps).
  *  upper_triangle: 1 evaluates each pair of points of two different query
  *                 groups once, from the group that comes first in tree

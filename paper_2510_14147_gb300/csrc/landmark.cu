@@ -44,7 +44,8 @@ struct LmInput {
 
 // Lemma 1's ghost test of point p (nearest-centre distance dmin) for cell k:
 // exact for Hamming (integers); for L2 with a relative margin of 2^-10 over
-// fp32 distances whose error is below 2^-17 (more ghosts never change rows).
+// fp32 distances whose error is below 2^-12 (a row's terms in one chain, up to
+// 4096 of them; more ghosts never change rows).
 __device__ __forceinline__ bool lm_ghost(const LmInput &in, float d, float dmin, float eps_up, int lev_k) {
     if (in.metric == CT_HAMMING_B1) return d <= dmin + 2.0f * (float)lev_k;
     return d <= fmaf(dmin + eps_up, 1.0f + 0x1p-10f, eps_up) + 0x1p-60f;

@@ -91,7 +91,8 @@ __device__ __forceinline__ bool ft_wait(FtShared &S, uint64_t *bar, uint32_t par
 // Every wait is bounded; a wait that gives up ends all roles (CT_ETIMEOUT).
 // 290 M candidate rows of 128 floats (2.2 M tiles): 7.5 ms, about 980 clocks a
 // tile and SM, of which the epilogue's warps are busy 650 and the producers'
-// 800; 292 M rows of 16 floats: 6.3 ms.
+// 800; 292 M rows of 16 floats: 6.3 ms.  (28 warps leave 72 registers a thread;
+// -Xptxas -v: 28 bytes of them spilled, 32 read back.)
 __global__ void __launch_bounds__(FT_T, 1) k_filter_tc(const __grid_constant__ Views V, Items items,
                                                        ItemWave wave, const uint32_t *__restrict__ cand, PairList out,
                                                        unsigned long long *__restrict__ next,

@@ -1,7 +1,9 @@
 // tc.cuh -- fifth-generation tensor core (tcgen05) primitives for sm_100+:
-// tensor-memory allocation, shared-memory operand descriptors, the BF16 MMA
+// tensor-memory allocation, shared-memory operand descriptors, the 16-bit MMA
 // with FP32 accumulation in tensor memory, commit to an mbarrier, and loads of
-// the accumulator back into registers.  All waits are bounded.
+// the accumulator back into registers.  All waits are bounded.  The filter
+// (leaf_tc.cuh) uses fp16 operands in the 128-byte-swizzled layout; BF16 and
+// the layout without swizzle serve the self-test of tc.cu alone.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -12,7 +14,7 @@ namespace tc {
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-// Operand tiles are K-major without swizzle: element (r, k) of a tile with 8-row
+// The self-test's BF16 operand tiles are K-major without swizzle: element (r, k) of a tile with 8-row
 // groups sits at byte  (r / 8) * SBO + (k / 8) * LBO + (r % 8) * 16 + (k % 8) * 2
 // (8 x 16-byte core matrices).  Rows are 128 bf16 (256 bytes) here, so one row
 // group spans 16 core matrices: LBO = 128, SBO = 2048.
