@@ -821,15 +821,17 @@ __global__ void __launch_bounds__(LEV_C) k_net_pairs_lev(Strings S, const int32_
 __global__ void __launch_bounds__(128) k_net_pick_lev(const int2 *__restrict__ hlist, Hubs hb, Batch bt, LevCands lc,
                                                       int mcap, int chunk_len, int32_t *__restrict__ active) {
     __shared__ float cd[LEV_C];
-    __shared__ uint16_t pd[LEV_C * LEV_C];
+    __shared__ __align__(4) uint16_t pd[LEV_C * LEV_C];
     __shared__ int picks[NET_M];
     const int2 hs = hlist[blockIdx.x];
     const int h = hs.x;
     if (hb.done[h]) return;
     const int n = lc.n[blockIdx.x], b = hb.begin[h], nc = hb.nc[h], K = lev_most_cands(hb.count[h], chunk_len);
     for (int i = threadIdx.x; i < n; i += blockDim.x) cd[i] = lc.d[b + i];
-    for (int i = threadIdx.x; i < n * K; i += blockDim.x)  // rows below n (entries at and past n are not read)
-        pd[i] = lc.pair[(size_t)b * LEV_PAIR_PP + i];
+    // rows below n, two entries at a time (those at and past n, and one past an odd end, are not read)
+    const uint32_t *pair = reinterpret_cast<const uint32_t *>(lc.pair + (size_t)b * LEV_PAIR_PP);
+#pragma unroll 4
+    for (int i = threadIdx.x; i < (n * K + 1) >> 1; i += 128) reinterpret_cast<uint32_t *>(pd)[i] = pair[i];
     __syncthreads();
     if (threadIdx.x >= 32) return;
     const int m = n ? net_greedy<LEV_C>(cd, n, hb.thr[h], mcap, picks,

@@ -3551,7 +3551,7 @@ void query_multi(int C, const ct_tree *const *trees, const QParams *qps, cudaStr
 
     // counters of the FP32 leaf launches, each used once (count: one or two; emit; rows emitted again)
     DBuf<unsigned long long> fp_ctr(8, s);
-    if (l2) CT_CHECK_CUDA(cudaMemsetAsync(fp_ctr.p, 0, 8 * sizeof(unsigned long long), s));
+    if (any_fp) CT_CHECK_CUDA(cudaMemsetAsync(fp_ctr.p, 0, 8 * sizeof(unsigned long long), s));
     int fp_launches = 0;
     unsigned long long *const fp_n = fp_ctr.p + 7;  // entries of the edge list
     DBuf<uint2> fp_e;

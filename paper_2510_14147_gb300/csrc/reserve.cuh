@@ -13,7 +13,7 @@ namespace ct {
 // some hundred thousand such walks wrap a 32-bit count, after which the stores
 // go before the list.  A compare-and-swap that leaves the count alone when the
 // entries do not fit is no way out: many walks stop at the same time, and the
-// walk of 121k x 16 uniform points took 6.6 ms instead of 3.0.)
+// walk of a million 256-bit codes took 11.2 ms instead of 5.1.)
 struct ListRoom {
     int begin;  // the first entry, cap if there is none
     bool fits;  // all the entries have room; else those from begin on are marked empty
