@@ -1632,7 +1632,7 @@ __device__ __forceinline__ void leaf_l2_item(
 // that five CTAs share an SM instead of three (a tile is a chain of copy,
 // barrier, arithmetic, barrier: more of them in flight; -Xptxas -v: 96
 // registers, the count form spills 32 bytes of them and reads 28 back).
-// 174k x 64 at 87 neighbours: count 16.3 -> 14.1 ms, bound by the shared-memory
+// 174k x 64 at 87 neighbours: count 16.3 -> 13.7 ms, bound by the shared-memory
 // reads of the micro-tiles (71 % of that pipe, four wavefronts per 16-byte
 // read whatever is broadcast) and the FP32 pipe (58 %).  The emit pass reads
 // the list of edges instead of the blocks' pairs: 4.8 -> 0.8 ms.
